@@ -1,10 +1,14 @@
 // CSR utilities of the sign solver: validation, the reproducible 1-norm and
 // scaling of step a1, prefix scans, block-diagonal assembly of batches and
 // deterministic per-matrix reductions.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 
 #include "common.cuh"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace sgn {
 
@@ -317,6 +321,13 @@ __global__ void k_fill_seg(int nb, const int64_t *moff, int64_t n, int32_t *seg)
 // the largest one, hi * 2^64 + lo, comes back as
 // ((double)hi * 2^64 + (double)lo) * 2^(e-62).
 
+// *p = max(*p, v). The value is read first: it only grows, so an entry at or
+// below it needs no atomic. A large matrix's rows otherwise queue on one
+// address (262144 rows: about 170 us for each of the three maxima).
+__device__ __forceinline__ void max_into(unsigned long long *p, unsigned long long v) {
+  if (*reinterpret_cast<volatile unsigned long long *>(p) < v) atomicMax(p, v);
+}
+
 __device__ __forceinline__ void add128(unsigned long long *lohi, unsigned long long q) {
   unsigned long long old = atomicAdd(&lohi[0], q);
   if (old + q < old) atomicAdd(&lohi[1], 1ULL);
@@ -331,7 +342,7 @@ __global__ void k_absmax(int64_t n, const int32_t *seg, const int64_t *rp, const
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o, 8));
     if (has && gl == 0 && m > 0.0)
-      atomicMax(&mmax[seg[r]], (unsigned long long)__double_as_longlong(m));
+      max_into(&mmax[seg[r]], (unsigned long long)__double_as_longlong(m));
   });
 }
 
@@ -355,14 +366,14 @@ __global__ void k_colmax_hi(int64_t n, const int32_t *seg, const unsigned long l
                             unsigned long long *maxhi) {
   for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
        j += int64_t(gridDim.x) * blockDim.x)
-    if (colsum[2 * j] | colsum[2 * j + 1]) atomicMax(&maxhi[seg[j]], colsum[2 * j + 1]);
+    if (colsum[2 * j] | colsum[2 * j + 1]) max_into(&maxhi[seg[j]], colsum[2 * j + 1]);
 }
 
 __global__ void k_colmax_lo(int64_t n, const int32_t *seg, const unsigned long long *colsum,
                             const unsigned long long *maxhi, unsigned long long *maxlo) {
   for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
        j += int64_t(gridDim.x) * blockDim.x)
-    if (colsum[2 * j + 1] == maxhi[seg[j]]) atomicMax(&maxlo[seg[j]], colsum[2 * j]);
+    if (colsum[2 * j + 1] == maxhi[seg[j]]) max_into(&maxlo[seg[j]], colsum[2 * j]);
 }
 
 __global__ void k_norm_final(int nb, const unsigned long long *mmax,
@@ -397,39 +408,68 @@ __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp,
 }
 
 // ------------------------------------------------------------ reductions
-constexpr int RED_T = 256;
-__global__ void __launch_bounds__(RED_T) k_seg_reduce(const int64_t *moff, const double *part,
-                                                      int ncomp, double *out) {
-  __shared__ double sm[RED_T];
-  int m = blockIdx.x;
-  int64_t b = moff[m], e = moff[m + 1];
-  for (int c = 0; c < ncomp; ++c) {
-    double acc = 0.0;
-    for (int64_t r = b + threadIdx.x; r < e; r += RED_T) acc += part[r * ncomp + c];
-    sm[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = RED_T / 2; s > 0; s >>= 1) {
-      if (threadIdx.x < s) sm[threadIdx.x] += sm[threadIdx.x + s];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[int64_t(m) * ncomp + c] = sm[0];
-    __syncthreads();
+// Sums per matrix. A matrix is served by a cluster of RED_C CTAs: with one CTA
+// a matrix of 262144 rows took 232 us per sum of two components and 267 us
+// per count (one SM's FP64 pipe and load latency bound it). With the clusters
+// and the 1-norm's maxima below, the mixed solve of the tridiagonal matrix of
+// that order went from 16.3 to 11.9 ms (GB300).
+constexpr int RED_T = 256;  // partial sums per component; their order is fixed
+constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
+constexpr int RED_LANES = RED_T / RED_C;
+constexpr int RED_U = 8;    // rows loaded at once
+static_assert(RED_LANES == 32, "one warp of each CTA per component");
+
+// Component c = threadIdx.y of matrix m: partial sum t (0 <= t < RED_T) adds
+// rows t, t + RED_T, ... one after another, and the partial sums are added
+// pairwise, t + s into t for s = RED_T / 2 .. 1. CTA q of the cluster holds the
+// partial sums 32 q .. 32 q + 31, a warp per component, so the FP64 additions
+// spread over RED_C SMs and the result does not depend on the split.
+__global__ void __cluster_dims__(RED_C, 1, 1)
+    k_seg_reduce(const int64_t *moff, const double *part, int ncomp, double *out) {
+  __shared__ double sm[2][RED_T];
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
+  const int c = threadIdx.y, t = q * RED_LANES + threadIdx.x;
+  cl.sync();  // CTA 0 has started: its shared memory may be written
+  const int64_t e = moff[m + 1];
+  double acc = 0.0;
+  int64_t r = moff[m] + t;
+  for (; r + (RED_U - 1) * RED_T < e; r += RED_U * RED_T) {
+    double v[RED_U];
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u) v[u] = part[(r + u * RED_T) * ncomp + c];
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u) acc += v[u];
   }
+  for (; r < e; r += RED_T) acc += part[r * ncomp + c];
+  *cl.map_shared_rank(&sm[c][t], 0) = acc;
+  cl.sync();
+  if (q != 0) return;
+  for (int s = RED_T / 2; s > 0; s >>= 1) {
+    for (int i = threadIdx.x; i < s; i += RED_LANES) sm[c][i] += sm[c][i + s];
+    __syncwarp();
+  }
+  if (threadIdx.x == 0) out[int64_t(m) * ncomp + c] = sm[c][0];
 }
 
-__global__ void __launch_bounds__(RED_T) k_seg_count(const int64_t *moff, const int64_t *rs,
-                                                     const int64_t *re, int64_t *out) {
-  __shared__ int64_t sm[RED_T];
-  int m = blockIdx.x;
-  int64_t acc = 0;
-  for (int64_t r = moff[m] + threadIdx.x; r < moff[m + 1]; r += RED_T) acc += re[r] - rs[r];
-  sm[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = RED_T / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sm[threadIdx.x] += sm[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[m] = sm[0];
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
+    k_seg_count(const int64_t *moff, const int64_t *rs, const int64_t *re, int64_t *out) {
+  __shared__ unsigned long long sm;  // CTA 0: the matrix's count
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
+  if (threadIdx.x == 0) sm = 0ULL;
+  cl.sync();
+  long long acc = 0;
+  const int64_t e = moff[m + 1];
+#pragma unroll 4
+  for (int64_t r = moff[m] + q * RED_T + threadIdx.x; r < e; r += RED_C * RED_T)
+    acc += re[r] - rs[r];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane_id() == 0 && acc)
+    atomicAdd(cl.map_shared_rank(&sm, 0), (unsigned long long)acc);
+  cl.sync();
+  if (q == 0 && threadIdx.x == 0) out[m] = int64_t(sm);
 }
 
 // One CTA per extracted matrix: rebased row pointers, shifted columns,
@@ -494,7 +534,7 @@ void launch_compact_rows(int64_t n, const int64_t *rs, const int64_t *re, const 
 void launch_seg_count(int nb, const int64_t *moff, const int64_t *rs, const int64_t *re,
                       int64_t *out, cudaStream_t s) {
   if (nb == 0) return;
-  k_seg_count<<<nb, RED_T, 0, s>>>(moff, rs, re, out);
+  k_seg_count<<<unsigned(nb) * RED_C, RED_T, 0, s>>>(moff, rs, re, out);
   SGN_LAUNCH_CHECK();
 }
 
@@ -609,7 +649,8 @@ void launch_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64
 void launch_seg_reduce(int nb, const int64_t *moff, const double *part, int ncomp, double *out,
                        cudaStream_t s) {
   if (nb == 0) return;
-  k_seg_reduce<<<nb, RED_T, 0, s>>>(moff, part, ncomp, out);
+  k_seg_reduce<<<unsigned(nb) * RED_C, dim3(RED_LANES, unsigned(ncomp)), 0, s>>>(moff, part, ncomp,
+                                                                             out);
   SGN_LAUNCH_CHECK();
 }
 
