@@ -13,29 +13,38 @@
 //
 // Products. For a digit pair (s, t) the tensor cores form the integer matrix
 // D_s E_t^T with FP32 accumulation: each product is at most 64 * 64 = 2^12 in
-// magnitude and K is taken in blocks of at most 4096, so every partial sum of
-// a block is an integer of magnitude at most 2^24 and its accumulation is
-// exact in any order. The epilogue adds, block by block,
-//   C_ij += (D_s E_t^T)_ij * 2^(e_i + 1) 2^(f_j + 1) 2^(-7 (s + t))
-// in FP64: the scale is a power of two, so each term is exact and is built
-// from the FP32 bits with integer operations; one FP64 addition per term.
-// The pairs with s + t <= 9 (36 of the 64) are kept, in the order of
-// increasing weight; the dropped ones and the rounding of the inputs to the
-// 2^-55 grid stay below 2^-41 * 2^(e_i + f_j) * K / 4096 in the worst case
-// (digits of equal sign), about the error bound of an FP64 dot product; the
-// FP64 sums of the blocks add their own rounding.
+// magnitude, so an accumulator that takes at most 4096 products per entry, of
+// one pair or of several of the same level s + t, only ever holds integers of
+// magnitude at most 2^24 and is exact in any order. The pairs with s + t <= 9
+// (36 of the 64) are kept; the dropped ones and the rounding of the inputs to
+// the 2^-55 grid stay below 2^-41 * 2^(e_i + f_j) * K / 4096 in the worst case
+// (digits of equal sign), about the error bound of an FP64 dot product.
+// The levels 9 .. 4 of a K block are added as 64-bit integers,
+//   L = sum_{l=4..9} 2^(7 (9 - l)) sum_{s+t=l} D_s E_t^T   (|L| < 2^62),
+// the levels 3 and 2 likewise as H, and the block's product is
+//   2^(e_i + f_j + 2) (2^-63 L + 2^-21 H),
+// two integers converted to FP64 and one or two FP64 additions per entry;
+// later blocks are added in FP64.
 //
 // Kernel: persistent, one CTA per SM, 320 threads, laid out as the
 // split-TF32 kernel but with eight epilogue warps (two per 32 TMEM lanes,
-// one per half of the columns). A work unit is one 128 x 256 tile of C; its
-// CTA runs the (digit pair, K block) steps one after another, each a K loop
-// into one of two 256-column TMEM accumulators, so that the epilogue warps add
-// step u into C while the MMAs of step u + 1 run. A thread's loads of C for a
-// 32-column chunk are all issued before its stores, to keep them in flight
-// together. The producer thread streams 32-wide K slices of the pair's A and
-// Bt digits with TMA into an eight-stage ring (64-byte swizzle); the MMA
-// thread issues two kind::f16 (BF16) MMAs per stage. Every wait has a clock
-// budget, as in the split-TF32 kernel.
+// one per half of the columns). A work unit is one 128 x 256 tile of C. Its
+// pairs are taken two levels at a time, (8, 9), (6, 7), (4, 5), (2, 3): step t
+// of the levels (l, l + 1) multiplies the digit planes A_(l-t) and A_(l+1-t)
+// by the same B_t into the two 256-column TMEM accumulators, one per level.
+// The producer thread streams 32-wide K slices of the three planes with TMA
+// into a six-stage ring (64-byte swizzle); the MMA thread issues two kind::f16
+// (BF16) MMAs per accumulator and stage. Steps share an accumulator while its
+// products stay within 4096 per entry (all of a level for K <= 512, one step
+// for K > 2048); then the epilogue warps drain both accumulators into the
+// CTA's tile of integers (global scratch, 256 KB, stays in L2).
+// What bounds it: the tensor pipe and, behind it, the L2 reads of the operand
+// planes, 16 KB per pair and slice here against 24 KB when every pair loads
+// its own two planes, and the FP64 pipe (16 cycles per warp instruction) when
+// every pair is added into C in FP64, as an earlier form did: 6.07 ms at
+// 4096^3 and 3.69 ms at 2744^3 (GB300), now 4.16 and 2.31 ms (1.19 PFLOP/s on
+// the tensor pipe at 4096^3; 512 tiles are 3.4 waves of 152 CTAs).
+// Every wait has a clock budget, as in the split-TF32 kernel.
 #include <stdint.h>
 
 #include <algorithm>
@@ -55,50 +64,42 @@ using namespace tc;
 constexpr int XM = 128;    // tile rows (UMMA M)
 constexpr int XN = 256;    // tile columns (UMMA N)
 constexpr int XK = 32;     // K slice per stage: 32 BF16 = 64 bytes = one swizzle span
-constexpr int XSTAGE = 8;  // ring of stages
+constexpr int XSTAGE = 6;  // ring of stages
 constexpr int XSPAN = XK * 2;
 constexpr int XA_BYTES = XM * XK * 2;  // 8 KB
 constexpr int XB_BYTES = XN * XK * 2;  // 16 KB
-constexpr int XSTAGE_BYTES = XA_BYTES + XB_BYTES;
+constexpr int XSTAGE_BYTES = 2 * XA_BYTES + XB_BYTES;  // A_(l-t), A_(l+1-t), B_t
 constexpr int XTHREADS = 320;  // producer, MMA, eight epilogue warps
 constexpr uint32_t XTMEM_COLS = 2 * XN;
 constexpr int XSMEM = XSTAGE * XSTAGE_BYTES + 1024;  // ring and alignment slack
 constexpr int DIGIT_BITS = 7;
-constexpr int MAX_LEVEL = F64X_DIGITS + 1;  // pairs with s + t <= MAX_LEVEL
 constexpr int KBLK = F64X_MAX_K / XK;       // K stages per exact block (integer sums <= 2^24)
+// Level pairs (l, l + 1), l = 8, 6, 4, 2: the pairs with s + t <= 9 and 8 digits.
+constexpr int XLP = 4;
+static_assert(F64X_DIGITS == 8 && DIGIT_BITS == 7, "level pairs (8, 9) .. (2, 3) of 8 digits");
+__host__ __device__ constexpr int lower_level(int lp) { return 8 - 2 * lp; }
+constexpr int XPAIRS = 36;  // sum over the level pairs of (l - 1) + l
+// the CTA's integer tile: 32-column chunks of a warp, column by column
+constexpr size_t XTILE_BYTES = size_t(XM) * XN * sizeof(long long);
 
-// The kept digit pairs, smallest weight first: s + t from MAX_LEVEL down to 2.
-struct PairList {
-  int n;
-  unsigned char s[F64X_DIGITS * F64X_DIGITS], t[F64X_DIGITS * F64X_DIGITS];
-};
-constexpr PairList make_pairs() {
-  PairList p{};
-  p.n = 0;
-  for (int lv = MAX_LEVEL; lv >= 2; --lv)
-    for (int s = 1; s <= F64X_DIGITS; ++s) {
-      int t = lv - s;
-      if (t >= 1 && t <= F64X_DIGITS) {
-        p.s[p.n] = (unsigned char)s;
-        p.t[p.n] = (unsigned char)t;
-        ++p.n;
-      }
-    }
-  return p;
-}
-constexpr PairList kPairs = make_pairs();
-__constant__ PairList c_pairs = kPairs;
-
-// v 2^sc as an FP64 value, built from the bits of the FP32 integer v (exact):
-// the epilogue then spends one FP64 addition per term, GB300's FP64 pipe
-// being the scarce unit there. Falls back to ldexp outside the normal range.
-__device__ __forceinline__ double exact_scaled(float v, int sc) {
-  const uint32_t b = __float_as_uint(v);
-  if ((b & 0x7FFFFFFFu) == 0u) return 0.0;
-  const int e = int((b >> 23) & 0xFFu) - 127 + sc + 1023;
-  if (e <= 0 || e >= 2047) return ldexp(double(v), sc);
+// v 2^sc as an FP64 value, rounded to nearest: built with integer operations,
+// the FP64 pipe being the scarce unit. Falls back to ldexp outside the
+// normal range.
+__device__ __forceinline__ double scaled_int(long long v, int sc) {
+  if (v == 0) return 0.0;
+  const unsigned long long a = v < 0 ? 0ULL - (unsigned long long)v : (unsigned long long)v;
+  const int z = __clzll((long long)a);
+  const unsigned long long m = a << z;  // top bit set
+  const int e = 63 - z + sc + 1022;     // biased exponent less one (the top bit adds one)
+  if (e < 0 || e >= 2045) return ldexp(double(v), sc);
+  const unsigned long long mant = (m >> 11) + ((m >> 10) & 1ULL);
   return __longlong_as_double(
-      (long long)((uint64_t(b >> 31) << 63) | (uint64_t(e) << 52) | (uint64_t(b & 0x7FFFFFu) << 29)));
+      (long long)((((unsigned long long)e << 52) + mant) | (v < 0 ? 1ULL << 63 : 0ULL)));
+}
+
+// The exact integers of an FP32 accumulator.
+__device__ __forceinline__ long long acc_int(uint32_t bits) {
+  return (long long)__float2int_rn(__uint_as_float(bits));
 }
 
 // Tile t of the launch -> job and tile origin (m0, n0); M blocks run fastest.
@@ -117,27 +118,25 @@ __device__ __forceinline__ void xtile_of(int t, const SliceJob *jobs, const int 
 }
 
 // maps[2 j]: the digits of A of job j as one (8 M) x K array, maps[2 j + 1]
-// those of Bt as (8 N) x K; digit s of row r is row (s - 1) rows + r.
+// those of Bt as (8 N) x K; digit s of row r is row (s - 1) rows + r. tiles: one
+// integer tile per CTA.
 __global__ void __launch_bounds__(XTHREADS, 1)
     k_gemm_slices(const SliceJob *jobs, const CUtensorMap *maps, const int *tile_start,
-                  int njobs, int ntiles, int *err) {
+                  int njobs, int ntiles, long long *tiles, int *err) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t full[XSTAGE], empty[XSTAGE], tfull[2], tempty[2], done;
+  __shared__ __align__(8) uint64_t full[XSTAGE], empty[XSTAGE], tfull, tempty, done;
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort, s_consumed;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   volatile int *abort = &s_abort;
-  const int npairs = c_pairs.n;
   if (tid == 0) {
     for (int i = 0; i < XSTAGE; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 8);
-    }
+    mbar_init(&tfull, 1);
+    mbar_init(&tempty, 8);
     mbar_init(&done, 1);
     s_abort = 0;
     s_consumed = 0;
@@ -160,17 +159,25 @@ __global__ void __launch_bounds__(XTHREADS, 1)
         xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
         const SliceJob &J = jobs[j];
         const CUtensorMap *mp = maps + 2 * j;
-        const int nk = (J.K + XK - 1) / XK, nblk = (nk + KBLK - 1) / KBLK;
-        for (int u = 0; u < npairs * nblk && !*abort; ++u) {
-          const int p = u / nblk, k0 = (u % nblk) * KBLK, k1 = min(nk, k0 + KBLK);
-          const int ya = (c_pairs.s[p] - 1) * J.M + m0, yb = (c_pairs.t[p] - 1) * J.N + n0;
-          for (int kb = k0; kb < k1; ++kb, ++issued) {
-            const int st = issued % XSTAGE;
-            if (!bounded_wait(&empty[st], ((issued / XSTAGE) & 1) ^ 1, abort)) break;
-            const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
-            mbar_expect_tx(&full[st], XSTAGE_BYTES);
-            tma_load_2d(d, mp + 0, kb * XK, ya, &full[st]);
-            tma_load_2d(d + XA_BYTES, mp + 1, kb * XK, yb, &full[st]);
+        const int nk = (J.K + XK - 1) / XK;
+        for (int k0 = 0; k0 < nk && !*abort; k0 += KBLK) {
+          const int k1 = min(nk, k0 + KBLK);
+          for (int lp = 0; lp < XLP && !*abort; ++lp) {
+            const int l = lower_level(lp);
+            for (int t2 = 1; t2 <= l && !*abort; ++t2) {
+              const bool both = t2 < l;  // step l has no pair of level l
+              const int y0 = (l - t2 - 1) * J.M + m0, y1 = (l - t2) * J.M + m0;
+              const int yb = (t2 - 1) * J.N + n0;
+              for (int kb = k0; kb < k1; ++kb, ++issued) {
+                const int st = issued % XSTAGE;
+                if (!bounded_wait(&empty[st], ((issued / XSTAGE) & 1) ^ 1, abort)) break;
+                const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
+                mbar_expect_tx(&full[st], both ? XSTAGE_BYTES : XSTAGE_BYTES - XA_BYTES);
+                if (both) tma_load_2d(d, mp + 0, kb * XK, y0, &full[st]);
+                tma_load_2d(d + XA_BYTES, mp + 0, kb * XK, y1, &full[st]);
+                tma_load_2d(d + 2 * XA_BYTES, mp + 1, kb * XK, yb, &full[st]);
+              }
+            }
           }
         }
       }
@@ -178,40 +185,51 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(XM, XN);
-      int it = 0, uc = 0;  // stages consumed, units (tile, pair) done
+      int it = 0, uc = 0;  // stages consumed, accumulations (both accumulators) done
       bool any = false, ok = true;
       for (int t = blockIdx.x; t < ntiles && ok && !*abort; t += gridDim.x) {
         int j, m0, n0;
         xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
-        const int nk = (jobs[j].K + XK - 1) / XK, nblk = (nk + KBLK - 1) / KBLK;
-        for (int u = 0; u < npairs * nblk && ok; ++u, ++uc) {
-          const int k0 = (u % nblk) * KBLK, k1 = min(nk, k0 + KBLK);
-          const int a = uc & 1;
-          if (!bounded_wait(&tempty[a], ((uc >> 1) & 1) ^ 1, abort)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t acc = tmem + uint32_t(a * XN);
-          for (int kb = k0; kb < k1; ++kb, ++it) {
-            const int st = it % XSTAGE;
-            if (!bounded_wait(&full[st], (it / XSTAGE) & 1, abort)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
+        const int nk = (jobs[j].K + XK - 1) / XK;
+        for (int k0 = 0; k0 < nk && ok; k0 += KBLK) {
+          const int k1 = min(nk, k0 + KBLK), group = KBLK / (k1 - k0);
+          for (int lp = 0; lp < XLP && ok; ++lp) {
+            const int l = lower_level(lp);
+            for (int ta = 1; ta <= l && ok; ta += group, ++uc) {
+              const int tb = min(l, ta + group - 1);  // steps ta .. tb accumulate together
+              if (!bounded_wait(&tempty, (uc & 1) ^ 1, abort)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              for (int t2 = ta; t2 <= tb && ok; ++t2) {
+                const bool both = t2 < l;
+                for (int kb = k0; kb < k1; ++kb, ++it) {
+                  const int st = it % XSTAGE;
+                  if (!bounded_wait(&full[st], (it / XSTAGE) & 1, abort)) {
+                    ok = false;
+                    break;
+                  }
+                  tc_fence_after();
+                  const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
+                  const uint32_t more = t2 > ta || kb > k0 ? 1u : 0u;
 #pragma unroll
-            for (int s = 0; s < XK / 16; ++s) {
-              const uint32_t ko = uint32_t(s) * 32u;
-              mma_bf16(acc, smem_desc_sw<XSPAN>(d + ko), smem_desc_sw<XSPAN>(d + XA_BYTES + ko),
-                       idesc, ((kb - k0) | s) != 0 ? 1u : 0u);
+                  for (int s = 0; s < XK / 16; ++s) {
+                    const uint32_t ko = uint32_t(s) * 32u;
+                    const uint64_t bd = smem_desc_sw<XSPAN>(d + 2 * XA_BYTES + ko);
+                    if (both)
+                      mma_bf16(tmem, smem_desc_sw<XSPAN>(d + ko), bd, idesc, s ? 1u : more);
+                    mma_bf16(tmem + XN, smem_desc_sw<XSPAN>(d + XA_BYTES + ko), bd, idesc,
+                             s ? 1u : more);
+                  }
+                  any = true;
+                  mma_commit(&empty[st]);
+                }
+              }
+              if (!ok) break;
+              mma_commit(&tfull);
             }
-            any = true;
-            mma_commit(&empty[st]);
           }
-          if (!ok) break;
-          mma_commit(&tfull[a]);
         }
       }
       s_consumed = it;
@@ -223,77 +241,109 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   } else {
     const int q = warp & 3;           // this warp's 32 TMEM lanes (rows)
     const int half = (warp - 2) >> 2;  // and its half of the tile's columns
+    // this warp's part of the CTA's integer tile: [chunk][column][lane]
+    long long *const low =
+        tiles + size_t(blockIdx.x) * (XM * XN) + size_t(warp - 2) * (XM * XN / 8) + lane;
+    const uint32_t trow = tmem + (uint32_t(q * 32) << 16);
     int uc = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    bool stop = false;
+    for (int t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
       int j, m0, n0;
       xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
       const SliceJob J = jobs[j];
       const int gr = m0 + q * 32 + lane;
       const int ea = gr < J.M ? J.ea[gr] : 0;
-      const int nk = (J.K + XK - 1) / XK, nblk = (nk + KBLK - 1) / KBLK;
-      bool stop = false;
-      for (int u = 0; u < npairs * nblk; ++u, ++uc) {
-        const int p = u / nblk;
-        const int a = uc & 1;
-        if (!bounded_wait(&tfull[a], (uc >> 1) & 1, abort)) {
-          stop = true;
-          break;
-        }
-        tc_fence_after();
-        // exponent of 2^(e_i + 1) 2^(-7 (s + t)); the column's is added per term
-        const int er = ea - DIGIT_BITS * (c_pairs.s[p] + c_pairs.t[p]);
+      const int nk = (J.K + XK - 1) / XK;
+      for (int k0 = 0; k0 < nk && !stop; k0 += KBLK) {
+        const int group = KBLK / (min(nk, k0 + KBLK) - k0);
+        for (int lp = 0; lp < XLP && !stop; ++lp) {
+          const int l = lower_level(lp);
+          for (int ta = 1; ta <= l; ta += group, ++uc) {
+            if (!bounded_wait(&tfull, uc & 1, abort)) {
+              stop = true;
+              break;
+            }
+            tc_fence_after();
+            const bool both = ta < l;  // the lower level's accumulator was written
 #pragma unroll 1
-        for (int c = 0; c < XN / 64; ++c) {
-          uint32_t v[32];
-          const int col = half * (XN / 2) + c * 32;  // this warp's columns of the tile
-          __syncwarp();
-          tmem_ld_32x32(tmem + (uint32_t(q * 32) << 16) + uint32_t(a * XN + col), v);
-          tmem_wait_ld();
-          const int gc = n0 + col;
-          if (gr >= J.M) continue;
-          double *crow = J.C + int64_t(gr) * J.ldc + gc;
-          const bool add = u != 0 || J.accum;  // C holds earlier terms
-          if (gc + 32 <= J.N) {
-            // all sixteen loads of the row's chunk in flight before any store
-            double2 c2[16];
-            if (add) {
+            for (int c = 0; c < XN / 64; ++c) {
+              uint32_t v0[32], v1[32];
+              const int col = half * (XN / 2) + c * 32;  // this warp's columns of the tile
+              __syncwarp();
+              if (both) tmem_ld_32x32(trow + uint32_t(col), v0);
+              tmem_ld_32x32(trow + uint32_t(XN + col), v1);
+              tmem_wait_ld();
+              if (!both) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) c2[i] = reinterpret_cast<const double2 *>(crow)[i];
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const int2 eb = reinterpret_cast<const int2 *>(J.eb + gc)[i];
-              double2 t2 = make_double2(exact_scaled(__uint_as_float(v[2 * i]), er + eb.x),
-                                        exact_scaled(__uint_as_float(v[2 * i + 1]), er + eb.y));
-              if (add) {
-                t2.x = c2[i].x + t2.x;
-                t2.y = c2[i].y + t2.y;
+                for (int i = 0; i < 32; ++i) v0[i] = 0u;
               }
-              reinterpret_cast<double2 *>(crow)[i] = t2;
-            }
-          } else {
-            // ragged last chunk (N and ldc even, C 16-byte aligned: column pairs)
+              long long *const lc = low + c * 32 * 32;
+              if (lp < XLP - 1) {  // levels 9 .. 4: into the integer tile
+                const bool first = lp == 0 && ta == 1;
+                const int sh = 2 * DIGIT_BITS * lp;
 #pragma unroll
-            for (int k = 0; k < 32; k += 2) {
-              if (gc + k >= J.N) break;
-              const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + k);
-              double2 t2 = make_double2(exact_scaled(__uint_as_float(v[k]), er + eb.x),
-                                        exact_scaled(__uint_as_float(v[k + 1]), er + eb.y));
-              double2 *cp = reinterpret_cast<double2 *>(crow + k);
-              if (add) {
-                const double2 c2 = *cp;
-                t2.x = c2.x + t2.x;
-                t2.y = c2.y + t2.y;
+                for (int h = 0; h < 2; ++h) {
+                  long long o[16];
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) o[i] = first ? 0ll : lc[(16 * h + i) * 32];
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) {
+                    const int x = 16 * h + i;
+                    lc[x * 32] =
+                        o[i] + (acc_int(v0[x]) * (1 << DIGIT_BITS) + acc_int(v1[x])) * (1ll << sh);
+                  }
+                }
+                continue;
               }
-              *cp = t2;
+              // levels 3 and 2: C = [C +] 2^(e_i + f_j - 63) L + 2^(e_i + f_j - 21) H
+              const int gc = n0 + col;
+              if (gr >= J.M) continue;
+              double *const crow = J.C + int64_t(gr) * J.ldc + gc;
+              const bool with_low = ta == 1;
+              const bool add = ta > 1 || k0 > 0 || J.accum;  // C holds earlier terms
+              auto pair_of = [&](int k, const double2 &old) {  // columns gc + k, gc + k + 1
+                const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + k);
+                double r[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                  const int sc = ea + (i ? eb.y : eb.x);
+                  r[i] = scaled_int(acc_int(v0[k + i]) * (1 << DIGIT_BITS) + acc_int(v1[k + i]),
+                                    sc - 3 * DIGIT_BITS);
+                  if (with_low) r[i] += scaled_int(lc[(k + i) * 32], sc - 9 * DIGIT_BITS);
+                  if (add) r[i] += i ? old.y : old.x;
+                }
+                return make_double2(r[0], r[1]);
+              };
+              if (gc + 32 <= J.N) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  double2 o[8];  // eight loads of the row in flight before any store
+                  if (add) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                      o[i] = reinterpret_cast<const double2 *>(crow)[8 * h + i];
+                  }
+#pragma unroll
+                  for (int i = 0; i < 8; ++i)
+                    reinterpret_cast<double2 *>(crow)[8 * h + i] =
+                        pair_of(16 * h + 2 * i, add ? o[i] : make_double2(0.0, 0.0));
+                }
+              } else {
+                // ragged last chunk (N and ldc even, C 16-byte aligned: column pairs)
+#pragma unroll
+                for (int k = 0; k < 32; k += 2) {
+                  if (gc + k >= J.N) break;
+                  double2 *const cp = reinterpret_cast<double2 *>(crow + k);
+                  *cp = pair_of(k, add ? *cp : make_double2(0.0, 0.0));
+                }
+              }
             }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty);
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[a]);
       }
-      if (stop) break;
     }
   }
 
@@ -440,10 +490,27 @@ size_t scratch_maps_x(int njobs) {
   return size_t(njobs) * 2 + (size_t(njobs + 1) * sizeof(int) + sizeof(CUtensorMap) - 1) /
                                  sizeof(CUtensorMap);
 }
+// the maps and tile offsets, then the CTAs' integer tiles
+size_t scratch_maps_bytes_x(int njobs) {
+  return (scratch_maps_x(njobs) * sizeof(CUtensorMap) + 255) & ~size_t(255);
+}
+
+// SMs of the device: the CTAs of k_gemm_slices.
+int slice_ctas() {
+  static const int nsm = [] {  // once, thread-safe
+    int dev = 0, n = 0;
+    SGN_CUDA(cudaGetDevice(&dev));
+    SGN_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    SGN_CUDA(cudaFuncSetAttribute(k_gemm_slices, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  XSMEM));
+    return n;
+  }();
+  return nsm;
+}
 
 }  // namespace
 
-int f64x_pairs() { return kPairs.n; }
+int f64x_pairs() { return XPAIRS; }
 
 void launch_densify64(int64_t n, const int32_t *seg, const int *dslot, const int64_t *moff,
                       const int64_t *rp, const int32_t *col, const double *val,
@@ -474,7 +541,9 @@ size_t f64x_digits_bytes(int rows, int ld) {
   return size_t(F64X_DIGITS) * size_t(rows) * size_t(ld) * sizeof(uint16_t);
 }
 
-size_t slice_jobs_scratch_bytes(int njobs) { return scratch_maps_x(njobs) * sizeof(CUtensorMap); }
+size_t slice_jobs_scratch_bytes(int njobs) {
+  return scratch_maps_bytes_x(njobs) + size_t(slice_ctas()) * XTILE_BYTES;
+}
 
 void launch_slices(int rows, int K, const double *x, int ldx, int transpose, uint16_t *digits,
                    int ld, int *w, cudaStream_t s) {
@@ -488,14 +557,6 @@ void launch_slices(int rows, int K, const double *x, int ldx, int transpose, uin
 void launch_slice_jobs(int njobs, const SliceJob *jobs_host, SliceJob *jobs_dev, void *scratch,
                        int *err, cudaStream_t s) {
   if (njobs <= 0) return;
-  static const int nsm = [] {  // once, thread-safe
-    int dev = 0, n = 0;
-    SGN_CUDA(cudaGetDevice(&dev));
-    SGN_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    SGN_CUDA(cudaFuncSetAttribute(k_gemm_slices, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  XSMEM));
-    return n;
-  }();
   thread_local std::vector<CUtensorMap> host;
   host.resize(scratch_maps_x(njobs));
   CUtensorMap *maps = host.data();
@@ -517,11 +578,11 @@ void launch_slice_jobs(int njobs, const SliceJob *jobs_host, SliceJob *jobs_dev,
                            cudaMemcpyHostToDevice, s));
   SGN_CUDA(cudaMemcpyAsync(jobs_dev, jobs_host, sizeof(SliceJob) * size_t(njobs),
                            cudaMemcpyHostToDevice, s));
-  const unsigned char *sc = static_cast<const unsigned char *>(scratch);
-  k_gemm_slices<<<std::min(ntiles, nsm), XTHREADS, XSMEM, s>>>(
+  unsigned char *sc = static_cast<unsigned char *>(scratch);
+  k_gemm_slices<<<std::min(ntiles, slice_ctas()), XTHREADS, XSMEM, s>>>(
       jobs_dev, reinterpret_cast<const CUtensorMap *>(sc),
       reinterpret_cast<const int *>(sc + size_t(njobs) * 2 * sizeof(CUtensorMap)), njobs, ntiles,
-      err);
+      reinterpret_cast<long long *>(sc + scratch_maps_bytes_x(njobs)), err);
   SGN_LAUNCH_CHECK();
 }
 
@@ -565,7 +626,7 @@ extern "C" sign_status sign_dense_product_f64(int M, int N, int K, const double 
     err.ensure(sizeof(int), s);
     SGN_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
     {
-      ProfScope ps(KC_DENSE64, s, 2.0 * kPairs.n * double(M) * double(N) * double(kp), 0.0);
+      ProfScope ps(KC_DENSE64, s, 2.0 * XPAIRS * double(M) * double(N) * double(kp), 0.0);
       launch_slice_jobs(1, &J, job.as<SliceJob>(), scratch.p, err.as<int>(), s);
     }
     int herr = 0;
