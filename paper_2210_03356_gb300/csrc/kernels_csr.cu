@@ -321,11 +321,23 @@ __global__ void k_fill_seg(int nb, const int64_t *moff, int64_t n, int32_t *seg)
 // the largest one, hi * 2^64 + lo, comes back as
 // ((double)hi * 2^64 + (double)lo) * 2^(e-62).
 
-// *p = max(*p, v). The value is read first: it only grows, so an entry at or
-// below it needs no atomic. A large matrix's rows otherwise queue on one
-// address (262144 rows: about 170 us for each of the three maxima).
-__device__ __forceinline__ void max_into(unsigned long long *p, unsigned long long v) {
-  if (*reinterpret_cast<volatile unsigned long long *>(p) < v) atomicMax(p, v);
+// p[m] = max(p[m], v) for every lane of the warp (v = 0: nothing to add). The
+// lanes of one matrix are reduced first, and the value is read before the
+// atomic: it only grows, so a maximum at or below it needs none. A large
+// matrix's rows otherwise queue on one address (262144 rows: about 170 us for
+// each of the three maxima).
+__device__ __forceinline__ void max_into(unsigned long long *p, int m, unsigned long long v) {
+  const int m0 = __shfl_sync(0xffffffffu, m, 0);
+  bool put = v != 0ULL;
+  if (__all_sync(0xffffffffu, m == m0)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+      v = w > v ? w : v;
+    }
+    put = v != 0ULL && lane_id() == 0;
+  }
+  if (put && *reinterpret_cast<volatile unsigned long long *>(p + m) < v) atomicMax(p + m, v);
 }
 
 __device__ __forceinline__ void add128(unsigned long long *lohi, unsigned long long q) {
@@ -341,8 +353,8 @@ __global__ void k_absmax(int64_t n, const int32_t *seg, const int64_t *rp, const
       for (int64_t p = rp[r] + gl; p < rp[r + 1]; p += 8) m = fmax(m, fabs(val[p]));
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o, 8));
-    if (has && gl == 0 && m > 0.0)
-      max_into(&mmax[seg[r]], (unsigned long long)__double_as_longlong(m));
+    max_into(mmax, seg[r],
+             has && gl == 0 && m > 0.0 ? (unsigned long long)__double_as_longlong(m) : 0ULL);
   });
 }
 
@@ -362,18 +374,24 @@ __global__ void k_colsum(int64_t n, const int32_t *seg, const int64_t *rp, const
   });
 }
 
+// A whole warp stays in the loop (max_into); its lanes past the end add nothing.
 __global__ void k_colmax_hi(int64_t n, const int32_t *seg, const unsigned long long *colsum,
                             unsigned long long *maxhi) {
-  for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
-       j += int64_t(gridDim.x) * blockDim.x)
-    if (colsum[2 * j] | colsum[2 * j + 1]) max_into(&maxhi[seg[j]], colsum[2 * j + 1]);
+  for (int64_t j0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane_id(); j0 < n;
+       j0 += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t j = j0 + lane_id() < n ? j0 + lane_id() : n - 1;
+    max_into(maxhi, seg[j], colsum[2 * j + 1]);
+  }
 }
 
 __global__ void k_colmax_lo(int64_t n, const int32_t *seg, const unsigned long long *colsum,
                             const unsigned long long *maxhi, unsigned long long *maxlo) {
-  for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
-       j += int64_t(gridDim.x) * blockDim.x)
-    if (colsum[2 * j + 1] == maxhi[seg[j]]) max_into(&maxlo[seg[j]], colsum[2 * j]);
+  for (int64_t j0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane_id(); j0 < n;
+       j0 += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t j = j0 + lane_id() < n ? j0 + lane_id() : n - 1;
+    const int m = seg[j];
+    max_into(maxlo, m, colsum[2 * j + 1] == maxhi[m] ? colsum[2 * j] : 0ULL);
+  }
 }
 
 __global__ void k_norm_final(int nb, const unsigned long long *mmax,
@@ -412,11 +430,12 @@ __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp,
 // a matrix of 262144 rows took 232 us per sum of two components and 267 us
 // per count (one SM's FP64 pipe and load latency bound it). With the clusters
 // and the 1-norm's maxima below, the mixed solve of the tridiagonal matrix of
-// that order went from 16.3 to 11.9 ms (GB300).
+// that order went from 16.3 to 11.9 ms, and to 11.0 with the rows prefetched
+// and the maxima reduced per warp (GB300).
 constexpr int RED_T = 256;  // partial sums per component; their order is fixed
 constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
 constexpr int RED_LANES = RED_T / RED_C;
-constexpr int RED_U = 8;    // rows loaded at once
+constexpr int RED_U = 16;   // rows loaded at once, the next ones while these are added
 static_assert(RED_LANES == 32, "one warp of each CTA per component");
 
 // Component c = threadIdx.y of matrix m: partial sum t (0 <= t < RED_T) adds
@@ -434,14 +453,30 @@ __global__ void __cluster_dims__(RED_C, 1, 1)
   const int64_t e = moff[m + 1];
   double acc = 0.0;
   int64_t r = moff[m] + t;
-  for (; r + (RED_U - 1) * RED_T < e; r += RED_U * RED_T) {
-    double v[RED_U];
+  double v[RED_U], w[RED_U];  // absent rows are loaded as -0, which adds nothing
+  auto fetch = [&](double (&d)[RED_U]) {
 #pragma unroll
-    for (int u = 0; u < RED_U; ++u) v[u] = part[(r + u * RED_T) * ncomp + c];
+    for (int u = 0; u < RED_U; ++u, r += RED_T) d[u] = r < e ? part[r * ncomp + c] : -0.0;
+  };
+  auto add = [&](const double (&d)[RED_U]) {
 #pragma unroll
-    for (int u = 0; u < RED_U; ++u) acc += v[u];
+    for (int u = 0; u < RED_U; ++u) acc += d[u];
+  };
+  fetch(v);
+  for (;;) {
+    if (r >= e) {
+      add(v);
+      break;
+    }
+    fetch(w);
+    add(v);
+    if (r >= e) {
+      add(w);
+      break;
+    }
+    fetch(v);
+    add(w);
   }
-  for (; r < e; r += RED_T) acc += part[r * ncomp + c];
   *cl.map_shared_rank(&sm[c][t], 0) = acc;
   cl.sync();
   if (q != 0) return;
