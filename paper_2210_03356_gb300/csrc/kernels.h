@@ -214,11 +214,14 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
 // Numeric product. Row i is written at cs[i] (exclusive scan of ub) and its
 // end stored in ce[i]. MODE_SQUARE: C = A A, and part[2i] = sum_j (C_ij -
 // delta_ij)^2, part[2i+1] = sum_k a_ik^2. MODE_UPDATE: C = 1.5 A - 0.5 A B.
+// The part entries of dense-path matrices (dslot nullable; dslot[seg[i]] >= 0)
+// are left to the dense path.
 template <typename T>
 void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int32_t *lo, const int32_t *len, const int32_t *lists,
-                    const int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
-                    double *part, cudaStream_t s);
+                    int mode, const int32_t *lo, const int32_t *len, const int32_t *seg,
+                    const int *dslot, const int32_t *lists, const int *counters,
+                    const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
+                    cudaStream_t s);
 
 // ---------------------------------------------------------------- filter
 // Per-matrix scalars after the check of the current iterates.

@@ -860,10 +860,13 @@ __global__ void __launch_bounds__(CTA_THREADS)
 
 // Rows with an empty column range: their slot stays empty (ce = cs) and, in
 // MODE_SQUARE, they still contribute (0 - 1)^2 = 1 for the missing diagonal
-// and sum_k a_ik^2 to the norms.
+// and sum_k a_ik^2 to the norms. The rows of dense-path matrices (dslot[seg]
+// >= 0) are empty here too, but their norms come from the dense blocks: their
+// values are not read (4096 full rows of 4096 entries: 610 us -> 4 us).
 template <typename T>
 __global__ void k_rows_empty(int64_t n, const int64_t *ars, const int64_t *are, const T *aval,
-                             const int32_t *len, const int64_t *cs, int64_t *ce, double *part) {
+                             const int32_t *len, const int32_t *seg, const int *dslot,
+                             const int64_t *cs, int64_t *ce, double *part) {
   int lane = lane_id();
   const int g = lane >> 3, gl = lane & 7;  // four groups of 8 lanes
   int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -885,14 +888,15 @@ __global__ void k_rows_empty(int64_t n, const int64_t *ars, const int64_t *are, 
       if (has && gl == 0) ce[r] = cs[r];
       if (!part) continue;
       double xs = 0.0;
-      if (has)
+      const bool norms = has && !(dslot && dslot[seg[r]] >= 0);
+      if (norms)
         for (int64_t p = ars[r] + gl; p < are[r]; p += 8) {
           double x = double(aval[p]);
           xs += x * x;
         }
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) xs += __shfl_xor_sync(0xffffffffu, xs, o, 8);
-      if (has && gl == 0) {
+      if (norms && gl == 0) {
         part[2 * r] = 1.0;
         part[2 * r + 1] = xs;
       }
@@ -976,13 +980,15 @@ static void num_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, c
 
 template <typename T>
 void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int32_t *lo, const int32_t *len, const int32_t *lists,
-                    const int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
-                    double *part, cudaStream_t s) {
+                    int mode, const int32_t *lo, const int32_t *len, const int32_t *seg,
+                    const int *dslot, const int32_t *lists, const int *counters,
+                    const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
+                    cudaStream_t s) {
   if (n == 0) return;
   int *ctr = const_cast<int *>(counters);
-  k_rows_empty<T><<<grid_cap(n, 8 * 32, 16), 256, 0, s>>>(n, A.rs, A.re, aval, len, cs, ce,
-                                                      mode == MODE_SQUARE ? part : nullptr);
+  k_rows_empty<T><<<grid_cap(n, 8 * 32, 16), 256, 0, s>>>(n, A.rs, A.re, aval, len, seg, dslot,
+                                                          cs, ce,
+                                                          mode == MODE_SQUARE ? part : nullptr);
   SGN_LAUNCH_CHECK();
   if (mode == MODE_SQUARE)
     num_launch<T, MODE_SQUARE>(n, A, aval, B, bval, lo, len, lists, ctr, cs, ce, ccol, cval, part,
@@ -994,11 +1000,13 @@ void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, cons
 
 template void launch_numeric<double>(int64_t, const Rows &, const double *, const Rows &,
                                      const double *, int, const int32_t *, const int32_t *,
-                                     const int32_t *, const int *, const int64_t *, int64_t *,
-                                     int32_t *, double *, double *, cudaStream_t);
+                                     const int32_t *, const int *, const int32_t *, const int *,
+                                     const int64_t *, int64_t *, int32_t *, double *, double *,
+                                     cudaStream_t);
 template void launch_numeric<float>(int64_t, const Rows &, const float *, const Rows &,
                                     const float *, int, const int32_t *, const int32_t *,
-                                    const int32_t *, const int *, const int64_t *, int64_t *,
-                                    int32_t *, float *, double *, cudaStream_t);
+                                    const int32_t *, const int *, const int32_t *, const int *,
+                                    const int64_t *, int64_t *, int32_t *, float *, double *,
+                                    cudaStream_t);
 
 }  // namespace sgn

@@ -522,7 +522,9 @@ struct Solver {
       // bytes: the row-wise class keeps the whole product's algorithmic bytes
       ProfScope ps(cls, s, fl - fl_band, by);
       launch_numeric<T>(N, A, aval, B, bval, mode, w.lo.as<int32_t>(), w.len.as<int32_t>(),
-                        w.wlist.as<int32_t>(), w.counters.as<int>(), C.rs.template as<int64_t>(),
+                        st.d_seg.template as<int32_t>(),
+                        dp && dp->any() ? w.dslot.as<int>() : nullptr, w.wlist.as<int32_t>(),
+                        w.counters.as<int>(), C.rs.template as<int64_t>(),
                         C.re.template as<int64_t>(), C.col.template as<int32_t>(), C.d_val(),
                         mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
     }
