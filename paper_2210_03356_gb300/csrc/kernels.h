@@ -439,11 +439,13 @@ void launch_dense_emit64(int64_t n, const int32_t *seg, const int *dslot, const 
 struct DenseBuf {
   float *X_hi, *X_lo, *XT_hi, *XT_lo, *TT_hi, *TT_lo, *P;
   int n, ld;
+  int64_t row0;  // the matrix's first row in the stage
 };
+// The nd dense blocks (leading dimensions up to max_ld) from the stage's CSR:
+// every element of X and X^T is written.
+void launch_densify(int nd, int max_ld, const int64_t *rp, const int32_t *col, const float *val,
+                    const DenseBuf *bufs, cudaStream_t s);
 // dslot[m] = index into bufs for matrices on the dense path, -1 otherwise.
-void launch_densify(int64_t n, const int32_t *seg, const int *dslot, const int64_t *moff,
-                    const int64_t *rp, const int32_t *col, const float *val, const DenseBuf *bufs,
-                    cudaStream_t s);
 void launch_dense_resid(int64_t n, const int32_t *seg, const int *dslot, const int64_t *moff,
                         const DenseBuf *bufs, double *part, unsigned long long *tcount,
                         cudaStream_t s);

@@ -609,6 +609,7 @@ struct Solver {
         DenseBuf b = {};
         b.n = int(n);
         b.ld = ld;
+        b.row0 = st.moff[i];
         dp.bufs.push_back(b);
       } else {
         DenseBuf64 b = {};
@@ -689,11 +690,8 @@ struct Solver {
       w.dscratch.ensure(dense_jobs_scratch_bytes(int(jobs.size())), s);
       const DenseBuf *bufs = w.dbufs.as<DenseBuf>();
       if (mode == MODE_SQUARE) {
-        size_t total = 0;
-        for (const DenseBuf &b : dp.bufs) total += 7 * size_t(b.ld) * size_t(b.ld);
-        SGN_CUDA(cudaMemsetAsync(w.dmem.p, 0, sizeof(float) * total, s));
-        launch_densify(N, st.d_seg.template as<int32_t>(), w.dslot.as<int>(),
-                       st.d_moff.template as<int64_t>(), st.X.d_rp(), st.X.d_col(),
+        // every element of X and X^T is written here and of T^T and P by the products
+        launch_densify(dp.nd, dp.max_ld, st.X.d_rp(), st.X.d_col(),
                        reinterpret_cast<const float *>(st.X.val.p), bufs, s);
       }
       {
