@@ -237,7 +237,7 @@ struct MatScalars {
   unsigned long long sel_q;  // q(b) = floor(b^2 / 2^(2e - 62))
   unsigned long long tiny;   // keys below this have q == 0 (all ones: no key is summed)
   int sel_e;                 // e + 1023, the biased exponent of b (1 for a subnormal b)
-  int sel_pad;
+  int sel_base;              // top 16 bits of the pivot's key (a little below b / sqrt(nnz_bar))
 };
 // From sums[2m] = sum (T-I)^2, sums[2m+1] = sum X^2: r, x, beta, b.
 void launch_matrix_scalars(int nb, const int64_t *moff, const double *sums, double c4,
@@ -264,46 +264,56 @@ void launch_budget_x2(int nb, const int64_t *moff, const double *x2, double swit
                       MatScalars *ms, cudaStream_t s);
 
 // The values a threshold is selected over: row r holds entries [rs[r], re[r])
-// of matrix seg[r]; rs == nullptr means one flat array of flat_nnz values of
-// matrix 0, cut into rows of kFlatRow values.
-constexpr int64_t kFlatRow = 16384;
+// of matrix seg[r], whose rows start at moff[m]; rs == nullptr means one flat
+// array of flat_nnz values of matrix 0, cut into rows of kFlatRow values.
+// cshift: the candidate room of a matrix is its entry count >> cshift.
+constexpr int64_t kFlatRow = 1024;
 struct SelRows {
   int64_t nrows;
   const int32_t *seg;
   const int64_t *rs;
   const int64_t *re;
   int64_t flat_nnz;
+  const int64_t *moff;
+  int cshift;
 };
 
 // Threshold selection (EXACT) for every active matrix; writes ms[m].tau.
-// The scratch holds, 256-byte aligned each: the level-0 histograms (1024
-// 128-bit sums per matrix), the digit histograms (256 per matrix), one
-// minimum per matrix, one select state of at most kSelStateBytes per matrix,
-// the candidate count, and room for cap candidates (8-byte key + row).
+// The scratch holds, 256-byte aligned each: the level-0 histograms
+// (kSelBuckets 128-bit sums per matrix), one minimum per matrix, one select
+// state of at most kSelStateBytes per matrix, the overflow flag and the
+// candidate counts, and room for cap candidates (8-byte key + row).
+// kSelBuckets: the buckets from b / sqrt(2^62) to b, 16 per octave, and one
+// sum below.
+constexpr int kSelBuckets = 512;
 constexpr size_t kSelStateBytes = 64;
 constexpr size_t sel_align(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t select_scratch_bytes(int nb, int64_t cap) {
-  return sel_align(size_t(nb) * 1024 * 2 * 8) + sel_align(size_t(nb) * 256 * 2 * 8) +
-         sel_align(size_t(nb) * 8) + sel_align(size_t(nb) * kSelStateBytes) + sel_align(8) +
+  return sel_align(size_t(nb) * kSelBuckets * 2 * 8) + sel_align(size_t(nb) * 8) +
+         sel_align(size_t(nb) * kSelStateBytes) + sel_align(size_t(nb + 1) * 8) +
          sel_align(size_t(cap > 0 ? cap : 1) * 8) + sel_align(size_t(cap > 0 ? cap : 1) * 4);
 }
-// cand_cap is the scratch's candidate room. Candidates past it are counted
-// but not kept, and the thresholds (and counts) are then not valid: the
-// caller compares the count (*select_cand_count) with cand_cap and selects
-// again with room for every value when it is exceeded.
+// nvals: the values (or slots) of all rows, which sizes the launches. nnz
+// (nullable): the entries per matrix, stored into ms[m].nnz_bar; else nnz_bar
+// holds them already.
+// cand_cap is the scratch's candidate room, at least nvals >> R.cshift. When a
+// matrix has more candidates than its room, *select_overflow is set and the
+// thresholds (and counts) are not valid: the caller selects again with room
+// for every value (cshift 0). With cshift 0 it cannot happen.
 // cnt, dropped (nullable, R.nrows each; R must have rows rs/re): the
 // filter's per-row kept counts and dropped sums of squares under the
 // selected tau, as launch_filter_count gives them, except that the squares of
 // the dropped entries of the crossing bucket are left out: add them per
 // matrix with launch_select_drop_fix once dropped is summed per matrix.
-void launch_select_exact(int nb, const SelRows &R, int64_t cand_cap, const int *active,
-                         const void *val, int val_f32, MatScalars *ms, void *scratch,
-                         int64_t *cnt, double *dropped, cudaStream_t s);
+void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
+                         const int *active, const void *val, int val_f32, const int64_t *nnz,
+                         MatScalars *ms, void *scratch, int64_t *cnt, double *dropped,
+                         cudaStream_t s);
 // sums[m] += the squares of matrix m's dropped entries of its crossing bucket
 // (after launch_select_exact with counts, on the same scratch).
 void launch_select_drop_fix(int nb, const int *active, void *scratch, const MatScalars *ms,
                             double *sums, cudaStream_t s);
-const unsigned long long *select_cand_count(void *scratch, int nb);
+const unsigned long long *select_overflow(void *scratch, int nb);
 // ms[m].nnz_bar = nnz[m].
 void launch_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms, cudaStream_t s);
 // BOUND: tau = b / sqrt(nnz_bar) per matrix.
@@ -314,10 +324,11 @@ void launch_select_bound(int nb, const int *active, MatScalars *ms, cudaStream_t
 void launch_filter_count(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,
                          const int64_t *re, const void *val, int val_f32, const MatScalars *ms,
                          int64_t *cnt, double *dropped, cudaStream_t s);
-void launch_filter_write(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,
-                         const int64_t *re, const int32_t *col, const void *val, int val_f32,
-                         const MatScalars *ms, const int64_t *orp, int32_t *ocol, void *oval,
-                         cudaStream_t s);
+// nvals: the values (or slots) of all rows, which sizes the launch.
+void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int *active,
+                         const int64_t *rs, const int64_t *re, const int32_t *col, const void *val,
+                         int val_f32, const MatScalars *ms, const int64_t *orp, int32_t *ocol,
+                         void *oval, cudaStream_t s);
 
 // ---------------------------------------------------------------- NMF (Alg. 3.1.1)
 // The inverse of the n x n FP64 matrix in lu (leading dimension ld; factored

@@ -10,22 +10,31 @@
 // dropped, every |x| >= tau kept, so equal magnitudes share their fate); if
 // all entries with |x| <= b fit, tau is the smallest magnitude above b
 // (+inf if there is none). It is found by a radix select on the IEEE bit
-// pattern of |x| (positive doubles order like unsigned integers): a
-// histogram of the top 16 bits over a 1024-bucket window below b, then six
-// 8-bit digits over the candidates of the crossing bucket. The squares are
+// pattern of |x| (positive doubles order like unsigned integers): a histogram
+// of the top 16 bits over the buckets that can hold the crossing, then 8-bit
+// digits over the candidates of the crossing bucket. The crossing is never
+// below b / sqrt(N), N the matrix's entries (N smaller squares fit b^2), so
+// everything below that is one sum kept in registers and only the entries of
+// [b / sqrt(N), b] go to a bucket. The squares are
 // summed as exact 128-bit integers on a fixed grid of the matrix, q(x) =
 // floor(x^2 / 2^(2e - 62)) with 2^e <= b < 2^(e+1), against Q = q(b): the
 // decision does not depend on the order of the additions, and it is the exact
 // one up to the flooring, less than one grid step (2^-62 b^2) per entry.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace sgn {
 
 namespace {
 
-constexpr int NB0 = 1024;        // level-0 buckets
-constexpr int NDIG = 256;        // digit buckets
+constexpr int NB0 = kSelBuckets;  // level-0 buckets: the sum below the pivot, then 16 per octave
+constexpr int NDIG = 256;         // digit buckets
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
@@ -64,22 +73,20 @@ struct SelState {
   int pad;
 };
 
-// Scratch: 128-bit sums (lo, hi) per bucket for the level-0 and digit
-// histograms, the smallest key above b per matrix, the select states, the
-// candidate count and the candidates (key, row of the values).
+// Scratch: 128-bit sums (lo, hi) per level-0 bucket, the smallest key above b
+// per matrix, the select states, the candidate counts and the candidates
+// (key, row of the values), each matrix's in a region of its own.
 struct SelScratch {
-  unsigned long long *hist0;    // nb * NB0 * 2
-  unsigned long long *hdig;     // nb * NDIG * 2
-  unsigned long long *minabove; // nb
-  SelState *st;                 // nb
-  unsigned long long *ncand;    // 1
-  unsigned long long *cand;     // cap
-  int *cand_r;                  // cap
-  unsigned long long cap;       // candidate room; *ncand may count past it (overflow)
+  unsigned long long *hist0;     // nb * NB0 * 2
+  unsigned long long *minabove;  // nb
+  SelState *st;                  // nb
+  unsigned long long *overflow;  // 1: set when a matrix has more candidates than room
+  unsigned long long *ncand;     // nb; may count past the room
+  unsigned long long *cand;      // cap
+  int *cand_r;                   // cap
 };
 
 static_assert(sizeof(SelState) <= kSelStateBytes, "select state outgrew its scratch slot");
-static_assert(NB0 == 1024 && NDIG == 256, "scratch layout in kernels.h assumes these sizes");
 
 inline size_t align_up(size_t x) { return sel_align(x); }
 
@@ -88,19 +95,27 @@ SelScratch carve(void *base, int nb, int64_t cap) {
   SelScratch s;
   s.hist0 = reinterpret_cast<unsigned long long *>(p);
   p += align_up(size_t(nb) * NB0 * 2 * 8);
-  s.hdig = reinterpret_cast<unsigned long long *>(p);
-  p += align_up(size_t(nb) * NDIG * 2 * 8);
   s.minabove = reinterpret_cast<unsigned long long *>(p);
   p += align_up(size_t(nb) * 8);
   s.st = reinterpret_cast<SelState *>(p);
   p += align_up(size_t(nb) * kSelStateBytes);
-  s.ncand = reinterpret_cast<unsigned long long *>(p);
-  p += align_up(8);
+  s.overflow = reinterpret_cast<unsigned long long *>(p);
+  s.ncand = s.overflow + 1;
+  p += align_up(size_t(nb + 1) * 8);
   s.cand = reinterpret_cast<unsigned long long *>(p);
   p += align_up(size_t(cap > 0 ? cap : 1) * 8);
   s.cand_r = reinterpret_cast<int *>(p);
-  s.cap = (unsigned long long)(cap > 0 ? cap : 1);
   return s;
+}
+
+// Matrix m's candidate region: its entries start at slot rs[moff[m]], and the
+// region is that range of slots (shifted right by cshift when the room is a
+// sixteenth of the slots), so the regions of different matrices are disjoint.
+__device__ __forceinline__ unsigned long long cand_base(const SelRows &R, int m) {
+  return R.rs ? (unsigned long long)(R.rs[R.moff[m]] >> R.cshift) : 0ULL;
+}
+__device__ __forceinline__ unsigned long long cand_room(const SelRows &R, const MatScalars &ms) {
+  return (unsigned long long)(ms.nnz_bar >> R.cshift);
 }
 
 // Rows of the values to select over: row r holds entries [rs[r], re[r]) and
@@ -155,6 +170,39 @@ __device__ __forceinline__ unsigned long long key_t<float>(float x) { return key
 template <>
 __device__ __forceinline__ unsigned long long key_t<double>(double x) { return key_f64(x); }
 
+// Keys in the width of the values: FP32 values are compared as 32-bit keys,
+// with every bound converted once per row. ceil_key(k): the smallest key of
+// the type whose magnitude is at least that of the 64-bit key k (all ones past
+// infinity); floor_key(k): the largest whose magnitude is at most that.
+template <typename T>
+struct KeyT;
+template <>
+struct KeyT<float> {
+  using K = uint32_t;
+  static constexpr K kInf = 0x7F800000u;
+  static __device__ __forceinline__ K of(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+  static __device__ __forceinline__ unsigned long long wide(K k) {
+    return key_f32(__uint_as_float(k));
+  }
+  static __device__ __forceinline__ K ceil_key(unsigned long long k) {
+    if (k > INF_KEY) return ~0u;
+    return __float_as_uint(__double2float_ru(__longlong_as_double((long long)k)));
+  }
+  static __device__ __forceinline__ K floor_key(unsigned long long k) {
+    if (k > INF_KEY) return 0x7FFFFFFFu;
+    return __float_as_uint(__double2float_rd(__longlong_as_double((long long)k)));
+  }
+};
+template <>
+struct KeyT<double> {
+  using K = unsigned long long;
+  static constexpr K kInf = INF_KEY;
+  static __device__ __forceinline__ K of(double x) { return key_f64(x); }
+  static __device__ __forceinline__ unsigned long long wide(K k) { return k; }
+  static __device__ __forceinline__ K ceil_key(unsigned long long k) { return k; }
+  static __device__ __forceinline__ K floor_key(unsigned long long k) { return k; }
+};
+
 // (hi, lo) += x^2 for FP32 x, exactly: the square's rounding error comes from
 // an FMA and the sum's from TwoSum; all in FP32, which this GPU runs at 64x
 // its FP64 rate. Inputs are scaled by 2^48 (exact), so that squares of
@@ -198,24 +246,59 @@ __device__ __forceinline__ unsigned long long qval(unsigned long long key, int e
   }
 }
 
-// Per matrix: e (the biased exponent of b, 1 for a subnormal b), Q = q(b) and
-// the smallest key with q >= 1 (the key of 2^(e - 31 - 1023)). b = 0, +inf or
-// NaN: no key is summed (tiny = all ones), every q counts as 0.
-__global__ void k_sel_prepare(int nb, MatScalars *ms) {
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nb) return;
+// q of a key of the values' own width, and its level-0 bucket (base: the top 16
+// bits of the pivot). FP32 keys of the normal range need 32-bit operations and
+// one 32 x 32-bit product.
+template <typename T>
+__device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, int eb, int base,
+                                                       int &bk) {
+  if constexpr (sizeof(T) == 4) {
+    if (key >= 0x00800000u) {
+      const int ex = int(key >> 23);
+      const unsigned m = (key & 0x7FFFFFu) | 0x800000u;
+      const unsigned long long m2 = (unsigned long long)m * m;  // < 2^48
+      const int sh = 16 - 2 * (eb - 896 - ex);  // q = m^2 2^sh; above -48 since q >= 1
+      bk = int(key >> 19) + (896 << 4) - base + 1;
+      return sh >= 0 ? m2 << sh : m2 >> -sh;
+    }
+  }
+  const unsigned long long wide = KeyT<T>::wide(key);
+  bk = int(wide >> 48) - base + 1;
+  return qval<T>(wide, eb);
+}
+
+// Per matrix, in a CTA of its own: nnz_bar = nnz[m] (nullable: as it is), e (the
+// biased exponent of b, 1 for a subnormal b), Q = q(b), the smallest key with
+// q >= 1 (the key of 2^(e - 31 - 1023)) and the pivot's bucket: a power of two
+// fraction below b / sqrt(nnz_bar), so that no rounding lifts it above. b = 0,
+// +inf or NaN: no key is summed (tiny = all ones), every q counts as 0.
+// Clears the matrix's histogram, minimum and candidate count.
+__global__ void __launch_bounds__(256)
+    k_sel_prepare(const int64_t *nnz, MatScalars *ms, SelScratch sc) {
+  const int m = blockIdx.x;
+  for (int t = threadIdx.x; t < 2 * NB0; t += 256) sc.hist0[size_t(m) * NB0 * 2 + t] = 0ULL;
+  if (threadIdx.x) return;
+  sc.minabove[m] = ~0ULL;
+  sc.ncand[m] = 0ULL;
+  if (m == 0) *sc.overflow = 0ULL;
+  if (nnz) ms[m].nnz_bar = nnz[m];
   const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
   const int e = int(bkey >> 52);
   if (bkey == 0ULL || e >= 0x7FF) {  // b <= 0 (sign bit) is caught here as well
     ms[m].sel_e = 0;
     ms[m].sel_q = 0ULL;
     ms[m].tiny = ~0ULL;
+    ms[m].sel_base = int((bkey & 0x7FFFFFFFFFFFFFFFULL) >> 48);
     return;
   }
   const int eb = e ? e : 1;
   ms[m].sel_e = eb;
   ms[m].sel_q = qval<double>(bkey, eb);
   ms[m].tiny = eb > 32 ? (unsigned long long)(eb - 31) << 52 : 0ULL;
+  const int64_t N = ms[m].nnz_bar > 1 ? ms[m].nnz_bar : 1;
+  const double pivot = ms[m].b / sqrt(double(N)) * 0.999;
+  const int base = int((unsigned long long)__double_as_longlong(pivot) >> 48);
+  ms[m].sel_base = pivot < 0x1p-1000 && base > 0 ? base - 1 : base;  // rounding near underflow
 }
 
 // (lo, hi) += (alo, ahi) atomically in memory; exact, order-independent.
@@ -226,19 +309,11 @@ __device__ __forceinline__ void add128(unsigned long long *lohi, unsigned long l
   if (ahi) atomicAdd(&lohi[1], ahi);
 }
 
-__device__ __forceinline__ int bucket0(unsigned long long key, unsigned long long bkey) {
-  long long base = (long long)(bkey >> 48) - (NB0 - 1);
-  long long t = (long long)(key >> 48);
-  if (base < 0) base = 0;
-  return t <= base ? 0 : int(t - base);
-}
-
 // A chunk of consecutive rows, their extents and matrices staged in shared
 // memory by one thread per row, so that a warp's loop over the chunk's rows
 // waits on the values only, not on the chain row -> matrix -> scalars.
 // Rows of inactive matrices are staged empty.
-constexpr int RPC = 64;  // rows per chunk (row lists); flat values: 32 rows of kFlatRow
-__device__ __forceinline__ int64_t chunk_rows(const SelRows &R) { return R.rs ? RPC : 32; }
+constexpr int RPC = 64;  // most rows of a chunk
 
 struct ChunkRows {
   int64_t b[RPC], e[RPC];
@@ -262,103 +337,136 @@ __device__ __forceinline__ int stage_rows(const SelRows &R, const int *active, i
   return t;
 }
 
-constexpr int HIST_LPR = 8;  // lanes per row of the level-0 histogram
+// How a pass over the rows is cut. LPR lanes per row: 8 for the short rows of
+// many (four rows per warp at a time), 32 for long rows, and for few rows,
+// where the chip is not full anyway and a row's latency counts. A chunk of
+// rows is what one CTA stages at a time: 64 rows (two turns of its 8 warps'
+// 8-lane groups), or 8 (a row per warp), so that 4096 rows of 4096 entries
+// make 512 chunks; as 64 chunks of 8-lane rows the three passes of a filter
+// over them took 690, 376 and 276 us, now 66, 43 and 47.
+struct SelCut {
+  int lpr, rpc;
+};
+SelCut sel_cut(int64_t nrows, int64_t nvals) {
+  // 152 SMs x 8 warps x 8 rows: fewer rows leave warps without one
+  const bool wide = nrows < 152 * 64 || nvals / (nrows > 0 ? nrows : 1) >= 512;
+  return wide ? SelCut{32, 8} : SelCut{8, RPC};
+}
 
-// Level-0 histogram. A CTA takes a chunk of consecutive rows, a warp
-// 32 / HIST_LPR rows at a time with HIST_LPR lanes each (the per-row work is
-// then spread over more entries per lane), each lane a contiguous run of the
-// row's entries. Neighbouring entries of a row have similar magnitudes, so a
-// lane sums its run per bucket in registers and adds the run's total once
-// when the bucket changes: into a shared histogram for the chunk's first
-// matrix (almost every row: matrices span many chunks), else into the global
-// one.
+// Adds q to bucket bk of a shared histogram of 96-bit sums kept as three
+// 32-bit words: 32-bit shared atomics are native, 64-bit ones are loops.
+__device__ __forceinline__ void add96(uint32_t (*h)[NB0], int bk, unsigned long long q) {
+  const uint32_t l = uint32_t(q), old = atomicAdd(&h[0][bk], l);
+  uint32_t c = old + l < old ? 1u : 0u;
+  const uint32_t u = uint32_t(q >> 32), v = u + c;
+  c = v < u ? 1u : 0u;
+  if (v) {
+    const uint32_t old1 = atomicAdd(&h[1][bk], v);
+    c += old1 + v < old1 ? 1u : 0u;
+  }
+  if (c) atomicAdd(&h[2][bk], c);
+}
 
-template <typename T>
+// Level-0 histogram. A warp takes 32 / LPR rows of the CTA's chunk at a time,
+// LPR lanes each, neighbouring lanes on neighbouring entries (which have
+// similar magnitudes, so they mostly take the same way). Of each entry's key:
+// above b, the smallest is kept; below the pivot's bucket, the squares are
+// summed in the lane's registers; between, they go to the bucket, in shared
+// memory for the chunk's first matrix (almost every row: matrices span many
+// chunks), else in the global histogram. Bound by instruction issue.
+template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS)
-    k_sel_hist0(SelRows R, const int *active, const T *val, const MatScalars *ms, SelScratch sc) {
-  __shared__ unsigned long long s_h[NB0 * 2];
-  __shared__ unsigned long long s_min;
+    k_sel_hist0(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
+                SelScratch sc) {
+  using K = typename KeyT<T>::K;
+  __shared__ uint32_t s_h[3][NB0];
+  __shared__ unsigned long long s_min, s_below[2];
   __shared__ ChunkRows cr;
-  __shared__ unsigned long long s_bkey[RPC], s_tiny[RPC];
-  __shared__ int s_eb[RPC];
+  __shared__ K s_b[RPC], s_tiny[RPC], s_base[RPC];
+  __shared__ int s_eb[RPC], s_top[RPC];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = SEL_THREADS / 32;
-  const int64_t rpc = chunk_rows(R);
+  constexpr int U = 4;  // loads in flight per lane
   const int64_t nchunks = (R.nrows + rpc - 1) / rpc;
   for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int64_t r0 = c * rpc, r1 = min(r0 + rpc, R.nrows);
-    for (int t = threadIdx.x; t < 2 * NB0; t += SEL_THREADS) s_h[t] = 0ULL;
-    if (threadIdx.x == 0) s_min = ~0ULL;
+    for (int t = threadIdx.x; t < 3 * NB0; t += SEL_THREADS) (&s_h[0][0])[t] = 0u;
+    if (threadIdx.x == 0) {
+      s_min = ~0ULL;
+      s_below[0] = s_below[1] = 0ULL;
+    }
     int mt = 0;
     const int t = stage_rows(R, active, r0, r1, cr, mt);
     if (t >= 0) {
-      s_bkey[t] = (unsigned long long)__double_as_longlong(ms[mt].b);
+      s_b[t] = KeyT<T>::floor_key((unsigned long long)__double_as_longlong(ms[mt].b));
+      s_tiny[t] = KeyT<T>::ceil_key(ms[mt].tiny);
+      s_base[t] = KeyT<T>::ceil_key((unsigned long long)ms[mt].sel_base << 48);
       s_eb[t] = ms[mt].sel_e;
-      s_tiny[t] = ms[mt].tiny;
+      s_top[t] = ms[mt].sel_base;
     }
     __syncthreads();
     const int m0 = cr.m[0];
-    // HIST_LPR lanes per row, 32 / HIST_LPR rows of the chunk per warp at a time
-    const int g = lane / HIST_LPR, gl = lane % HIST_LPR;
+    const int g = lane / LPR, gl = lane % LPR;
     const int nr = int(r1 - r0);
-    for (int i0 = warp * (32 / HIST_LPR); i0 < nr; i0 += nw * (32 / HIST_LPR)) {
-      const int i = i0 + g;
-      const bool has = i < nr;
-      const int64_t e0 = has ? cr.b[i] : 0, e1 = has ? cr.e[i] : 0;
-      const int m = has ? cr.m[i] : m0;
-      const unsigned long long bkey = has ? s_bkey[i] : 0ULL, tiny = has ? s_tiny[i] : ~0ULL;
-      const int eb = has ? s_eb[i] : 0;
-      unsigned long long *hist = m == m0 ? s_h : sc.hist0 + size_t(m) * NB0 * 2;
-      const int64_t per = (e1 - e0 + HIST_LPR - 1) / HIST_LPR;
-      const int64_t p0 = e0 + gl * per, p1 = min(p0 + per, e1);
-      int cur = -1;
-      unsigned long long clo = 0, chi = 0, mymin = ~0ULL;
-      // four independent loads in flight, then the entries in order
-      for (int64_t pb = p0; pb < p1; pb += 4) {
-        unsigned long long keys[4];
+    unsigned long long blo = 0, bhi = 0;  // squares below the pivot (matrix m0)
+    K mymin = ~K(0);                      // smallest key above b (matrix m0)
+    for (int i = warp * (32 / LPR) + g; i < nr; i += nw * (32 / LPR)) {
+      const int64_t e1 = cr.e[i];
+      const int m = cr.m[i];
+      const K bk_ = s_b[i], tiny = s_tiny[i], base = s_base[i];
+      const int eb = s_eb[i], top = s_top[i];
+      for (int64_t p = cr.b[i] + gl; p < e1; p += U * LPR) {
+        T x[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) keys[u] = pb + u < p1 ? key_t<T>(val[pb + u]) : 0ULL;
+        for (int u = 0; u < U; ++u) x[u] = p + u * LPR < e1 ? val[p + u * LPR] : T(0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const unsigned long long key = keys[u];
-          if (pb + u >= p1) break;
-          if (key > bkey) {
-            mymin = key < mymin ? key : mymin;
-            continue;
-          }
-          if (key < tiny) continue;
-          unsigned long long q = qval<T>(key, eb);
-          if (!q) continue;
-          int bk = bucket0(key, bkey);
-          if (bk != cur) {
-            if (cur >= 0) add128(hist + 2 * cur, clo, chi);
-            cur = bk;
-            clo = q;
-            chi = 0;
-          } else {
-            clo += q;
-            if (clo < q) ++chi;
+        for (int u = 0; u < U; ++u) {
+          const K key = KeyT<T>::of(x[u]);
+          if (key > bk_) {
+            if (m == m0)
+              mymin = key < mymin ? key : mymin;
+            else
+              atomicMin(&sc.minabove[m], KeyT<T>::wide(key));
+          } else if (key >= tiny && key != 0) {
+            int bk;
+            const unsigned long long q = q_bucket<T>(key, eb, top, bk);
+            if (m == m0) {
+              if (key >= base) {
+                add96(s_h, bk, q);
+              } else {
+                blo += q;
+                bhi += blo < q ? 1ULL : 0ULL;
+              }
+            } else {
+              add128(sc.hist0 + (size_t(m) * NB0 + (key >= base ? bk : 0)) * 2, q, 0ULL);
+            }
           }
         }
       }
-      if (cur >= 0) add128(hist + 2 * cur, clo, chi);
+    }
 #pragma unroll
-      for (int o = HIST_LPR / 2; o > 0; o >>= 1) {
-        const unsigned long long w = __shfl_xor_sync(0xffffffffu, mymin, o, HIST_LPR);
-        mymin = w < mymin ? w : mymin;
-      }
-      if (gl == 0 && has && mymin != ~0ULL) {
-        if (m == m0)
-          atomicMin(&s_min, mymin);
-        else
-          atomicMin(&sc.minabove[m], mymin);
-      }
+    for (int o = 16; o > 0; o >>= 1) {
+      const K y = __shfl_xor_sync(0xffffffffu, mymin, o);
+      mymin = y < mymin ? y : mymin;
+      const unsigned long long l2 = __shfl_xor_sync(0xffffffffu, blo, o);
+      const unsigned long long h2 = __shfl_xor_sync(0xffffffffu, bhi, o);
+      blo += l2;
+      bhi += h2 + (blo < l2 ? 1ULL : 0ULL);
+    }
+    if (lane == 0) {
+      if (mymin != ~K(0)) atomicMin(&s_min, KeyT<T>::wide(mymin));
+      if (blo | bhi) add128(s_below, blo, bhi);
     }
     __syncthreads();
     if (active[m0]) {
-      unsigned long long *g = sc.hist0 + size_t(m0) * NB0 * 2;
-      for (int t2 = threadIdx.x; t2 < NB0; t2 += SEL_THREADS)
-        if (s_h[2 * t2] | s_h[2 * t2 + 1]) add128(g + 2 * t2, s_h[2 * t2], s_h[2 * t2 + 1]);
-      if (threadIdx.x == 0 && s_min != ~0ULL) atomicMin(&sc.minabove[m0], s_min);
+      unsigned long long *gh = sc.hist0 + size_t(m0) * NB0 * 2;
+      for (int t2 = threadIdx.x; t2 < NB0; t2 += SEL_THREADS) {
+        const unsigned long long lo = s_h[0][t2] | ((unsigned long long)s_h[1][t2] << 32);
+        if (lo | s_h[2][t2]) add128(gh + 2 * t2, lo, s_h[2][t2]);
+      }
+      if (threadIdx.x == 0) {
+        if (s_below[0] | s_below[1]) add128(gh, s_below[0], s_below[1]);
+        if (s_min != ~0ULL) atomicMin(&sc.minabove[m0], s_min);
+      }
     }
     __syncthreads();
   }
@@ -414,22 +522,22 @@ __device__ __forceinline__ int warp_crossing(const unsigned long long *h, int nb
   return -1;
 }
 
-// One warp per matrix: the level-0 bucket where the exact sums cross Q.
+// One warp per matrix: the level-0 bucket where the exact sums cross Q (never
+// the sum below the pivot, bucket 0).
 __global__ void k_sel_find0(int nb, const int *active, const MatScalars *ms, SelScratch sc) {
   const int m = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (m == 0 && lane == 0) *sc.ncand = 0ULL;
   if (m >= nb) return;
   SelState st = {};
   if (active[m]) {
-    unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
-    long long base = (long long)(bkey >> 48) - (NB0 - 1);
-    if (base < 0) base = 0;
+    const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
+    const int base = ms[m].sel_base;
+    const int nbk = min(NB0, int(bkey >> 48) - base + 2);  // up to b's own bucket
     unsigned long long lo = 0, hi = 0;
-    const int c = warp_crossing(sc.hist0 + size_t(m) * NB0 * 2, NB0, ms[m].sel_q, lo, hi);
+    const int c = warp_crossing(sc.hist0 + size_t(m) * NB0 * 2, nbk, ms[m].sel_q, lo, hi);
     if (c >= 0) {
       st.found = 1;
-      st.prefix = (unsigned long long)(base + c) << 48;
+      st.prefix = (unsigned long long)(base + c - 1) << 48;
       st.below_lo = st.below0_lo = lo;
       st.below_hi = st.below0_hi = hi;
     }
@@ -466,28 +574,30 @@ struct DropSum {
 };
 
 constexpr int EX_U = 4;  // entries per lane of a row loaded at once
-constexpr int FLT_LPR = 8;  // lanes per row of the candidate pass and the filter write
 
 // Candidates: the entries of the crossing bucket (top 16 bits of the key equal
-// to the prefix, 0 < key <= b), appended with one atomic per warp.
+// to the prefix, 0 < key <= b), appended to the matrix's region with one atomic
+// per row's lanes and load round.
 // With cnt (the filter of a solve) the same pass also counts, per row, what
 // does not depend on where tau falls inside the crossing bucket: entries
 // above the bucket or above b are kept (cnt[r]); entries below it are
 // dropped, their squares summed into dropped[r] as in k_filter_count. A
 // matrix without a crossing already has its tau (the smallest key above b),
-// so every entry is decided here. k_sel_cand_keep adds the kept candidates
+// so every entry is decided here. k_sel_digits adds the kept candidates
 // once tau is final; the dropped candidates' squares come from the select's
 // exact sums (k_sel_drop_fix). Rows of inactive matrices get 0 and 0.
-template <typename T>
+// Per row two bounds on the keys decide: below s_lo an entry is dropped, from
+// s_up on it is kept, between it is a candidate (a NaN is dropped).
+template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS)
-    k_sel_extract(SelRows R, const int *active, const T *val, const MatScalars *ms,
+    k_sel_extract(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
                   SelScratch sc, int64_t *cnt, double *dropped) {
+  using K = typename KeyT<T>::K;
   __shared__ ChunkRows cr;
-  __shared__ unsigned long long s_bkey[RPC], s_top[RPC], s_tkey[RPC];
+  __shared__ K s_lo[RPC], s_up[RPC];
   __shared__ int s_found[RPC];
+  __shared__ unsigned long long s_cbase[RPC], s_room[RPC];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = SEL_THREADS / 32;
-  const unsigned lt = (1u << lane) - 1u;
-  const int64_t rpc = chunk_rows(R);
   const int64_t nchunks = (R.nrows + rpc - 1) / rpc;
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const int64_t r0 = ch * rpc, r1 = min(r0 + rpc, R.nrows);
@@ -496,94 +606,87 @@ __global__ void __launch_bounds__(SEL_THREADS)
     const int t = stage_rows(R, active, r0, r1, cr, mt);
     if (t >= 0) {
       const bool found = active[mt] && sc.st[mt].found != 0;
-      const unsigned long long above = sc.minabove[mt];
       s_found[t] = found;
-      s_bkey[t] = (unsigned long long)__double_as_longlong(ms[mt].b);
-      s_top[t] = found ? sc.st[mt].prefix >> 48 : 0ULL;
-      s_tkey[t] = above == ~0ULL ? INF_KEY : above;  // tau without a crossing
+      if (found) {
+        const unsigned long long lo = sc.st[mt].prefix, next = lo + (1ULL << 48);
+        s_lo[t] = KeyT<T>::ceil_key(lo);
+        const K top = KeyT<T>::ceil_key(next);
+        const K above = KeyT<T>::floor_key((unsigned long long)__double_as_longlong(ms[mt].b)) + 1;
+        s_up[t] = above < top ? above : top;
+        s_cbase[t] = cand_base(R, mt);
+        s_room[t] = cand_room(R, ms[mt]);
+      } else {
+        const unsigned long long above = sc.minabove[mt];  // tau without a crossing
+        s_lo[t] = s_up[t] = KeyT<T>::ceil_key(above == ~0ULL ? INF_KEY : above);
+      }
     }
     __syncthreads();
-    // FLT_LPR lanes per row, 32 / FLT_LPR rows of the chunk per warp at a time
-    const int g = lane / FLT_LPR, gl = lane % FLT_LPR;
+    const int g = lane / LPR, gl = lane % LPR;
+    const unsigned gmask = LPR == 32 ? 0xffffffffu : ((1u << (LPR & 31)) - 1u) << (g * LPR);
+    const unsigned below = gmask & ((1u << lane) - 1u);
     const int nr = int(r1 - r0);
-    for (int i0 = warp * (32 / FLT_LPR); i0 < nr; i0 += nw * (32 / FLT_LPR)) {
+    for (int i0 = warp * (32 / LPR); i0 < nr; i0 += nw * (32 / LPR)) {
       const int i = i0 + g;
       const bool has = i < nr && (cnt || s_found[i] != 0);
       const int64_t r = r0 + i;
-      const bool found = has && s_found[i] != 0;
       // empty for inactive matrices: 0 and 0 written
       const int64_t e0 = has ? cr.b[i] : 0, e1 = has ? cr.e[i] : 0;
-      const unsigned long long bkey = has ? s_bkey[i] : 0ULL, top = has ? s_top[i] : 0ULL;
-      const unsigned long long tkey = has ? s_tkey[i] : INF_KEY;
+      const K lo = has ? s_lo[i] : K(0), up = has ? s_up[i] : K(0);
       int c = 0;
       DropSum ds;
-      for (int64_t p0 = e0;; p0 += FLT_LPR * EX_U) {
-        if (!__any_sync(0xffffffffu, p0 < e1)) break;  // every row of the warp done
+      for (int64_t p0 = e0;; p0 += LPR * EX_U) {
+        // the warp's rows together (loops of their own would run one by one)
+        if (!__any_sync(0xffffffffu, p0 < e1)) break;
         T x[EX_U];
 #pragma unroll
         for (int u = 0; u < EX_U; ++u) {
-          const int64_t p = p0 + FLT_LPR * u + gl;
+          const int64_t p = p0 + LPR * u + gl;
           x[u] = p < e1 ? val[p] : T(0);  // a zero is neither counted nor dropped
         }
-        bool take[EX_U];
+        unsigned take[EX_U];
+        int n = 0;
 #pragma unroll
         for (int u = 0; u < EX_U; ++u) {
-          const unsigned long long key = key_t<T>(x[u]);
-          take[u] = false;
-          if (key == 0ULL) continue;
-          bool drop;
-          if (found) {
-            const unsigned long long t16 = key >> 48;
-            take[u] = key <= bkey && t16 == top;
-            if (take[u] || !cnt) continue;
-            drop = !(key <= INF_KEY && (t16 > top || key > bkey));
-          } else {
-            drop = !keep_key(key, tkey);
-          }
-          if (drop)
-            ds.add(x[u]);
-          else
+          const K key = KeyT<T>::of(x[u]);
+          const bool cand = key >= lo && key < up && key != 0;
+          take[u] = __ballot_sync(0xffffffffu, cand) & gmask;
+          n += __popc(take[u]);
+          if (!cnt || cand || key == 0) continue;
+          if (key >= up && key <= KeyT<T>::kInf)
             ++c;
+          else
+            ds.add(x[u]);
         }
+        if (n) {  // the row's candidates of this round, in one reservation
+          const int m = cr.m[i];
+          unsigned long long at = 0;
+          if (gl == 0) at = atomicAdd(&sc.ncand[m], (unsigned long long)n);
+          at = __shfl_sync(gmask, at, g * LPR);
+          const unsigned long long cb = s_cbase[i], room = s_room[i];
 #pragma unroll
-        for (int u = 0; u < EX_U; ++u) {
-          const unsigned mask = __ballot_sync(0xffffffffu, take[u]);
-          if (!mask) continue;
-          unsigned long long base = 0;
-          if (lane == 0) base = atomicAdd(sc.ncand, (unsigned long long)__popc(mask));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (take[u]) {
-            const unsigned long long slot = base + __popc(mask & lt);
-            if (slot < sc.cap) {  // past the room: counted only (the caller retries with more)
-              sc.cand[slot] = key_t<T>(x[u]);
-              sc.cand_r[slot] = int(r);
+          for (int u = 0; u < EX_U; ++u) {
+            if ((take[u] >> lane) & 1u) {
+              const unsigned long long slot = at + __popc(take[u] & below);
+              if (slot < room) {
+                sc.cand[cb + slot] = KeyT<T>::wide(KeyT<T>::of(x[u]));
+                sc.cand_r[cb + slot] = int(r);
+              } else {  // past the room: the caller selects again with more
+                *sc.overflow = 1ULL;
+              }
             }
+            at += __popc(take[u]);
           }
         }
       }
       if (!cnt) continue;
 #pragma unroll
-      for (int o = FLT_LPR / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o, FLT_LPR);
-      const double d = ds.group_total<T, FLT_LPR>();
+      for (int o = LPR / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o, LPR);
+      const double d = ds.group_total<T, LPR>();
       if (gl == 0 && has) {
         cnt[r] = c;
         dropped[r] = d;
       }
     }
-  }
-}
-
-// The kept candidates (key >= tau, tau final) into their rows' counts.
-__global__ void k_sel_cand_keep(SelRows R, const MatScalars *ms, SelScratch sc, int64_t *cnt) {
-  unsigned long long total = *sc.ncand;
-  if (total > sc.cap) total = sc.cap;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const int64_t r = sc.cand_r[i];
-    const unsigned long long tkey =
-        (unsigned long long)__double_as_longlong(ms[row_mat(R, r)].tau);
-    if (keep_key(sc.cand[i], tkey))
-      atomicAdd(reinterpret_cast<unsigned long long *>(cnt + r), 1ULL);
   }
 }
 
@@ -603,49 +706,124 @@ __global__ void k_sel_drop_fix(int nb, const int *active, SelScratch sc, const M
   sums[m] = __dadd_rn(sums[m], ldexp(q, 2 * (ms[m].sel_e - 1023) - 62));
 }
 
-__global__ void k_sel_hist_digit(SelRows R, const MatScalars *ms, SelScratch sc, int shift) {
-  unsigned long long total = *sc.ncand;
-  if (total > sc.cap) total = sc.cap;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    int m = row_mat(R, sc.cand_r[i]);
-    unsigned long long key = sc.cand[i];
-    if ((key >> (shift + 8)) != (sc.st[m].prefix >> (shift + 8))) continue;
-    int d = int((key >> shift) & 255ULL);
-    unsigned long long q = qval<double>(key, ms[m].sel_e);
-    if (q) add128(sc.hdig + (size_t(m) * NDIG + d) * 2, q, 0ULL);
+// The digits below the crossing bucket, tau and the kept candidates' counts of
+// a matrix, in one cluster of DG_C CTAs: per digit every CTA sums its part of
+// the candidates into a shared histogram, CTA 0 adds the histograms over
+// distributed shared memory and finds the crossing. The candidates that match
+// the first digit are kept in shared memory for the later ones when they fit.
+// LEVELS: 6 digits cover the 48 bits of an FP64 key, 3 those of an FP32 value
+// (its FP64 key's low 29 bits are zero). Up to DG_ONE candidates CTA 0 works
+// alone. Twelve launches over all candidates did this before: 6 x (5.0 + 5.2)
+// us for one matrix of 500 rows, now 13 in all.
+constexpr int DG_C = 8, DG_T = 512, DG_KEEP = 2048, DG_ONE = 4096;
+template <int LEVELS>
+__global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
+    k_sel_digits(SelRows R, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
+  __shared__ uint32_t h[3][NDIG];
+  __shared__ unsigned long long sum[NDIG * 2];
+  __shared__ unsigned long long keep[DG_KEEP];
+  __shared__ unsigned long long s_res[3];  // CTA 0: prefix and sum below it
+  __shared__ int s_nkeep;
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / DG_C, rank = int(cl.block_rank()), tid = threadIdx.x;
+  if (!active[m]) return;  // the whole cluster, as every return before the loop
+  const SelState st = sc.st[m];
+  if (!st.found) {
+    if (rank == 0 && tid == 0) {
+      const unsigned long long k = sc.minabove[m];
+      ms[m].tau = k == ~0ULL ? __longlong_as_double(0x7ff0000000000000LL)
+                             : __longlong_as_double((long long)k);
+    }
+    return;
   }
-}
-
-// One warp per matrix: the digit at `shift` where the sums cross Q.
-__global__ void k_sel_find_digit(int nb, const MatScalars *ms, SelScratch sc, int shift) {
-  const int m = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
-  if (m >= nb) return;
-  SelState &st = sc.st[m];
-  if (!st.found) return;
-  unsigned long long lo = st.below_lo, hi = st.below_hi;
-  unsigned long long *h = sc.hdig + size_t(m) * NDIG * 2;
-  const int d = warp_crossing(h, NDIG, ms[m].sel_q, lo, hi);
-  __syncwarp();
-  // the buckets are read: cleared here for the next digit, instead of a memset
-  for (int c = threadIdx.x & 31; c < 2 * NDIG; c += 32) h[c] = 0ULL;
-  if (d >= 0 && (threadIdx.x & 31) == 0) {
-    st.prefix |= (unsigned long long)d << shift;
-    st.below_lo = lo;
-    st.below_hi = hi;
+  const unsigned long long room = cand_room(R, ms[m]), cb = cand_base(R, m);
+  const unsigned long long total = sc.ncand[m] < room ? sc.ncand[m] : room;
+  const bool one = total <= DG_ONE;
+  if (one && rank != 0) return;
+  const int nc = one ? 1 : DG_C;
+  const int eb = ms[m].sel_e;
+  const unsigned long long Q = ms[m].sel_q;
+  unsigned long long prefix = st.prefix, lo = st.below_lo, hi = st.below_hi;
+  bool local = false;  // the survivors of the first digit are in keep
+  for (int level = 0; level < LEVELS; ++level) {
+    const int shift = 40 - 8 * level;
+    for (int t = tid; t < 3 * NDIG; t += DG_T) (&h[0][0])[t] = 0u;
+    if (level == 1 && tid == 0) s_nkeep = 0;
+    __syncthreads();
+    auto digit = [&](unsigned long long key) {
+      if ((key >> (shift + 8)) != (prefix >> (shift + 8))) return false;
+      const unsigned long long q = qval<double>(key, eb);
+      const int d = int((key >> shift) & 255ULL);
+      const uint32_t l = uint32_t(q), old = atomicAdd(&h[0][d], l);
+      uint32_t c = old + l < old ? 1u : 0u;
+      const uint32_t u = uint32_t(q >> 32), v = u + c;
+      c = v < u ? 1u : 0u;
+      if (v) {
+        const uint32_t old1 = atomicAdd(&h[1][d], v);
+        c += old1 + v < old1 ? 1u : 0u;
+      }
+      if (c) atomicAdd(&h[2][d], c);
+      return true;
+    };
+    if (local) {
+      for (int i = tid; i < s_nkeep; i += DG_T) digit(keep[i]);
+    } else {
+#pragma unroll 4
+      for (unsigned long long i = (unsigned long long)rank * DG_T + tid; i < total;
+           i += (unsigned long long)nc * DG_T) {
+        const unsigned long long key = sc.cand[cb + i];
+        if (digit(key) && level == 1) {
+          const int at = atomicAdd(&s_nkeep, 1);
+          if (at < DG_KEEP) keep[at] = key;
+        }
+      }
+    }
+    if (nc > 1) cl.sync(); else __syncthreads();
+    if (level == 1) local = s_nkeep <= DG_KEEP;
+    if (rank == 0) {
+      if (tid < NDIG) {
+        unsigned long long a = 0, b = 0;
+        for (int q = 0; q < nc; ++q) {
+          const uint32_t *hq = nc > 1 ? cl.map_shared_rank(&h[0][0], q) : &h[0][0];
+          const unsigned long long w =
+              hq[tid] | ((unsigned long long)hq[NDIG + tid] << 32);
+          a += w;
+          b += hq[2 * NDIG + tid] + (a < w ? 1ULL : 0ULL);
+        }
+        sum[2 * tid] = a;
+        sum[2 * tid + 1] = b;
+      }
+      __syncthreads();
+      if (tid < 32) {
+        unsigned long long l2 = lo, h2 = hi;
+        const int d = warp_crossing(sum, NDIG, Q, l2, h2);
+        if (tid == 0) {
+          s_res[0] = d >= 0 ? prefix | ((unsigned long long)d << shift) : prefix;
+          s_res[1] = d >= 0 ? l2 : lo;
+          s_res[2] = d >= 0 ? h2 : hi;
+        }
+      }
+    }
+    if (nc > 1) cl.sync(); else __syncthreads();
+    const unsigned long long *res = nc > 1 ? cl.map_shared_rank(s_res, 0) : s_res;
+    prefix = res[0];
+    lo = res[1];
+    hi = res[2];
   }
-}
-
-__global__ void k_sel_final(int nb, const int *active, SelScratch sc, MatScalars *ms) {
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nb || !active[m]) return;
-  if (sc.st[m].found) {
-    ms[m].tau = __longlong_as_double((long long)sc.st[m].prefix);
-  } else {
-    unsigned long long k = sc.minabove[m];
-    ms[m].tau = k == ~0ULL ? __longlong_as_double(0x7ff0000000000000LL)
-                           : __longlong_as_double((long long)k);
+  if (rank == 0 && tid == 0) {
+    ms[m].tau = __longlong_as_double((long long)prefix);
+    sc.st[m].prefix = prefix;
+    sc.st[m].below_lo = lo;
+    sc.st[m].below_hi = hi;
   }
+  // the kept candidates (key >= tau) into their rows' counts
+  if (cnt) {
+    for (unsigned long long i = (unsigned long long)rank * DG_T + tid; i < total;
+         i += (unsigned long long)nc * DG_T)
+      if (keep_key(sc.cand[cb + i], prefix))
+        atomicAdd(reinterpret_cast<unsigned long long *>(cnt + sc.cand_r[cb + i]), 1ULL);
+  }
+  if (nc > 1) cl.sync();  // CTA 0's shared memory is read until here
 }
 
 // ------------------------------------------------------------ filter
@@ -707,55 +885,62 @@ __global__ void k_filter_count(int64_t n, const int32_t *seg, const int *active,
   }
 }
 
-template <typename T>
+template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS)
-    k_filter_write(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,
+    k_filter_write(int64_t n, int rpc, const int32_t *seg, const int *active, const int64_t *rs,
                    const int64_t *re, const int32_t *col, const T *val, const MatScalars *ms,
                    const int64_t *orp, int32_t *ocol, T *oval) {
+  using K = typename KeyT<T>::K;
   __shared__ ChunkRows cr;
   __shared__ int64_t s_out[RPC], s_oend[RPC];
-  __shared__ unsigned long long s_tkey[RPC];
+  __shared__ K s_tkey[RPC];
   const int lane = lane_id(), warp = threadIdx.x >> 5, nw = SEL_THREADS / 32;
-  const SelRows R{n, seg, rs, re, 0};
-  const int64_t nchunks = (n + RPC - 1) / RPC;
+  SelRows R{};
+  R.nrows = n;
+  R.seg = seg;
+  R.rs = rs;
+  R.re = re;
+  const int64_t nchunks = (n + rpc - 1) / rpc;
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int64_t r0 = ch * RPC, r1 = min(r0 + RPC, n);
+    const int64_t r0 = ch * rpc, r1 = min(r0 + rpc, n);
     __syncthreads();  // the previous chunk's rows are read
     int mt = 0;
     const int t = stage_rows(R, active, r0, r1, cr, mt);
     if (t >= 0) {
       s_out[t] = orp[r0 + t];
       s_oend[t] = orp[r0 + t + 1];
-      s_tkey[t] = (unsigned long long)__double_as_longlong(ms[mt].tau);
+      s_tkey[t] = KeyT<T>::ceil_key((unsigned long long)__double_as_longlong(ms[mt].tau));
     }
     __syncthreads();
-    // FLT_LPR lanes per row, 32 / FLT_LPR rows of the chunk per warp at a time
-    const int g = lane / FLT_LPR, gl = lane % FLT_LPR;
-    const unsigned gbits = (1u << FLT_LPR) - 1u, glt = (1u << gl) - 1u;
+    // LPR lanes per row, 32 / LPR rows of the chunk per warp at a time
+    const int g = lane / LPR, gl = lane % LPR;
+    const unsigned gmask = LPR == 32 ? 0xffffffffu : ((1u << (LPR & 31)) - 1u) << (g * LPR);
+    const unsigned below = gmask & ((1u << lane) - 1u);
     const int nr = int(r1 - r0);
-    for (int i0 = warp * (32 / FLT_LPR); i0 < nr; i0 += nw * (32 / FLT_LPR)) {
+    for (int i0 = warp * (32 / LPR); i0 < nr; i0 += nw * (32 / LPR)) {
       const int i = i0 + g;
       const bool has = i < nr;
       // the row's room from the counts; the same rule decides both, and the
       // bound keeps a write inside the row whatever the values are
-      const unsigned long long tkey = has ? s_tkey[i] : INF_KEY;
+      const K tkey = has ? s_tkey[i] : ~K(0);
       int64_t out = has ? s_out[i] : 0;
       const int64_t oend = has ? s_oend[i] : 0, b = has ? cr.b[i] : 0, e = has ? cr.e[i] : 0;
-      for (int64_t p0 = b;; p0 += FLT_LPR * EX_U) {
+      for (int64_t p0 = b;; p0 += LPR * EX_U) {
         if (!__any_sync(0xffffffffu, p0 < e)) break;  // every row of the warp done
         T x[EX_U];
         int32_t c[EX_U];
 #pragma unroll
         for (int u = 0; u < EX_U; ++u) {
-          const int64_t p = p0 + FLT_LPR * u + gl;
+          const int64_t p = p0 + LPR * u + gl;
           x[u] = p < e ? val[p] : T(0);  // a zero is never kept
           c[u] = p < e ? col[p] : 0;
         }
 #pragma unroll
         for (int u = 0; u < EX_U; ++u) {
-          const bool keep = keep_key(key_t<T>(x[u]), tkey);
-          const unsigned gm = (__ballot_sync(0xffffffffu, keep) >> (g * FLT_LPR)) & gbits;
-          const int64_t pos = out + __popc(gm & glt);
+          const K key = KeyT<T>::of(x[u]);
+          const bool keep = key >= tkey && key != 0 && key <= KeyT<T>::kInf;
+          const unsigned gm = __ballot_sync(0xffffffffu, keep) & gmask;
+          const int64_t pos = out + __popc(gm & below);
           if (keep && pos < oend) {
             ocol[pos] = c[u];
             oval[pos] = x[u];
@@ -798,64 +983,61 @@ void launch_select_bound(int nb, const int *active, MatScalars *ms, cudaStream_t
   SGN_LAUNCH_CHECK();
 }
 
-const unsigned long long *select_cand_count(void *scratch, int nb) {
-  return carve(scratch, nb, 1).ncand;
+const unsigned long long *select_overflow(void *scratch, int nb) {
+  return carve(scratch, nb, 1).overflow;
 }
 
-void launch_select_exact(int nb, const SelRows &R, int64_t cand_cap, const int *active,
-                         const void *val, int val_f32, MatScalars *ms, void *scratch,
-                         int64_t *cnt, double *dropped, cudaStream_t s) {
-  SelScratch sc = carve(scratch, nb, cand_cap);
-  SGN_CUDA(cudaMemsetAsync(sc.hist0, 0, size_t(nb) * NB0 * 2 * 8, s));
-  SGN_CUDA(cudaMemsetAsync(sc.minabove, 0xff, size_t(nb) * 8, s));
-  k_sel_prepare<<<(nb + 127) / 128, 128, 0, s>>>(nb, ms);
-  SGN_LAUNCH_CHECK();
-  const int64_t rpc = R.rs ? RPC : 32;
+// f(lanes per row as a constant, rows per chunk, CTAs) of a pass over the rows
+template <typename F>
+static void sel_pass(int64_t nrows, int64_t nvals, F f) {
+  if (nrows <= 0) return;
+  const SelCut c = sel_cut(nrows, nvals);
+  const int g = grid_for(nrows, c.rpc, 152 * 8);
+  if (c.lpr == 32)
+    f(std::integral_constant<int, 32>{}, c.rpc, g);
+  else
+    f(std::integral_constant<int, 8>{}, c.rpc, g);
+}
+
+template <typename T>
+static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *active, const T *val,
+                         const int64_t *nnz, MatScalars *ms, const SelScratch &sc, int64_t *cnt,
+                         double *dropped, cudaStream_t s) {
   {
     ProfScope ps(KC_SEL_HIST, s, 0.0, 0.0);
-    if (R.nrows > 0) {
-      const int g = grid_for((R.nrows + rpc - 1) / rpc, 1, 152 * 8);
-      if (val_f32)
-        k_sel_hist0<float><<<g, SEL_THREADS, 0, s>>>(R, active, static_cast<const float *>(val),
-                                                     ms, sc);
-      else
-        k_sel_hist0<double><<<g, SEL_THREADS, 0, s>>>(R, active,
-                                                      static_cast<const double *>(val), ms, sc);
+    k_sel_prepare<<<nb, 256, 0, s>>>(nnz, ms, sc);
+    SGN_LAUNCH_CHECK();
+    sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
+      k_sel_hist0<T, lpr.value><<<g, SEL_THREADS, 0, s>>>(R, rpc, active, val, ms, sc);
       SGN_LAUNCH_CHECK();
-    }
+    });
     k_sel_find0<<<(nb + 3) / 4, 128, 0, s>>>(nb, active, ms, sc);
     SGN_LAUNCH_CHECK();
   }
   {
     ProfScope ps(KC_SEL_EXTRACT, s, 0.0, 0.0);
-    if (R.nrows > 0) {
-      const int g = grid_for((R.nrows + rpc - 1) / rpc, 1, 152 * 8);
-      if (val_f32)
-        k_sel_extract<float><<<g, SEL_THREADS, 0, s>>>(R, active, static_cast<const float *>(val),
-                                                       ms, sc, cnt, dropped);
-      else
-        k_sel_extract<double><<<g, SEL_THREADS, 0, s>>>(
-            R, active, static_cast<const double *>(val), ms, sc, cnt, dropped);
+    sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
+      k_sel_extract<T, lpr.value><<<g, SEL_THREADS, 0, s>>>(R, rpc, active, val, ms, sc, cnt,
+                                                           dropped);
       SGN_LAUNCH_CHECK();
-    }
+    });
   }
   ProfScope ps(KC_SEL_DIGITS, s, 0.0, 0.0);
-  // zeroed once; after each level the matrices that fill buckets (those with
-  // a crossing) clear them again in k_sel_find_digit
-  SGN_CUDA(cudaMemsetAsync(sc.hdig, 0, size_t(nb) * NDIG * 2 * 8, s));
-  for (int level = 0; level < 6; ++level) {
-    int shift = 40 - 8 * level;
-    k_sel_hist_digit<<<152 * 4, 256, 0, s>>>(R, ms, sc, shift);
-    SGN_LAUNCH_CHECK();
-    k_sel_find_digit<<<(nb + 3) / 4, 128, 0, s>>>(nb, ms, sc, shift);
-    SGN_LAUNCH_CHECK();
-  }
-  k_sel_final<<<(nb + 127) / 128, 128, 0, s>>>(nb, active, sc, ms);
+  k_sel_digits<sizeof(T) == 4 ? 3 : 6><<<unsigned(nb) * DG_C, DG_T, 0, s>>>(R, active, sc, ms, cnt);
   SGN_LAUNCH_CHECK();
-  if (cnt) {
-    k_sel_cand_keep<<<152 * 2, 256, 0, s>>>(R, ms, sc, cnt);
-    SGN_LAUNCH_CHECK();
-  }
+}
+
+void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
+                         const int *active, const void *val, int val_f32, const int64_t *nnz,
+                         MatScalars *ms, void *scratch, int64_t *cnt, double *dropped,
+                         cudaStream_t s) {
+  const SelScratch sc = carve(scratch, nb, cand_cap);
+  if (val_f32)
+    select_exact<float>(nb, R, nvals, active, static_cast<const float *>(val), nnz, ms, sc, cnt,
+                        dropped, s);
+  else
+    select_exact<double>(nb, R, nvals, active, static_cast<const double *>(val), nnz, ms, sc, cnt,
+                         dropped, s);
 }
 
 void launch_select_drop_fix(int nb, const int *active, void *scratch, const MatScalars *ms,
@@ -873,20 +1055,21 @@ void launch_filter_count(int64_t n, const int32_t *seg, const int *active, const
   SGN_LAUNCH_CHECK();
 }
 
-void launch_filter_write(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,
-                         const int64_t *re, const int32_t *col, const void *val, int val_f32,
-                         const MatScalars *ms, const int64_t *orp, int32_t *ocol, void *oval,
-                         cudaStream_t s) {
-  if (n == 0) return;
-  if (val_f32)
-    k_filter_write<float><<<grid_for(n, RPC, 152 * 8), SEL_THREADS, 0, s>>>(
-        n, seg, active, rs, re, col, static_cast<const float *>(val), ms, orp, ocol,
-        static_cast<float *>(oval));
-  else
-    k_filter_write<double><<<grid_for(n, RPC, 152 * 8), SEL_THREADS, 0, s>>>(
-        n, seg, active, rs, re, col, static_cast<const double *>(val), ms, orp, ocol,
-        static_cast<double *>(oval));
-  SGN_LAUNCH_CHECK();
+void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int *active,
+                         const int64_t *rs, const int64_t *re, const int32_t *col, const void *val,
+                         int val_f32, const MatScalars *ms, const int64_t *orp, int32_t *ocol,
+                         void *oval, cudaStream_t s) {
+  sel_pass(n, nvals, [&](auto lpr, int rpc, int g) {
+    if (val_f32)
+      k_filter_write<float, lpr.value><<<g, SEL_THREADS, 0, s>>>(
+          n, rpc, seg, active, rs, re, col, static_cast<const float *>(val), ms, orp, ocol,
+          static_cast<float *>(oval));
+    else
+      k_filter_write<double, lpr.value><<<g, SEL_THREADS, 0, s>>>(
+          n, rpc, seg, active, rs, re, col, static_cast<const double *>(val), ms, orp, ocol,
+          static_cast<double *>(oval));
+    SGN_LAUNCH_CHECK();
+  });
 }
 
 }  // namespace sgn

@@ -192,7 +192,7 @@ struct Work {
   BandBuf bx, bt;  // bands of the iterate X and of T = X X (FP32 stage)
   DevBuf bandrow;  // rows of T written by the square's band tiles (1) or not (0)
   DevBuf n2v, n2y, n2z, n2part, n2zacc, n2xmax, n2ymax, n2nrm, x2;  // budget_norm
-  int64_t sel_cap = 0;  // candidate room of the last threshold select
+  int sel_shift = 0;    // > 0: the last threshold select had room for entries >> sel_shift
   DevBuf binfo;         // per row of a product's B: first/last column, length
   DevBuf nmf_int, nmf_dbl;  // NMF: permutation, pivot, singular flags; ||X^-1||
   bool bt_rows_done = false;  // the square's band tiles wrote their rows of T's band
@@ -999,8 +999,9 @@ struct Solver {
         mb[dp.mat[d]] = n * n * n;
       }
     }
-    // per-matrix nnz(Xbar) straight into the device scalars (BOUND needs it)
-    launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
+    // per-matrix nnz(Xbar) straight into the device scalars (the threshold selects do it themselves)
+    if (o.filter == SIGN_FILTER_NONE)
+      launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
     // the iterate is not read again this round: a large one's memory can take
     // the filtered update (reuse is ordered after the update on this stream)
     if (st.X.col.cap + st.X.val.cap > BIG_BUFFER) {
@@ -1113,7 +1114,6 @@ struct Solver {
     }
     launch_seg_count(nb, st.d_moff.template as<int64_t>(), C.rs.as<int64_t>(), C.re.as<int64_t>(),
                      w.nnzc.as<int64_t>(), s);
-    launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
     int live = 0;
     for (int a : st.alive) live += a;
     if (live == 0) wait();  // the extraction reads X and the pinned block list
@@ -1130,14 +1130,21 @@ struct Solver {
     int nb = int(st.mats.size());
     if (o.filter == SIGN_FILTER_EXACT) {
       const int64_t big = int64_t(1) << 28;
-      w.sel_cap = full_room || in.slots <= big ? in.slots : std::max(big, in.slots / 16);
-      w.sel.ensure(select_scratch_bytes(nb, w.sel_cap), s);
+      w.sel_shift = full_room || in.slots <= big ? 0 : 4;
+      const int64_t cap = w.sel_shift ? std::max(big, in.slots >> w.sel_shift) : in.slots;
+      w.sel.ensure(select_scratch_bytes(nb, cap), s);
       w.dropped.ensure(sizeof(double) * size_t(N > 0 ? N : 1), s);
       w.cnt.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
-      SelRows R{N, st.d_seg.template as<int32_t>(), in.rs.template as<int64_t>(),
-                in.re.template as<int64_t>(), 0};
-      launch_select_exact(nb, R, w.sel_cap, d_act, in.val.p, is_f32<T>(), w.ms.as<MatScalars>(),
-                          w.sel.p, w.cnt.as<int64_t>(), w.dropped.as<double>(), s);
+      SelRows R{N,
+                st.d_seg.template as<int32_t>(),
+                in.rs.template as<int64_t>(),
+                in.re.template as<int64_t>(),
+                0,
+                st.d_moff.template as<int64_t>(),
+                w.sel_shift};
+      launch_select_exact(nb, R, in.slots, cap, d_act, in.val.p, is_f32<T>(),
+                          w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), w.sel.p,
+                          w.cnt.as<int64_t>(), w.dropped.as<double>(), s);
     } else {
       ProfScope psel(KC_SELECT, s);
       launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
@@ -1181,11 +1188,11 @@ struct Solver {
       d2h(hm.tot, out.d_rp() + N, 1, s);
       d2h(hm.ms, w.ms.p, size_t(nb), s);
       d2h(hm.dsum, w.sums.p, size_t(nb), s);
-      const bool capped = exact && w.sel_cap < in.slots;
+      const bool capped = exact && w.sel_shift > 0;
       if (capped) d2h(reinterpret_cast<unsigned long long *>(hm.tot + 3),
-                      select_cand_count(w.sel.p, nb), 1, s);
+                      select_overflow(w.sel.p, nb), 1, s);
       wait();
-      if (!capped || uint64_t(hm.tot[3]) <= uint64_t(w.sel_cap)) break;
+      if (!capped || hm.tot[3] == 0) break;
       select_threshold(st, in, d_act, true);  // the crossing bucket outgrew the room
     }
     int64_t nnz = hm.tot[0];
@@ -1196,10 +1203,10 @@ struct Solver {
     {
       ProfScope pw(KC_FILTER, s, 0.0,
                    double(in.slots + nnz) * (sizeof(T) + 4.0) + 24.0 * double(N));
-      launch_filter_write(N, st.d_seg.template as<int32_t>(), d_act, in.rs.template as<int64_t>(),
-                          in.re.template as<int64_t>(), in.col.template as<int32_t>(), in.val.p,
-                          is_f32<T>(), w.ms.as<MatScalars>(), out.d_rp(), out.d_col(), out.val.p,
-                          s);
+      launch_filter_write(N, in.slots, st.d_seg.template as<int32_t>(), d_act,
+                          in.rs.template as<int64_t>(), in.re.template as<int64_t>(),
+                          in.col.template as<int32_t>(), in.val.p, is_f32<T>(),
+                          w.ms.as<MatScalars>(), out.d_rp(), out.d_col(), out.val.p, s);
     }
     ex.assign(hm.ex, hm.ex + nb + 1);
     if (dsum) dsum->assign(hm.dsum, hm.dsum + nb);
