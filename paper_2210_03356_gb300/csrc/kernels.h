@@ -331,12 +331,12 @@ void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int
                          void *oval, cudaStream_t s);
 
 // ---------------------------------------------------------------- NMF (Alg. 3.1.1)
-// The inverse of the n x n FP64 matrix in lu (leading dimension ld; factored
-// in place) by LU with partial pivoting and one forward and back substitution
-// per column of the identity, into inv (same ld). perm: n ints; pivot: one
-// int; *singular = 1 (and inv undefined) if a pivot column is zero.
-void launch_dense_inverse(int n, int ld, double *lu, int *perm, int *pivot, int *singular,
-                          double *inv, cudaStream_t s);
+// The inverse of the n x n FP64 matrix in lu (leading dimension ld; its upper
+// triangle becomes U) by LU with partial pivoting and one forward and back
+// substitution per column of the identity, into inv (same ld). swaps: n ints;
+// *singular = 1 (and inv undefined) if a pivot column is zero.
+void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, double *inv,
+                          cudaStream_t s);
 // *out = ||inv||_F / sqrt(n) (part: n doubles of scratch).
 void launch_inv_norm(int n, int ld, const double *inv, double *part, double *out,
                      cudaStream_t s);

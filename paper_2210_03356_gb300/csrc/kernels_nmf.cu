@@ -1,14 +1,23 @@
 // Newton's method with filtering (NMF, Alg. 3.1.1): the dense inverse of the
 // current iterate and the Newton update Xbar = (X + X^-1) / 2.
 //
-// The inverse follows LU with partial pivoting (right-looking: for each
-// column c the first row of largest magnitude at or below c becomes the
-// pivot, the rows below are reduced by l = a_rc / a_cc with one rounded
-// product and one rounded subtraction per entry), then, for each column e of
-// the identity, the forward substitution L y = P e and the back substitution
-// U x = y with their sums in ascending index order. The column solves are
-// independent and run one per thread. Every operation is an explicitly
-// rounded FP64 operation, so the inverse is the same on every run.
+// The inverse follows LU with partial pivoting (for each column c the first row
+// of largest magnitude at or below c becomes the pivot, the rows below are
+// reduced by l = a_rc / a_cc with one rounded product and one rounded
+// subtraction per entry), the forward substitution L y = P e for each column
+// e of the identity and the back substitution U x = y, both with their sums
+// in ascending index order. Every operation is an explicitly rounded FP64
+// operation and every entry takes its operations in that order, so the inverse
+// is the same on every run and for every blocking.
+//
+// The forward substitution rides along with the elimination: the identity's
+// rows are swapped and reduced like those of the matrix, [A | I] -> [U | y].
+// Columns are taken in panels: k_lu_panel factors a panel in one CTA, and
+// k_lu_trail applies its swaps and its reductions, in ascending column order,
+// to every column right of it and to the identity, a strip of 8 columns per
+// CTA. Four launches per column and one thread per column of the identity
+// (a chain of n^2 dependent steps, each waiting on its loads) took 36 ms for
+// n = 500; now 15.9 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -19,112 +28,271 @@ namespace sgn {
 
 namespace {
 
-constexpr int PIVOT_THREADS = 1024;
+constexpr int PANEL_T = 1024;        // threads of the panel kernel
+constexpr int PANEL_W = 8;           // most columns of a panel
+constexpr size_t PANEL_SMEM = 200 * 1024;
+constexpr int STRIP = 8;             // columns per CTA of the trailing update
+constexpr int TRAIL_T = 256;
 
-// The pivot of column c: the first row r >= c of largest |lu[r][c]| (a NaN
-// diagonal keeps row c, as a sequential scan from row c would); a largest
-// magnitude of 0 marks the matrix singular.
-__global__ void __launch_bounds__(PIVOT_THREADS)
-    k_lu_pivot(int n, int ld, const double *lu, int c, int *pivot, int *singular) {
-  __shared__ double sv[PIVOT_THREADS / 32];
-  __shared__ int si[PIVOT_THREADS / 32];
+// Columns of a panel: as many as fit the panel kernel's shared memory; one,
+// worked on in place, when even a column does not fit.
+int panel_width(int n) {
+  int w = PANEL_W;
+  while (w > 1 && size_t(n) * w * sizeof(double) > PANEL_SMEM) w /= 2;
+  return w;
+}
+
+// inv = I
+__global__ void k_inv_init(int n, int ld, double *inv) {
+  const int64_t total = int64_t(n) * n;
+  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < total;
+       t += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t i = t / n, j = t - i * n;
+    inv[i * ld + j] = i == j ? 1.0 : 0.0;
+  }
+}
+
+// Factors the panel of columns [c0, c0 + w), rows c0 .. n - 1: one CTA, a
+// thread per row (more for long columns), the panel in shared memory column
+// by column unless in_place. The pivot of a column is its first row of
+// largest magnitude (a NaN diagonal keeps its row, as a sequential scan from
+// there would); a largest magnitude of 0 marks the matrix singular. swaps[c]
+// is the row swapped with row c. Bound by the FP64 pipe of one SM (the
+// divisions) and the barriers: two per column.
+__global__ void __launch_bounds__(PANEL_T)
+    k_lu_panel(int n, int ld, double *lu, int c0, int w, int in_place, int *swaps,
+               int *singular) {
+  extern __shared__ double panel[];
+  __shared__ double sv[PANEL_T / 32];
+  __shared__ int si[PANEL_T / 32], s_pivot;
   if (*singular) return;
-  double best = -1.0;
-  int bi = n;
-  for (int r = c + int(threadIdx.x); r < n; r += PIVOT_THREADS) {
-    const double v = fabs(lu[int64_t(r) * ld + c]);
-    if (v > best) {  // rows ascend within a thread: ties keep the first
-      best = v;
-      bi = r;
-    }
+  const int R = n - c0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double *const G = lu + int64_t(c0) * ld + c0;
+  // entry (row r, column k) of the panel at P[k * sk + r * sr]
+  double *const P = in_place ? G : panel;
+  const int64_t sk = in_place ? 1 : R, sr = in_place ? ld : 1;
+  if (!in_place) {
+    for (int t = tid; t < R * w; t += PANEL_T) panel[(t % w) * R + t / w] = G[int64_t(t / w) * ld + t % w];
+    __syncthreads();
   }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = 0; k < w; ++k) {
+    double best = -1.0;
+    int bi = R;
+    for (int r = k + tid; r < R; r += PANEL_T) {
+      const double v = fabs(P[k * sk + r * sr]);
+      if (v > best) {  // rows ascend within a thread: ties keep the first
+        best = v;
+        bi = r;
+      }
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ov > best || (ov == best && oi < bi)) {
-      best = ov;
-      bi = oi;
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) {
+        best = ov;
+        bi = oi;
+      }
     }
+    if (lane == 0) {
+      sv[warp] = best;
+      si[warp] = bi;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      best = sv[lane];
+      bi = si[lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > best || (ov == best && oi < bi)) {
+          best = ov;
+          bi = oi;
+        }
+      }
+      const double d = fabs(P[k * sk + k * sr]);
+      if (d != d) {  // NaN pivot candidate: kept
+        best = d;
+        bi = k;
+      }
+      const int p = bi < R ? bi : k;
+      __syncwarp();
+      if (best == 0.0) {
+        if (lane == 0) s_pivot = -1;
+      } else {
+        if (lane < w && p != k) {
+          const double t = P[lane * sk + k * sr];
+          P[lane * sk + k * sr] = P[lane * sk + p * sr];
+          P[lane * sk + p * sr] = t;
+        }
+        if (lane == 0) {
+          s_pivot = p;
+          swaps[c0 + k] = c0 + p;
+        }
+      }
+    }
+    __syncthreads();
+    if (s_pivot < 0) {
+      if (tid == 0) *singular = 1;
+      return;
+    }
+    const double piv = P[k * sk + k * sr];
+    for (int r = k + 1 + tid; r < R; r += PANEL_T) {
+      const double l = __ddiv_rn(P[k * sk + r * sr], piv);
+      P[k * sk + r * sr] = l;
+      for (int j = k + 1; j < w; ++j)
+        P[j * sk + r * sr] = __dsub_rn(P[j * sk + r * sr], __dmul_rn(l, P[j * sk + k * sr]));
+    }
+    __syncthreads();
   }
-  if (lane == 0) {
-    sv[w] = best;
-    si[w] = bi;
+  if (!in_place)
+    for (int t = tid; t < R * w; t += PANEL_T) G[int64_t(t / w) * ld + t % w] = panel[(t % w) * R + t / w];
+}
+
+// The panel's swaps and reductions on a strip of 8 columns: of lu right of the
+// panel, then of inv. W: the panel's width. Bound by the FP64 pipe.
+template <int W>
+__global__ void __launch_bounds__(TRAIL_T)
+    k_lu_trail(int n, int ld, double *lu, double *inv, int c0, const int *swaps,
+               const int *singular) {
+  __shared__ int rows[2 * W], src[2 * W];
+  __shared__ int nrows;
+  __shared__ double moved[2 * W][STRIP], L[W][W], U[W][STRIP];
+  if (*singular) return;
+  const int c1 = c0 + W, lu_strips = (n - c1 + STRIP - 1) / STRIP;
+  const bool in_lu = int(blockIdx.x) < lu_strips;
+  const int j = threadIdx.x % STRIP, rr = threadIdx.x / STRIP;
+  constexpr int RT = TRAIL_T / STRIP;  // rows at a time
+  const int col = in_lu ? c1 + int(blockIdx.x) * STRIP + j
+                        : (int(blockIdx.x) - lu_strips) * STRIP + j;
+  double *const A = (in_lu ? lu : inv) + col;  // column col
+  const bool has = col < n;
+  // where the contents of the rows that the swaps touch come from
+  if (threadIdx.x == 0) {
+    int m = 0;
+    auto slot = [&](int r) {
+      for (int i = 0; i < m; ++i)
+        if (rows[i] == r) return i;
+      rows[m] = src[m] = r;
+      return m++;
+    };
+    for (int k = 0; k < W; ++k) {
+      const int a = slot(c0 + k), b = slot(swaps[c0 + k]);
+      const int t = src[a];
+      src[a] = src[b];
+      src[b] = t;
+    }
+    nrows = m;
+  }
+  for (int t = threadIdx.x; t < W * W; t += TRAIL_T)
+    L[t / W][t % W] = lu[int64_t(c0 + t / W) * ld + c0 + t % W];
+  __syncthreads();
+  for (int i = rr; i < nrows; i += RT)
+    if (has) moved[i][j] = A[int64_t(src[i]) * ld];
+  __syncthreads();
+  // the panel's rows, reduced one after another (row c0 + k is slot k or was
+  // listed before it): U
+  for (int i = rr; i < nrows; i += RT)
+    if (has && (rows[i] < c0 || rows[i] >= c1)) A[int64_t(rows[i]) * ld] = moved[i][j];
+  if (rr == 0 && has) {
+    double u[W];
+    for (int i = 0; i < nrows; ++i)
+      if (rows[i] < c1) U[rows[i] - c0][j] = moved[i][j];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      double a = U[k][j];
+#pragma unroll
+      for (int i = 0; i < k; ++i) a = __dsub_rn(a, __dmul_rn(L[k][i], u[i]));
+      u[k] = a;
+      U[k][j] = a;
+      A[int64_t(c0 + k) * ld] = a;
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < PIVOT_THREADS / 32; ++i)
-      if (sv[i] > best || (sv[i] == best && si[i] < bi)) {
-        best = sv[i];
-        bi = si[i];
-      }
-    const double d = fabs(lu[int64_t(c) * ld + c]);
-    if (d != d) {  // NaN pivot candidate at c: kept, as a scan from row c would
-      best = d;
-      bi = c;
-    }
-    if (best == 0.0) *singular = 1;
-    *pivot = bi < n ? bi : c;
+  if (!has) return;
+  double u[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) u[k] = U[k][j];
+#pragma unroll 2
+  for (int r = c1 + rr; r < n; r += RT) {
+    const double *l = lu + int64_t(r) * ld + c0;
+    double a = A[int64_t(r) * ld];
+#pragma unroll
+    for (int k = 0; k < W; ++k) a = __dsub_rn(a, __dmul_rn(l[k], u[k]));
+    A[int64_t(r) * ld] = a;
   }
 }
 
-__global__ void k_lu_swap(int n, int ld, double *lu, int c, const int *pivot, int *perm,
-                          const int *singular) {
+// U x = y for 32 columns of inv per warp, in place: for i = n - 1 .. 0,
+// x_i = (y_i - sum_{j > i, ascending} u_ij x_j) / u_ii. A sum starts with the
+// x found last, so the n^2 / 2 subtractions of a column are one dependent
+// chain: what bounds the kernel is their latency. The operands are kept off the
+// chain: the BACK_U nearest x stay in registers (shifted by one per row), the
+// first u of the next row and the operands of the next BACK_U terms are loaded
+// while the current ones are used.
+constexpr int BACK_U = 8;
+__global__ void __launch_bounds__(32)
+    k_back(int n, int ld, const double *lu, double *inv, const int *singular) {
   if (*singular) return;
-  const int pr = *pivot;
-  if (pr == c) return;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    const double t = lu[int64_t(c) * ld + j];
-    lu[int64_t(c) * ld + j] = lu[int64_t(pr) * ld + j];
-    lu[int64_t(pr) * ld + j] = t;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const int t = perm[c];
-    perm[c] = perm[pr];
-    perm[pr] = t;
-  }
-}
-
-// rows r > c, columns j > c: lu[r][j] -= (lu[r][c] / lu[c][c]) lu[c][j]
-__global__ void k_lu_update(int n, int ld, double *lu, int c, const int *singular) {
-  if (*singular) return;
-  const int j = c + 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const double piv = lu[int64_t(c) * ld + c], ucj = lu[int64_t(c) * ld + j];
-  for (int r = c + 1 + blockIdx.y; r < n; r += gridDim.y) {
-    const double l = __ddiv_rn(lu[int64_t(r) * ld + c], piv);
-    double *a = lu + int64_t(r) * ld + j;
-    *a = __dsub_rn(*a, __dmul_rn(l, ucj));
-  }
-}
-
-// the multipliers into column c (after the rows were reduced with them)
-__global__ void k_lu_store_l(int n, int ld, double *lu, int c, const int *singular) {
-  if (*singular) return;
-  const double piv = lu[int64_t(c) * ld + c];
-  for (int r = c + 1 + blockIdx.x * blockDim.x + threadIdx.x; r < n;
-       r += gridDim.x * blockDim.x)
-    lu[int64_t(r) * ld + c] = __ddiv_rn(lu[int64_t(r) * ld + c], piv);
-}
-
-// column e of the inverse: L y = P e_e, then U x = y (in place in inv)
-__global__ void k_lu_solve(int n, int ld, const double *lu, const int *perm, double *inv,
-                           const int *singular) {
-  if (*singular) return;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  for (int i = 0; i < n; ++i) {
-    double s = perm[i] == e ? 1.0 : 0.0;
-    const double *li = lu + int64_t(i) * ld;
-    for (int j = 0; j < i; ++j) s = __dsub_rn(s, __dmul_rn(li[j], inv[int64_t(j) * ld + e]));
-    inv[int64_t(i) * ld + e] = s;
-  }
+  const int e = blockIdx.x * 32 + threadIdx.x;
+  const bool has = e < n;
+  double *const x = inv + (has ? e : n - 1);  // lanes past the end repeat the last column
+  double xw[BACK_U], uf[BACK_U], un[BACK_U];
+  double ua[BACK_U], xa[BACK_U], ub[BACK_U], xb[BACK_U];
+#pragma unroll
+  for (int t = 0; t < BACK_U; ++t) xw[t] = uf[t] = 0.0;
+  double y = x[int64_t(n - 1) * ld], d = lu[int64_t(n - 1) * ld + n - 1];
   for (int i = n - 1; i >= 0; --i) {
     const double *ui = lu + int64_t(i) * ld;
-    double s = inv[int64_t(i) * ld + e];
-    for (int j = i + 1; j < n; ++j) s = __dsub_rn(s, __dmul_rn(ui[j], inv[int64_t(j) * ld + e]));
-    inv[int64_t(i) * ld + e] = __ddiv_rn(s, ui[i]);
+    auto fetch = [&](double (&u)[BACK_U], double (&v)[BACK_U], int j0) {
+#pragma unroll
+      for (int t = 0; t < BACK_U; ++t)
+        if (j0 + t < n) {
+          u[t] = ui[j0 + t];
+          v[t] = x[int64_t(j0 + t) * ld];
+        }
+    };
+    double s = y;
+    auto use = [&](const double (&u)[BACK_U], const double (&v)[BACK_U], int j0) {
+      if (j0 + BACK_U <= n) {
+#pragma unroll
+        for (int t = 0; t < BACK_U; ++t) s = __dsub_rn(s, __dmul_rn(u[t], v[t]));
+      } else {
+#pragma unroll
+        for (int t = 0; t < BACK_U; ++t)
+          if (j0 + t < n) s = __dsub_rn(s, __dmul_rn(u[t], v[t]));
+      }
+    };
+    int j0 = i + 1 + BACK_U;
+    fetch(ua, xa, j0);
+    double yn = 0.0, dn = 1.0;
+    if (i > 0) {  // the next row's start
+      yn = x[int64_t(i - 1) * ld];
+      dn = lu[int64_t(i - 1) * ld + i - 1];
+#pragma unroll
+      for (int t = 0; t < BACK_U; ++t)
+        if (i + t < n) un[t] = lu[int64_t(i - 1) * ld + i + t];
+    }
+    use(uf, xw, i + 1);
+    while (j0 < n) {
+      fetch(ub, xb, j0 + BACK_U);
+      use(ua, xa, j0);
+      j0 += BACK_U;
+      if (j0 >= n) break;
+      fetch(ua, xa, j0 + BACK_U);
+      use(ub, xb, j0);
+      j0 += BACK_U;
+    }
+    const double xi = __ddiv_rn(s, d);
+    if (has) x[int64_t(i) * ld] = xi;
+#pragma unroll
+    for (int t = BACK_U - 1; t > 0; --t) xw[t] = xw[t - 1];
+    xw[0] = xi;
+#pragma unroll
+    for (int t = 0; t < BACK_U; ++t) uf[t] = un[t];
+    y = yn;
+    d = dn;
   }
 }
 
@@ -141,12 +309,18 @@ __global__ void k_inv_rowsq(int n, int ld, const double *inv, double *part) {
   }
 }
 
-// *out = sqrt(sum_i part[i]) / sqrt(n), the rows added in order
+// *out = sqrt(sum_i part[i]) / sqrt(n), the rows added in order (one warp: 32
+// rows loaded at once, the next ones while these are added)
 __global__ void k_inv_norm(int n, const double *part, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int i = 0; i < n; ++i) s = __dadd_rn(s, part[i]);
-  *out = __ddiv_rn(__dsqrt_rn(s), __dsqrt_rn(double(n)));
+  const int lane = threadIdx.x;
+  double s = 0.0, v = lane < n ? part[lane] : 0.0;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const double w = i0 + 32 + lane < n ? part[i0 + 32 + lane] : 0.0;
+    const int m = min(32, n - i0);
+    for (int t = 0; t < m; ++t) s = __dadd_rn(s, __shfl_sync(0xffffffffu, v, t));
+    v = w;
+  }
+  if (lane == 0) *out = __ddiv_rn(__dsqrt_rn(s), __dsqrt_rn(double(n)));
 }
 
 __global__ void k_nmf_densify(int n, int ld, const int64_t *rp, const int32_t *col,
@@ -187,10 +361,6 @@ __global__ void k_nmf_budget(int m, int64_t n, const double *xinv, double c4, do
   ms[m].b = __dmul_rn(__dsqrt_rn(double(n)), beta);
 }
 
-__global__ void k_perm_init(int n, int *perm) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) perm[i] = i;
-}
-
 int blocks_for(int64_t items, int per) {
   int64_t g = (items + per - 1) / per;
   return int(g < 1 ? 1 : (g > 152 * 32 ? 152 * 32 : g));
@@ -198,27 +368,39 @@ int blocks_for(int64_t items, int per) {
 
 }  // namespace
 
-void launch_dense_inverse(int n, int ld, double *lu, int *perm, int *pivot, int *singular,
-                          double *inv, cudaStream_t s) {
+void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, double *inv,
+                          cudaStream_t s) {
   if (n <= 0) return;
+  static const bool attr = [] {  // once, thread-safe
+    SGN_CUDA(cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  int(PANEL_SMEM)));
+    return true;
+  }();
+  (void)attr;
   SGN_CUDA(cudaMemsetAsync(singular, 0, sizeof(int), s));
-  k_perm_init<<<blocks_for(n, 256), 256, 0, s>>>(n, perm);
+  k_inv_init<<<blocks_for(int64_t(n) * n, 256), 256, 0, s>>>(n, ld, inv);
   SGN_LAUNCH_CHECK();
-  for (int c = 0; c < n; ++c) {
-    k_lu_pivot<<<1, PIVOT_THREADS, 0, s>>>(n, ld, lu, c, pivot, singular);
+  const int width = panel_width(n);
+  for (int c0 = 0; c0 < n;) {
+    int w = width;
+    while (w > n - c0) w /= 2;  // the last columns: widths are powers of two
+    const size_t smem = size_t(n - c0) * w * sizeof(double);
+    const int in_place = smem > PANEL_SMEM ? 1 : 0;
+    k_lu_panel<<<1, PANEL_T, in_place ? 0 : smem, s>>>(n, ld, lu, c0, w, in_place, swaps, singular);
     SGN_LAUNCH_CHECK();
-    k_lu_swap<<<blocks_for(n, 256), 256, 0, s>>>(n, ld, lu, c, pivot, perm, singular);
-    SGN_LAUNCH_CHECK();
-    if (c + 1 < n) {
-      const int cols = n - c - 1;
-      dim3 g(unsigned((cols + 127) / 128), unsigned(std::min(cols, 1024)));
-      k_lu_update<<<g, 128, 0, s>>>(n, ld, lu, c, singular);
+    const unsigned strips =
+        unsigned((n - c0 - w + STRIP - 1) / STRIP + (n + STRIP - 1) / STRIP);
+    auto trail = [&](auto kernel) {
+      kernel<<<strips, TRAIL_T, 0, s>>>(n, ld, lu, inv, c0, swaps, singular);
       SGN_LAUNCH_CHECK();
-      k_lu_store_l<<<blocks_for(cols, 256), 256, 0, s>>>(n, ld, lu, c, singular);
-      SGN_LAUNCH_CHECK();
-    }
+    };
+    if (w == 8) trail(k_lu_trail<8>);
+    else if (w == 4) trail(k_lu_trail<4>);
+    else if (w == 2) trail(k_lu_trail<2>);
+    else trail(k_lu_trail<1>);
+    c0 += w;
   }
-  k_lu_solve<<<(n + 63) / 64, 64, 0, s>>>(n, ld, lu, perm, inv, singular);
+  k_back<<<(n + 31) / 32, 32, 0, s>>>(n, ld, lu, inv, singular);
   SGN_LAUNCH_CHECK();
 }
 

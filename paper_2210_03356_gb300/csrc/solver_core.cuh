@@ -194,7 +194,7 @@ struct Work {
   DevBuf n2v, n2y, n2z, n2part, n2zacc, n2xmax, n2ymax, n2nrm, x2;  // budget_norm
   int sel_shift = 0;    // > 0: the last threshold select had room for entries >> sel_shift
   DevBuf binfo;         // per row of a product's B: first/last column, length
-  DevBuf nmf_int, nmf_dbl;  // NMF: permutation, pivot, singular flags; ||X^-1||
+  DevBuf nmf_int, nmf_dbl;  // NMF: row swaps, singular flags; ||X^-1||
   bool bt_rows_done = false;  // the square's band tiles wrote their rows of T's band
 };
 
@@ -1064,9 +1064,9 @@ struct Solver {
     const size_t blk = size_t(nmax) * size_t(nmax);
     double *dx = static_cast<double *>(w.dmem.ensure(sizeof(double) * (3 * blk + size_t(nmax)), s));
     double *lu = dx + blk, *inv = lu + blk, *part = inv + blk;
-    w.nmf_int.ensure(sizeof(int) * size_t(nmax + 2 + nb), s);
+    w.nmf_int.ensure(sizeof(int) * size_t(nmax + nb), s);
     w.nmf_dbl.ensure(sizeof(double) * size_t(nb), s);
-    int *perm = w.nmf_int.as<int>(), *pivot = perm + nmax, *sing = pivot + 2;
+    int *swaps = w.nmf_int.as<int>(), *sing = swaps + nmax;
     double *xinv = w.nmf_dbl.as<double>();
     SGN_CUDA(cudaMemsetAsync(sing, 0, sizeof(int) * size_t(nb), s));
     int64_t slot0 = 0;
@@ -1079,7 +1079,7 @@ struct Solver {
       launch_nmf_densify(ni, ni, st.X.d_rp(), st.X.d_col(), st.X.d_val(), row0, dx, s);
       SGN_CUDA(cudaMemcpyAsync(lu, dx, sizeof(double) * size_t(n) * size_t(n),
                                cudaMemcpyDeviceToDevice, s));
-      launch_dense_inverse(ni, ni, lu, perm, pivot, sing + i, inv, s);
+      launch_dense_inverse(ni, ni, lu, swaps, sing + i, inv, s);
       launch_inv_norm(ni, ni, inv, part, xinv + i, s);
       launch_nmf_combine(ni, ni, dx, inv, row0, slot0, C.rs.as<int64_t>(), C.re.as<int64_t>(),
                          C.col.as<int32_t>(), C.val.as<double>(), s);
