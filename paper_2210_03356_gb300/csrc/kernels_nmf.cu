@@ -17,7 +17,7 @@
 // to every column right of it and to the identity, a strip of 8 columns per
 // CTA. Four launches per column and one thread per column of the identity
 // (a chain of n^2 dependent steps, each waiting on its loads) took 36 ms for
-// n = 500; now 15.9 ms.
+// n = 500; now 8.7 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -27,6 +27,28 @@
 namespace sgn {
 
 namespace {
+
+// Product and difference, each rounded once, as fused multiply-adds with an
+// exact factor or addend: fma(a, b, -0) is a b rounded (and keeps the sign of
+// a zero product), fma(b, -1, a) is a - b rounded. One FP64 warp instruction
+// occupies its quarter of the SM for 64 cycles as a DFMA and 76 as a DADD
+// (measured), and takes as long in a dependent chain.
+// In inline PTX, so that the compiler does not see a product and a difference
+// that it could contract into one rounding.
+__device__ __forceinline__ double fma_ptx(double a, double b, double c) {
+  double r;
+  asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
+  return r;
+}
+__device__ __forceinline__ double mul_rn(double a, double b) { return fma_ptx(a, b, -0.0); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return fma_ptx(b, -1.0, a); }
+
+// |v| as an integer that orders like it; a NaN orders below everything, as in
+// a scan with v > best.
+__device__ __forceinline__ long long mag_key(double v) {
+  const long long k = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+  return k > 0x7FF0000000000000ll ? -1ll : k;
+}
 
 constexpr int PANEL_T = 1024;        // threads of the panel kernel
 constexpr int PANEL_W = 8;           // most columns of a panel
@@ -63,7 +85,7 @@ __global__ void __launch_bounds__(PANEL_T)
     k_lu_panel(int n, int ld, double *lu, int c0, int w, int in_place, int *swaps,
                int *singular) {
   extern __shared__ double panel[];
-  __shared__ double sv[PANEL_T / 32];
+  __shared__ long long sv[PANEL_T / 32];
   __shared__ int si[PANEL_T / 32], s_pivot;
   if (*singular) return;
   const int R = n - c0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -76,10 +98,10 @@ __global__ void __launch_bounds__(PANEL_T)
     __syncthreads();
   }
   for (int k = 0; k < w; ++k) {
-    double best = -1.0;
+    long long best = -1;
     int bi = R;
     for (int r = k + tid; r < R; r += PANEL_T) {
-      const double v = fabs(P[k * sk + r * sr]);
+      const long long v = mag_key(P[k * sk + r * sr]);
       if (v > best) {  // rows ascend within a thread: ties keep the first
         best = v;
         bi = r;
@@ -87,7 +109,7 @@ __global__ void __launch_bounds__(PANEL_T)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
       const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
       if (ov > best || (ov == best && oi < bi)) {
         best = ov;
@@ -104,21 +126,21 @@ __global__ void __launch_bounds__(PANEL_T)
       bi = si[lane];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ov > best || (ov == best && oi < bi)) {
           best = ov;
           bi = oi;
         }
       }
-      const double d = fabs(P[k * sk + k * sr]);
+      const double d = P[k * sk + k * sr];
       if (d != d) {  // NaN pivot candidate: kept
-        best = d;
+        best = 1;
         bi = k;
       }
       const int p = bi < R ? bi : k;
       __syncwarp();
-      if (best == 0.0) {
+      if (best == 0) {
         if (lane == 0) s_pivot = -1;
       } else {
         if (lane < w && p != k) {
@@ -142,7 +164,7 @@ __global__ void __launch_bounds__(PANEL_T)
       const double l = __ddiv_rn(P[k * sk + r * sr], piv);
       P[k * sk + r * sr] = l;
       for (int j = k + 1; j < w; ++j)
-        P[j * sk + r * sr] = __dsub_rn(P[j * sk + r * sr], __dmul_rn(l, P[j * sk + k * sr]));
+        P[j * sk + r * sr] = sub_rn(P[j * sk + r * sr], mul_rn(l, P[j * sk + k * sr]));
     }
     __syncthreads();
   }
@@ -203,7 +225,7 @@ __global__ void __launch_bounds__(TRAIL_T)
     for (int k = 0; k < W; ++k) {
       double a = U[k][j];
 #pragma unroll
-      for (int i = 0; i < k; ++i) a = __dsub_rn(a, __dmul_rn(L[k][i], u[i]));
+      for (int i = 0; i < k; ++i) a = sub_rn(a, mul_rn(L[k][i], u[i]));
       u[k] = a;
       U[k][j] = a;
       A[int64_t(c0 + k) * ld] = a;
@@ -219,80 +241,89 @@ __global__ void __launch_bounds__(TRAIL_T)
     const double *l = lu + int64_t(r) * ld + c0;
     double a = A[int64_t(r) * ld];
 #pragma unroll
-    for (int k = 0; k < W; ++k) a = __dsub_rn(a, __dmul_rn(l[k], u[k]));
+    for (int k = 0; k < W; ++k) a = sub_rn(a, mul_rn(l[k], u[k]));
     A[int64_t(r) * ld] = a;
   }
 }
 
-// U x = y for 32 columns of inv per warp, in place: for i = n - 1 .. 0,
+// U x = y for 32 columns of inv per CTA, in place: for i = n - 1 .. 0,
 // x_i = (y_i - sum_{j > i, ascending} u_ij x_j) / u_ii. A sum starts with the
 // x found last, so the n^2 / 2 subtractions of a column are one dependent
-// chain: what bounds the kernel is their latency. The operands are kept off the
-// chain: the BACK_U nearest x stay in registers (shifted by one per row), the
-// first u of the next row and the operands of the next BACK_U terms are loaded
-// while the current ones are used.
-constexpr int BACK_U = 8;
-__global__ void __launch_bounds__(32)
+// chain of 64-cycle instructions, which bounds the kernel. Warp 0 runs the
+// chain and nothing else; warps 1 .. 3, on the other quarters of the SM,
+// prepare the products, BACK_C at a time, one chunk ahead, through shared
+// memory. Only the product with the x found last is left to warp 0: the
+// chunks of row i start at j = i + 2, whose x is known a row earlier. One warp
+// doing both took 186 cycles per term (11.2 ms for n = 500), now 87 (5.6 ms).
+constexpr int BACK_P = 16;          // products per producer warp and chunk
+constexpr int BACK_C = 3 * BACK_P;  // products per chunk
+__global__ void __launch_bounds__(128)
     k_back(int n, int ld, const double *lu, double *inv, const int *singular) {
+  __shared__ double prod[2][BACK_C][32];
   if (*singular) return;
-  const int e = blockIdx.x * 32 + threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
   const bool has = e < n;
   double *const x = inv + (has ? e : n - 1);  // lanes past the end repeat the last column
-  double xw[BACK_U], uf[BACK_U], un[BACK_U];
-  double ua[BACK_U], xa[BACK_U], ub[BACK_U], xb[BACK_U];
-#pragma unroll
-  for (int t = 0; t < BACK_U; ++t) xw[t] = uf[t] = 0.0;
-  double y = x[int64_t(n - 1) * ld], d = lu[int64_t(n - 1) * ld + n - 1];
-  for (int i = n - 1; i >= 0; --i) {
+  // products of the chunk of row i that starts at column j0
+  auto produce = [&](double (*p)[32], int i, int j0) {
     const double *ui = lu + int64_t(i) * ld;
-    auto fetch = [&](double (&u)[BACK_U], double (&v)[BACK_U], int j0) {
+    const int j1 = j0 + (warp - 1) * BACK_P;
+    double u[BACK_P], v[BACK_P];
 #pragma unroll
-      for (int t = 0; t < BACK_U; ++t)
-        if (j0 + t < n) {
-          u[t] = ui[j0 + t];
-          v[t] = x[int64_t(j0 + t) * ld];
-        }
-    };
-    double s = y;
-    auto use = [&](const double (&u)[BACK_U], const double (&v)[BACK_U], int j0) {
-      if (j0 + BACK_U <= n) {
-#pragma unroll
-        for (int t = 0; t < BACK_U; ++t) s = __dsub_rn(s, __dmul_rn(u[t], v[t]));
-      } else {
-#pragma unroll
-        for (int t = 0; t < BACK_U; ++t)
-          if (j0 + t < n) s = __dsub_rn(s, __dmul_rn(u[t], v[t]));
+    for (int t = 0; t < BACK_P; ++t)
+      if (j1 + t < n) {
+        u[t] = ui[j1 + t];
+        v[t] = x[int64_t(j1 + t) * ld];
       }
-    };
-    int j0 = i + 1 + BACK_U;
-    fetch(ua, xa, j0);
-    double yn = 0.0, dn = 1.0;
-    if (i > 0) {  // the next row's start
-      yn = x[int64_t(i - 1) * ld];
-      dn = lu[int64_t(i - 1) * ld + i - 1];
 #pragma unroll
-      for (int t = 0; t < BACK_U; ++t)
-        if (i + t < n) un[t] = lu[int64_t(i - 1) * ld + i + t];
+    for (int t = 0; t < BACK_P; ++t)
+      if (j1 + t < n) p[(warp - 1) * BACK_P + t][lane] = mul_rn(u[t], v[t]);
+  };
+  // the chunks in order: row i, columns from j0; every row has at least one
+  int i = n - 1, j0 = n + 1, buf = 0;
+  if (warp > 0) produce(prod[0], i, j0);
+  __syncthreads();
+  double s = 0.0, xl = 0.0;  // the row's sum, the x found last
+  double y = 0.0, d = 0.0, u1 = 0.0;
+  if (warp == 0) {
+    y = x[int64_t(i) * ld];
+    d = lu[int64_t(i) * ld + i];
+  }
+  for (bool first = true; i >= 0;) {
+    const bool last = j0 + BACK_C >= n;  // the row's last chunk
+    const int ni = last ? i - 1 : i, nj0 = last ? i + 1 : j0 + BACK_C;
+    if (warp > 0) {
+      if (ni >= 0) produce(prod[buf ^ 1], ni, nj0);
+    } else {
+      if (first) s = i + 1 < n ? sub_rn(y, mul_rn(u1, xl)) : y;
+      double yn = 0.0, dn = 0.0, un = 0.0;
+      if (last && i > 0) {  // the next row's start
+        yn = x[int64_t(i - 1) * ld];
+        dn = lu[int64_t(i - 1) * ld + i - 1];
+        un = lu[int64_t(i - 1) * ld + i];
+      }
+      const int m = min(BACK_C, n - j0);
+      if (m == BACK_C) {
+#pragma unroll 16
+        for (int t = 0; t < BACK_C; ++t) s = sub_rn(s, prod[buf][t][lane]);
+      } else {
+#pragma unroll 4
+        for (int t = 0; t < m; ++t) s = sub_rn(s, prod[buf][t][lane]);
+      }
+      if (last) {
+        xl = __ddiv_rn(s, d);
+        if (has) x[int64_t(i) * ld] = xl;
+        y = yn;
+        d = dn;
+        u1 = un;
+      }
     }
-    use(uf, xw, i + 1);
-    while (j0 < n) {
-      fetch(ub, xb, j0 + BACK_U);
-      use(ua, xa, j0);
-      j0 += BACK_U;
-      if (j0 >= n) break;
-      fetch(ua, xa, j0 + BACK_U);
-      use(ub, xb, j0);
-      j0 += BACK_U;
-    }
-    const double xi = __ddiv_rn(s, d);
-    if (has) x[int64_t(i) * ld] = xi;
-#pragma unroll
-    for (int t = BACK_U - 1; t > 0; --t) xw[t] = xw[t - 1];
-    xw[0] = xi;
-#pragma unroll
-    for (int t = 0; t < BACK_U; ++t) uf[t] = un[t];
-    y = yn;
-    d = dn;
+    __syncthreads();
+    first = last;
+    i = ni;
+    j0 = nj0;
+    buf ^= 1;
   }
 }
 
@@ -400,7 +431,7 @@ void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, 
     else trail(k_lu_trail<1>);
     c0 += w;
   }
-  k_back<<<(n + 31) / 32, 32, 0, s>>>(n, ld, lu, inv, singular);
+  k_back<<<(n + 31) / 32, 128, 0, s>>>(n, ld, lu, inv, singular);
   SGN_LAUNCH_CHECK();
 }
 
