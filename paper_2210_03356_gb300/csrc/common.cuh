@@ -34,16 +34,9 @@ void count_launch();
   } while (0)
 
 // Shared-memory row accumulators: rows whose column range fits WARP_W slots
-// are handled by one warp; wider rows by one CTA in chunks of CTA_W slots.
+// are handled by one warp; wider rows in windows of WARP_W columns.
 constexpr int WARP_W = 1024;
 constexpr int WARPS_PER_CTA = 4;
-constexpr int CTA_THREADS = 256;
-template <typename T> struct CtaW;
-template <> struct CtaW<double> { static constexpr int value = 12288; };
-template <> struct CtaW<float> { static constexpr int value = 20480; };
-// symbolic pass of wide rows: one bitmap covering up to SYM_BITS columns
-constexpr int SYM_BITS = 1 << 18;
-constexpr int K_BATCH = 256;  // k entries whose B-row ranges are located at once
 
 // Kernel classes timed when profiling is on (sign_prof_enable).
 enum KClass {

@@ -132,7 +132,7 @@ struct Rows {
 };
 
 // Row classes of the numeric kernels: groups of 32, 16 or 8 lanes per row,
-// one CTA per row, or band tiles of 16 rows (FP32 only; the list holds each
+// windows of wide rows (RC_CTA), or band tiles of 16 rows (FP32 only; the list holds each
 // tile's first row).
 enum RowClass { RC_G32 = 0, RC_CTA = 1, RC_G16 = 2, RC_G8 = 3, RC_BAND = 4, RC_NONE = 5, RC_N = 5 };
 constexpr int RC_QUEUE = RC_N;        // counters[RC_QUEUE + c]: work-queue head of class c
@@ -211,7 +211,7 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
                          const int32_t *len, const int32_t *lists, int *counters,
                          const int64_t *cs, int64_t *ce, int32_t *ccol, float *cval, double *part,
                          cudaStream_t s);
-// Numeric product. Row i is written at cs[i] (exclusive scan of ub) and its
+// Numeric product of the rows up to WARP_W columns wide. Row i is written at cs[i] (exclusive scan of ub) and its
 // end stored in ce[i]. MODE_SQUARE: C = A A, and part[2i] = sum_j (C_ij -
 // delta_ij)^2, part[2i+1] = sum_k a_ik^2. MODE_UPDATE: C = 1.5 A - 0.5 A B.
 // The part entries of dense-path matrices (dslot nullable; dslot[seg[i]] >= 0)
@@ -222,6 +222,25 @@ void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, cons
                     const int *dslot, const int32_t *lists, const int *counters,
                     const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                     cudaStream_t s);
+
+// The rows of more than WARP_W columns (the RC_CTA list, `rows` of them).
+// mean_b: the mean length of the B rows that products read. off: scratch of
+// n * wt.stride ints for B's column-block table, or null (binary search in
+// its place); wt: the rows' matrices, the block width 1 << sh and the table's
+// row stride, (max matrix order >> sh) + 2.
+struct WideTable {
+  const int32_t *seg;
+  const int64_t *moff;
+  const int *off;
+  int sh, stride;
+};
+int wide_block_shift(int64_t max_n);
+template <typename T>
+void launch_numeric_wide(int64_t n, int rows, double mean_b, const Rows &A, const T *aval,
+                         const Rows &B, const T *bval, int mode, WideTable wt, int *off,
+                         const int32_t *lo, const int32_t *len, const int32_t *lists,
+                         int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
+                         double *part, cudaStream_t s);
 
 // ---------------------------------------------------------------- filter
 // Per-matrix scalars after the check of the current iterates.

@@ -9,8 +9,9 @@
 // Row i of C = A B is accumulated in shared memory over its column range
 // [lo_i, lo_i + len_i) (union of the ranges of the rows B_k, k in A_i), indexed
 // by column - lo_i, so the output comes out in ascending column order without
-// hashing or sorting. Rows with len <= WARP_W go to one warp each; wider rows
-// to one CTA each, in chunks of CTA_W columns.
+// hashing or sorting. Rows with len <= WARP_W go to one warp each; the columns
+// of wider rows are split over the windows of one or several warps, each of
+// which runs through all k on its own columns.
 //
 // No symbolic pass: each output row gets a slot of ub_i = min(len_i, work_i)
 // entries (work_i = multiply-adds of the row, plus the row of A itself in
@@ -718,97 +719,186 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
   }
 }
 
-template <typename T>
-constexpr size_t num_cta_smem() {
-  return size_t(CtaW<T>::value) * (sizeof(T) + 1) + 2 * K_BATCH * sizeof(int64_t);
+// Column blocks of B's rows: off[k * stride + b] is the number of entries of
+// row k in columns before block b (blocks of 1 << sh columns from the first
+// column of the row's matrix), b = 0 .. stride - 1. A warp per row.
+__global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
+                             const int32_t *seg, const int64_t *moff, int sh, int stride,
+                             int *off) {
+  const int lane = lane_id();
+  const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+  for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
+    const int64_t a = rs[r], e = re[r], base = moff[seg[r]];
+    int *o = off + r * stride;
+    int last = -1;  // block of the entry before the chunk
+    for (int64_t p0 = a; p0 < e; p0 += 32) {
+      const int64_t p = p0 + lane;
+      const int b = p < e ? int((col[p] - base) >> sh) : stride - 1;
+      int prev = __shfl_up_sync(0xffffffffu, b, 1);
+      if (lane == 0) prev = last;
+      if (p < e)
+        for (int i = prev + 1; i <= b; ++i) o[i] = int(p - a);
+      last = __shfl_sync(0xffffffffu, b, int(min(int64_t(31), e - 1 - p0)));
+    }
+    for (int i = last + 1 + lane; i < stride; i += 32) o[i] = int(e - a);
+  }
 }
 
-template <typename T, int MODE>
-__global__ void __launch_bounds__(CTA_THREADS)
-    k_num_cta(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
-              const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
-              const int32_t *lo, const int32_t *len, const int32_t *clist, int *counters,
-              const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
-  constexpr int CW = CtaW<T>::value;
-  // the CTA class uses counters[RC_CTA] (length) and counters[RC_QUEUE + RC_CTA] (queue head)
-  constexpr int NW = CTA_THREADS / 32;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int64_t *ks = reinterpret_cast<int64_t *>(smem_raw);
-  int64_t *ke = ks + K_BATCH;
-  T *acc = reinterpret_cast<T *>(ke + K_BATCH);
-  unsigned char *f = reinterpret_cast<unsigned char *>(acc + CW);
-  __shared__ int s_idx;
-  __shared__ int s_cnt[NW];
-  __shared__ double s_red[2][NW];
-  int lane = lane_id(), w = threadIdx.x >> 5;
+// Rows of more than WARP_W columns. P warps (a power of two up to 8) take a row
+// together, each a window of at most WARP_W columns of it at a time: the warp
+// runs through the k of A_i in ascending order and adds the part of B_k that
+// falls in its window, found in the column-block table (or, without one, by
+// binary search), so no barrier separates the k; the warps of a row meet only
+// to add up their entry counts before each writes its part. P follows the
+// mean length of B's rows: enough entries of B_k per warp to fill its lanes
+// (an FP64 instruction costs the pipe the same whatever its active lanes).
+// One CTA per row with a barrier per k took 12.0 and 6.0 ms for the update and
+// the square of the 16^3 Laplacian's FP32 iterate just below the dense path's
+// density, now 7.8 and 4.0.
+constexpr int WIDE_WARPS = 8;
+constexpr int WIDE_K = 4;  // k whose first 32 entries are loaded ahead
+template <typename T>
+constexpr int wide_occ() { return sizeof(T) == 8 ? 3 : 5; }  // CTAs per SM
+template <typename T>
+constexpr size_t wide_smem() { return size_t(WIDE_WARPS) * WARP_W * (sizeof(T) + 1); }
+
+template <typename T, int MODE, int P>
+__global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
+    k_num_wide(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
+               const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
+               const int32_t *seg, const int64_t *moff, const int *off, int sh, int stride,
+               const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
+               const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool MARK = sizeof(T) == 4;  // untouched FP32 slots hold -0 (see mac)
+  constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
+  extern __shared__ __align__(16) unsigned char wide_smem_raw[];
+  __shared__ int s_idx[NG], s_cnt[WIDE_WARPS];
+  __shared__ double s_red[2][WIDE_WARPS];
+  __shared__ int s_diag[WIDE_WARPS];
+  const int lane = lane_id(), w = threadIdx.x >> 5, g = w / P, wr = w % P;
   const unsigned lt = (1u << lane) - 1u;
+  T *acc = reinterpret_cast<T *>(wide_smem_raw) + w * WARP_W;
+  unsigned char *f = wide_smem_raw + size_t(WIDE_WARPS) * WARP_W * sizeof(T) + w * WARP_W;
+  // the warps of one row
+  auto row_sync = [&] {
+    if constexpr (P == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(P * 32) : "memory");
+  };
+  const int total = counters[RC_CTA];
   for (;;) {
-    if (threadIdx.x == 0) s_idx = atomicAdd(&counters[RC_QUEUE + RC_CTA], 1);
-    __syncthreads();
-    int idx = s_idx;
-    __syncthreads();
-    if (idx >= counters[RC_CTA]) break;
-    int32_t r = clist[idx];
-    int64_t L = len[r];
-    int64_t base = lo[r];
-    int64_t a0 = ars[r], a1 = are[r];
-    int64_t nA = a1 - a0;
-    bool multi = L > CW;
+    if (wr == 0 && lane == 0) s_idx[g] = atomicAdd(&counters[RC_QUEUE + RC_CTA], 1);
+    row_sync();
+    const int idx = s_idx[g];
+    if (idx >= total) break;
+    const int32_t r = list[idx];
+    const int64_t base = moff[seg[r]], a0 = ars[r], a1 = are[r];
+    const int b0 = int((lo[r] - base) >> sh), b1 = int((int64_t(lo[r]) + len[r] - 1 - base) >> sh);
+    const int bpw = min(WARP_W >> sh, (b1 - b0 + P) / P);  // blocks per warp and window
     int64_t out = cs[r];
     double rs = 0.0;
     bool diag = false;
-    for (int64_t c0 = base; c0 < base + L; c0 += CW) {
-      int W = int(min(int64_t(CW), base + L - c0));
-      for (int s = threadIdx.x; s < W; s += CTA_THREADS) {
-        acc[s] = T(0);
-        f[s] = 0;
+    for (int win = b0; win <= b1; win += P * bpw) {
+      const int w0 = win + wr * bpw, w1 = min(w0 + bpw, b1 + 1);  // this warp's blocks
+      const bool has = w0 < w1;
+      const int64_t c0 = base + (int64_t(w0) << sh);
+      const int W = has ? (w1 - w0) << sh : 0;  // its columns
+      for (int s = lane; s < W; s += 32) {
+        acc[s] = MARK ? T(-0.0) : T(0);
+        if (!MARK || MODE == MODE_UPDATE) f[s] = 0;
       }
-      __syncthreads();
-      for (int64_t kb = 0; kb < nA; kb += K_BATCH) {
-        int nk = int(min(int64_t(K_BATCH), nA - kb));
-        if (threadIdx.x < nk) {
-          int32_t k = acol[a0 + kb + threadIdx.x];
-          int64_t s = brs[k], e = bre[k];
-          if (multi) {
-            s = lower_bound(bcol, s, e, c0);
-            e = lower_bound(bcol, s, e, c0 + W);
+      __syncwarp();
+      if (has) {
+        for (int64_t pb = a0; pb < a1; pb += 32) {
+          T av = T(0);
+          int64_t qs = 0;
+          int qn = 0;
+          if (pb + lane < a1) {
+            const int32_t k = acol[pb + lane];
+            av = aval[pb + lane];
+            qs = brs[k];
+            if (off) {
+              const int *o = off + int64_t(k) * stride;
+              const int o0 = o[w0];
+              qn = o[w1] - o0;
+              qs += o0;
+            } else {
+              const int64_t e = bre[k];
+              qs = lower_bound(bcol, qs, e, c0);
+              qn = int(lower_bound(bcol, qs, e, c0 + W) - qs);
+            }
           }
-          ks[threadIdx.x] = s;
-          ke[threadIdx.x] = e;
-        }
-        __syncthreads();
-        for (int t = 0; t < nk; ++t) {  // ascending k
-          accumulate_k<T, CTA_THREADS>(aval[a0 + kb + t], ks[t], ke[t], bcol, bval, c0, acc, f,
-                                       threadIdx.x);
-          __syncthreads();
-        }
-      }
-      if (MODE == MODE_UPDATE) {
-        for (int64_t p = a0 + threadIdx.x; p < a1; p += CTA_THREADS) {
-          int64_t j = int64_t(acol[p]) - c0;
-          if (j >= 0 && j < W) {
-            acc[j] = ns_combine(aval[p], acc[j]);
-            f[j] = 3;
+          unsigned todo = __ballot_sync(FULL, qn > 0);
+          while (todo) {  // ascending k, WIDE_K at a time
+            T a[WIDE_K], v[WIDE_K];
+            int64_t q0[WIDE_K];
+            int nn[WIDE_K], j[WIDE_K];
+#pragma unroll
+            for (int t = 0; t < WIDE_K; ++t) {
+              const int src = todo ? __ffs(todo) - 1 : 0;
+              const bool any = todo != 0;
+              todo &= todo - 1;
+              a[t] = __shfl_sync(FULL, av, src);
+              q0[t] = __shfl_sync(FULL, qs, src);
+              nn[t] = __shfl_sync(FULL, qn, src);
+              if (!any) nn[t] = 0;
+              if (lane < nn[t]) {
+                j[t] = int(bcol[q0[t] + lane] - c0);
+                v[t] = bval[q0[t] + lane];
+              }
+            }
+#pragma unroll
+            for (int t = 0; t < WIDE_K; ++t) {
+              if (lane < nn[t]) mac<T, MARK>(acc, f, j[t], a[t], v[t]);
+              if (nn[t] > 32)
+                accumulate_k<T, 32, MARK>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, f,
+                                          lane);
+              __syncwarp();
+            }
           }
         }
-        __syncthreads();
-      }
-      // ordered emission: round g covers words g*NW .. g*NW+NW-1, warp w one word
-      for (int s0 = 0; s0 < W; s0 += 32 * NW) {
-        int s = s0 + w * 32 + lane;
-        int fl = s < W ? f[s] : 0;
-        unsigned m = __ballot_sync(0xffffffffu, fl != 0);
-        if (lane == 0) s_cnt[w] = __popc(m);
-        __syncthreads();
-        int64_t wbase = out;
-        int64_t round_total = 0;
-        for (int i = 0; i < NW; ++i) {
-          if (i < w) wbase += s_cnt[i];
-          round_total += s_cnt[i];
+        if (MODE == MODE_UPDATE) {  // x_ij of the window
+          const int64_t x0 = lower_bound(acol, a0, a1, c0), x1 = lower_bound(acol, x0, a1, c0 + W);
+          for (int64_t p = x0 + lane; p < x1; p += 32) {
+            const int jx = int(acol[p] - c0);
+            T xt = acc[jx];
+            if (untouched<T, MARK>(xt)) xt = T(0);
+            acc[jx] = ns_combine(aval[p], xt);
+            f[jx] = 3;
+          }
+          __syncwarp();
         }
+      }
+      auto touched = [&](int s) -> int {
+        if (s >= W) return 0;
+        if (!MARK) return f[s];
+        int fl = MODE == MODE_UPDATE ? f[s] : 0;
+        if (!fl && !untouched<T, MARK>(acc[s])) fl = 1;
+        return fl;
+      };
+      int cnt = 0;
+      for (int s0 = 0; s0 < W; s0 += 32)
+        cnt += __popc(__ballot_sync(FULL, touched(s0 + lane) != 0));
+      int64_t at = out;
+      if constexpr (P > 1) {
+        if (lane == 0) s_cnt[w] = cnt;
+        row_sync();
+        for (int i = 0; i < P; ++i) {
+          const int ci = s_cnt[g * P + i];
+          if (i < wr) at += ci;
+          out += ci;
+        }
+      } else {
+        out += cnt;
+      }
+      for (int s0 = 0; s0 < W; s0 += 32) {
+        const int s = s0 + lane, fl = touched(s);
+        const unsigned mk = __ballot_sync(FULL, fl != 0);
         if (fl) {
-          int64_t pos = wbase + __popc(m & lt);
-          int64_t cj = c0 + s;
+          const int64_t pos = at + __popc(mk & lt);
+          const int64_t cj = c0 + s;
           T v = acc[s];
           if (MODE == MODE_UPDATE && !(fl & 2)) v = ns_combine(T(0), v);
           ccol[pos] = int32_t(cj);
@@ -822,39 +912,42 @@ __global__ void __launch_bounds__(CTA_THREADS)
             rs += d * d;
           }
         }
-        out += round_total;
-        __syncthreads();
+        at += __popc(mk);
       }
+      row_sync();  // s_cnt and the accumulators are free again
     }
-    if (threadIdx.x == 0) ce[r] = out;
+    if (wr == 0 && lane == 0) ce[r] = out;
     if (MODE == MODE_SQUARE) {
       double xs = 0.0;
-      for (int64_t p = a0 + threadIdx.x; p < a1; p += CTA_THREADS) {
-        double x = double(aval[p]);
+      for (int64_t p = a0 + wr * 32 + lane; p < a1; p += P * 32) {
+        const double x = double(aval[p]);
         xs += x * x;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        rs += __shfl_xor_sync(0xffffffffu, rs, o);
-        xs += __shfl_xor_sync(0xffffffffu, xs, o);
+        rs += __shfl_xor_sync(FULL, rs, o);
+        xs += __shfl_xor_sync(FULL, xs, o);
       }
-      int any_diag = __syncthreads_or(diag ? 1 : 0);
+      const bool dg = __any_sync(FULL, diag);
       if (lane == 0) {
         s_red[0][w] = rs;
         s_red[1][w] = xs;
+        s_diag[w] = dg ? 1 : 0;
       }
-      __syncthreads();
-      if (threadIdx.x == 0) {
+      row_sync();
+      if (wr == 0 && lane == 0) {
         double a = 0.0, b = 0.0;
-        for (int i = 0; i < NW; ++i) {
-          a += s_red[0][i];
-          b += s_red[1][i];
+        int any = 0;
+        for (int i = 0; i < P; ++i) {
+          a += s_red[0][w + i];
+          b += s_red[1][w + i];
+          any |= s_diag[w + i];
         }
-        part[2 * int64_t(r)] = any_diag ? a : a + 1.0;
+        part[2 * int64_t(r)] = any ? a : a + 1.0;
         part[2 * int64_t(r) + 1] = b;
       }
-      __syncthreads();
     }
+    row_sync();  // s_idx and s_red are read
   }
 }
 
@@ -965,18 +1058,80 @@ static void num_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, c
                                             ce, ccol, cval, part, s);
   group_launch<T, MODE, 8>(n, A, aval, B, bval, lo, len, lists, ctr, RC_G8, cs, ce, ccol, cval,
                            part, s);
-  constexpr size_t sm = num_cta_smem<T>();
+}
+
+template <typename T, int MODE, int P>
+static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, const T *bval,
+                        const WideTable &wt, const int32_t *lo, const int32_t *len,
+                        const int32_t *list, int *ctr, const int64_t *cs, int64_t *ce,
+                        int32_t *ccol, T *cval, double *part, cudaStream_t s) {
+  constexpr size_t sm = wide_smem<T>();
   static const bool attr = [] {  // once, thread-safe
-    SGN_CUDA(cudaFuncSetAttribute(k_num_cta<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  int(sm)));
+    SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
     return true;
   }();
   (void)attr;
-  k_num_cta<T, MODE><<<grid_cap(n, 1, 2), CTA_THREADS, sm, s>>>(
-      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, lo, len, lists + int64_t(RC_CTA) * n, ctr,
-      cs, ce, ccol, cval, part);
+  k_num_wide<T, MODE, P><<<grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()), WIDE_WARPS * 32, sm, s>>>(
+      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg, wt.moff, wt.off, wt.sh, wt.stride,
+      lo, len, list, ctr, cs, ce, ccol, cval, part);
   SGN_LAUNCH_CHECK();
 }
+
+template <typename T, int MODE>
+static void wide_launch_p(int rows, int p, const Rows &A, const T *aval, const Rows &B,
+                          const T *bval, const WideTable &wt, const int32_t *lo,
+                          const int32_t *len, const int32_t *list, int *ctr, const int64_t *cs,
+                          int64_t *ce, int32_t *ccol, T *cval, double *part, cudaStream_t s) {
+#define SGN_WIDE(P) \
+  wide_launch<T, MODE, P>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cs, ce, ccol, cval, part, s)
+  if (p >= 8) SGN_WIDE(8);
+  else if (p >= 4) SGN_WIDE(4);
+  else if (p >= 2) SGN_WIDE(2);
+  else SGN_WIDE(1);
+#undef SGN_WIDE
+}
+
+int wide_block_shift(int64_t max_n) {
+  int sh = 7;
+  while (sh < 9 && (max_n >> sh) >= 64) ++sh;
+  return sh;
+}
+
+template <typename T>
+void launch_numeric_wide(int64_t n, int rows, double mean_b, const Rows &A, const T *aval,
+                         const Rows &B, const T *bval, int mode, WideTable wt, int *off,
+                         const int32_t *lo, const int32_t *len, const int32_t *lists,
+                         int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
+                         double *part, cudaStream_t s) {
+  if (rows <= 0) return;
+  if (off) {
+    k_col_blocks<<<grid_cap(n, 8, 16), 256, 0, s>>>(n, B.rs, B.re, B.col, wt.seg, wt.moff, wt.sh,
+                                                    wt.stride, off);
+    SGN_LAUNCH_CHECK();
+  }
+  wt.off = off;
+  // warps per row: about 64 (FP32) or 128 (FP64) entries of a B row per warp
+  const double per = sizeof(T) == 8 ? 128.0 : 64.0;
+  const int p = mean_b >= 8 * per ? 8 : mean_b >= 4 * per ? 4 : mean_b >= 2 * per ? 2 : 1;
+  const int32_t *list = lists + int64_t(RC_CTA) * n;
+  if (mode == MODE_SQUARE)
+    wide_launch_p<T, MODE_SQUARE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cs, ce,
+                                  ccol, cval, part, s);
+  else
+    wide_launch_p<T, MODE_UPDATE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cs, ce,
+                                  ccol, cval, part, s);
+}
+template void launch_numeric_wide<double>(int64_t, int, double, const Rows &, const double *,
+                                          const Rows &, const double *, int, WideTable, int *,
+                                          const int32_t *, const int32_t *, const int32_t *, int *,
+                                          const int64_t *, int64_t *, int32_t *, double *,
+                                          double *, cudaStream_t);
+template void launch_numeric_wide<float>(int64_t, int, double, const Rows &, const float *,
+                                         const Rows &, const float *, int, WideTable, int *,
+                                         const int32_t *, const int32_t *, const int32_t *, int *,
+                                         const int64_t *, int64_t *, int32_t *, float *, double *,
+                                         cudaStream_t);
 
 template <typename T>
 void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,

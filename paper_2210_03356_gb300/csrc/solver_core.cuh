@@ -189,6 +189,7 @@ struct Work {
   DevBuf lo, len, ub, wlist, clist, counters, part, scan_tmp, eoff, sums, ms, active, sel,
       asm_blocks, asm_off, asm_lens, dropped, norm_work, norm, work, mults, cnt, nnzc, xblocks,
       dslot, dmem, dbufs, djobs, dscratch, dcount, derr;
+  DevBuf wide;     // column-block table of a product's B (wide rows)
   BandBuf bx, bt;  // bands of the iterate X and of T = X X (FP32 stage)
   DevBuf bandrow;  // rows of T written by the square's band tiles (1) or not (0)
   DevBuf n2v, n2y, n2z, n2part, n2zacc, n2xmax, n2ymax, n2nrm, x2;  // budget_norm
@@ -454,7 +455,6 @@ struct Solver {
                       w.scan_tmp.as<int64_t>(), s);
           d2h(hm.tot + 2, w.bt.pos.as<int64_t>() + N, 1, s);
         }
-        d2h(hm.ctr, w.counters.p, RC_COUNTERS, s);
         d2h(hm.dsum, band_work_dev(), 1, s);
       }
     }
@@ -467,6 +467,7 @@ struct Solver {
     }
     d2h(hm.tot, C.rs.template as<int64_t>() + N, 1, s);
     d2h(hm.mults, w.mults.p, size_t(nb), s);
+    d2h(hm.ctr, w.counters.p, RC_COUNTERS, s);
     wait();
     int64_t slots = hm.tot[0];
     const bool band_tiles = band && hm.ctr[RC_BAND] > 0;
@@ -527,6 +528,25 @@ struct Solver {
                         w.counters.as<int>(), C.rs.template as<int64_t>(),
                         C.re.template as<int64_t>(), C.col.template as<int32_t>(), C.d_val(),
                         mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
+      if (hm.ctr[RC_CTA] > 0) {
+        int64_t max_n = 0;
+        for (size_t i = 0; i + 1 < st.moff.size(); ++i)
+          max_n = std::max(max_n, st.moff[i + 1] - st.moff[i]);
+        const int sh = wide_block_shift(max_n), stride = int(max_n >> sh) + 2;
+        // B's column-block table when its rows mostly hold more entries than the
+        // table has columns; shorter rows are searched
+        int *off = nullptr;
+        if (double(nnzB) >= double(N) * double(stride))
+          off = static_cast<int *>(w.wide.ensure(sizeof(int) * size_t(N) * size_t(stride), s));
+        launch_numeric_wide<T>(N, hm.ctr[RC_CTA], fl / (2.0 * double(nnzA > 0 ? nnzA : 1)), A,
+                               aval, B, bval, mode,
+                               WideTable{st.d_seg.template as<int32_t>(),
+                                         st.d_moff.template as<int64_t>(), nullptr, sh, stride},
+                               off, w.lo.as<int32_t>(), w.len.as<int32_t>(), w.wlist.as<int32_t>(),
+                               w.counters.as<int>(), C.rs.template as<int64_t>(),
+                               C.re.template as<int64_t>(), C.col.template as<int32_t>(),
+                               C.d_val(), mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
+      }
     }
     if (band_tiles) {
       ProfScope ps(mode == MODE_SQUARE ? KC_BAND_SQUARE : KC_BAND_UPDATE, s, fl_band, 0.0);
