@@ -159,7 +159,8 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // multiply-adds are added to *band_work (nullable; zeroed by the caller);
 // bandrow (nullable) gets 1 for the rows of band tiles, 0 for the others.
 // binfo: scratch of n records (B's rows' first/last column and length; B has
-// n rows, as every operand of a stage).
+// n rows, as every operand of a stage). ends (nullable; FP64 products): n
+// records for the numeric product (columns near the ends of B's long rows).
 // dslot (nullable, per matrix): matrices with dslot[m] >= 0 take the dense
 // path; their rows get no sparse work, and in MODE_UPDATE a whole row of
 // slots (moff gives the matrix sizes).
@@ -167,7 +168,8 @@ void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, 
                    int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, double *work,
-                   double *band_work, unsigned char *bandrow, int4 *binfo, cudaStream_t s);
+                   double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
+                   cudaStream_t s);
 
 // Band layout of the rows of an FP32 operand: row k's values dense over the
 // columns [fc[k], fc[k] + nf[k]) (fc and nf multiples of 4, holes +0) at
@@ -215,11 +217,11 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
 // end stored in ce[i]. MODE_SQUARE: C = A A, and part[2i] = sum_j (C_ij -
 // delta_ij)^2, part[2i+1] = sum_k a_ik^2. MODE_UPDATE: C = 1.5 A - 0.5 A B.
 // The part entries of dense-path matrices (dslot nullable; dslot[seg[i]] >= 0)
-// are left to the dense path.
+// are left to the dense path. ends: from launch_bounds (FP64; null for FP32).
 template <typename T>
 void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int32_t *lo, const int32_t *len, const int32_t *seg,
-                    const int *dslot, const int32_t *lists, const int *counters,
+                    int mode, const int2 *ends, const int32_t *lo, const int32_t *len,
+                    const int32_t *seg, const int *dslot, const int32_t *lists, const int *counters,
                     const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                     cudaStream_t s);
 

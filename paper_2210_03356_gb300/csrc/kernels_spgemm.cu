@@ -110,14 +110,22 @@ __device__ __forceinline__ float lane_use(float avg, int g) {
   return avg / (rounds * float(g));
 }
 
+// B rows of at least this mean length keep their row on 32 lanes: below about
+// 62 entries a banded row's head and tail overlap its neighbours' too much to
+// be streamed.
+constexpr float STREAM_AVG = 64.0f;
+
 // Per row k of B: (first column, last column, entries, 0), so that k_bounds
-// reads one 16-byte record per k instead of a chain of dependent loads.
+// reads one 16-byte record per k instead of a chain of dependent loads. ends
+// (nullable; FP64 products): of a row with at least 32 entries, the 31st
+// column and the 31st from its end (see stream_rows).
 __global__ void k_row_info(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
-                           int4 *info) {
+                           int4 *info, int2 *ends) {
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     const int64_t a = rs[r], b = re[r];
     info[r] = b > a ? make_int4(col[a], col[b - 1], int(b - a), 0) : make_int4(0, -1, 0, 0);
+    if (ends && b - a >= 32) ends[r] = make_int2(col[a + 30], col[b - 31]);
   }
 }
 
@@ -150,7 +158,8 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
       cls = L <= WARP_W / 2 ? RC_G16 : RC_G32;
     } else {
       const float avg = float(wk) / float(na > 0 ? na : 1);
-      const float u32 = lane_use(avg, 32), u16 = lane_use(avg, 16), u8 = lane_use(avg, 8);
+      // long B rows run one after another through full passes (stream_rows)
+      const float u32 = avg >= STREAM_AVG ? 1.0f : lane_use(avg, 32), u16 = lane_use(avg, 16), u8 = lane_use(avg, 8);
       cls = RC_G32;
       if (L <= WARP_W / 2 && u16 > u32 + group_margin) cls = RC_G16;
       if (L <= WARP_W / 4 && u8 > (cls == RC_G16 ? u16 : u32) + group_margin) cls = RC_G8;
@@ -346,38 +355,40 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
   }
 }
 
-// Touched slots. With MARK = false every product sets the slot's byte flag
-// f[j] = 1. With MARK = true (FP32 accumulators) an untouched slot holds -0.0
-// and no flag is written: each product is fma(a, b, acc) + 0, and adding +0
-// turns a -0 result into +0 and leaves every other value as it is. A slot
-// reads -0 only until its first product, and its values are those of an
+// Untouched slots are marked by their value, so that a product stores nothing
+// but the sum (a flag byte per product was one of eight shared-memory
+// wavefronts of an FP64 pass, whose kernels run that unit at 75%).
+// FP32: an untouched slot holds -0.0; each product is fma(a, b, acc) + 0, and
+// adding +0 turns a -0 result into +0 and leaves every other value as it is. A
+// slot reads -0 only until its first product, and its values are those of an
 // accumulation from +0 (which can never produce -0) bit for bit.
-template <typename T, bool MARK>
-__device__ __forceinline__ bool untouched(T v) {
-  if constexpr (MARK)
-    return __float_as_uint(v) == 0x80000000u;
+// FP64: an untouched slot holds a NaN of a payload that no operation produces;
+// a product that finds it starts from +0.
+constexpr int kEmptyHi = int(0xFFF85E17u);  // high word of the FP64 mark
+__device__ __forceinline__ bool untouched(float v) { return __float_as_uint(v) == 0x80000000u; }
+__device__ __forceinline__ bool untouched(double v) { return __double2hiint(v) == kEmptyHi; }
+template <typename T>
+__device__ __forceinline__ T empty_slot() {
+  if constexpr (sizeof(T) == 4)
+    return -0.0f;
   else
-    return false;
+    return __hiloint2double(kEmptyHi, 0);
 }
-template <typename T, bool MARK>
-__device__ __forceinline__ void mac(T *acc, unsigned char *f, int j, T a, T v) {
-  static_assert(!MARK || sizeof(T) == 4, "the -0 marker is used for FP32 accumulators");
-  if constexpr (MARK) {
-    acc[j] = __fadd_rn(fma_rn(a, v, acc[j]), 0.0f);
-  } else {
-    acc[j] = fma_rn(a, v, acc[j]);
-    f[j] = 1;
-  }
+__device__ __forceinline__ void mac(float *acc, int j, float a, float v) {
+  acc[j] = __fadd_rn(fma_rn(a, v, acc[j]), 0.0f);
+}
+__device__ __forceinline__ void mac(double *acc, int j, double a, double v) {
+  const double c = acc[j];
+  acc[j] = fma_rn(a, v, untouched(c) ? 0.0 : c);
 }
 
 // One k of the accumulation: lanes stride over B_k = [q0, q1) and add
 // a * b_kj into acc[col - c0], up to four independent products per lane in
 // flight. The columns of B_k are distinct, so the slots of one call never
 // collide.
-template <typename T, int STRIDE, bool MARK = false>
+template <typename T, int STRIDE>
 __device__ __forceinline__ void accumulate_k(T a, int64_t q0, int64_t q1, const int32_t *bcol,
-                                             const T *bval, int64_t c0, T *acc,
-                                             unsigned char *f, int tid) {
+                                             const T *bval, int64_t c0, T *acc, int tid) {
   if constexpr (sizeof(T) == 8) {
     // FP64 (DFMA-bound): passes of STRIDE entries taken four, then two, then
     // one at a time, the same for every lane of the group, so that only the
@@ -395,21 +406,21 @@ __device__ __forceinline__ void accumulate_k(T a, int64_t q0, int64_t q1, const 
       const int j3 = ok3 ? int(bcol[q + 3 * STRIDE] - c0) : 0;
       const T v0 = bval[q], v1 = bval[q + STRIDE], v2 = bval[q + 2 * STRIDE];
       const T v3 = ok3 ? bval[q + 3 * STRIDE] : T(0);
-      mac<T, MARK>(acc, f, j0, a, v0);
-      mac<T, MARK>(acc, f, j1, a, v1);
-      mac<T, MARK>(acc, f, j2, a, v2);
-      if (ok3) mac<T, MARK>(acc, f, j3, a, v3);
+      mac(acc, j0, a, v0);
+      mac(acc, j1, a, v1);
+      mac(acc, j2, a, v2);
+      if (ok3) mac(acc, j3, a, v3);
     }
     if (pass + 2 <= np) {
       const bool ok1 = q + STRIDE < q1;
       const int j0 = int(bcol[q] - c0), j1 = ok1 ? int(bcol[q + STRIDE] - c0) : 0;
       const T v0 = bval[q], v1 = ok1 ? bval[q + STRIDE] : T(0);
-      mac<T, MARK>(acc, f, j0, a, v0);
-      if (ok1) mac<T, MARK>(acc, f, j1, a, v1);
+      mac(acc, j0, a, v0);
+      if (ok1) mac(acc, j1, a, v1);
       pass += 2;
       q += 2 * STRIDE;
     }
-    if (pass < np && q < q1) mac<T, MARK>(acc, f, int(bcol[q] - c0), a, bval[q]);
+    if (pass < np && q < q1) mac(acc, int(bcol[q] - c0), a, bval[q]);
   } else {
     // FP32 (issue-bound): 32-bit offsets from the start of B_k, one 64-bit
     // address per k (~4% faster)
@@ -422,29 +433,101 @@ __device__ __forceinline__ void accumulate_k(T a, int64_t q0, int64_t q1, const 
       int j0 = bc[i] - cz, j1 = bc[i + STRIDE] - cz;
       int j2 = bc[i + 2 * STRIDE] - cz, j3 = bc[i + 3 * STRIDE] - cz;
       T v0 = bv[i], v1 = bv[i + STRIDE], v2 = bv[i + 2 * STRIDE], v3 = bv[i + 3 * STRIDE];
-      mac<T, MARK>(acc, f, j0, a, v0);
-      mac<T, MARK>(acc, f, j1, a, v1);
-      mac<T, MARK>(acc, f, j2, a, v2);
-      mac<T, MARK>(acc, f, j3, a, v3);
+      mac(acc, j0, a, v0);
+      mac(acc, j1, a, v1);
+      mac(acc, j2, a, v2);
+      mac(acc, j3, a, v3);
     }
     if (i + STRIDE < n) {
       int j0 = bc[i] - cz, j1 = bc[i + STRIDE] - cz;
       T v0 = bv[i], v1 = bv[i + STRIDE];
-      mac<T, MARK>(acc, f, j0, a, v0);
-      mac<T, MARK>(acc, f, j1, a, v1);
+      mac(acc, j0, a, v0);
+      mac(acc, j1, a, v1);
       i += 2 * STRIDE;
     }
-    if (i < n) mac<T, MARK>(acc, f, bc[i] - cz, a, bv[i]);
+    if (i < n) mac(acc, bc[i] - cz, a, bv[i]);
   }
+}
+
+// The products of up to 32 consecutive k (lane t < nk holds a_t and the B row
+// [qs, qs + len)) as one stream of entries, 32 per pass, so that every pass but
+// the last is full: a DFMA costs the FP64 pipe the same whatever its active
+// lanes, and with a pass structure per k a B row of 145 entries left 10% of
+// the lanes idle. A pass may hold the tail of B_t and the head of B_(t+1); it
+// stays free of collisions, and every slot keeps its ascending k, when each
+// row has at least 32 entries (so a pass meets at most two rows) and the last
+// 31 columns of B_t all lie above the first 31 of B_(t+1) (ends). Returns false,
+// doing nothing, when that does not hold for all nk rows. Up to eight passes'
+// loads are in flight.
+__device__ __forceinline__ bool stream_rows(int nk, double av, int64_t qs, int len, int2 ends,
+                                            const int32_t *bcol, const double *bval, int32_t c0,
+                                            double *acc, int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int next_head = __shfl_down_sync(FULL, ends.x, 1);
+  const bool ok = lane >= nk || (len >= 32 && (lane == nk - 1 || ends.y > next_head));
+  if (!__all_sync(FULL, ok)) return false;
+  int end = lane < nk ? len : 0;  // inclusive prefix: where row t ends in the stream
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(FULL, end, o);
+    if (lane >= o) end += y;
+  }
+  const int total = __shfl_sync(FULL, end, 31);
+  const int64_t off = qs - (end - len);  // stream position p of row t is entry off + p
+  // row t of the pass's first entry (uniform) and row t + 1: where t ends, the
+  // factors and the offsets, fetched from their lanes when t advances
+  int t = 0, e = __shfl_sync(FULL, end, 0);
+  double at = __shfl_sync(FULL, av, 0), an = __shfl_sync(FULL, av, 1);
+  int64_t ot = __shfl_sync(FULL, off, 0), on = __shfl_sync(FULL, off, 1);
+  int j[4], jn[4];
+  double a[4], v[4], aw[4], vw[4];
+  auto fetch = [&](int p0, int (&j)[4], double (&a)[4], double (&v)[4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = p0 + 32 * u + lane;
+      const bool head = p >= e;  // of row t + 1
+      a[u] = head ? an : at;
+      const int64_t q = (head ? on : ot) + p;
+      j[u] = -1;
+      if (p < total) {
+        j[u] = bcol[q] - c0;
+        v[u] = bval[q];
+      }
+      if (p0 + 32 * (u + 1) >= e && t < 31) {
+        ++t;
+        e = __shfl_sync(FULL, end, t);
+        at = an;
+        ot = on;
+        const int nx = min(t + 1, 31);
+        an = __shfl_sync(FULL, av, nx);
+        on = __shfl_sync(FULL, off, nx);
+      }
+    }
+  };
+  auto add = [&](const int (&j)[4], const double (&a)[4], const double (&v)[4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (j[u] >= 0) mac(acc, j[u], a[u], v[u]);
+      __syncwarp();
+    }
+  };
+  fetch(0, j, a, v);
+  for (int p0 = 0; p0 < total; p0 += 256) {  // the next four passes load while four are added
+    if (p0 + 128 < total) fetch(p0 + 128, jn, aw, vw);
+    add(j, a, v);
+    if (p0 + 128 >= total) break;
+    if (p0 + 256 < total) fetch(p0 + 256, j, a, v);
+    add(jn, aw, vw);
+  }
+  return true;
 }
 
 // accumulate_k for one k shared by two rows (a_ik and a_i'k): every entry of
 // B_k is loaded once and added into both rows' accumulators.
-template <typename T, bool MARK>
+template <typename T>
 __device__ __forceinline__ void accumulate_k2(T a, T b, int64_t q0, int64_t q1,
                                               const int32_t *bcol, const T *bval, int32_t ca,
-                                              T *acca, unsigned char *fa, int32_t cb, T *accb,
-                                              unsigned char *fb, int tid) {
+                                              T *acca, int32_t cb, T *accb, int tid) {
   const int n = int(q1 - q0);
   const int32_t *bc = bcol + q0;
   const T *bv = bval + q0;
@@ -452,30 +535,30 @@ __device__ __forceinline__ void accumulate_k2(T a, T b, int64_t q0, int64_t q1,
   for (; i + 96 < n; i += 128) {
     int32_t c0 = bc[i], c1 = bc[i + 32], c2 = bc[i + 64], c3 = bc[i + 96];
     T v0 = bv[i], v1 = bv[i + 32], v2 = bv[i + 64], v3 = bv[i + 96];
-    mac<T, MARK>(acca, fa, c0 - ca, a, v0);
-    mac<T, MARK>(acca, fa, c1 - ca, a, v1);
-    mac<T, MARK>(acca, fa, c2 - ca, a, v2);
-    mac<T, MARK>(acca, fa, c3 - ca, a, v3);
-    mac<T, MARK>(accb, fb, c0 - cb, b, v0);
-    mac<T, MARK>(accb, fb, c1 - cb, b, v1);
-    mac<T, MARK>(accb, fb, c2 - cb, b, v2);
-    mac<T, MARK>(accb, fb, c3 - cb, b, v3);
+    mac(acca, c0 - ca, a, v0);
+    mac(acca, c1 - ca, a, v1);
+    mac(acca, c2 - ca, a, v2);
+    mac(acca, c3 - ca, a, v3);
+    mac(accb, c0 - cb, b, v0);
+    mac(accb, c1 - cb, b, v1);
+    mac(accb, c2 - cb, b, v2);
+    mac(accb, c3 - cb, b, v3);
   }
   // at most three entries per lane are left: two loaded together, then one
   if (i + 32 < n) {
     int32_t c0 = bc[i], c1 = bc[i + 32];
     T v0 = bv[i], v1 = bv[i + 32];
-    mac<T, MARK>(acca, fa, c0 - ca, a, v0);
-    mac<T, MARK>(acca, fa, c1 - ca, a, v1);
-    mac<T, MARK>(accb, fb, c0 - cb, b, v0);
-    mac<T, MARK>(accb, fb, c1 - cb, b, v1);
+    mac(acca, c0 - ca, a, v0);
+    mac(acca, c1 - ca, a, v1);
+    mac(accb, c0 - cb, b, v0);
+    mac(accb, c1 - cb, b, v1);
     i += 64;
   }
   if (i < n) {
     int32_t c = bc[i];
     T v = bv[i];
-    mac<T, MARK>(acca, fa, c - ca, a, v);
-    mac<T, MARK>(accb, fb, c - cb, b, v);
+    mac(acca, c - ca, a, v);
+    mac(accb, c - cb, b, v);
   }
 }
 
@@ -486,15 +569,14 @@ __device__ __forceinline__ void accumulate_k2(T a, T b, int64_t q0, int64_t q1,
 // ascending order, one FMA per slot per k, exactly as with a warp of its own.
 // Rows of a banded iterate that are neighbours share almost all of their k,
 // so the pair gathers B about half as often as two warps would.
-// Row x has k entries [pa, ea) and accumulator (acca, fa) for columns from
+// Row x has k entries [pa, ea) and accumulator acca for columns from
 // ca; row y likewise (an absent row has pb == eb).
-template <typename T, bool MARK>
+template <typename T>
 __device__ __forceinline__ void pair_rows(int64_t pa, int64_t ea, int64_t pb, int64_t eb,
                                           const int32_t *acol, const T *aval,
                                           const int64_t *brs, const int64_t *bre,
                                           const int32_t *bcol, const T *bval, int32_t ca,
-                                          T *acca, unsigned char *fa, int32_t cb, T *accb,
-                                          unsigned char *fb, int lane) {
+                                          T *acca, int32_t cb, T *accb, int lane) {
   constexpr unsigned FULL = 0xffffffffu;
   // lane l holds the (k, a_k, start, length) of the l-th k of each row's window
   int ka = INT_MAX, kb = INT_MAX, na = 0, nb = 0;
@@ -548,20 +630,20 @@ __device__ __forceinline__ void pair_rows(int64_t pa, int64_t ea, int64_t pb, in
       const T a = __shfl_sync(FULL, va, ia), b = __shfl_sync(FULL, vb, ib);
       const int64_t q0 = __shfl_sync(FULL, qa, ia);
       const int n = __shfl_sync(FULL, na, ia);
-      accumulate_k2<T, MARK>(a, b, q0, q0 + n, bcol, bval, ca, acca, fa, cb, accb, fb, lane);
+      accumulate_k2<T>(a, b, q0, q0 + n, bcol, bval, ca, acca, cb, accb, lane);
       ++ia;
       ++ib;
     } else if (ha < hb) {
       const T a = __shfl_sync(FULL, va, ia);
       const int64_t q0 = __shfl_sync(FULL, qa, ia);
       const int n = __shfl_sync(FULL, na, ia);
-      accumulate_k<T, 32, MARK>(a, q0, q0 + n, bcol, bval, ca, acca, fa, lane);
+      accumulate_k<T, 32>(a, q0, q0 + n, bcol, bval, ca, acca, lane);
       ++ia;
     } else {
       const T b = __shfl_sync(FULL, vb, ib);
       const int64_t q0 = __shfl_sync(FULL, qb, ib);
       const int n = __shfl_sync(FULL, nb, ib);
-      accumulate_k<T, 32, MARK>(b, q0, q0 + n, bcol, bval, cb, accb, fb, lane);
+      accumulate_k<T, 32>(b, q0, q0 + n, bcol, bval, cb, accb, lane);
       ++ib;
     }
     __syncwarp();
@@ -583,10 +665,10 @@ template <typename T, int MODE, int G, bool PAIR = false>
 __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<T>::value)
     k_num_group(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
                 const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
-                const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
-                int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
+                const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *list,
+                int *counters, int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
+                double *part) {
   static_assert(!PAIR || G == 16, "pairs are two 16-lane groups");
-  constexpr bool MARK = sizeof(T) == 4;  // untouched FP32 slots hold -0 (see mac)
   constexpr int NG = 32 / G;
   constexpr int SLOTS = WARP_W / NG;
   // group bases staggered across shared-memory banks: without it the groups of
@@ -594,14 +676,15 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
   // their lanes, which touch neighbouring slots, collide
   constexpr int PAD = G == 32 ? 0 : (sizeof(T) == 4 ? G : (G == 8 ? 8 : 0));
   __shared__ T acc_all[WARPS_PER_CTA][WARP_W + 3 * PAD];
-  __shared__ unsigned char flags[WARPS_PER_CTA][WARP_W + 3 * PAD];
+  // MODE_UPDATE: slots that hold x_ij, written once per entry of X_i
+  __shared__ unsigned char flags[WARPS_PER_CTA][MODE == MODE_UPDATE ? WARP_W + 3 * PAD : 1];
   const int lane = lane_id(), w = threadIdx.x >> 5;
   const int g = lane / G, gl = lane % G;
   const unsigned gbits = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
   const unsigned gmask = gbits << (g * G);
   const unsigned lt = (1u << gl) - 1u;
   T *acc = acc_all[w] + g * (SLOTS + PAD);
-  unsigned char *f = flags[w] + g * (SLOTS + PAD);
+  unsigned char *f = flags[w] + (MODE == MODE_UPDATE ? g * (SLOTS + PAD) : 0);
   const int total = counters[cls];
   for (;;) {
     int base = 0;
@@ -615,18 +698,17 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
       const int L = has ? len[r] : 0;
       const int32_t c0 = has ? lo[r] : 0;
       for (int s = gl; s < L; s += G) {
-        acc[s] = MARK ? T(-0.0) : T(0);
-        if (!MARK || MODE == MODE_UPDATE) f[s] = 0;
+        acc[s] = empty_slot<T>();
+        if (MODE == MODE_UPDATE) f[s] = 0;
       }
       const int64_t a0 = has ? ars[r] : 0, a1 = has ? are[r] : 0;
       if (PAIR) {
         __syncwarp();
         constexpr unsigned FULL = 0xffffffffu;
-        pair_rows<T, MARK>(__shfl_sync(FULL, a0, 0), __shfl_sync(FULL, a1, 0),
+        pair_rows<T>(__shfl_sync(FULL, a0, 0), __shfl_sync(FULL, a1, 0),
                      __shfl_sync(FULL, a0, G), __shfl_sync(FULL, a1, G), acol, aval, brs, bre,
-                     bcol, bval, __shfl_sync(FULL, c0, 0), acc_all[w], flags[w],
-                     __shfl_sync(FULL, c0, G), acc_all[w] + (SLOTS + PAD),
-                     flags[w] + (SLOTS + PAD), lane);
+                     bcol, bval, __shfl_sync(FULL, c0, 0), acc_all[w], __shfl_sync(FULL, c0, G),
+                     acc_all[w] + (SLOTS + PAD), lane);
       } else {
         __syncwarp(gmask);
         // ascending k; the (a_ik, start, end) of G k at a time are fetched by
@@ -635,17 +717,22 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
           const int nk = int(min(int64_t(G), a1 - pb));
           T av = T(0);
           int64_t qs = 0, qe = 0;
+          int2 be = make_int2(0, 0);
           if (gl < nk) {
             int32_t k = acol[pb + gl];
             av = aval[pb + gl];
             qs = brs[k];
             qe = bre[k];
+            if constexpr (sizeof(T) == 8 && G == 32) be = ends[k];
+          }
+          if constexpr (sizeof(T) == 8 && G == 32) {
+            if (stream_rows(nk, av, qs, int(qe - qs), be, bcol, bval, c0, acc, lane)) continue;
           }
           for (int t = 0; t < nk; ++t) {
             T a = __shfl_sync(gmask, av, t, G);
             int64_t q0 = __shfl_sync(gmask, qs, t, G);
             int64_t q1 = __shfl_sync(gmask, qe, t, G);
-            accumulate_k<T, G, MARK>(a, q0, q1, bcol, bval, c0, acc, f, gl);
+            accumulate_k<T, G>(a, q0, q1, bcol, bval, c0, acc, gl);
             __syncwarp(gmask);
           }
         }
@@ -655,9 +742,9 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
           for (int64_t p = a0 + gl; p < a1; p += G) {
             int j = acol[p] - c0;
             T xt = acc[j];
-            if (untouched<T, MARK>(xt)) xt = T(0);
+            if (untouched(xt)) xt = T(0);
             acc[j] = ns_combine(aval[p], xt);
-            f[j] = 3;
+            f[j] = 2;
           }
           __syncwarp(gmask);
         }
@@ -669,12 +756,9 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
           int s = s0 + gl;
           int fl = 0;
           if (s < L) {
-            if (MARK) {  // touched: a product (acc is not -0) or, in an update, x_ij
-              fl = MODE == MODE_UPDATE ? f[s] : 0;
-              if (!fl && !untouched<T, MARK>(acc[s])) fl = 1;
-            } else {
-              fl = f[s];
-            }
+            // touched: a product or, in an update, x_ij
+            fl = MODE == MODE_UPDATE ? f[s] : 0;
+            if (!fl && !untouched(acc[s])) fl = 1;
           }
           unsigned m = (__ballot_sync(gmask, fl != 0) >> (g * G)) & gbits;
           if (fl) {
@@ -759,8 +843,10 @@ constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_K = 4;  // k whose first 32 entries are loaded ahead
 template <typename T>
 constexpr int wide_occ() { return sizeof(T) == 8 ? 3 : 5; }  // CTAs per SM
-template <typename T>
-constexpr size_t wide_smem() { return size_t(WIDE_WARPS) * WARP_W * (sizeof(T) + 1); }
+template <typename T, int MODE>
+constexpr size_t wide_smem() {
+  return size_t(WIDE_WARPS) * WARP_W * (sizeof(T) + (MODE == MODE_UPDATE ? 1 : 0));
+}
 
 template <typename T, int MODE, int P>
 __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
@@ -770,7 +856,6 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
                const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
                const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
   constexpr unsigned FULL = 0xffffffffu;
-  constexpr bool MARK = sizeof(T) == 4;  // untouched FP32 slots hold -0 (see mac)
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
   __shared__ int s_idx[NG], s_cnt[WIDE_WARPS];
@@ -806,8 +891,8 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
       const int64_t c0 = base + (int64_t(w0) << sh);
       const int W = has ? (w1 - w0) << sh : 0;  // its columns
       for (int s = lane; s < W; s += 32) {
-        acc[s] = MARK ? T(-0.0) : T(0);
-        if (!MARK || MODE == MODE_UPDATE) f[s] = 0;
+        acc[s] = empty_slot<T>();
+        if (MODE == MODE_UPDATE) f[s] = 0;
       }
       __syncwarp();
       if (has) {
@@ -851,10 +936,9 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
             }
 #pragma unroll
             for (int t = 0; t < WIDE_K; ++t) {
-              if (lane < nn[t]) mac<T, MARK>(acc, f, j[t], a[t], v[t]);
+              if (lane < nn[t]) mac(acc, j[t], a[t], v[t]);
               if (nn[t] > 32)
-                accumulate_k<T, 32, MARK>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, f,
-                                          lane);
+                accumulate_k<T, 32>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, lane);
               __syncwarp();
             }
           }
@@ -864,18 +948,17 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
           for (int64_t p = x0 + lane; p < x1; p += 32) {
             const int jx = int(acol[p] - c0);
             T xt = acc[jx];
-            if (untouched<T, MARK>(xt)) xt = T(0);
+            if (untouched(xt)) xt = T(0);
             acc[jx] = ns_combine(aval[p], xt);
-            f[jx] = 3;
+            f[jx] = 2;
           }
           __syncwarp();
         }
       }
       auto touched = [&](int s) -> int {
         if (s >= W) return 0;
-        if (!MARK) return f[s];
         int fl = MODE == MODE_UPDATE ? f[s] : 0;
-        if (!fl && !untouched<T, MARK>(acc[s])) fl = 1;
+        if (!fl && !untouched(acc[s])) fl = 1;
         return fl;
       };
       int cnt = 0;
@@ -1021,9 +1104,10 @@ void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, 
                    int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, double *work,
-                   double *band_work, unsigned char *bandrow, int4 *binfo, cudaStream_t s) {
+                   double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
+                   cudaStream_t s) {
   if (n == 0) return;
-  k_row_info<<<grid_cap(n, 256, 8), 256, 0, s>>>(n, B.rs, B.re, B.col, binfo);
+  k_row_info<<<grid_cap(n, 256, 8), 256, 0, s>>>(n, B.rs, B.re, B.col, binfo, ends);
   SGN_LAUNCH_CHECK();
   int tiles = int((n + BOUNDS_TILE - 1) / BOUNDS_TILE);
   int g = tiles < sm_count() * 8 ? tiles : sm_count() * 8;
@@ -1035,28 +1119,28 @@ void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, 
 
 template <typename T, int MODE, int G, bool PAIR = false>
 static void group_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                         const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
+                         const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
                          int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
                          double *part, cudaStream_t s) {
   k_num_group<T, MODE, G, PAIR><<<grid_cap(n, WARPS_PER_CTA * (32 / G),
                                            PAIR ? PAIR_OCC : WarpOcc<T>::value),
                                   WARPS_PER_CTA * 32, 0, s>>>(
-      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, lo, len, lists + int64_t(cls) * n, ctr,
+      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, ends, lo, len, lists + int64_t(cls) * n, ctr,
       cls, cs, ce, ccol, cval, part);
   SGN_LAUNCH_CHECK();
 }
 
 template <typename T, int MODE>
 static void num_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                       const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
+                       const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
                        const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                        cudaStream_t s) {
-  group_launch<T, MODE, 32>(n, A, aval, B, bval, lo, len, lists, ctr, RC_G32, cs, ce, ccol, cval,
+  group_launch<T, MODE, 32>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G32, cs, ce, ccol, cval,
                             part, s);
   // FP32: the 16-lane class holds row pairs (GROUPS_PAIRS)
-  group_launch<T, MODE, 16, sizeof(T) == 4>(n, A, aval, B, bval, lo, len, lists, ctr, RC_G16, cs,
+  group_launch<T, MODE, 16, sizeof(T) == 4>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G16, cs,
                                             ce, ccol, cval, part, s);
-  group_launch<T, MODE, 8>(n, A, aval, B, bval, lo, len, lists, ctr, RC_G8, cs, ce, ccol, cval,
+  group_launch<T, MODE, 8>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G8, cs, ce, ccol, cval,
                            part, s);
 }
 
@@ -1065,7 +1149,7 @@ static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, c
                         const WideTable &wt, const int32_t *lo, const int32_t *len,
                         const int32_t *list, int *ctr, const int64_t *cs, int64_t *ce,
                         int32_t *ccol, T *cval, double *part, cudaStream_t s) {
-  constexpr size_t sm = wide_smem<T>();
+  constexpr size_t sm = wide_smem<T, MODE>();
   static const bool attr = [] {  // once, thread-safe
     SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
@@ -1135,8 +1219,8 @@ template void launch_numeric_wide<float>(int64_t, int, double, const Rows &, con
 
 template <typename T>
 void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int32_t *lo, const int32_t *len, const int32_t *seg,
-                    const int *dslot, const int32_t *lists, const int *counters,
+                    int mode, const int2 *ends, const int32_t *lo, const int32_t *len,
+                    const int32_t *seg, const int *dslot, const int32_t *lists, const int *counters,
                     const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                     cudaStream_t s) {
   if (n == 0) return;
@@ -1146,22 +1230,22 @@ void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, cons
                                                           mode == MODE_SQUARE ? part : nullptr);
   SGN_LAUNCH_CHECK();
   if (mode == MODE_SQUARE)
-    num_launch<T, MODE_SQUARE>(n, A, aval, B, bval, lo, len, lists, ctr, cs, ce, ccol, cval, part,
+    num_launch<T, MODE_SQUARE>(n, A, aval, B, bval, ends, lo, len, lists, ctr, cs, ce, ccol, cval, part,
                                s);
   else
-    num_launch<T, MODE_UPDATE>(n, A, aval, B, bval, lo, len, lists, ctr, cs, ce, ccol, cval, part,
+    num_launch<T, MODE_UPDATE>(n, A, aval, B, bval, ends, lo, len, lists, ctr, cs, ce, ccol, cval, part,
                                s);
 }
 
 template void launch_numeric<double>(int64_t, const Rows &, const double *, const Rows &,
-                                     const double *, int, const int32_t *, const int32_t *,
-                                     const int32_t *, const int *, const int32_t *, const int *,
-                                     const int64_t *, int64_t *, int32_t *, double *, double *,
+                                     const double *, int, const int2 *, const int32_t *,
+                                     const int32_t *, const int32_t *, const int *,
+                                     const int32_t *, const int *, const int64_t *, int64_t *, int32_t *, double *, double *,
                                      cudaStream_t);
 template void launch_numeric<float>(int64_t, const Rows &, const float *, const Rows &,
-                                    const float *, int, const int32_t *, const int32_t *,
-                                    const int32_t *, const int *, const int32_t *, const int *,
-                                    const int64_t *, int64_t *, int32_t *, float *, double *,
+                                    const float *, int, const int2 *, const int32_t *,
+                                    const int32_t *, const int32_t *, const int *, const int32_t *,
+                                    const int *, const int64_t *, int64_t *, int32_t *, float *, double *,
                                     cudaStream_t);
 
 }  // namespace sgn

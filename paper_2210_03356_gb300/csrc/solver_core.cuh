@@ -195,6 +195,7 @@ struct Work {
   DevBuf n2v, n2y, n2z, n2part, n2zacc, n2xmax, n2ymax, n2nrm, x2;  // budget_norm
   int sel_shift = 0;    // > 0: the last threshold select had room for entries >> sel_shift
   DevBuf binfo;         // per row of a product's B: first/last column, length
+  DevBuf ends;          // and (FP64) columns near its ends
   DevBuf nmf_int, nmf_dbl;  // NMF: row swaps, singular flags; ||X^-1||
   bool bt_rows_done = false;  // the square's band tiles wrote their rows of T's band
 };
@@ -405,6 +406,9 @@ struct Solver {
     // the slot total below; the band tiles write the rows of T's band they
     // compute, and the update fills in the other rows of T it needs
     const bool band = sizeof(T) == 4 && o.fp32_band;
+    int2 *ends = sizeof(T) == 8
+                     ? static_cast<int2 *>(w.ends.ensure(sizeof(int2) * size_t(N > 0 ? N : 1), s))
+                     : nullptr;
     {
       ProfScope ps(KC_BOUNDS, s);
       if (band && mode == MODE_SQUARE) w.bandrow.ensure(size_t(N > 0 ? N : 1), s);
@@ -418,7 +422,7 @@ struct Solver {
                     w.counters.as<int>(), w.work.as<double>(), band_work_dev(),
                     band && mode == MODE_SQUARE ? w.bandrow.as<unsigned char>() : nullptr,
                     static_cast<int4 *>(w.binfo.ensure(sizeof(int4) * size_t(N > 0 ? N : 1), s)),
-                    s);
+                    ends, s);
       launch_seg_reduce(nb, st.d_moff.template as<int64_t>(), w.work.as<double>(), 1,
                         w.mults.as<double>(), s);
       if (band) {
@@ -522,7 +526,7 @@ struct Solver {
     {
       // bytes: the row-wise class keeps the whole product's algorithmic bytes
       ProfScope ps(cls, s, fl - fl_band, by);
-      launch_numeric<T>(N, A, aval, B, bval, mode, w.lo.as<int32_t>(), w.len.as<int32_t>(),
+      launch_numeric<T>(N, A, aval, B, bval, mode, ends, w.lo.as<int32_t>(), w.len.as<int32_t>(),
                         st.d_seg.template as<int32_t>(),
                         dp && dp->any() ? w.dslot.as<int>() : nullptr, w.wlist.as<int32_t>(),
                         w.counters.as<int>(), C.rs.template as<int64_t>(),
