@@ -218,18 +218,22 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
 // delta_ij)^2, part[2i+1] = sum_k a_ik^2. MODE_UPDATE: C = 1.5 A - 0.5 A B.
 // The part entries of dense-path matrices (dslot nullable; dslot[seg[i]] >= 0)
 // are left to the dense path. ends: from launch_bounds (FP64; null for FP32).
+// rows: the list lengths (counters[RC_*]) on the host; empty classes are not
+// launched. few: every listed row is in the 32-lane class (groups = 0) and runs
+// with its loads ahead of its sums (rows too few to hide them otherwise); shared:
+// they are left to launch_numeric_wide.
 template <typename T>
-void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int2 *ends, const int32_t *lo, const int32_t *len,
-                    const int32_t *seg, const int *dslot, const int32_t *lists, const int *counters,
-                    const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
-                    cudaStream_t s);
-
-// The rows of more than WARP_W columns (the RC_CTA list, `rows` of them).
-// mean_b: the mean length of the B rows that products read. off: scratch of
-// n * wt.stride ints for B's column-block table, or null (binary search in
-// its place); wt: the rows' matrices, the block width 1 << sh and the table's
-// row stride, (max matrix order >> sh) + 2.
+void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Rows &A, const T *aval,
+                    const Rows &B, const T *bval, int mode, const int2 *ends, const int32_t *lo,
+                    const int32_t *len, const int32_t *seg, const int *dslot,
+                    const int32_t *lists, int *counters, const int64_t *cs, int64_t *ce,
+                    int32_t *ccol, T *cval, double *part, cudaStream_t s);
+// The rows of more than WARP_W columns (cls = RC_CTA, `rows` of them), or the few
+// rows of the 32-lane class (cls = RC_G32), by windows of several warps.
+// mean_b: the mean length of the B rows that products read. wt: the rows'
+// matrices, the column-block table of B (launch_col_blocks: n * stride ints;
+// null: binary search in its place), its block width 1 << sh and row stride,
+// (max matrix order >> sh) + 2.
 struct WideTable {
   const int32_t *seg;
   const int64_t *moff;
@@ -237,9 +241,11 @@ struct WideTable {
   int sh, stride;
 };
 int wide_block_shift(int64_t max_n);
+void launch_col_blocks(int64_t n, const Rows &B, const int32_t *seg, const int64_t *moff, int sh,
+                       int stride, int *off, cudaStream_t s);
 template <typename T>
-void launch_numeric_wide(int64_t n, int rows, double mean_b, const Rows &A, const T *aval,
-                         const Rows &B, const T *bval, int mode, WideTable wt, int *off,
+void launch_numeric_wide(int64_t n, int cls, int rows, double mean_b, const Rows &A, const T *aval,
+                         const Rows &B, const T *bval, int mode, const WideTable &wt,
                          const int32_t *lo, const int32_t *len, const int32_t *lists,
                          int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
                          double *part, cudaStream_t s);

@@ -522,6 +522,80 @@ __device__ __forceinline__ bool stream_rows(int nk, double av, int64_t qs, int l
   return true;
 }
 
+// The k-loop of one row by one warp when rows are few and latency counts: the
+// B rows of 32 k are located together (the next 32 while these run), and the
+// first 64 entries of four k are loaded while the four before them are added.
+// The k still run one after another, one fused multiply-add per slot each.
+template <typename T>
+__device__ __forceinline__ void ahead_rows(int64_t a0, int64_t a1, const int32_t *acol,
+                                           const T *aval, const int64_t *brs, const int64_t *bre,
+                                           const int32_t *bcol, const T *bval, int32_t c0, T *acc,
+                                           int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int D = 4;
+  struct Four {
+    T a[D], v0[D], v1[D];
+    int64_t q[D];
+    int n[D], j0[D], j1[D];
+  };
+  T av = T(0), nav = T(0);
+  int64_t qs = 0, nqs = 0;
+  int qn = 0, nqn = 0;
+  auto locate = [&](int64_t p, T &a, int64_t &q, int &n) {
+    n = 0;
+    if (p < a1) {
+      const int32_t k = acol[p];
+      a = aval[p];
+      q = brs[k];
+      n = int(bre[k] - q);
+    }
+  };
+  auto load = [&](Four &x, int t0) {
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      x.a[t] = __shfl_sync(FULL, av, t0 + t);
+      x.q[t] = __shfl_sync(FULL, qs, t0 + t);
+      x.n[t] = __shfl_sync(FULL, qn, t0 + t);
+      if (lane < x.n[t]) {
+        x.j0[t] = int(bcol[x.q[t] + lane] - c0);
+        x.v0[t] = bval[x.q[t] + lane];
+      }
+      if (lane + 32 < x.n[t]) {
+        x.j1[t] = int(bcol[x.q[t] + lane + 32] - c0);
+        x.v1[t] = bval[x.q[t] + lane + 32];
+      }
+    }
+  };
+  auto add = [&](const Four &x) {
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      if (lane < x.n[t]) mac(acc, x.j0[t], x.a[t], x.v0[t]);
+      if (lane + 32 < x.n[t]) mac(acc, x.j1[t], x.a[t], x.v1[t]);
+      if (x.n[t] > 64)
+        accumulate_k<T, 32>(x.a[t], x.q[t] + 64, x.q[t] + x.n[t], bcol, bval, c0, acc, lane);
+      __syncwarp();
+    }
+  };
+  locate(a0 + lane, av, qs, qn);
+  Four x, y;
+  for (int64_t pb = a0; pb < a1; pb += 32) {
+    const int nk = int(min(int64_t(32), a1 - pb));
+    locate(pb + 32 + lane, nav, nqs, nqn);
+    load(x, 0);
+    for (int t = 0; t < nk; t += 2 * D) {  // lanes past nk hold empty rows
+      if (t + D < nk) load(y, t + D);
+      add(x);
+      if (t + D < nk) {
+        if (t + 2 * D < nk) load(x, t + 2 * D);
+        add(y);
+      }
+    }
+    av = nav;
+    qs = nqs;
+    qn = nqn;
+  }
+}
+
 // accumulate_k for one k shared by two rows (a_ik and a_i'k): every entry of
 // B_k is loaded once and added into both rows' accumulators.
 template <typename T>
@@ -650,6 +724,7 @@ __device__ __forceinline__ void pair_rows(int64_t pa, int64_t ea, int64_t pb, in
   }
 }
 
+constexpr int AHEAD_OCC = 4;  // CTAs per SM of the ahead_rows kernels (registers for loads in flight)
 constexpr int PAIR_OCC = 8;  // CTAs per SM of the pair kernel: 64 registers, no spills
 template <typename T>
 struct WarpOcc;  // CTAs per SM of the warp kernel (shared memory and registers)
@@ -659,16 +734,24 @@ template <> struct WarpOcc<float> { static constexpr int value = 10; };
 // G lanes per row, 32/G rows per warp; each group owns WARP_W*G/32 slots of
 // its warp's accumulator and runs the ascending-k accumulation of its own row
 // with group-wide barriers, so the result is the same as with a whole warp.
-// PAIR (with G = 16): the two rows of a warp share its k-loop (pair_rows);
-// the rest of the kernel is that of 16-lane groups.
-template <typename T, int MODE, int G, bool PAIR = false>
-__global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<T>::value)
+// LOOP: LOOP_PAIR (with G = 16): the two rows of a warp share its k-loop
+// (pair_rows); the rest of the kernel is that of 16-lane groups. LOOP_AHEAD
+// (with G = 32): the k-loop of ahead_rows.
+enum { LOOP_ROW = 0, LOOP_PAIR = 1, LOOP_AHEAD = 2 };
+template <typename T, int LOOP>
+constexpr int group_occ() {
+  return LOOP == LOOP_PAIR ? PAIR_OCC : LOOP == LOOP_AHEAD ? AHEAD_OCC : WarpOcc<T>::value;
+}
+template <typename T, int MODE, int G, int LOOP = LOOP_ROW>
+__global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
     k_num_group(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
                 const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
                 const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *list,
                 int *counters, int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
                 double *part) {
+  constexpr bool PAIR = LOOP == LOOP_PAIR;
   static_assert(!PAIR || G == 16, "pairs are two 16-lane groups");
+  static_assert(LOOP != LOOP_AHEAD || G == 32, "a warp per row");
   constexpr int NG = 32 / G;
   constexpr int SLOTS = WARP_W / NG;
   // group bases staggered across shared-memory banks: without it the groups of
@@ -702,13 +785,16 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, PAIR ? PAIR_OCC : WarpOcc<
         if (MODE == MODE_UPDATE) f[s] = 0;
       }
       const int64_t a0 = has ? ars[r] : 0, a1 = has ? are[r] : 0;
-      if (PAIR) {
+      if constexpr (PAIR) {
         __syncwarp();
         constexpr unsigned FULL = 0xffffffffu;
         pair_rows<T>(__shfl_sync(FULL, a0, 0), __shfl_sync(FULL, a1, 0),
                      __shfl_sync(FULL, a0, G), __shfl_sync(FULL, a1, G), acol, aval, brs, bre,
                      bcol, bval, __shfl_sync(FULL, c0, 0), acc_all[w], __shfl_sync(FULL, c0, G),
                      acc_all[w] + (SLOTS + PAD), lane);
+      } else if constexpr (LOOP == LOOP_AHEAD) {
+        __syncwarp();
+        ahead_rows<T>(a0, a1, acol, aval, brs, bre, bcol, bval, c0, acc, lane);
       } else {
         __syncwarp(gmask);
         // ascending k; the (a_ik, start, end) of G k at a time are fetched by
@@ -854,7 +940,7 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
                const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
                const int32_t *seg, const int64_t *moff, const int *off, int sh, int stride,
                const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
-               const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
+               int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
@@ -872,9 +958,9 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
     else
       asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(P * 32) : "memory");
   };
-  const int total = counters[RC_CTA];
+  const int total = counters[cls];
   for (;;) {
-    if (wr == 0 && lane == 0) s_idx[g] = atomicAdd(&counters[RC_QUEUE + RC_CTA], 1);
+    if (wr == 0 && lane == 0) s_idx[g] = atomicAdd(&counters[RC_QUEUE + cls], 1);
     row_sync();
     const int idx = s_idx[g];
     if (idx >= total) break;
@@ -1117,37 +1203,44 @@ void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, 
   SGN_LAUNCH_CHECK();
 }
 
-template <typename T, int MODE, int G, bool PAIR = false>
-static void group_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                         const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
-                         int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
-                         double *part, cudaStream_t s) {
-  k_num_group<T, MODE, G, PAIR><<<grid_cap(n, WARPS_PER_CTA * (32 / G),
-                                           PAIR ? PAIR_OCC : WarpOcc<T>::value),
+template <typename T, int MODE, int G, int LOOP = LOOP_ROW>
+static void group_launch(int rows, int64_t n, const Rows &A, const T *aval, const Rows &B,
+                         const T *bval, const int2 *ends, const int32_t *lo, const int32_t *len,
+                         const int32_t *lists, int *ctr, int cls, const int64_t *cs, int64_t *ce,
+                         int32_t *ccol, T *cval, double *part, cudaStream_t s) {
+  if (rows <= 0) return;
+  k_num_group<T, MODE, G, LOOP><<<grid_cap(rows, WARPS_PER_CTA * (32 / G), group_occ<T, LOOP>()),
                                   WARPS_PER_CTA * 32, 0, s>>>(
-      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, ends, lo, len, lists + int64_t(cls) * n, ctr,
-      cls, cs, ce, ccol, cval, part);
+      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, ends, lo, len, lists + int64_t(cls) * n,
+      ctr, cls, cs, ce, ccol, cval, part);
   SGN_LAUNCH_CHECK();
 }
 
 template <typename T, int MODE>
-static void num_launch(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                       const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *lists, int *ctr,
-                       const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
-                       cudaStream_t s) {
-  group_launch<T, MODE, 32>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G32, cs, ce, ccol, cval,
-                            part, s);
+static void num_launch(int64_t n, const int *rows, bool few, const Rows &A, const T *aval,
+                       const Rows &B, const T *bval, const int2 *ends, const int32_t *lo,
+                       const int32_t *len, const int32_t *lists, int *ctr, const int64_t *cs,
+                       int64_t *ce, int32_t *ccol, T *cval, double *part, cudaStream_t s) {
+  if (few) {
+    group_launch<T, MODE, 32, LOOP_AHEAD>(rows[RC_G32], n, A, aval, B, bval, ends, lo, len, lists,
+                                          ctr, RC_G32, cs, ce, ccol, cval, part, s);
+    return;
+  }
+  group_launch<T, MODE, 32>(rows[RC_G32], n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G32,
+                            cs, ce, ccol, cval, part, s);
   // FP32: the 16-lane class holds row pairs (GROUPS_PAIRS)
-  group_launch<T, MODE, 16, sizeof(T) == 4>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G16, cs,
-                                            ce, ccol, cval, part, s);
-  group_launch<T, MODE, 8>(n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G8, cs, ce, ccol, cval,
-                           part, s);
+  group_launch<T, MODE, 16, sizeof(T) == 4 ? LOOP_PAIR : LOOP_ROW>(
+      rows[RC_G16], n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G16, cs, ce, ccol, cval,
+      part, s);
+  if constexpr (sizeof(T) == 8)
+    group_launch<T, MODE, 8>(rows[RC_G8], n, A, aval, B, bval, ends, lo, len, lists, ctr, RC_G8,
+                             cs, ce, ccol, cval, part, s);
 }
 
 template <typename T, int MODE, int P>
 static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, const T *bval,
                         const WideTable &wt, const int32_t *lo, const int32_t *len,
-                        const int32_t *list, int *ctr, const int64_t *cs, int64_t *ce,
+                        const int32_t *list, int *ctr, int cls, const int64_t *cs, int64_t *ce,
                         int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   constexpr size_t sm = wide_smem<T, MODE>();
   static const bool attr = [] {  // once, thread-safe
@@ -1158,22 +1251,31 @@ static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, c
   (void)attr;
   k_num_wide<T, MODE, P><<<grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()), WIDE_WARPS * 32, sm, s>>>(
       A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg, wt.moff, wt.off, wt.sh, wt.stride,
-      lo, len, list, ctr, cs, ce, ccol, cval, part);
+      lo, len, list, ctr, cls, cs, ce, ccol, cval, part);
   SGN_LAUNCH_CHECK();
 }
 
 template <typename T, int MODE>
 static void wide_launch_p(int rows, int p, const Rows &A, const T *aval, const Rows &B,
                           const T *bval, const WideTable &wt, const int32_t *lo,
-                          const int32_t *len, const int32_t *list, int *ctr, const int64_t *cs,
-                          int64_t *ce, int32_t *ccol, T *cval, double *part, cudaStream_t s) {
+                          const int32_t *len, const int32_t *list, int *ctr, int cls,
+                          const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
+                          cudaStream_t s) {
 #define SGN_WIDE(P) \
-  wide_launch<T, MODE, P>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cs, ce, ccol, cval, part, s)
+  wide_launch<T, MODE, P>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cls, cs, ce, ccol, cval, \
+                          part, s)
   if (p >= 8) SGN_WIDE(8);
   else if (p >= 4) SGN_WIDE(4);
   else if (p >= 2) SGN_WIDE(2);
   else SGN_WIDE(1);
 #undef SGN_WIDE
+}
+
+void launch_col_blocks(int64_t n, const Rows &B, const int32_t *seg, const int64_t *moff, int sh,
+                       int stride, int *off, cudaStream_t s) {
+  if (n == 0) return;
+  k_col_blocks<<<grid_cap(n, 8, 16), 256, 0, s>>>(n, B.rs, B.re, B.col, seg, moff, sh, stride, off);
+  SGN_LAUNCH_CHECK();
 }
 
 int wide_block_shift(int64_t max_n) {
@@ -1183,69 +1285,67 @@ int wide_block_shift(int64_t max_n) {
 }
 
 template <typename T>
-void launch_numeric_wide(int64_t n, int rows, double mean_b, const Rows &A, const T *aval,
-                         const Rows &B, const T *bval, int mode, WideTable wt, int *off,
+void launch_numeric_wide(int64_t n, int cls, int rows, double mean_b, const Rows &A, const T *aval,
+                         const Rows &B, const T *bval, int mode, const WideTable &wt,
                          const int32_t *lo, const int32_t *len, const int32_t *lists,
                          int *counters, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
                          double *part, cudaStream_t s) {
   if (rows <= 0) return;
-  if (off) {
-    k_col_blocks<<<grid_cap(n, 8, 16), 256, 0, s>>>(n, B.rs, B.re, B.col, wt.seg, wt.moff, wt.sh,
-                                                    wt.stride, off);
-    SGN_LAUNCH_CHECK();
-  }
-  wt.off = off;
-  // warps per row: about 64 (FP32) or 128 (FP64) entries of a B row per warp
-  const double per = sizeof(T) == 8 ? 128.0 : 64.0;
+  // warps per row: about 64 (FP32) or 128 (FP64) entries of a B row per warp, a
+  // pass for each where rows are few
+  const double per = cls != RC_CTA ? 32.0 : sizeof(T) == 8 ? 128.0 : 64.0;
   const int p = mean_b >= 8 * per ? 8 : mean_b >= 4 * per ? 4 : mean_b >= 2 * per ? 2 : 1;
-  const int32_t *list = lists + int64_t(RC_CTA) * n;
+  const int32_t *list = lists + int64_t(cls) * n;
   if (mode == MODE_SQUARE)
-    wide_launch_p<T, MODE_SQUARE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cs, ce,
-                                  ccol, cval, part, s);
+    wide_launch_p<T, MODE_SQUARE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cls, cs,
+                                  ce, ccol, cval, part, s);
   else
-    wide_launch_p<T, MODE_UPDATE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cs, ce,
-                                  ccol, cval, part, s);
+    wide_launch_p<T, MODE_UPDATE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cls, cs,
+                                  ce, ccol, cval, part, s);
 }
-template void launch_numeric_wide<double>(int64_t, int, double, const Rows &, const double *,
-                                          const Rows &, const double *, int, WideTable, int *,
+template void launch_numeric_wide<double>(int64_t, int, int, double, const Rows &, const double *,
+                                          const Rows &, const double *, int, const WideTable &,
                                           const int32_t *, const int32_t *, const int32_t *, int *,
                                           const int64_t *, int64_t *, int32_t *, double *,
                                           double *, cudaStream_t);
-template void launch_numeric_wide<float>(int64_t, int, double, const Rows &, const float *,
-                                         const Rows &, const float *, int, WideTable, int *,
+template void launch_numeric_wide<float>(int64_t, int, int, double, const Rows &, const float *,
+                                         const Rows &, const float *, int, const WideTable &,
                                          const int32_t *, const int32_t *, const int32_t *, int *,
                                          const int64_t *, int64_t *, int32_t *, float *, double *,
                                          cudaStream_t);
 
 template <typename T>
-void launch_numeric(int64_t n, const Rows &A, const T *aval, const Rows &B, const T *bval,
-                    int mode, const int2 *ends, const int32_t *lo, const int32_t *len,
-                    const int32_t *seg, const int *dslot, const int32_t *lists, const int *counters,
-                    const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
-                    cudaStream_t s) {
+void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Rows &A, const T *aval,
+                    const Rows &B, const T *bval, int mode, const int2 *ends, const int32_t *lo,
+                    const int32_t *len, const int32_t *seg, const int *dslot,
+                    const int32_t *lists, int *counters, const int64_t *cs, int64_t *ce,
+                    int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   if (n == 0) return;
-  int *ctr = const_cast<int *>(counters);
-  k_rows_empty<T><<<grid_cap(n, 8 * 32, 16), 256, 0, s>>>(n, A.rs, A.re, aval, len, seg, dslot,
-                                                          cs, ce,
-                                                          mode == MODE_SQUARE ? part : nullptr);
-  SGN_LAUNCH_CHECK();
+  int64_t listed = 0;
+  for (int c = 0; c < RC_N; ++c) listed += int64_t(rows[c]) * (c == RC_BAND ? 16 : 1);
+  if (listed < n) {
+    k_rows_empty<T><<<grid_cap(n, 8 * 32, 16), 256, 0, s>>>(
+        n, A.rs, A.re, aval, len, seg, dslot, cs, ce, mode == MODE_SQUARE ? part : nullptr);
+    SGN_LAUNCH_CHECK();
+  }
+  if (shared) return;
   if (mode == MODE_SQUARE)
-    num_launch<T, MODE_SQUARE>(n, A, aval, B, bval, ends, lo, len, lists, ctr, cs, ce, ccol, cval, part,
-                               s);
+    num_launch<T, MODE_SQUARE>(n, rows, few, A, aval, B, bval, ends, lo, len, lists, counters, cs,
+                               ce, ccol, cval, part, s);
   else
-    num_launch<T, MODE_UPDATE>(n, A, aval, B, bval, ends, lo, len, lists, ctr, cs, ce, ccol, cval, part,
-                               s);
+    num_launch<T, MODE_UPDATE>(n, rows, few, A, aval, B, bval, ends, lo, len, lists, counters, cs,
+                               ce, ccol, cval, part, s);
 }
 
-template void launch_numeric<double>(int64_t, const Rows &, const double *, const Rows &,
-                                     const double *, int, const int2 *, const int32_t *,
-                                     const int32_t *, const int32_t *, const int *,
-                                     const int32_t *, const int *, const int64_t *, int64_t *, int32_t *, double *, double *,
-                                     cudaStream_t);
-template void launch_numeric<float>(int64_t, const Rows &, const float *, const Rows &,
-                                    const float *, int, const int2 *, const int32_t *,
-                                    const int32_t *, const int32_t *, const int *, const int32_t *,
-                                    const int *, const int64_t *, int64_t *, int32_t *, float *, double *,
-                                    cudaStream_t);
+template void launch_numeric<double>(int64_t, const int *, bool, bool, const Rows &, const double *,
+                                     const Rows &, const double *, int, const int2 *,
+                                     const int32_t *, const int32_t *, const int32_t *,
+                                     const int *, const int32_t *, int *, const int64_t *,
+                                     int64_t *, int32_t *, double *, double *, cudaStream_t);
+template void launch_numeric<float>(int64_t, const int *, bool, bool, const Rows &, const float *,
+                                    const Rows &, const float *, int, const int2 *,
+                                    const int32_t *, const int32_t *, const int32_t *, const int *,
+                                    const int32_t *, int *, const int64_t *, int64_t *, int32_t *,
+                                    float *, double *, cudaStream_t);
 
 }  // namespace sgn
