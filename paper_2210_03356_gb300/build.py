@@ -13,7 +13,7 @@ SOURCES = ["kernels_csr.cu", "kernels_spgemm.cu", "kernels_select.cu", "solver.c
            "memory.cu", "threshold.cu", "threshold_noalloc.cu", "kernels_dense.cu", "server.cu",
            "kernels_f64x.cu", "kernels_band.cu", "kernels_norm2.cu",
            "kernels_nmf.cu"]
-HEADERS = [os.path.join(CSRC, h) for h in ("common.cuh", "kernels.h", "solver_core.cuh", "tc.cuh")] + [
+HEADERS = [os.path.join(CSRC, h) for h in ("common.cuh", "kernels.h", "seg.cuh", "solver_core.cuh", "tc.cuh")] + [
     os.path.join(ROOT, "include", "sign.h")]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",

@@ -49,9 +49,12 @@ void launch_gersh(int64_t n, const int64_t *rp, const int32_t *col, const double
                   GershStats *g, cudaStream_t s);
 
 // out[0] = 0, out[i+1] = sum_{r<=i} cnt[r] for i < n. tmp holds
-// scan_tmp_elems(n) int64 values.
+// scan_tmp_elems(n) int64 values. seg, eoff (nullable): row r belongs to matrix
+// seg[r] (ascending, no matrix empty); eoff[0] = 0 and eoff[m + 1] the value at
+// the end of matrix m. total (nullable): out[n] once more.
 int64_t scan_tmp_elems(int64_t n);
-void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s);
+void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s,
+                 const int32_t *seg = nullptr, int64_t *eoff = nullptr, int64_t *total = nullptr);
 
 // One block of a block-diagonal assembly: rows [row0, row0+nrows) of a source
 // CSR whose column indices are shifted by col_shift on the way.
@@ -115,9 +118,9 @@ void launch_extract(int nblocks, const ExtractBlock *blocks, int64_t max_entries
 void launch_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64_t *out,
                            cudaStream_t s);
 
-// out[m*ncomp + c] = sum over rows r of matrix m of part[r*ncomp + c], in a
-// fixed order (deterministic).
-void launch_seg_reduce(int nb, const int64_t *moff, const double *part, int ncomp, double *out,
+// out[m] = sum over the rows r of matrix m of part[r], in a fixed order
+// (deterministic).
+void launch_seg_reduce(int nb, const int64_t *moff, const double *part, double *out,
                        cudaStream_t s);
 
 // ---------------------------------------------------------------- spgemm
@@ -141,7 +144,8 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // Per row i of C = A B (rows of inactive matrices are empty): the column
 // range [lo, lo+len) of the row (including A's own row in MODE_UPDATE), the
 // slot size ub[i] = min(len, work + (UPDATE ? nnz(A_i) : 0)) >= nnz(C_i), and
-// work[i] = sum_{k in A_i} nnz(B_k), the multiply-adds of the row. Non-empty
+// work of the row = sum_{k in A_i} nnz(B_k), its multiply-adds, added into
+// mults[m] (zeroed by the caller). Non-empty
 // rows are listed, in row order within tiles, by the numeric kernel that takes
 // them: lists holds RC_N lists of n entries (32-, 16- or 8-lane groups, one
 // CTA per row, band tiles); counters[c] is the length of list c and
@@ -167,7 +171,7 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, const int *active,
                    int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
-                   int64_t *ub, int32_t *lists, int *counters, double *work,
+                   int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
                    cudaStream_t s);
 
@@ -266,9 +270,12 @@ struct MatScalars {
   int sel_e;                 // e + 1023, the biased exponent of b (1 for a subnormal b)
   int sel_base;              // top 16 bits of the pivot's key (a little below b / sqrt(nnz_bar))
 };
-// From sums[2m] = sum (T-I)^2, sums[2m+1] = sum X^2: r, x, beta, b.
-void launch_matrix_scalars(int nb, const int64_t *moff, const double *sums, double c4,
-                           double tol_stage, double switch_resid, MatScalars *ms, cudaStream_t s);
+// The check of the iterates: from part (part[2r], part[2r+1] per row: the
+// squares of T - I and of X) r, x, beta and b, and nnz[m] = the entries of T in
+// matrix m's rows [rs, re).
+void launch_check_scalars(int nb, const int64_t *moff, const double *part, const int64_t *rs,
+                          const int64_t *re, double c4, double tol_stage, double switch_resid,
+                          MatScalars *ms, int64_t *nnz, cudaStream_t s);
 // ---------------------------------------------------------------- 2-norm
 // ||X||_2 estimates for the budget_norm variant (see kernels_norm2.cu):
 // v_0 = (1,...,1)/sqrt(n), NORM2_STEPS steps v <- X^T X v / ||X^T X v||, then
@@ -320,9 +327,9 @@ constexpr size_t select_scratch_bytes(int nb, int64_t cap) {
          sel_align(size_t(nb) * kSelStateBytes) + sel_align(size_t(nb + 1) * 8) +
          sel_align(size_t(cap > 0 ? cap : 1) * 8) + sel_align(size_t(cap > 0 ? cap : 1) * 4);
 }
-// nvals: the values (or slots) of all rows, which sizes the launches. nnz
-// (nullable): the entries per matrix, stored into ms[m].nnz_bar; else nnz_bar
-// holds them already.
+// nvals: the values (or slots) of all rows, which sizes the launches. With row
+// lists the entries per matrix are counted into ms[m].nnz_bar; for a flat array
+// nnz_bar holds them already.
 // cand_cap is the scratch's candidate room, at least nvals >> R.cshift. When a
 // matrix has more candidates than its room, *select_overflow is set and the
 // thresholds (and counts) are not valid: the caller selects again with room
@@ -330,16 +337,17 @@ constexpr size_t select_scratch_bytes(int nb, int64_t cap) {
 // cnt, dropped (nullable, R.nrows each; R must have rows rs/re): the
 // filter's per-row kept counts and dropped sums of squares under the
 // selected tau, as launch_filter_count gives them, except that the squares of
-// the dropped entries of the crossing bucket are left out: add them per
-// matrix with launch_select_drop_fix once dropped is summed per matrix.
+// the dropped entries of the crossing bucket are left out: launch_drop_sums
+// adds them per matrix.
 void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
-                         const int *active, const void *val, int val_f32, const int64_t *nnz,
-                         MatScalars *ms, void *scratch, int64_t *cnt, double *dropped,
+                         const int *active, const void *val, int val_f32, MatScalars *ms,
+                         void *scratch, int64_t *cnt, double *dropped,
                          cudaStream_t s);
-// sums[m] += the squares of matrix m's dropped entries of its crossing bucket
-// (after launch_select_exact with counts, on the same scratch).
-void launch_select_drop_fix(int nb, const int *active, void *scratch, const MatScalars *ms,
-                            double *sums, cudaStream_t s);
+// sums[m] = the dropped squares of matrix m's rows; with the scratch of a
+// launch_select_exact with counts (nullable), those of its crossing bucket are
+// added.
+void launch_drop_sums(int nb, const int64_t *moff, const double *dropped, const int *active,
+                      void *scratch, const MatScalars *ms, double *sums, cudaStream_t s);
 const unsigned long long *select_overflow(void *scratch, int nb);
 // ms[m].nnz_bar = nnz[m].
 void launch_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms, cudaStream_t s);

@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "seg.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -217,22 +218,19 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(int64_t n, const int64_t
   if (threadIdx.x == 0) tmp[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_blocks(int64_t nblocks, int64_t *tmp) {
+// A tile's scan: the tiles before it are added from their totals in tmp (a
+// single tile has none). seg, eoff (nullable): the scan's value at the end of
+// each matrix; total (nullable): the sum of all.
+__global__ void __launch_bounds__(SCAN_T)
+    k_scan_final(int64_t n, const int64_t *cnt, const int64_t *tmp, int64_t *out,
+                 const int32_t *seg, int64_t *eoff, int64_t *total) {
   __shared__ int64_t sm[33];
-  int64_t carry = 0;
-  for (int64_t b0 = 0; b0 < nblocks; b0 += SCAN_T) {
-    int64_t i = b0 + threadIdx.x;
-    int64_t v = i < nblocks ? tmp[i] : 0;
-    int64_t total;
-    int64_t ex = block_excl_scan(v, sm, &total);
-    if (i < nblocks) tmp[i] = carry + ex;
-    carry += total;
+  int64_t before = 0;
+  if (blockIdx.x > 0) {
+    int64_t v = 0;
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += SCAN_T) v += tmp[i];
+    block_excl_scan(v, sm, &before);
   }
-}
-
-__global__ void __launch_bounds__(SCAN_T) k_scan_final(int64_t n, const int64_t *cnt,
-                                                       const int64_t *tmp, int64_t *out) {
-  __shared__ int64_t sm[33];
   int64_t base = int64_t(blockIdx.x) * SCAN_TILE + int64_t(threadIdx.x) * SCAN_ITEMS;
   int64_t v[SCAN_ITEMS];
   int64_t s = 0;
@@ -241,13 +239,20 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_final(int64_t n, const int64_t 
     v[i] = base + i < n ? cnt[base + i] : 0;
     s += v[i];
   }
-  int64_t ex = block_excl_scan(s, sm, nullptr) + tmp[blockIdx.x];
+  int64_t ex = block_excl_scan(s, sm, nullptr) + before;
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     ex += v[i];
-    if (base + i < n) out[base + i + 1] = ex;
+    const int64_t r = base + i;
+    if (r >= n) break;
+    out[r + 1] = ex;
+    if (eoff && (r + 1 == n || seg[r + 1] != seg[r])) eoff[seg[r] + 1] = ex;
+    if (total && r + 1 == n) *total = ex;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    out[0] = 0;
+    if (eoff) eoff[0] = 0;
+  }
 }
 
 // ------------------------------------------------------------ assembly
@@ -432,59 +437,62 @@ __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp,
 // and the 1-norm's maxima below, the mixed solve of the tridiagonal matrix of
 // that order went from 16.3 to 11.9 ms, and to 11.0 with the rows prefetched
 // and the maxima reduced per warp (GB300).
-constexpr int RED_T = 256;  // partial sums per component; their order is fixed
-constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
-constexpr int RED_LANES = RED_T / RED_C;
-constexpr int RED_U = 16;   // rows loaded at once, the next ones while these are added
-static_assert(RED_LANES == 32, "one warp of each CTA per component");
 
-// Component c = threadIdx.y of matrix m: partial sum t (0 <= t < RED_T) adds
-// rows t, t + RED_T, ... one after another, and the partial sums are added
-// pairwise, t + s into t for s = RED_T / 2 .. 1. CTA q of the cluster holds the
-// partial sums 32 q .. 32 q + 31, a warp per component, so the FP64 additions
-// spread over RED_C SMs and the result does not depend on the split.
-__global__ void __cluster_dims__(RED_C, 1, 1)
-    k_seg_reduce(const int64_t *moff, const double *part, int ncomp, double *out) {
-  __shared__ double sm[2][RED_T];
+// out[m] = the sum of part over matrix m's rows.
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
+    k_seg_reduce(const int64_t *moff, const double *part, double *out) {
+  __shared__ double sm[RED_T];
   cg::cluster_group cl = cg::this_cluster();
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
-  const int c = threadIdx.y, t = q * RED_LANES + threadIdx.x;
+  const int t = q * RED_LANES + threadIdx.x;
   cl.sync();  // CTA 0 has started: its shared memory may be written
-  const int64_t e = moff[m + 1];
-  double acc = 0.0;
-  int64_t r = moff[m] + t;
-  double v[RED_U], w[RED_U];  // absent rows are loaded as -0, which adds nothing
-  auto fetch = [&](double (&d)[RED_U]) {
-#pragma unroll
-    for (int u = 0; u < RED_U; ++u, r += RED_T) d[u] = r < e ? part[r * ncomp + c] : -0.0;
-  };
-  auto add = [&](const double (&d)[RED_U]) {
-#pragma unroll
-    for (int u = 0; u < RED_U; ++u) acc += d[u];
-  };
-  fetch(v);
-  for (;;) {
-    if (r >= e) {
-      add(v);
-      break;
-    }
-    fetch(w);
-    add(v);
-    if (r >= e) {
-      add(w);
-      break;
-    }
-    fetch(v);
-    add(w);
-  }
-  *cl.map_shared_rank(&sm[c][t], 0) = acc;
+  *cl.map_shared_rank(&sm[t], 0) = seg_partial(part, 1, 0, moff[m], moff[m + 1], t);
   cl.sync();
   if (q != 0) return;
-  for (int s = RED_T / 2; s > 0; s >>= 1) {
-    for (int i = threadIdx.x; i < s; i += RED_LANES) sm[c][i] += sm[c][i + s];
-    __syncwarp();
+  seg_tree(sm);
+  if (threadIdx.x == 0) out[m] = sm[0];
+}
+
+// The check of a round in one launch: per matrix the sums of the two columns of
+// part (warps 0 and 1 of each CTA), the entries of T (warp 2) and from them r,
+// x, beta and b.
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(3 * RED_LANES)
+    k_check_scalars(const int64_t *moff, const double *part, const int64_t *rs, const int64_t *re,
+                    double c4, double tol_stage, double switch_resid, MatScalars *ms,
+                    int64_t *nnz) {
+  __shared__ double sm[2][RED_T];
+  __shared__ unsigned long long s_cnt;
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / RED_C, q = int(cl.block_rank()), c = threadIdx.x / RED_LANES;
+  const int t = q * RED_LANES + lane_id();
+  if (threadIdx.x == 0) s_cnt = 0ULL;
+  cl.sync();  // CTA 0 has started: its shared memory may be written
+  const int64_t b = moff[m], e = moff[m + 1];
+  if (c < 2) {
+    *cl.map_shared_rank(&sm[c][t], 0) = seg_partial(part, 2, c, b, e, t);
+  } else {
+    const unsigned long long k = seg_entries(rs, re, b, e, t, RED_T);
+    if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
   }
-  if (threadIdx.x == 0) out[int64_t(m) * ncomp + c] = sm[c][0];
+  cl.sync();
+  if (q != 0) return;
+  if (c < 2) seg_tree(sm[c]);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double sn = __dsqrt_rn(double(e - b));
+  const double r = __ddiv_rn(__dsqrt_rn(sm[0][0]), sn);
+  const double x = __ddiv_rn(__dsqrt_rn(sm[1][0]), sn);
+  double beta;
+  if (r >= switch_resid)
+    beta = __dmul_rn(c4, tol_stage);
+  else
+    beta = __ddiv_rn(__dmul_rn(__dmul_rn(0.75, r), r),
+                     __dadd_rn(__dmul_rn(3.0, x), __dmul_rn(__dmul_rn(x, x), x)));
+  ms[m].r = r;
+  ms[m].x = x;
+  ms[m].beta = beta;
+  ms[m].b = __dmul_rn(sn, beta);
+  nnz[m] = int64_t(s_cnt);
 }
 
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
@@ -494,15 +502,9 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
   if (threadIdx.x == 0) sm = 0ULL;
   cl.sync();
-  long long acc = 0;
-  const int64_t e = moff[m + 1];
-#pragma unroll 4
-  for (int64_t r = moff[m] + q * RED_T + threadIdx.x; r < e; r += RED_C * RED_T)
-    acc += re[r] - rs[r];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane_id() == 0 && acc)
-    atomicAdd(cl.map_shared_rank(&sm, 0), (unsigned long long)acc);
+  const unsigned long long k = seg_entries(rs, re, moff[m], moff[m + 1], q * RED_T + threadIdx.x,
+                                           RED_C * RED_T);
+  if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&sm, 0), k);
   cl.sync();
   if (q == 0 && threadIdx.x == 0) out[m] = int64_t(sm);
 }
@@ -610,17 +612,20 @@ void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s) {
 
 int64_t scan_tmp_elems(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
 
-void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s) {
+void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s,
+                 const int32_t *seg, int64_t *eoff, int64_t *total) {
   int64_t nblocks = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (nblocks == 0) {
     SGN_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), s));
+    if (eoff) SGN_CUDA(cudaMemsetAsync(eoff, 0, sizeof(int64_t), s));
+    if (total) SGN_CUDA(cudaMemsetAsync(total, 0, sizeof(int64_t), s));
     return;
   }
-  k_scan_reduce<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp);
-  SGN_LAUNCH_CHECK();
-  k_scan_blocks<<<1, SCAN_T, 0, s>>>(nblocks, tmp);
-  SGN_LAUNCH_CHECK();
-  k_scan_final<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp, out);
+  if (nblocks > 1) {
+    k_scan_reduce<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp);
+    SGN_LAUNCH_CHECK();
+  }
+  k_scan_final<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp, out, seg, eoff, total);
   SGN_LAUNCH_CHECK();
 }
 
@@ -681,11 +686,19 @@ void launch_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64
   SGN_LAUNCH_CHECK();
 }
 
-void launch_seg_reduce(int nb, const int64_t *moff, const double *part, int ncomp, double *out,
+void launch_seg_reduce(int nb, const int64_t *moff, const double *part, double *out,
                        cudaStream_t s) {
   if (nb == 0) return;
-  k_seg_reduce<<<unsigned(nb) * RED_C, dim3(RED_LANES, unsigned(ncomp)), 0, s>>>(moff, part, ncomp,
-                                                                             out);
+  k_seg_reduce<<<unsigned(nb) * RED_C, RED_LANES, 0, s>>>(moff, part, out);
+  SGN_LAUNCH_CHECK();
+}
+
+void launch_check_scalars(int nb, const int64_t *moff, const double *part, const int64_t *rs,
+                          const int64_t *re, double c4, double tol_stage, double switch_resid,
+                          MatScalars *ms, int64_t *nnz, cudaStream_t s) {
+  if (nb == 0) return;
+  k_check_scalars<<<unsigned(nb) * RED_C, 3 * RED_LANES, 0, s>>>(moff, part, rs, re, c4, tol_stage,
+                                                                switch_resid, ms, nnz);
   SGN_LAUNCH_CHECK();
 }
 

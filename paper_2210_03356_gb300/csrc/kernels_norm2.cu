@@ -205,11 +205,11 @@ void launch_norm2_est(int nb, const int64_t *moff, const int32_t *seg, int64_t n
     SGN_LAUNCH_CHECK();
     k_n2_zfinal<<<gr, 256, 0, s>>>(n, seg, ms, sw, wk.xmax, wk.ymax, wk.zacc, wk.z, wk.part);
     SGN_LAUNCH_CHECK();
-    launch_seg_reduce(nb, moff, wk.part, 1, wk.nrm, s);
+    launch_seg_reduce(nb, moff, wk.part, wk.nrm, s);
     k_n2_scale<<<gr, 256, 0, s>>>(n, seg, ms, sw, wk.z, wk.nrm, wk.v);
     SGN_LAUNCH_CHECK();
   }
-  launch_seg_reduce(nb, moff, wk.part, 1, wk.nrm, s);
+  launch_seg_reduce(nb, moff, wk.part, wk.nrm, s);
   k_n2_final<<<(nb + 127) / 128, 128, 0, s>>>(nb, wk.nrm, x2);
   SGN_LAUNCH_CHECK();
 }

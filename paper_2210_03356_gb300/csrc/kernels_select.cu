@@ -26,6 +26,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "seg.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -37,25 +38,6 @@ constexpr int NB0 = kSelBuckets;  // level-0 buckets: the sum below the pivot, t
 constexpr int NDIG = 256;         // digit buckets
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
-
-__global__ void k_matrix_scalars(int nb, const int64_t *moff, const double *sums, double c4,
-                                 double tol_stage, double switch_resid, MatScalars *ms) {
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nb) return;
-  double sn = __dsqrt_rn(double(moff[m + 1] - moff[m]));
-  double r = __ddiv_rn(__dsqrt_rn(sums[2 * m]), sn);
-  double x = __ddiv_rn(__dsqrt_rn(sums[2 * m + 1]), sn);
-  double beta;
-  if (r >= switch_resid)
-    beta = __dmul_rn(c4, tol_stage);
-  else
-    beta = __ddiv_rn(__dmul_rn(__dmul_rn(0.75, r), r),
-                     __dadd_rn(__dmul_rn(3.0, x), __dmul_rn(__dmul_rn(x, x), x)));
-  ms[m].r = r;
-  ms[m].x = x;
-  ms[m].beta = beta;
-  ms[m].b = __dmul_rn(sn, beta);
-}
 
 __global__ void k_select_bound(int nb, const int *active, MatScalars *ms) {
   int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -267,21 +249,32 @@ __device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, 
   return qval<T>(wide, eb);
 }
 
-// Per matrix, in a CTA of its own: nnz_bar = nnz[m] (nullable: as it is), e (the
-// biased exponent of b, 1 for a subnormal b), Q = q(b), the smallest key with
+// Per matrix, by a cluster: nnz_bar = its entries (row lists), e (the biased
+// exponent of b, 1 for a subnormal b), Q = q(b), the smallest key with
 // q >= 1 (the key of 2^(e - 31 - 1023)) and the pivot's bucket: a power of two
 // fraction below b / sqrt(nnz_bar), so that no rounding lifts it above. b = 0,
 // +inf or NaN: no key is summed (tiny = all ones), every q counts as 0.
 // Clears the matrix's histogram, minimum and candidate count.
-__global__ void __launch_bounds__(256)
-    k_sel_prepare(const int64_t *nnz, MatScalars *ms, SelScratch sc) {
-  const int m = blockIdx.x;
-  for (int t = threadIdx.x; t < 2 * NB0; t += 256) sc.hist0[size_t(m) * NB0 * 2 + t] = 0ULL;
-  if (threadIdx.x) return;
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
+    k_sel_prepare(SelRows R, MatScalars *ms, SelScratch sc) {
+  __shared__ unsigned long long s_cnt;  // CTA 0: the matrix's entries
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
+  if (threadIdx.x == 0) s_cnt = 0ULL;
+  cl.sync();
+  for (int t = q * RED_T + threadIdx.x; t < 2 * NB0; t += RED_C * RED_T)
+    sc.hist0[size_t(m) * NB0 * 2 + t] = 0ULL;
+  if (R.rs) {
+    const unsigned long long k = seg_entries(R.rs, R.re, R.moff[m], R.moff[m + 1],
+                                             q * RED_T + threadIdx.x, RED_C * RED_T);
+    if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
+  }
+  cl.sync();
+  if (q != 0 || threadIdx.x) return;
   sc.minabove[m] = ~0ULL;
   sc.ncand[m] = 0ULL;
   if (m == 0) *sc.overflow = 0ULL;
-  if (nnz) ms[m].nnz_bar = nnz[m];
+  if (R.rs) ms[m].nnz_bar = int64_t(s_cnt);
   const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
   const int e = int(bkey >> 52);
   if (bkey == 0ULL || e >= 0x7FF) {  // b <= 0 (sign bit) is caught here as well
@@ -690,20 +683,35 @@ __global__ void __launch_bounds__(SEL_THREADS)
   }
 }
 
-// sums[m] += the squares of the dropped candidates: the exact sum of their q
+// sums[m] = the dropped squares of matrix m's rows plus, with the select's
+// scratch, those of the dropped candidates: the exact sum of their q
 // (the select's sum below tau minus its sum below the crossing bucket) in
 // grid steps 2^(2e - 62). A candidate's magnitude is at least b / sqrt(1.1
 // nnz) (a bucket spans a factor 2^(1/16)), so its q is above 2^62 / (1.1 nnz)
 // and its flooring to an integer is far below the FP64 rounding of the sum.
-__global__ void k_sel_drop_fix(int nb, const int *active, SelScratch sc, const MatScalars *ms,
-                               double *sums) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nb || !active[m] || !sc.st[m].found) return;
-  const SelState st = sc.st[m];
-  const unsigned long long lo = st.below_lo - st.below0_lo;
-  const unsigned long long hi = st.below_hi - st.below0_hi - (st.below_lo < st.below0_lo ? 1ULL : 0ULL);
-  const double q = __fma_rn(double(hi), 18446744073709551616.0, double(lo));
-  sums[m] = __dadd_rn(sums[m], ldexp(q, 2 * (ms[m].sel_e - 1023) - 62));
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
+    k_drop_sums(const int64_t *moff, const double *dropped, const int *active, int exact,
+                SelScratch sc, const MatScalars *ms, double *sums) {
+  __shared__ double sm[RED_T];
+  cg::cluster_group cl = cg::this_cluster();
+  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
+  const int t = q * RED_LANES + threadIdx.x;
+  cl.sync();  // CTA 0 has started: its shared memory may be written
+  *cl.map_shared_rank(&sm[t], 0) = seg_partial(dropped, 1, 0, moff[m], moff[m + 1], t);
+  cl.sync();
+  if (q != 0) return;
+  seg_tree(sm);
+  if (threadIdx.x != 0) return;
+  double sum = sm[0];
+  if (exact && active[m] && sc.st[m].found) {
+    const SelState st = sc.st[m];
+    const unsigned long long lo = st.below_lo - st.below0_lo;
+    const unsigned long long hi =
+        st.below_hi - st.below0_hi - (st.below_lo < st.below0_lo ? 1ULL : 0ULL);
+    const double qs = __fma_rn(double(hi), 18446744073709551616.0, double(lo));
+    sum = __dadd_rn(sum, ldexp(qs, 2 * (ms[m].sel_e - 1023) - 62));
+  }
+  sums[m] = sum;
 }
 
 // The digits below the crossing bucket, tau and the kept candidates' counts of
@@ -966,13 +974,6 @@ __global__ void k_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms) {
 
 }  // namespace
 
-void launch_matrix_scalars(int nb, const int64_t *moff, const double *sums, double c4,
-                           double tol_stage, double switch_resid, MatScalars *ms, cudaStream_t s) {
-  k_matrix_scalars<<<(nb + 127) / 128, 128, 0, s>>>(nb, moff, sums, c4, tol_stage, switch_resid,
-                                                    ms);
-  SGN_LAUNCH_CHECK();
-}
-
 void launch_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms, cudaStream_t s) {
   k_store_nnz_bar<<<(nb + 127) / 128, 128, 0, s>>>(nb, nnz, ms);
   SGN_LAUNCH_CHECK();
@@ -1001,11 +1002,11 @@ static void sel_pass(int64_t nrows, int64_t nvals, F f) {
 
 template <typename T>
 static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *active, const T *val,
-                         const int64_t *nnz, MatScalars *ms, const SelScratch &sc, int64_t *cnt,
-                         double *dropped, cudaStream_t s) {
+                         MatScalars *ms, const SelScratch &sc, int64_t *cnt, double *dropped,
+                         cudaStream_t s) {
   {
     ProfScope ps(KC_SEL_HIST, s, 0.0, 0.0);
-    k_sel_prepare<<<nb, 256, 0, s>>>(nnz, ms, sc);
+    k_sel_prepare<<<unsigned(nb) * RED_C, RED_T, 0, s>>>(R, ms, sc);
     SGN_LAUNCH_CHECK();
     sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
       k_sel_hist0<T, lpr.value><<<g, SEL_THREADS, 0, s>>>(R, rpc, active, val, ms, sc);
@@ -1028,21 +1029,23 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *act
 }
 
 void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
-                         const int *active, const void *val, int val_f32, const int64_t *nnz,
-                         MatScalars *ms, void *scratch, int64_t *cnt, double *dropped,
-                         cudaStream_t s) {
+                         const int *active, const void *val, int val_f32, MatScalars *ms,
+                         void *scratch, int64_t *cnt, double *dropped, cudaStream_t s) {
   const SelScratch sc = carve(scratch, nb, cand_cap);
   if (val_f32)
-    select_exact<float>(nb, R, nvals, active, static_cast<const float *>(val), nnz, ms, sc, cnt,
-                        dropped, s);
+    select_exact<float>(nb, R, nvals, active, static_cast<const float *>(val), ms, sc, cnt, dropped,
+                        s);
   else
-    select_exact<double>(nb, R, nvals, active, static_cast<const double *>(val), nnz, ms, sc, cnt,
+    select_exact<double>(nb, R, nvals, active, static_cast<const double *>(val), ms, sc, cnt,
                          dropped, s);
 }
 
-void launch_select_drop_fix(int nb, const int *active, void *scratch, const MatScalars *ms,
-                            double *sums, cudaStream_t s) {
-  k_sel_drop_fix<<<(nb + 127) / 128, 128, 0, s>>>(nb, active, carve(scratch, nb, 1), ms, sums);
+void launch_drop_sums(int nb, const int64_t *moff, const double *dropped, const int *active,
+                      void *scratch, const MatScalars *ms, double *sums, cudaStream_t s) {
+  if (nb == 0) return;
+  const SelScratch sc = scratch ? carve(scratch, nb, 1) : SelScratch{};
+  k_drop_sums<<<unsigned(nb) * RED_C, RED_LANES, 0, s>>>(moff, dropped, active, scratch ? 1 : 0, sc,
+                                                        ms, sums);
   SGN_LAUNCH_CHECK();
 }
 

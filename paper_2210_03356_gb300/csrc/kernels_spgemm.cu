@@ -134,11 +134,11 @@ constexpr int64_t BOUNDS_LONG = 256;
 
 // The bounds and class of one row of sparse work, from its k hull [kf, kl],
 // its column hull [mn, mx] (mx < 0: no output) and its multiply-adds wk;
-// writes lo, len, ub, work of row r and, for band tiles, the row's statistics.
+// writes lo, len, ub of row r and, for band tiles, the row's statistics.
 __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t mn, int32_t mx,
                                           int32_t kf, int32_t kl, int64_t wk, int mode,
                                           int groups, float group_margin, int band, int32_t *lo,
-                                          int32_t *len, int64_t *ub, double *work, int *sseg,
+                                          int32_t *len, int64_t *ub, int *sseg,
                                           int *slo, int *sL, int *skf, int *skl, int *sna,
                                           float *swk) {
   int cls = RC_NONE;
@@ -146,7 +146,6 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
     ub[r] = 0;
     len[r] = 0;
     lo[r] = 0;
-    work[r] = double(wk);
   } else {
     const int32_t L = mx - mn + 1;
     const int64_t bound = wk + (mode == MODE_UPDATE ? na : 0);
@@ -167,7 +166,6 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
     lo[r] = mn;
     len[r] = L;
     ub[r] = bound < L ? bound : L;
-    work[r] = double(wk);
   }
   if (band) {
     *sseg = m;
@@ -188,7 +186,8 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
              const int *active, int mode, int groups, float group_margin, int band,
              float band_min_eff, const int *dslot,
              const int64_t *moff, int32_t *lo, int32_t *len, int64_t *ub, int32_t *lists,
-             int *counters, double *work, double *band_work, unsigned char *bandrow) {
+             int *counters, unsigned long long *mults, double *band_work,
+             unsigned char *bandrow) {
   __shared__ unsigned char s_cls[BOUNDS_TILE];
   __shared__ int s_cnt[BOUNDS_TILE / 32][RC_N];
   __shared__ int s_base[RC_N];
@@ -212,6 +211,7 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
     s_seg[i] = -1;  // not eligible for a band tile
     int m = 0;
     int64_t a0 = 0, a1 = 0;
+    unsigned long long mywork = 0;  // the row's multiply-adds
     if (r < n) {
       m = seg[r];
       if (!active[m] || (dslot && dslot[m] >= 0)) {
@@ -221,7 +221,6 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
         ub[r] = dense && mode == MODE_UPDATE ? moff[m + 1] - moff[m] : 0;
         len[r] = 0;
         lo[r] = 0;
-        work[r] = 0.0;
       } else {
         a0 = ars[r];
         a1 = are[r];
@@ -251,8 +250,9 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
             mn = min(mn, kf);
             mx = max(mx, kl);
           }
+          mywork = (unsigned long long)wk;
           cls = bounds_row(r, m, a1 - a0, mn, mx, kf, kl, wk, mode, groups, group_margin, band,
-                           lo, len, ub, work, s_seg + i, s_lo + i, s_L + i, s_kf + i, s_kl + i,
+                           lo, len, ub, s_seg + i, s_lo + i, s_L + i, s_kf + i, s_kl + i,
                            s_na + i, s_wk + i);
         }
       }
@@ -287,11 +287,21 @@ __global__ void __launch_bounds__(BOUNDS_TILE)
           mn = min(mn, kf);
           mx = max(mx, kl);
         }
+        mywork = (unsigned long long)wk;
         s_cls[li] = (unsigned char)bounds_row(lr, lmat, la1 - la0, mn, mx, kf, kl, wk, mode,
-                                              groups, group_margin, band, lo, len, ub, work,
+                                              groups, group_margin, band, lo, len, ub,
                                               s_seg + li, s_lo + li, s_L + li, s_kf + li,
                                               s_kl + li, s_na + li, s_wk + li);
       }
+    }
+    // multiply-adds per matrix: one atomic per warp where its rows are of one matrix
+    if (__all_sync(0xffffffffu, m == __shfl_sync(0xffffffffu, m, 0) || mywork == 0)) {
+      unsigned long long sum = mywork;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0 && sum) atomicAdd(&mults[m], sum);
+    } else if (mywork) {
+      atomicAdd(&mults[m], mywork);
     }
     __syncthreads();
     // band tiles: aligned groups of 16 rows of one matrix, all with sparse
@@ -1189,7 +1199,7 @@ int grid_cap(int64_t items, int per_block, int per_sm) {
 void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, const int *active,
                    int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
-                   int64_t *ub, int32_t *lists, int *counters, double *work,
+                   int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
                    cudaStream_t s) {
   if (n == 0) return;
@@ -1199,7 +1209,7 @@ void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, 
   int g = tiles < sm_count() * 8 ? tiles : sm_count() * 8;
   k_bounds<<<g, BOUNDS_TILE, 0, s>>>(n, A.rs, A.re, A.col, binfo, seg, active, mode, groups,
                                      group_margin, band, band_min_eff, dslot, moff, lo, len, ub,
-                                     lists, counters, work, band_work, bandrow);
+                                     lists, counters, mults, band_work, bandrow);
   SGN_LAUNCH_CHECK();
 }
 
@@ -1279,7 +1289,7 @@ void launch_col_blocks(int64_t n, const Rows &B, const int32_t *seg, const int64
 }
 
 int wide_block_shift(int64_t max_n) {
-  int sh = 7;
+  int sh = 5;
   while (sh < 9 && (max_n >> sh) >= 64) ++sh;
   return sh;
 }

@@ -1,0 +1,83 @@
+// Sums over the rows of a matrix by a cluster of RED_C CTAs, one warp of each
+// per summed component.
+#pragma once
+
+#include <cooperative_groups.h>
+#include <stdint.h>
+
+namespace sgn {
+
+constexpr int RED_T = 256;  // partial sums per component; their order is fixed
+constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
+constexpr int RED_LANES = RED_T / RED_C;
+constexpr int RED_U = 16;   // rows loaded at once, the next ones while these are added
+static_assert(RED_LANES == 32, "one warp of each CTA per component");
+
+// acc + v as a fused multiply-add (v * 1 is exact): in a chain of dependent FP64
+// additions a DFMA takes 64 cycles, a DADD 76. In PTX, so that it stays one.
+__device__ __forceinline__ double chain_add(double acc, double v) {
+  double r;
+  asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(v), "d"(1.0), "d"(acc));
+  return r;
+}
+
+// Partial sum t of component c: rows b + t, b + t + RED_T, ... below e, one after
+// another.
+__device__ __forceinline__ double seg_partial(const double *part, int ncomp, int c, int64_t b,
+                                              int64_t e, int t) {
+  double acc = 0.0;
+  int64_t r = b + t;
+  double v[RED_U], w[RED_U];  // absent rows are loaded as -0, which adds nothing
+  auto fetch = [&](double (&d)[RED_U]) {
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u, r += RED_T) d[u] = r < e ? part[r * ncomp + c] : -0.0;
+  };
+  auto add = [&](const double (&d)[RED_U]) {
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u) acc = chain_add(acc, d[u]);
+  };
+  if (e - b <= RED_U / 2 * RED_T) {  // short matrices: no rows to load ahead
+    for (; r < e; r += RED_T) acc = chain_add(acc, part[r * ncomp + c]);
+    return acc;
+  }
+  fetch(v);
+  for (;;) {
+    if (r >= e) {
+      add(v);
+      break;
+    }
+    fetch(w);
+    add(v);
+    if (r >= e) {
+      add(w);
+      break;
+    }
+    fetch(v);
+    add(w);
+  }
+  return acc;
+}
+
+// One warp: the partial sums sm[0 .. RED_T) added pairwise, t + s into t for
+// s = RED_T / 2 .. 1, into sm[0].
+__device__ __forceinline__ void seg_tree(double *sm) {
+  const int lane = threadIdx.x & 31;
+  for (int s = RED_T / 2; s > 0; s >>= 1) {
+    for (int i = lane; i < s; i += 32) sm[i] += sm[i + s];
+    __syncwarp();
+  }
+}
+
+// Warp q of a matrix's cluster: its share of the entries of the rows [b, e).
+__device__ __forceinline__ unsigned long long seg_entries(const int64_t *rs, const int64_t *re,
+                                                          int64_t b, int64_t e, int first,
+                                                          int step) {
+  long long acc = 0;
+#pragma unroll 8
+  for (int64_t r = b + first; r < e; r += step) acc += re[r] - rs[r];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return (unsigned long long)acc;
+}
+
+}  // namespace sgn

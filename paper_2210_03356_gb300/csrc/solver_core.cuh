@@ -18,6 +18,7 @@
 #pragma once
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <memory>
@@ -194,8 +195,8 @@ struct BandBuf {
 
 // Shared scratch of one solve call.
 struct Work {
-  DevBuf lo, len, ub, wlist, clist, counters, part, scan_tmp, eoff, sums, ms, active, sel,
-      asm_blocks, asm_off, asm_lens, dropped, norm_work, norm, work, mults, cnt, nnzc, xblocks,
+  DevBuf lo, len, ub, wlist, clist, counters, part, scan_tmp, eoff, ms, active, sel,
+      asm_blocks, asm_off, asm_lens, dropped, norm_work, norm, cnt, xblocks,
       dslot, dmem, dbufs, djobs, dscratch, dcount, derr;
   DevBuf wide;     // column-block table of a product's B (wide rows)
   BandBuf bx, bt;  // bands of the iterate X and of T = X X (FP32 stage)
@@ -219,21 +220,51 @@ struct DensePlan {
   bool any() const { return nd > 0; }
 };
 
+// What the host reads back at a wait lies in one block, on the device (Work) and
+// in its host mirror, and is copied at once.
+// A product: class counters, band-tile multiply-adds, totals of the slots and
+// of the two bands, multiply-adds per matrix.
+struct ProductHead {
+  int ctr[RC_COUNTERS];
+  double band_work;
+  int64_t tot[3];
+  unsigned long long mults[1];  // per matrix
+  static size_t bytes(int nb) { return offsetof(ProductHead, mults) + 8 * size_t(nb); }
+};
+static_assert(offsetof(ProductHead, band_work) % 8 == 0 && offsetof(ProductHead, mults) % 8 == 0,
+              "8-byte fields");
+// A check or a filter: scalars, dropped squares, entry offsets, entries.
+struct MatPack {
+  MatScalars *ms;
+  double *dsum;
+  int64_t *ex, *nnz;
+  static MatPack at(void *p, int nb) {
+    MatPack k;
+    k.ms = static_cast<MatScalars *>(p);
+    k.dsum = reinterpret_cast<double *>(k.ms + nb);
+    k.ex = reinterpret_cast<int64_t *>(k.dsum + nb);
+    k.nnz = k.ex + nb + 1;
+    return k;
+  }
+  static size_t bytes(int nb) { return (sizeof(MatScalars) + 24) * size_t(nb) + 8; }
+};
+
 // Page-locked host mirrors of the per-matrix values read back every round.
 // Kept per host thread and grown only (cudaFreeHost would synchronize the
 // device), so repeated solves reuse them.
 struct HostMirror {
   void *p = nullptr;
   size_t cap = 0;
-  MatScalars *ms = nullptr;
-  int64_t *ex = nullptr, *nnz_t = nullptr, *nnz_bar = nullptr, *tot = nullptr;
-  double *mults = nullptr, *dsum = nullptr;
+  MatPack pack;
+  ProductHead *head = nullptr;
+  double *mults = nullptr;  // of the last product, per matrix
+  int64_t *tot = nullptr;
   ExtractBlock *xb = nullptr;
-  int *ctr = nullptr;  // the product's class counters
-  void alloc(int nb) {
-    size_t bytes = sizeof(MatScalars) * nb + sizeof(int64_t) * (4 * size_t(nb) + 8) +
-                   sizeof(double) * 2 * size_t(nb) + sizeof(ExtractBlock) * nb +
-                   sizeof(int) * RC_COUNTERS + 1024;
+  int nb = 0;
+  void alloc(int n) {
+    nb = n;
+    size_t bytes = MatPack::bytes(nb) + ProductHead::bytes(nb) + sizeof(double) * size_t(nb) +
+                   sizeof(ExtractBlock) * nb + 64 + 1024;
     if (bytes > cap) {
       if (p) cudaFreeHost(p);
       p = nullptr;
@@ -246,15 +277,11 @@ struct HostMirror {
       c += (b + 63) & ~size_t(63);
       return r;
     };
-    ms = reinterpret_cast<MatScalars *>(take(sizeof(MatScalars) * nb));
-    ex = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * (nb + 1)));
-    nnz_t = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * nb));
-    nnz_bar = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * nb));
-    tot = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * 4));
+    pack = MatPack::at(take(MatPack::bytes(nb)), nb);
+    head = reinterpret_cast<ProductHead *>(take(ProductHead::bytes(nb)));
     mults = reinterpret_cast<double *>(take(sizeof(double) * nb));
-    dsum = reinterpret_cast<double *>(take(sizeof(double) * nb));
+    tot = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * 4));
     xb = reinterpret_cast<ExtractBlock *>(take(sizeof(ExtractBlock) * nb));
-    ctr = reinterpret_cast<int *>(take(sizeof(int) * RC_COUNTERS));
   }
   ~HostMirror() {
     if (p) cudaFreeHost(p);
@@ -384,15 +411,16 @@ struct Solver {
                          dst.d_col(), dst.val.p, is_f32<TD>(), s);
   }
 
-  // the band tiles' multiply-adds, a double after the class counters
-  double *band_work_dev() {
-    return reinterpret_cast<double *>(w.counters.as<char>() + sizeof(int) * RC_COUNTERS);
+  // the last product's values for the host, and the round's per-matrix values
+  ProductHead *head_dev() { return w.counters.as<ProductHead>(); }
+  MatPack pack_dev(int nb) { return MatPack::at(w.ms.ensure(MatPack::bytes(nb), s), nb); }
+  void read_pack(int nb) {
+    d2h(reinterpret_cast<char *>(hm.pack.ms), w.ms.p, MatPack::bytes(nb), s);
   }
 
   // ---------------------------------------------------------------- product
   // C = A B for a stage. Enqueues everything; on return C is allocated and the
-  // product queued, hm.mults holds the per-matrix multiply-adds (synced) and
-  // w.nnzc the per-matrix nnz of C (device, read with the next sync).
+  // product queued and hm.mults holds the per-matrix multiply-adds (synced).
   template <typename T>
   void product(Stage<T> &st, const Rows &A, const T *aval, int64_t nnzA, const Rows &B,
                const T *bval, int64_t nnzB, int mode, Slotted<T> &C, const int *active,
@@ -403,12 +431,10 @@ struct Solver {
     w.len.ensure(sizeof(int32_t) * size_t(N), s);
     w.ub.ensure(sizeof(int64_t) * size_t(N), s);
     w.wlist.ensure(sizeof(int32_t) * size_t(RC_N) * size_t(N), s);
-    w.work.ensure(sizeof(double) * size_t(N), s);
-    w.mults.ensure(sizeof(double) * size_t(nb), s);
-    w.nnzc.ensure(sizeof(int64_t) * size_t(nb), s);
-    w.counters.ensure(sizeof(int) * RC_COUNTERS + sizeof(double), s);  // + band multiply-adds
+    w.counters.ensure(ProductHead::bytes(nb), s);
+    ProductHead *const head = head_dev();
     w.scan_tmp.ensure(sizeof(int64_t) * size_t(scan_tmp_elems(N)), s);
-    SGN_CUDA(cudaMemsetAsync(w.counters.p, 0, sizeof(int) * RC_COUNTERS + sizeof(double), s));
+    SGN_CUDA(cudaMemsetAsync(head, 0, ProductHead::bytes(nb), s));
     // band tiles (FP32): in SQUARE the bands of X (both operands) and of T
     // (the output, for the update) are laid out here, their sizes read with
     // the slot total below; the band tiles write the rows of T's band they
@@ -430,12 +456,10 @@ struct Solver {
                     dp && dp->any() ? w.dslot.as<int>() : nullptr,
                     st.d_moff.template as<int64_t>(), w.lo.as<int32_t>(),
                     w.len.as<int32_t>(), w.ub.as<int64_t>(), w.wlist.as<int32_t>(),
-                    w.counters.as<int>(), w.work.as<double>(), band_work_dev(),
+                    head->ctr, head->mults, &head->band_work,
                     band && mode == MODE_SQUARE ? w.bandrow.as<unsigned char>() : nullptr,
                     static_cast<int4 *>(w.binfo.ensure(sizeof(int4) * size_t(N > 0 ? N : 1), s)),
                     ends, s);
-      launch_seg_reduce(nb, st.d_moff.template as<int64_t>(), w.work.as<double>(), 1,
-                        w.mults.as<double>(), s);
       if (band) {
         if (mode == MODE_SQUARE) {
           for (BandBuf *b : {&w.bx, &w.bt}) {
@@ -449,14 +473,12 @@ struct Solver {
           launch_band_spans(N, B, w.bx.fc.as<int32_t>(), w.bx.nf.as<int32_t>(),
                             w.bx.span.as<int64_t>(), s);
           launch_scan(N, w.bx.span.as<int64_t>(), w.bx.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s);
+                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[1]);
           launch_band_spans_range(N, w.lo.as<int32_t>(), w.len.as<int32_t>(),
                                   w.bt.fc.as<int32_t>(), w.bt.nf.as<int32_t>(),
                                   w.bt.span.as<int64_t>(), s);
           launch_scan(N, w.bt.span.as<int64_t>(), w.bt.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s);
-          d2h(hm.tot + 1, w.bx.pos.as<int64_t>() + N, 1, s);
-          d2h(hm.tot + 2, w.bt.pos.as<int64_t>() + N, 1, s);
+                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[2]);
         } else if (!b_is_square_t) {  // B is not the square's T: its own layout
           w.bt.filled = false;
           w.bt_rows_done = false;
@@ -467,10 +489,8 @@ struct Solver {
           launch_band_spans(N, B, w.bt.fc.as<int32_t>(), w.bt.nf.as<int32_t>(),
                             w.bt.span.as<int64_t>(), s);
           launch_scan(N, w.bt.span.as<int64_t>(), w.bt.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s);
-          d2h(hm.tot + 2, w.bt.pos.as<int64_t>() + N, 1, s);
+                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[2]);
         }
-        d2h(hm.dsum, band_work_dev(), 1, s);
       }
     }
     C.n = N;
@@ -478,19 +498,20 @@ struct Solver {
     C.re.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
     {
       ProfScope ps(KC_SCAN, s);
-      launch_scan(N, w.ub.as<int64_t>(), C.rs.template as<int64_t>(), w.scan_tmp.as<int64_t>(), s);
+      launch_scan(N, w.ub.as<int64_t>(), C.rs.template as<int64_t>(), w.scan_tmp.as<int64_t>(), s,
+                  nullptr, nullptr, &head->tot[0]);
     }
-    d2h(hm.tot, C.rs.template as<int64_t>() + N, 1, s);
-    d2h(hm.mults, w.mults.p, size_t(nb), s);
-    d2h(hm.ctr, w.counters.p, RC_COUNTERS, s);
+    d2h(reinterpret_cast<char *>(hm.head), head, ProductHead::bytes(nb), s);
     wait();
-    int64_t slots = hm.tot[0];
-    const bool band_tiles = band && hm.ctr[RC_BAND] > 0;
+    const int *const ctr = hm.head->ctr;
+    for (int i = 0; i < nb; ++i) hm.mults[i] = double(hm.head->mults[i]);
+    int64_t slots = hm.head->tot[0];
+    const bool band_tiles = band && ctr[RC_BAND] > 0;
     if (band && mode == MODE_SQUARE) {
-      w.bx.total = hm.tot[1];
-      w.bt.total = hm.tot[2];
+      w.bx.total = hm.head->tot[1];
+      w.bt.total = hm.head->tot[2];
     } else if (band && !b_is_square_t) {
-      w.bt.total = hm.tot[2];
+      w.bt.total = hm.head->tot[2];
     }
     if (band_tiles) {
       auto alloc = [&](BandBuf &b) {
@@ -525,7 +546,7 @@ struct Solver {
     if (mode == MODE_SQUARE) w.part.ensure(sizeof(double) * size_t(2 * N), s);
     double fl = 0.0;
     for (int i = 0; i < nb; ++i) fl += 2.0 * hm.mults[i];
-    const double fl_band = band_tiles ? 2.0 * hm.dsum[0] : 0.0;  // the band tiles' share
+    const double fl_band = band_tiles ? 2.0 * hm.head->band_work : 0.0;  // the band tiles' share
     double per = 4.0 + sizeof(T);
     // algorithmic bytes: A and B read once, C written once (its size is known
     // after the launch; the slot total bounds it and is used here)
@@ -541,12 +562,12 @@ struct Solver {
       const double mean_b = fl / (2.0 * double(nnzA > 0 ? nnzA : 1));
       const bool shared = few && mean_b >= SHARED_B;
       int rows[RC_N];
-      std::copy(hm.ctr, hm.ctr + RC_N, rows);
+      std::copy(ctr, ctr + RC_N, rows);
       const int wide_rows[2] = {rows[RC_CTA], shared ? rows[RC_G32] : 0};
       launch_numeric<T>(N, rows, shared, few, A, aval, B, bval, mode, ends, w.lo.as<int32_t>(),
                         w.len.as<int32_t>(), st.d_seg.template as<int32_t>(),
                         dp && dp->any() ? w.dslot.as<int>() : nullptr, w.wlist.as<int32_t>(),
-                        w.counters.as<int>(), C.rs.template as<int64_t>(),
+                        head->ctr, C.rs.template as<int64_t>(),
                         C.re.template as<int64_t>(), C.col.template as<int32_t>(), C.d_val(),
                         mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
       if (wide_rows[0] + wide_rows[1] > 0) {
@@ -567,7 +588,7 @@ struct Solver {
         for (int i = 0; i < 2; ++i)
           launch_numeric_wide<T>(N, i ? RC_G32 : RC_CTA, wide_rows[i], mean_b, A, aval, B, bval,
                                  mode, wt, w.lo.as<int32_t>(), w.len.as<int32_t>(),
-                                 w.wlist.as<int32_t>(), w.counters.as<int>(),
+                                 w.wlist.as<int32_t>(), head->ctr,
                                  C.rs.template as<int64_t>(), C.re.template as<int64_t>(),
                                  C.col.template as<int32_t>(), C.d_val(),
                                  mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
@@ -584,14 +605,20 @@ struct Solver {
       launch_band_product(N, mode, A, reinterpret_cast<const float *>(aval), w.bx.view(),
                           mode == MODE_SQUARE ? w.bx.view() : w.bt.view(), tout,
                           w.lo.as<int32_t>(), w.len.as<int32_t>(), w.wlist.as<int32_t>(),
-                          w.counters.as<int>(), C.rs.template as<int64_t>(),
+                          head->ctr, C.rs.template as<int64_t>(),
                           C.re.template as<int64_t>(), C.col.template as<int32_t>(),
                           reinterpret_cast<float *>(C.val.p),
                           mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
     }
     if (dp && dp->any()) dense_step(st, mode, C, active, *dp);
-    launch_seg_count(nb, st.d_moff.template as<int64_t>(), C.rs.template as<int64_t>(),
-                     C.re.template as<int64_t>(), w.nnzc.as<int64_t>(), s);
+  }
+
+  // Entries per matrix of slotted rows into the pack (the EXACT select and the
+  // check count their rows themselves).
+  template <typename T>
+  void count_entries(Stage<T> &st, const Slotted<T> &C, int64_t *nnz) {
+    launch_seg_count(int(st.mats.size()), st.d_moff.template as<int64_t>(),
+                     C.rs.template as<int64_t>(), C.re.template as<int64_t>(), nnz, s);
   }
 
   // ---------------------------------------------------------------- dense path (a9)
@@ -879,15 +906,13 @@ struct Solver {
     product(st, xr, st.X.d_val(), st.X.nnz, xr, st.X.d_val(), st.X.nnz, MODE_SQUARE, st.Tm, d_act,
             &dp);
     std::vector<double> mt(hm.mults, hm.mults + nb);  // sparse multiply-adds of T
-    w.sums.ensure(sizeof(double) * size_t(2 * nb), s);
-    w.ms.ensure(sizeof(MatScalars) * size_t(nb), s);
+    const MatPack pk = pack_dev(nb);
     double tol_stage = st.prec == 32 ? o.fp32_until : o.tol;
     {
       ProfScope ps(KC_REDUCE, s);
-      launch_seg_reduce(nb, st.d_moff.template as<int64_t>(), w.part.as<double>(), 2,
-                        w.sums.as<double>(), s);
-      launch_matrix_scalars(nb, st.d_moff.template as<int64_t>(), w.sums.as<double>(), o.c4,
-                            tol_stage, o.switch_resid, w.ms.as<MatScalars>(), s);
+      launch_check_scalars(nb, st.d_moff.template as<int64_t>(), w.part.as<double>(),
+                           st.Tm.rs.template as<int64_t>(), st.Tm.re.template as<int64_t>(), o.c4,
+                           tol_stage, o.switch_resid, pk.ms, pk.nnz, s);
     }
     if (o.budget_norm) {  // variant: x = ||X||_2 in Eq. (1.18)
       ProfScope ps(KC_REDUCE, s);
@@ -909,19 +934,18 @@ struct Solver {
       launch_budget_x2(nb, st.d_moff.template as<int64_t>(), w.x2.as<double>(), o.switch_resid,
                        w.ms.as<MatScalars>(), s);
     }
-    d2h(hm.ms, w.ms.p, size_t(nb), s);
-    d2h(hm.nnz_t, w.nnzc.p, size_t(nb), s);
+    read_pack(nb);
     std::vector<unsigned long long> dcount(dp.nd);
     if (dp.any()) d2h(dcount.data(), w.dcount.p, size_t(dp.nd), s);
     wait();
     for (int d = 0; d < dp.nd; ++d) {  // the dense path's T: its nonzeros and multiply-adds
       int i = dp.mat[d];
-      hm.nnz_t[i] += int64_t(dcount[d]);
+      hm.pack.nnz[i] += int64_t(dcount[d]);
       double n = double(st.moff[i + 1] - st.moff[i]);
       mt[i] = n * n * n;
     }
     hcheck.stop();
-    std::vector<MatScalars> hms(hm.ms, hm.ms + nb);
+    std::vector<MatScalars> hms(hm.pack.ms, hm.pack.ms + nb);
     // ---- per-matrix decisions (steps a7, a8); leavers copied out in one launch
     HostScope hdecide(KH_DECIDE);
     int nx = 0;
@@ -932,7 +956,7 @@ struct Solver {
       if (!st.alive[i]) continue;
       MatState &ms = m[st.mats[i]];
       double r = hms[i].r;
-      trace_put(ms, ex[i + 1] - ex[i], hm.nnz_t[i], r, hms[i].x, st.prec, mt[i]);
+      trace_put(ms, ex[i + 1] - ex[i], hm.pack.nnz[i], r, hms[i].x, st.prec, mt[i]);
       ms.resid = r;
       int decision = 0;  // 0 update, 1 retire, 2 move
       if (st.prec == 64 && r <= o.tol) {
@@ -1016,7 +1040,7 @@ struct Solver {
     // ---- update: Xbar = 1.5 X - 0.5 X T (step a3), or NMF's (X + X^-1) / 2
     HostScope hupdate(KH_UPDATE);
     int64_t nnz_t_all = 0;
-    for (int i = 0; i < nb; ++i) nnz_t_all += hm.nnz_t[i];
+    for (int i = 0; i < nb; ++i) nnz_t_all += hm.pack.nnz[i];
     std::vector<double> mb(nb, 0.0);
     bool nmf = false;
     if constexpr (sizeof(T) == 8) nmf = o.method == SIGN_METHOD_NMF;
@@ -1045,8 +1069,10 @@ struct Solver {
       }
     }
     // per-matrix nnz(Xbar) straight into the device scalars (the threshold selects do it themselves)
-    if (o.filter == SIGN_FILTER_NONE)
-      launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
+    if (o.filter == SIGN_FILTER_NONE) {
+      count_entries(st, st.Xb, pk.nnz);
+      launch_store_nnz_bar(nb, pk.nnz, pk.ms, s);
+    }
     // the iterate is not read again this round: a large one's memory can take
     // the filtered update (reuse is ordered after the update on this stream)
     if (st.X.col.cap + st.X.val.cap > BIG_BUFFER) {
@@ -1157,8 +1183,6 @@ struct Solver {
       launch_extract(nx, w.xblocks.as<ExtractBlock>(), xmax, s);
       put(w.active.p, st.alive.data(), st.alive.size());
     }
-    launch_seg_count(nb, st.d_moff.template as<int64_t>(), C.rs.as<int64_t>(), C.re.as<int64_t>(),
-                     w.nnzc.as<int64_t>(), s);
     int live = 0;
     for (int a : st.alive) live += a;
     if (live == 0) wait();  // the extraction reads X and the pinned block list
@@ -1188,12 +1212,14 @@ struct Solver {
                 st.d_moff.template as<int64_t>(),
                 w.sel_shift};
       launch_select_exact(nb, R, in.slots, cap, d_act, in.val.p, is_f32<T>(),
-                          w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), w.sel.p,
-                          w.cnt.as<int64_t>(), w.dropped.as<double>(), s);
+                          w.ms.as<MatScalars>(), w.sel.p, w.cnt.as<int64_t>(),
+                          w.dropped.as<double>(), s);
     } else {
       ProfScope psel(KC_SELECT, s);
-      launch_store_nnz_bar(nb, w.nnzc.as<int64_t>(), w.ms.as<MatScalars>(), s);
-      launch_select_bound(nb, d_act, w.ms.as<MatScalars>(), s);
+      const MatPack pk = pack_dev(nb);
+      count_entries(st, in, pk.nnz);
+      launch_store_nnz_bar(nb, pk.nnz, pk.ms, s);
+      launch_select_bound(nb, d_act, pk.ms, s);
     }
   }
 
@@ -1208,7 +1234,7 @@ struct Solver {
     w.dropped.ensure(sizeof(double) * size_t(N > 0 ? N : 1), s);
     w.cnt.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
     out.rp.ensure(sizeof(int64_t) * size_t(N + 1), s);
-    w.eoff.ensure(sizeof(int64_t) * size_t(nb + 1), s);
+    const MatPack pk = pack_dev(nb);
     const bool exact = o.filter == SIGN_FILTER_EXACT;
     for (;;) {
       {
@@ -1220,27 +1246,20 @@ struct Solver {
                               in.rs.template as<int64_t>(), in.re.template as<int64_t>(),
                               in.val.p, is_f32<T>(), w.ms.as<MatScalars>(), w.cnt.as<int64_t>(),
                               w.dropped.as<double>(), s);
-        launch_scan(N, w.cnt.as<int64_t>(), out.d_rp(), w.scan_tmp.as<int64_t>(), s);
-        launch_seg_reduce(nb, st.d_moff.template as<int64_t>(), w.dropped.as<double>(), 1,
-                          w.sums.as<double>(), s);
-        if (exact)
-          launch_select_drop_fix(nb, d_act, w.sel.p, w.ms.as<MatScalars>(), w.sums.as<double>(),
-                                 s);
-        launch_gather_offsets(nb, st.d_moff.template as<int64_t>(), out.d_rp(),
-                              w.eoff.as<int64_t>(), s);
+        launch_scan(N, w.cnt.as<int64_t>(), out.d_rp(), w.scan_tmp.as<int64_t>(), s,
+                    st.d_seg.template as<int32_t>(), pk.ex);
+        launch_drop_sums(nb, st.d_moff.template as<int64_t>(), w.dropped.as<double>(), d_act,
+                         exact ? w.sel.p : nullptr, pk.ms, pk.dsum, s);
       }
-      d2h(hm.ex, w.eoff.p, size_t(nb + 1), s);
-      d2h(hm.tot, out.d_rp() + N, 1, s);
-      d2h(hm.ms, w.ms.p, size_t(nb), s);
-      d2h(hm.dsum, w.sums.p, size_t(nb), s);
+      read_pack(nb);
       const bool capped = exact && w.sel_shift > 0;
-      if (capped) d2h(reinterpret_cast<unsigned long long *>(hm.tot + 3),
-                      select_overflow(w.sel.p, nb), 1, s);
+      if (capped)
+        d2h(reinterpret_cast<unsigned long long *>(hm.tot), select_overflow(w.sel.p, nb), 1, s);
       wait();
-      if (!capped || hm.tot[3] == 0) break;
+      if (!capped || hm.tot[0] == 0) break;
       select_threshold(st, in, d_act, true);  // the crossing bucket outgrew the room
     }
-    int64_t nnz = hm.tot[0];
+    int64_t nnz = hm.pack.ex[nb];
     out.n = N;
     out.nnz = nnz;
     out.col.ensure(sizeof(int32_t) * size_t(nnz > 0 ? nnz : 1), s);
@@ -1253,8 +1272,8 @@ struct Solver {
                           in.col.template as<int32_t>(), in.val.p, is_f32<T>(),
                           w.ms.as<MatScalars>(), out.d_rp(), out.d_col(), out.val.p, s);
     }
-    ex.assign(hm.ex, hm.ex + nb + 1);
-    if (dsum) dsum->assign(hm.dsum, hm.dsum + nb);
+    ex.assign(hm.pack.ex, hm.pack.ex + nb + 1);
+    if (dsum) dsum->assign(hm.pack.dsum, hm.pack.dsum + nb);
   }
 
   // Filter + compaction (step a6): Xh = entries of Xb with |x| >= tau, x != 0.
@@ -1265,9 +1284,9 @@ struct Solver {
     std::vector<double> dsum;
     filter_rows(st, st.Xb, st.Xh, d_act, ex, &dsum);
     for (int i = 0; i < nb; ++i) {
-      hms[i].tau = hm.ms[i].tau;
-      hms[i].nnz_bar = hm.ms[i].nnz_bar;
-      hms[i].beta = hm.ms[i].beta;  // NMF sets its own budget after the check
+      hms[i].tau = hm.pack.ms[i].tau;
+      hms[i].nnz_bar = hm.pack.ms[i].nnz_bar;
+      hms[i].beta = hm.pack.ms[i].beta;  // NMF sets its own budget after the check
       hms[i].fnorm = std::sqrt(dsum[i]);
     }
     st.ex = ex;
@@ -1282,20 +1301,17 @@ struct Solver {
     launch_row_lengths(N, st.Xb.rs.template as<int64_t>(), st.Xb.re.template as<int64_t>(),
                        w.cnt.as<int64_t>(), s);
     st.Xh.rp.ensure(sizeof(int64_t) * size_t(N + 1), s);
-    launch_scan(N, w.cnt.as<int64_t>(), st.Xh.d_rp(), w.scan_tmp.as<int64_t>(), s);
     int nbm = int(st.mats.size());
-    w.eoff.ensure(sizeof(int64_t) * size_t(nbm + 1), s);
-    launch_gather_offsets(nbm, st.d_moff.template as<int64_t>(), st.Xh.d_rp(), w.eoff.as<int64_t>(), s);
-    d2h(hm.ex, w.eoff.p, size_t(nbm + 1), s);
-    d2h(hm.tot, st.Xh.d_rp() + N, 1, s);
-    d2h(hm.ms, w.ms.p, size_t(nbm), s);
+    launch_scan(N, w.cnt.as<int64_t>(), st.Xh.d_rp(), w.scan_tmp.as<int64_t>(), s,
+                st.d_seg.template as<int32_t>(), pack_dev(nbm).ex);
+    read_pack(nbm);
     wait();
     for (int i = 0; i < nbm; ++i) {
-      hms[i].nnz_bar = hm.ms[i].nnz_bar;
-      hms[i].beta = hm.ms[i].beta;  // NMF sets its own budget after the check
+      hms[i].nnz_bar = hm.pack.ms[i].nnz_bar;
+      hms[i].beta = hm.pack.ms[i].beta;  // NMF sets its own budget after the check
     }
-    st.ex.assign(hm.ex, hm.ex + nbm + 1);
-    int64_t nnz = hm.tot[0];
+    st.ex.assign(hm.pack.ex, hm.pack.ex + nbm + 1);
+    int64_t nnz = hm.pack.ex[nbm];
     st.Xh.n = N;
     st.Xh.nnz = nnz;
     st.Xh.col.ensure(sizeof(int32_t) * size_t(nnz > 0 ? nnz : 1), s);
