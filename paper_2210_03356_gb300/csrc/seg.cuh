@@ -10,7 +10,7 @@ namespace sgn {
 constexpr int RED_T = 256;  // partial sums per component; their order is fixed
 constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
 constexpr int RED_LANES = RED_T / RED_C;
-constexpr int RED_U = 16;   // rows loaded at once, the next ones while these are added
+constexpr int RED_U = 32;   // rows loaded at once, the next ones while these are added
 static_assert(RED_LANES == 32, "one warp of each CTA per component");
 
 // acc + v as a fused multiply-add (v * 1 is exact): in a chain of dependent FP64
@@ -36,7 +36,7 @@ __device__ __forceinline__ double seg_partial(const double *part, int ncomp, int
 #pragma unroll
     for (int u = 0; u < RED_U; ++u) acc = chain_add(acc, d[u]);
   };
-  if (e - b <= RED_U / 2 * RED_T) {  // short matrices: no rows to load ahead
+  if (e - b <= 8 * RED_T) {  // short matrices: no rows to load ahead
     for (; r < e; r += RED_T) acc = chain_add(acc, part[r * ncomp + c]);
     return acc;
   }
@@ -73,7 +73,7 @@ __device__ __forceinline__ unsigned long long seg_entries(const int64_t *rs, con
                                                           int64_t b, int64_t e, int first,
                                                           int step) {
   long long acc = 0;
-#pragma unroll 8
+#pragma unroll 16
   for (int64_t r = b + first; r < e; r += step) acc += re[r] - rs[r];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
