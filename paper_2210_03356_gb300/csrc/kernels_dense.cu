@@ -66,9 +66,14 @@ __device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
   lo = __fsub_rn(x, hi);
 }
 
-// Tile t of the launch -> job and tile origin (m0, n0); M blocks run fastest.
-__device__ __forceinline__ void tile_of(int t, const DenseJob *jobs, const int *tile_start,
-                                        int njobs, int &j, int &m0, int &n0) {
+// Work units of a launch: the first nfull tiles are whole (128 x 256); the
+// tiles after them, the last wave's, are cut into two halves of 128 columns
+// (tile_halves). Unit u -> job, origin (m0, n0) and width nw; M blocks run
+// fastest.
+__device__ __forceinline__ void unit_of(int u, int nfull, const DenseJob *jobs,
+                                        const int *tile_start, int njobs, int &j, int &m0,
+                                        int &n0, int &nw) {
+  const int t = u < nfull ? u : nfull + (u - nfull) / 2;
   int lo = 0, hi = njobs - 1;
   while (lo < hi) {  // last job with tile_start[j] <= t
     int mid = (lo + hi + 1) >> 1;
@@ -79,12 +84,18 @@ __device__ __forceinline__ void tile_of(int t, const DenseJob *jobs, const int *
   const int tm = (jobs[j].M + DM - 1) / DM;
   m0 = (local % tm) * DM;
   n0 = (local / tm) * DN;
+  nw = DN;
+  if (u >= nfull) {
+    nw = DN / 2;
+    n0 += ((u - nfull) & 1) * nw;
+  }
 }
 
-// maps[4 j + 0..3]: A_hi, A_lo, Bt_hi, Bt_lo of job j (boxes DK x DM and DK x DN).
+// maps[4 j + 0..3]: A_hi, A_lo, Bt_hi, Bt_lo of job j (boxes DK x DM; Bt's 256
+// rows take two).
 __global__ void __launch_bounds__(DTHREADS, 1)
     k_gemm_nt(const DenseJob *jobs, const CUtensorMap *maps, const int *tile_start, int njobs,
-              int ntiles, int *err) {
+              int nfull, int nunits, int *err) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[NSTAGE], empty[NSTAGE], tfull[2], tempty[2], done;
   __shared__ uint32_t tmem_slot;
@@ -120,31 +131,34 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x) {
-        int j, m0, n0;
-        tile_of(t, jobs, tile_start, njobs, j, m0, n0);
+      for (int t = blockIdx.x; t < nunits && !*abort; t += gridDim.x) {
+        int j, m0, n0, nw;
+        unit_of(t, nfull, jobs, tile_start, njobs, j, m0, n0, nw);
         const CUtensorMap *mp = maps + 4 * j;
         const int nk = (jobs[j].K + DK - 1) / DK;
         for (int kb = 0; kb < nk; ++kb, ++issued) {
           const int st = issued % NSTAGE;
           if (!bounded_wait(&empty[st], ((issued / NSTAGE) & 1) ^ 1, abort)) break;
           const uint32_t d = sbase + uint32_t(st * STAGE_BYTES);
-          mbar_expect_tx(&full[st], STAGE_BYTES);
+          mbar_expect_tx(&full[st], nw == DN ? STAGE_BYTES : STAGE_BYTES - B_BYTES);
           tma_load_2d(d, mp + 0, kb * DK, m0, &full[st]);
           tma_load_2d(d + A_BYTES, mp + 1, kb * DK, m0, &full[st]);
-          tma_load_2d(d + 2 * A_BYTES, mp + 2, kb * DK, n0, &full[st]);
-          tma_load_2d(d + 2 * A_BYTES + B_BYTES, mp + 3, kb * DK, n0, &full[st]);
+          for (int h = 0; h < nw; h += DM) {
+            const uint32_t db = d + 2 * A_BYTES + uint32_t(h * DK * 4);
+            tma_load_2d(db, mp + 2, kb * DK, n0 + h, &full[st]);
+            tma_load_2d(db + B_BYTES, mp + 3, kb * DK, n0 + h, &full[st]);
+          }
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = idesc_tf32(DM, DN);
       int it = 0, tc = 0;
       bool any = false;
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x, ++tc) {
-        int j, m0, n0;
-        tile_of(t, jobs, tile_start, njobs, j, m0, n0);
+      for (int t = blockIdx.x; t < nunits && !*abort; t += gridDim.x, ++tc) {
+        int j, m0, n0, nw;
+        unit_of(t, nfull, jobs, tile_start, njobs, j, m0, n0, nw);
+        const uint32_t idesc = idesc_tf32(DM, nw);
         const int nkj = (jobs[j].K + DK - 1) / DK;
         const int a = tc & 1;
         if (!bounded_wait(&tempty[a], ((tc >> 1) & 1) ^ 1, abort)) break;
@@ -184,9 +198,9 @@ __global__ void __launch_bounds__(DTHREADS, 1)
   } else {
     const int q = warp & 3;  // this warp's 32 TMEM lanes
     int tc = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tc) {
-      int j, m0, n0;
-      tile_of(t, jobs, tile_start, njobs, j, m0, n0);
+    for (int t = blockIdx.x; t < nunits; t += gridDim.x, ++tc) {
+      int j, m0, n0, nw;
+      unit_of(t, nfull, jobs, tile_start, njobs, j, m0, n0, nw);
       const DenseJob J = jobs[j];
       const int a = tc & 1;
       if (!bounded_wait(&tfull[a], (tc >> 1) & 1, abort)) break;
@@ -195,7 +209,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
       float *dh = J.C + int64_t(gr) * J.ldc;
       float *dl = J.C_lo ? J.C_lo + int64_t(gr) * J.ldc : nullptr;
 #pragma unroll 1
-      for (int c = 0; c < DN / 32; ++c) {
+      for (int c = 0; c < nw / 32; ++c) {
         uint32_t v[32];
         __syncwarp();
         tmem_ld_32x32(tmem + (uint32_t(q * 32) << 16) + uint32_t(a * DN + c * 32), v);
@@ -240,20 +254,55 @@ __global__ void __launch_bounds__(DTHREADS, 1)
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// Split into hi/lo, optionally transposing: out[i][j] = in[i][j] (or in[j][i]),
-// rows x cols of out, padded columns up to ldo zeroed.
-__global__ void k_split(int rows, int cols, const float *in, int ldi, int transpose, float *hi,
-                        float *lo, int ldo) {
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < int64_t(rows) * ldo;
+// Split into hi/lo: out[i][j] = in[i][j], padded columns up to ldo zeroed.
+// HBM-bound (4 B read, 8 B written per element), four columns per thread; ldi
+// and ldo are multiples of 4 and the rows 16-byte aligned.
+__global__ void __launch_bounds__(256)
+    k_split_rows(int rows, int cols, const float *in, int ldi, float *hi, float *lo, int ldo) {
+  const int q = ldo / 4;
+  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < int64_t(rows) * q;
        t += int64_t(gridDim.x) * blockDim.x) {
-    int i = int(t / ldo), j = int(t % ldo);
-    float x = 0.0f;
-    if (j < cols) x = transpose ? in[int64_t(j) * ldi + i] : in[int64_t(i) * ldi + j];
-    float h, l;
-    split_tf32(x, h, l);
-    hi[t] = h;
-    lo[t] = l;
+    const int64_t i = t / q;
+    const int j = int(t - i * q) * 4;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f), h, l;
+    if (j < cols) x = *reinterpret_cast<const float4 *>(in + i * ldi + j);  // cols: a multiple of 4
+    split_tf32(x.x, h.x, l.x);
+    split_tf32(x.y, h.y, l.y);
+    split_tf32(x.z, h.z, l.z);
+    split_tf32(x.w, h.w, l.w);
+    reinterpret_cast<float4 *>(hi)[t] = h;
+    reinterpret_cast<float4 *>(lo)[t] = l;
   }
+}
+
+// The same of the transpose: out[i][j] = in[j][i], through a 64 x 64 tile, so that
+// both sides move whole 128-byte lines.
+constexpr int ST = 64;
+__global__ void __launch_bounds__(256)
+    k_split_cols(int rows, int cols, const float *in, int ldi, float *hi, float *lo, int ldo) {
+  __shared__ float tile[ST][ST + 1];
+  const int i0 = blockIdx.x * ST, j0 = blockIdx.y * ST;  // of out
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+#pragma unroll
+  for (int a = 0; a < ST; a += 8)
+#pragma unroll
+    for (int b = 0; b < ST; b += 32) {
+      const int j = j0 + a + ty, i = i0 + b + tx;
+      tile[a + ty][b + tx] = j < cols && i < rows ? in[int64_t(j) * ldi + i] : 0.0f;
+    }
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < ST; a += 8)
+#pragma unroll
+    for (int b = 0; b < ST; b += 32) {
+      const int i = i0 + a + ty, j = j0 + b + tx;
+      if (i < rows && j < ldo) {
+        float h, l;
+        split_tf32(tile[b + tx][a + ty], h, l);
+        hi[int64_t(i) * ldo + j] = h;
+        lo[int64_t(i) * ldo + j] = l;
+      }
+    }
 }
 
 // Densify: the rows of the dense-path matrices of a stage CSR into their
@@ -349,23 +398,37 @@ __global__ void k_dense_resid(int64_t n, const int32_t *seg, const int *dslot, c
     float rh = 0.f, rl = 0.f, xh = 0.f, xl = 0.f;
     double rdiag = 0.0;
     unsigned cnt = 0;
-    for (int j = lane; j < Bf.n; j += 32) {
-      float t = __fadd_rn(Bf.TT_hi[i * Bf.ld + j], Bf.TT_lo[i * Bf.ld + j]);
-      float x = __fadd_rn(Bf.X_hi[i * Bf.ld + j], Bf.X_lo[i * Bf.ld + j]);
-      cnt += t != 0.0f;
-      if (j == i) {
-        double dd = double(t) - 1.0;
-        rdiag = dd * dd;
-      } else {
-        float pp = __fmul_rn(t, t), ee = __fmaf_rn(t, t, -pp);
-        float s = __fadd_rn(rh, pp), bb = __fsub_rn(s, rh);
-        rl = __fadd_rn(rl, __fadd_rn(__fadd_rn(__fsub_rn(rh, __fsub_rn(s, bb)), __fsub_rn(pp, bb)), ee));
-        rh = s;
+    const float *th = Bf.TT_hi + i * Bf.ld, *tl = Bf.TT_lo + i * Bf.ld;
+    const float *xhp = Bf.X_hi + i * Bf.ld, *xlp = Bf.X_lo + i * Bf.ld;
+    constexpr int U = 8;  // columns per lane in flight (the sums keep their order)
+    for (int j0 = lane; j0 < Bf.n; j0 += 32 * U) {
+      float tv[U], xv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 32 * u;
+        tv[u] = j < Bf.n ? __fadd_rn(th[j], tl[j]) : 0.0f;
+        xv[u] = j < Bf.n ? __fadd_rn(xhp[j], xlp[j]) : 0.0f;
       }
-      float px = __fmul_rn(x, x), ex = __fmaf_rn(x, x, -px);
-      float sx = __fadd_rn(xh, px), bx = __fsub_rn(sx, xh);
-      xl = __fadd_rn(xl, __fadd_rn(__fadd_rn(__fsub_rn(xh, __fsub_rn(sx, bx)), __fsub_rn(px, bx)), ex));
-      xh = sx;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 32 * u;
+        if (j >= Bf.n) break;
+        const float t = tv[u], x = xv[u];
+        cnt += t != 0.0f;
+        if (j == i) {
+          double dd = double(t) - 1.0;
+          rdiag = dd * dd;
+        } else {
+          float pp = __fmul_rn(t, t), ee = __fmaf_rn(t, t, -pp);
+          float s = __fadd_rn(rh, pp), bb = __fsub_rn(s, rh);
+          rl = __fadd_rn(rl, __fadd_rn(__fadd_rn(__fsub_rn(rh, __fsub_rn(s, bb)), __fsub_rn(pp, bb)), ee));
+          rh = s;
+        }
+        float px = __fmul_rn(x, x), ex = __fmaf_rn(x, x, -px);
+        float sx = __fadd_rn(xh, px), bx = __fsub_rn(sx, xh);
+        xl = __fadd_rn(xl, __fadd_rn(__fadd_rn(__fsub_rn(xh, __fsub_rn(sx, bx)), __fsub_rn(px, bx)), ex));
+        xh = sx;
+      }
     }
     double rs = double(rh) + double(rl) + rdiag, xs = double(xh) + double(xl);
 #pragma unroll
@@ -398,21 +461,28 @@ __global__ void k_dense_emit(int64_t n, const int32_t *seg, const int *dslot, co
     const DenseBuf Bf = bufs[d];
     int64_t r0 = moff[m], i = r - r0;
     int64_t out = cs[r];
-    for (int j0 = 0; j0 < Bf.n; j0 += 32) {
-      int j = j0 + lane;
-      float v = 0.0f;
-      if (j < Bf.n) {
-        float x = __fadd_rn(Bf.X_hi[i * Bf.ld + j], Bf.X_lo[i * Bf.ld + j]);
-        v = __fsub_rn(__fmul_rn(1.5f, x), __fmul_rn(0.5f, Bf.P[i * Bf.ld + j]));
+    const float *xhp = Bf.X_hi + i * Bf.ld, *xlp = Bf.X_lo + i * Bf.ld, *pp = Bf.P + i * Bf.ld;
+    constexpr int U = 4;  // columns per lane in flight
+    for (int j0 = 0; j0 < Bf.n; j0 += 32 * U) {
+      float v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 32 * u + lane;
+        v[u] = 0.0f;
+        if (j < Bf.n)
+          v[u] = __fsub_rn(__fmul_rn(1.5f, __fadd_rn(xhp[j], xlp[j])), __fmul_rn(0.5f, pp[j]));
       }
-      bool keep = v != 0.0f;
-      unsigned mk = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        int64_t pos = out + __popc(mk & lt);
-        ccol[pos] = int32_t(r0 + j);
-        cval[pos] = v;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool keep = v[u] != 0.0f;
+        const unsigned mk = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+          const int64_t pos = out + __popc(mk & lt);
+          ccol[pos] = int32_t(r0 + j0 + 32 * u + lane);
+          cval[pos] = v[u];
+        }
+        out += __popc(mk);
       }
-      out += __popc(mk);
     }
     if (lane == 0) ce[r] = out;
   }
@@ -458,8 +528,8 @@ void launch_dense_jobs(int njobs, const DenseJob *jobs_host, DenseJob *jobs_dev,
     const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     maps[4 * j + 0] = tc::operand_map(J.A_hi, f32, 4, J.M, J.K, J.lda, DK, DM);
     maps[4 * j + 1] = tc::operand_map(J.A_lo, f32, 4, J.M, J.K, J.lda, DK, DM);
-    maps[4 * j + 2] = tc::operand_map(J.B_hi, f32, 4, J.N, J.K, J.ldb, DK, DN);
-    maps[4 * j + 3] = tc::operand_map(J.B_lo, f32, 4, J.N, J.K, J.ldb, DK, DN);
+    maps[4 * j + 2] = tc::operand_map(J.B_hi, f32, 4, J.N, J.K, J.ldb, DK, DM);
+    maps[4 * j + 3] = tc::operand_map(J.B_lo, f32, 4, J.N, J.K, J.ldb, DK, DM);
     tile_start[j] = ntiles;
     ntiles += ((J.M + DM - 1) / DM) * ((J.N + DN - 1) / DN);
   }
@@ -470,19 +540,30 @@ void launch_dense_jobs(int njobs, const DenseJob *jobs_host, DenseJob *jobs_dev,
   SGN_CUDA(cudaMemcpyAsync(jobs_dev, jobs_host, sizeof(DenseJob) * size_t(njobs),
                            cudaMemcpyHostToDevice, s));
   const unsigned char *sc = static_cast<const unsigned char *>(scratch);
-  k_gemm_nt<<<std::min(ntiles, nsm), DTHREADS, dense_gemm_smem(), s>>>(
+  // a last wave of at most nsm / 2 tiles runs as halves: 4096^3 has 512 tiles, 3
+  // waves of 152 and 56 more (0.497 ms with whole tiles, 0.468 with halves);
+  // every entry is still summed by one accumulator in the same order
+  const int tail = ntiles % nsm;
+  const int nfull = tail > 0 && 2 * tail <= nsm ? ntiles - tail : ntiles;
+  const int nunits = nfull + 2 * (ntiles - nfull);
+  k_gemm_nt<<<std::min(nunits, nsm), DTHREADS, dense_gemm_smem(), s>>>(
       jobs_dev, reinterpret_cast<const CUtensorMap *>(sc),
-      reinterpret_cast<const int *>(sc + size_t(njobs) * 4 * sizeof(CUtensorMap)), njobs, ntiles,
-      err);
+      reinterpret_cast<const int *>(sc + size_t(njobs) * 4 * sizeof(CUtensorMap)), njobs, nfull,
+      nunits, err);
   SGN_LAUNCH_CHECK();
 }
 
 void launch_split(int rows, int cols, const float *in, int ldi, int transpose, float *hi,
                   float *lo, int ldo, cudaStream_t s) {
-  int64_t total = int64_t(rows) * ldo;
-  if (total == 0) return;
-  int g = int(std::min<int64_t>((total + 255) / 256, 152 * 32));
-  k_split<<<g, 256, 0, s>>>(rows, cols, in, ldi, transpose, hi, lo, ldo);
+  if (rows <= 0 || ldo <= 0) return;
+  if (transpose) {
+    const dim3 grid(unsigned((rows + ST - 1) / ST), unsigned((ldo + ST - 1) / ST));
+    k_split_cols<<<grid, 256, 0, s>>>(rows, cols, in, ldi, hi, lo, ldo);
+  } else {
+    const int64_t total = int64_t(rows) * (ldo / 4);
+    k_split_rows<<<int(std::min<int64_t>((total + 255) / 256, 152 * 32)), 256, 0, s>>>(
+        rows, cols, in, ldi, hi, lo, ldo);
+  }
   SGN_LAUNCH_CHECK();
 }
 
