@@ -438,7 +438,9 @@ struct SliceJob {
   int accum;  // 1: C += A Bt^T (a later K block); 0: C = A Bt^T
 };
 size_t f64x_digits_bytes(int rows, int ld);
-size_t slice_jobs_scratch_bytes(int njobs);
+// Device scratch of launch_slice_jobs for njobs jobs of ntiles tiles in all.
+int slice_tiles(int M, int N);
+size_t slice_jobs_scratch_bytes(int njobs, int ntiles);
 // Digit planes and scales of the rows of x (rows x K, leading dimension ldx),
 // or of its columns when transpose; digits zero for K <= k < ld.
 void launch_slices(int rows, int K, const double *x, int ldx, int transpose, uint16_t *digits,

@@ -42,8 +42,12 @@
 // planes, 16 KB per pair and slice here against 24 KB when every pair loads
 // its own two planes, and the FP64 pipe (16 cycles per warp instruction) when
 // every pair is added into C in FP64, as an earlier form did: 6.07 ms at
-// 4096^3 and 3.69 ms at 2744^3 (GB300), now 4.16 and 2.31 ms (1.19 PFLOP/s on
-// the tensor pipe at 4096^3; 512 tiles are 3.4 waves of 152 CTAs).
+// 4096^3 and 3.69 ms at 2744^3 (GB300), now 3.70 and 1.98 ms (1.34 PFLOP/s on
+// the tensor pipe at 4096^3).
+// Tiles of a last, partial wave are cut into S parts of about equal pairs, each
+// a work unit of its own that leaves its integers in scratch; k_slices_finish
+// adds them up (exactly, in any order) and writes C. 2744^3 has 242 tiles: two
+// waves of 152 become 1 2/3 (2.31 -> 1.98 ms), 1024^3 has 32: 0.29 -> 0.088 ms.
 // Every wait has a clock budget, as in the split-TF32 kernel.
 #include <stdint.h>
 
@@ -78,9 +82,59 @@ constexpr int KBLK = F64X_MAX_K / XK;       // K stages per exact block (integer
 constexpr int XLP = 4;
 static_assert(F64X_DIGITS == 8 && DIGIT_BITS == 7, "level pairs (8, 9) .. (2, 3) of 8 digits");
 __host__ __device__ constexpr int lower_level(int lp) { return 8 - 2 * lp; }
+// The steps (level pair, t) of a tile in the order in which a unit takes them: a
+// whole tile from the smallest weight up, the levels 3 and 2 last; for parts
+// the level pairs ordered so that halves, thirds and sixths of the pairs end
+// between steps.
+constexpr int XSTEPS = 20, XMAX_PARTS = 6;
+struct StepList {
+  unsigned char lp[2][XSTEPS], t[2][XSTEPS];  // [0] whole tiles, [1] parts
+};
+constexpr StepList make_steps() {
+  StepList s{};
+  const int order[2][XLP] = {{0, 1, 2, 3}, {0, 3, 1, 2}};
+  for (int k = 0; k < 2; ++k) {
+    int n = 0;
+    for (int i = 0; i < XLP; ++i)
+      for (int t = 1; t <= lower_level(order[k][i]); ++t, ++n) {
+        s.lp[k][n] = (unsigned char)order[k][i];
+        s.t[k][n] = (unsigned char)t;
+      }
+  }
+  return s;
+}
+constexpr StepList kSteps = make_steps();
+__constant__ StepList c_steps = kSteps;
+constexpr int step_pairs(int i) {  // of the parts' order
+  return kSteps.t[1][i] < lower_level(kSteps.lp[1][i]) ? 2 : 1;
+}
+// The units of a launch: nfull whole tiles, then S parts of each tile after them;
+// part p takes the steps bound[p] .. bound[p + 1] - 1.
+struct XPlan {
+  int nfull, ntail, parts;
+  int bound[XMAX_PARTS + 1];
+  __host__ __device__ int units() const { return nfull + ntail * parts; }
+};
 constexpr int XPAIRS = 36;  // sum over the level pairs of (l - 1) + l
-// the CTA's integer tile: 32-column chunks of a warp, column by column
+// an integer tile: 32-column chunks of a warp, column by column
 constexpr size_t XTILE_BYTES = size_t(XM) * XN * sizeof(long long);
+
+// Unit u -> its tile and steps [s0, s1) of the list k.
+struct XUnit {
+  int tile, k, s0, s1;
+};
+__device__ __forceinline__ XUnit unit_at(int u, const XPlan &pl) {
+  if (u < pl.nfull) return XUnit{u, 0, 0, XSTEPS};
+  const int v = u - pl.nfull, p = v % pl.parts;
+  return XUnit{pl.nfull + v / pl.parts, 1, pl.bound[p], pl.bound[p + 1]};
+}
+// The end of the run of steps from i that share an accumulator: one level pair,
+// at most `group` of them.
+__device__ __forceinline__ int run_end(const XUnit &un, int i, int group) {
+  int e = i + 1;
+  while (e < un.s1 && e - i < group && c_steps.lp[un.k][e] == c_steps.lp[un.k][i]) ++e;
+  return e;
+}
 
 // v 2^sc as an FP64 value, rounded to nearest: built with integer operations,
 // the FP64 pipe being the scarce unit. Falls back to ldexp outside the
@@ -119,10 +173,10 @@ __device__ __forceinline__ void xtile_of(int t, const SliceJob *jobs, const int 
 
 // maps[2 j]: the digits of A of job j as one (8 M) x K array, maps[2 j + 1]
 // those of Bt as (8 N) x K; digit s of row r is row (s - 1) rows + r. tiles: one
-// integer tile per CTA.
+// integer tile per CTA; parts: two per part (levels 9 .. 4, levels 3 and 2).
 __global__ void __launch_bounds__(XTHREADS, 1)
     k_gemm_slices(const SliceJob *jobs, const CUtensorMap *maps, const int *tile_start,
-                  int njobs, int ntiles, long long *tiles, int *err) {
+                  int njobs, XPlan pl, long long *tiles, long long *parts, int *err) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[XSTAGE], empty[XSTAGE], tfull, tempty, done;
   __shared__ uint32_t tmem_slot;
@@ -130,6 +184,7 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   volatile int *abort = &s_abort;
+  const int nunits = pl.units();
   if (tid == 0) {
     for (int i = 0; i < XSTAGE; ++i) {
       mbar_init(&full[i], 1);
@@ -154,29 +209,28 @@ __global__ void __launch_bounds__(XTHREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x) {
+      for (int u = blockIdx.x; u < nunits && !*abort; u += gridDim.x) {
+        const XUnit un = unit_at(u, pl);
         int j, m0, n0;
-        xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
+        xtile_of(un.tile, jobs, tile_start, njobs, j, m0, n0);
         const SliceJob &J = jobs[j];
         const CUtensorMap *mp = maps + 2 * j;
         const int nk = (J.K + XK - 1) / XK;
         for (int k0 = 0; k0 < nk && !*abort; k0 += KBLK) {
           const int k1 = min(nk, k0 + KBLK);
-          for (int lp = 0; lp < XLP && !*abort; ++lp) {
-            const int l = lower_level(lp);
-            for (int t2 = 1; t2 <= l && !*abort; ++t2) {
-              const bool both = t2 < l;  // step l has no pair of level l
-              const int y0 = (l - t2 - 1) * J.M + m0, y1 = (l - t2) * J.M + m0;
-              const int yb = (t2 - 1) * J.N + n0;
-              for (int kb = k0; kb < k1; ++kb, ++issued) {
-                const int st = issued % XSTAGE;
-                if (!bounded_wait(&empty[st], ((issued / XSTAGE) & 1) ^ 1, abort)) break;
-                const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
-                mbar_expect_tx(&full[st], both ? XSTAGE_BYTES : XSTAGE_BYTES - XA_BYTES);
-                if (both) tma_load_2d(d, mp + 0, kb * XK, y0, &full[st]);
-                tma_load_2d(d + XA_BYTES, mp + 0, kb * XK, y1, &full[st]);
-                tma_load_2d(d + 2 * XA_BYTES, mp + 1, kb * XK, yb, &full[st]);
-              }
+          for (int i = un.s0; i < un.s1 && !*abort; ++i) {
+            const int l = lower_level(c_steps.lp[un.k][i]), t = c_steps.t[un.k][i];
+            const bool both = t < l;  // step l has no pair of level l
+            const int y0 = (l - t - 1) * J.M + m0, y1 = (l - t) * J.M + m0;
+            const int yb = (t - 1) * J.N + n0;
+            for (int kb = k0; kb < k1; ++kb, ++issued) {
+              const int st = issued % XSTAGE;
+              if (!bounded_wait(&empty[st], ((issued / XSTAGE) & 1) ^ 1, abort)) break;
+              const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
+              mbar_expect_tx(&full[st], both ? XSTAGE_BYTES : XSTAGE_BYTES - XA_BYTES);
+              if (both) tma_load_2d(d, mp + 0, kb * XK, y0, &full[st]);
+              tma_load_2d(d + XA_BYTES, mp + 0, kb * XK, y1, &full[st]);
+              tma_load_2d(d + 2 * XA_BYTES, mp + 1, kb * XK, yb, &full[st]);
             }
           }
         }
@@ -187,48 +241,48 @@ __global__ void __launch_bounds__(XTHREADS, 1)
       const uint32_t idesc = idesc_bf16(XM, XN);
       int it = 0, uc = 0;  // stages consumed, accumulations (both accumulators) done
       bool any = false, ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok && !*abort; t += gridDim.x) {
+      for (int u = blockIdx.x; u < nunits && ok && !*abort; u += gridDim.x) {
+        const XUnit un = unit_at(u, pl);
         int j, m0, n0;
-        xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
+        xtile_of(un.tile, jobs, tile_start, njobs, j, m0, n0);
         const int nk = (jobs[j].K + XK - 1) / XK;
         for (int k0 = 0; k0 < nk && ok; k0 += KBLK) {
           const int k1 = min(nk, k0 + KBLK), group = KBLK / (k1 - k0);
-          for (int lp = 0; lp < XLP && ok; ++lp) {
-            const int l = lower_level(lp);
-            for (int ta = 1; ta <= l && ok; ta += group, ++uc) {
-              const int tb = min(l, ta + group - 1);  // steps ta .. tb accumulate together
-              if (!bounded_wait(&tempty, (uc & 1) ^ 1, abort)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              for (int t2 = ta; t2 <= tb && ok; ++t2) {
-                const bool both = t2 < l;
-                for (int kb = k0; kb < k1; ++kb, ++it) {
-                  const int st = it % XSTAGE;
-                  if (!bounded_wait(&full[st], (it / XSTAGE) & 1, abort)) {
-                    ok = false;
-                    break;
-                  }
-                  tc_fence_after();
-                  const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
-                  const uint32_t more = t2 > ta || kb > k0 ? 1u : 0u;
-#pragma unroll
-                  for (int s = 0; s < XK / 16; ++s) {
-                    const uint32_t ko = uint32_t(s) * 32u;
-                    const uint64_t bd = smem_desc_sw<XSPAN>(d + 2 * XA_BYTES + ko);
-                    if (both)
-                      mma_bf16(tmem, smem_desc_sw<XSPAN>(d + ko), bd, idesc, s ? 1u : more);
-                    mma_bf16(tmem + XN, smem_desc_sw<XSPAN>(d + XA_BYTES + ko), bd, idesc,
-                             s ? 1u : more);
-                  }
-                  any = true;
-                  mma_commit(&empty[st]);
-                }
-              }
-              if (!ok) break;
-              mma_commit(&tfull);
+          for (int i = un.s0; i < un.s1 && ok; ++uc) {
+            const int e = run_end(un, i, group);  // steps i .. e - 1 accumulate together
+            const int l = lower_level(c_steps.lp[un.k][i]);
+            if (!bounded_wait(&tempty, (uc & 1) ^ 1, abort)) {
+              ok = false;
+              break;
             }
+            tc_fence_after();
+            for (int q = i; q < e && ok; ++q) {
+              const bool both = c_steps.t[un.k][q] < l;
+              for (int kb = k0; kb < k1; ++kb, ++it) {
+                const int st = it % XSTAGE;
+                if (!bounded_wait(&full[st], (it / XSTAGE) & 1, abort)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+                const uint32_t d = sbase + uint32_t(st * XSTAGE_BYTES);
+                const uint32_t more = q > i || kb > k0 ? 1u : 0u;
+#pragma unroll
+                for (int s = 0; s < XK / 16; ++s) {
+                  const uint32_t ko = uint32_t(s) * 32u;
+                  const uint64_t bd = smem_desc_sw<XSPAN>(d + 2 * XA_BYTES + ko);
+                  if (both)
+                    mma_bf16(tmem, smem_desc_sw<XSPAN>(d + ko), bd, idesc, s ? 1u : more);
+                  mma_bf16(tmem + XN, smem_desc_sw<XSPAN>(d + XA_BYTES + ko), bd, idesc,
+                           s ? 1u : more);
+                }
+                any = true;
+                mma_commit(&empty[st]);
+              }
+            }
+            if (!ok) break;
+            mma_commit(&tfull);
+            i = e;
           }
         }
       }
@@ -241,30 +295,39 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   } else {
     const int q = warp & 3;           // this warp's 32 TMEM lanes (rows)
     const int half = (warp - 2) >> 2;  // and its half of the tile's columns
-    // this warp's part of the CTA's integer tile: [chunk][column][lane]
-    long long *const low =
-        tiles + size_t(blockIdx.x) * (XM * XN) + size_t(warp - 2) * (XM * XN / 8) + lane;
     const uint32_t trow = tmem + (uint32_t(q * 32) << 16);
     int uc = 0;
     bool stop = false;
-    for (int t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
+    for (int u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+      const XUnit un = unit_at(u, pl);
+      const bool part = un.k != 0;
       int j, m0, n0;
-      xtile_of(t, jobs, tile_start, njobs, j, m0, n0);
+      xtile_of(un.tile, jobs, tile_start, njobs, j, m0, n0);
       const SliceJob J = jobs[j];
+      // this warp's part of the integer tiles: [chunk][column][lane]; a part has a
+      // second one for the levels 3 and 2
+      long long *const low =
+          (part ? parts + size_t(u - pl.nfull) * (2 * XM * XN) : tiles + size_t(blockIdx.x) * (XM * XN)) +
+          size_t(warp - 2) * (XM * XN / 8) + lane;
       const int gr = m0 + q * 32 + lane;
       const int ea = gr < J.M ? J.ea[gr] : 0;
       const int nk = (J.K + XK - 1) / XK;
       for (int k0 = 0; k0 < nk && !stop; k0 += KBLK) {
         const int group = KBLK / (min(nk, k0 + KBLK) - k0);
-        for (int lp = 0; lp < XLP && !stop; ++lp) {
-          const int l = lower_level(lp);
-          for (int ta = 1; ta <= l; ta += group, ++uc) {
+        bool first_low = true, first_high = true;
+        {
+          for (int i = un.s0; i < un.s1; ++uc) {
+            const int e = run_end(un, i, group);
+            const int lp = c_steps.lp[un.k][i], ta = c_steps.t[un.k][i], l = lower_level(lp);
+            i = e;
             if (!bounded_wait(&tfull, uc & 1, abort)) {
               stop = true;
               break;
             }
             tc_fence_after();
             const bool both = ta < l;  // the lower level's accumulator was written
+            const bool high = lp == XLP - 1;
+            const bool first = high ? first_high : first_low;
 #pragma unroll 1
             for (int c = 0; c < XN / 64; ++c) {
               uint32_t v0[32], v1[32];
@@ -277,10 +340,9 @@ __global__ void __launch_bounds__(XTHREADS, 1)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v0[i] = 0u;
               }
-              long long *const lc = low + c * 32 * 32;
-              if (lp < XLP - 1) {  // levels 9 .. 4: into the integer tile
-                const bool first = lp == 0 && ta == 1;
-                const int sh = 2 * DIGIT_BITS * lp;
+              long long *const lc = low + c * 32 * 32 + (high && part ? XM * XN : 0);
+              if (!high || part) {  // into an integer tile
+                const int sh = high ? 0 : 2 * DIGIT_BITS * lp;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                   long long o[16];
@@ -299,8 +361,8 @@ __global__ void __launch_bounds__(XTHREADS, 1)
               const int gc = n0 + col;
               if (gr >= J.M) continue;
               double *const crow = J.C + int64_t(gr) * J.ldc + gc;
-              const bool with_low = ta == 1;
-              const bool add = ta > 1 || k0 > 0 || J.accum;  // C holds earlier terms
+              const bool with_low = first;
+              const bool add = !first || k0 > 0 || J.accum;  // C holds earlier terms
               auto pair_of = [&](int k, const double2 &old) {  // columns gc + k, gc + k + 1
                 const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + k);
                 double r[2];
@@ -338,6 +400,7 @@ __global__ void __launch_bounds__(XTHREADS, 1)
                 }
               }
             }
+            if (high) first_high = false; else first_low = false;
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty);
@@ -360,6 +423,49 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc(tmem, XTMEM_COLS);
+}
+
+// C of the tiles that were cut into parts: the parts' integers added, then as in
+// k_gemm_slices. low, high: bit p set if part p has steps of the levels 9 .. 4,
+// or of 3 and 2. A CTA per 32 x 32 block of a tile; a thread writes 32 B.
+__global__ void __launch_bounds__(256)
+    k_slices_finish(const SliceJob *jobs, const int *tile_start, int njobs, XPlan pl,
+                    const long long *parts, unsigned low, unsigned high) {
+  const int tt = blockIdx.x / 32, blk = blockIdx.x % 32;
+  int j, m0, n0;
+  xtile_of(pl.nfull + tt, jobs, tile_start, njobs, j, m0, n0);
+  const SliceJob J = jobs[j];
+  const int w = blk / 4, c = blk % 4, lane = threadIdx.x & 31, i0 = (threadIdx.x >> 5) * 4;
+  const int gr = m0 + ((w + 2) & 3) * 32 + lane;  // the layout of epilogue warp w + 2
+  const int gc = n0 + (w >> 2) * (XN / 2) + c * 32 + i0;
+  if (gr >= J.M || gc >= J.N) return;
+  const long long *t = parts + size_t(tt) * pl.parts * (2 * XM * XN) + size_t(w) * (XM * XN / 8) +
+                       c * 32 * 32 + lane;
+  long long L[4] = {0, 0, 0, 0}, H[4] = {0, 0, 0, 0};
+  for (int p = 0; p < pl.parts; ++p, t += 2 * XM * XN)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if ((low >> p) & 1u) L[i] += t[(i0 + i) * 32];
+      if ((high >> p) & 1u) H[i] += t[XM * XN + (i0 + i) * 32];
+    }
+  const int ea = J.ea[gr];
+  double *const crow = J.C + int64_t(gr) * J.ldc + gc;
+#pragma unroll
+  for (int i = 0; i < 4; i += 2) {
+    if (gc + i >= J.N) break;  // N is even
+    const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + i);
+    double2 v;
+    v.x = scaled_int(H[i], ea + eb.x - 3 * DIGIT_BITS) + scaled_int(L[i], ea + eb.x - 9 * DIGIT_BITS);
+    v.y = scaled_int(H[i + 1], ea + eb.y - 3 * DIGIT_BITS) +
+          scaled_int(L[i + 1], ea + eb.y - 9 * DIGIT_BITS);
+    double2 *const cp = reinterpret_cast<double2 *>(crow + i);
+    if (J.accum) {
+      const double2 o = *cp;
+      v.x += o.x;
+      v.y += o.y;
+    }
+    *cp = v;
+  }
 }
 
 // Digit planes. HBM-bound: an entry is read as 8 B (twice: row maximum, then
@@ -663,8 +769,50 @@ size_t f64x_digits_bytes(int rows, int ld) {
   return size_t(F64X_DIGITS) * size_t(rows) * size_t(ld) * sizeof(uint16_t);
 }
 
-size_t slice_jobs_scratch_bytes(int njobs) {
-  return scratch_maps_bytes_x(njobs) + size_t(slice_ctas()) * XTILE_BYTES;
+int slice_tiles(int M, int N) { return ((M + XM - 1) / XM) * ((N + XN - 1) / XN); }
+
+// Parts for the tiles of a partial last wave: the number that ends soonest, by
+// the most pairs of a part, each part's drain costing about a hundredth of a
+// tile; at most two units per CTA. Tiles of several K blocks stay whole.
+static XPlan slice_plan(int ntiles, bool one_block) {
+  const int nsm = slice_ctas();
+  XPlan best{};
+  best.nfull = ntiles;
+  best.parts = 1;
+  const int tail = ntiles % nsm;
+  if (!one_block || tail == 0) return best;
+  double cost = 1.0;
+  for (int S = 2; S <= XMAX_PARTS; ++S) {
+    if (tail * S > 2 * nsm) break;
+    XPlan pl{};
+    pl.nfull = ntiles - tail;
+    pl.ntail = tail;
+    pl.parts = S;
+    int most = 0, sum = 0, at = 0, prev = 0;
+    for (int i = 0; i < XSTEPS; ++i) {
+      sum += step_pairs(i);
+      if (at + 1 < S && sum * S >= XPAIRS * (at + 1)) {
+        pl.bound[++at] = i + 1;
+        most = std::max(most, sum - prev);
+        prev = sum;
+      }
+    }
+    most = std::max(most, XPAIRS - prev);
+    pl.bound[S] = XSTEPS;
+    const int waves = (tail * S + nsm - 1) / nsm;
+    const double c = waves * (double(most) / XPAIRS + 0.01) + 0.04;
+    if (at == S - 1 && c < cost) {
+      cost = c;
+      best = pl;
+    }
+  }
+  return best;
+}
+
+size_t slice_jobs_scratch_bytes(int njobs, int ntiles) {
+  const XPlan pl = slice_plan(ntiles, true);
+  return scratch_maps_bytes_x(njobs) +
+         XTILE_BYTES * (size_t(std::min(ntiles, slice_ctas())) + 2 * size_t(pl.ntail) * pl.parts);
 }
 
 void launch_slices(int rows, int K, const double *x, int ldx, int transpose, uint16_t *digits,
@@ -701,16 +849,29 @@ void launch_slice_jobs(int njobs, const SliceJob *jobs_host, SliceJob *jobs_dev,
     ntiles += ((J.M + XM - 1) / XM) * ((J.N + XN - 1) / XN);
   }
   tile_start[njobs] = ntiles;
+  bool one_block = true;
+  for (int j = 0; j < njobs; ++j) one_block = one_block && jobs_host[j].K <= F64X_MAX_K;
+  const XPlan pl = slice_plan(ntiles, one_block);
   SGN_CUDA(cudaMemcpyAsync(scratch, host.data(), host.size() * sizeof(CUtensorMap),
                            cudaMemcpyHostToDevice, s));
   SGN_CUDA(cudaMemcpyAsync(jobs_dev, jobs_host, sizeof(SliceJob) * size_t(njobs),
                            cudaMemcpyHostToDevice, s));
   unsigned char *sc = static_cast<unsigned char *>(scratch);
-  k_gemm_slices<<<std::min(ntiles, slice_ctas()), XTHREADS, XSMEM, s>>>(
-      jobs_dev, reinterpret_cast<const CUtensorMap *>(sc),
-      reinterpret_cast<const int *>(sc + size_t(njobs) * 2 * sizeof(CUtensorMap)), njobs, ntiles,
-      reinterpret_cast<long long *>(sc + scratch_maps_bytes_x(njobs)), err);
+  const int *starts = reinterpret_cast<const int *>(sc + size_t(njobs) * 2 * sizeof(CUtensorMap));
+  long long *tiles = reinterpret_cast<long long *>(sc + scratch_maps_bytes_x(njobs));
+  long long *parts = tiles + size_t(std::min(ntiles, slice_ctas())) * (XM * XN);
+  k_gemm_slices<<<std::min(pl.units(), slice_ctas()), XTHREADS, XSMEM, s>>>(
+      jobs_dev, reinterpret_cast<const CUtensorMap *>(sc), starts, njobs, pl, tiles, parts, err);
   SGN_LAUNCH_CHECK();
+  if (pl.ntail > 0) {
+    unsigned low = 0, high = 0;
+    for (int p = 0; p < pl.parts; ++p)
+      for (int i = pl.bound[p]; i < pl.bound[p + 1]; ++i)
+        (kSteps.lp[1][i] == XLP - 1 ? high : low) |= 1u << p;
+    k_slices_finish<<<unsigned(pl.ntail) * 32, 256, 0, s>>>(jobs_dev, starts, njobs, pl, parts, low,
+                                                          high);
+    SGN_LAUNCH_CHECK();
+  }
 }
 
 }  // namespace sgn
@@ -749,7 +910,7 @@ extern "C" sign_status sign_dense_product_f64(int M, int N, int K, const double 
     launch_slices(N, K, B, ldb, 1, db, kp, wb, s);  // Bt = B^T: the columns of B
     SliceJob J{M, N, kp, da, kp, db, kp, wa, wb, C, ldc};  // digits are zero for K <= k < kp
     job.ensure(sizeof(SliceJob), s);
-    scratch.ensure(slice_jobs_scratch_bytes(1), s);
+    scratch.ensure(slice_jobs_scratch_bytes(1, slice_tiles(M, N)), s);
     err.ensure(sizeof(int), s);
     SGN_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
     {

@@ -797,7 +797,6 @@ struct Solver {
       // A = X^T, read transposed from X, and Bt = X; UPDATE: C = P = X T with
       // A = X and Bt = T^T)
       w.djobs.ensure(sizeof(SliceJob) * size_t(dp.nd), s);
-      w.dscratch.ensure(slice_jobs_scratch_bytes(dp.nd), s);
       std::vector<SliceJob> jobs;
       for (int64_t k0 = 0; k0 < dp.max_ld; k0 += F64X_MAX_K) {
         jobs.clear();
@@ -819,6 +818,9 @@ struct Solver {
           }
           fl += 2.0 * f64x_pairs() * double(b.ld) * double(b.ld) * double(K);
         }
+        int ntiles = 0;
+        for (const SliceJob &jb : jobs) ntiles += slice_tiles(jb.M, jb.N);
+        w.dscratch.ensure(slice_jobs_scratch_bytes(int(jobs.size()), ntiles), s);
         ProfScope ps(KC_DENSE64, s, fl, 0.0);
         launch_slice_jobs(int(jobs.size()), jobs.data(), w.djobs.as<SliceJob>(), w.dscratch.p,
                           w.derr.as<int>(), s);
