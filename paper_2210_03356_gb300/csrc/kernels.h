@@ -369,9 +369,9 @@ void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int
 // The inverse of the n x n FP64 matrix in lu (leading dimension ld; its upper
 // triangle becomes U) by LU with partial pivoting and one forward and back
 // substitution per column of the identity, into inv (same ld). swaps: n ints;
-// *singular = 1 (and inv undefined) if a pivot column is zero.
-void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, double *inv,
-                          cudaStream_t s);
+// *singular = 1 (and inv undefined) if a pivot column is zero; wild: one int.
+void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, int *wild,
+                          double *inv, cudaStream_t s);
 // *out = ||inv||_F / sqrt(n) (part: n doubles of scratch).
 void launch_inv_norm(int n, int ld, const double *inv, double *part, double *out,
                      cudaStream_t s);

@@ -14,10 +14,10 @@
 // rows are swapped and reduced like those of the matrix, [A | I] -> [U | y].
 // Columns are taken in panels: k_lu_panel factors a panel in one CTA, and
 // k_lu_trail applies its swaps and its reductions, in ascending column order,
-// to every column right of it and to the identity, a strip of 8 columns per
+// to every column right of it and to the identity, a strip of 4 columns per
 // CTA. Four launches per column and one thread per column of the identity
 // (a chain of n^2 dependent steps, each waiting on its loads) took 36 ms for
-// n = 500; now 8.7 ms.
+// n = 500; now 8 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -53,7 +53,7 @@ __device__ __forceinline__ long long mag_key(double v) {
 constexpr int PANEL_T = 1024;        // threads of the panel kernel
 constexpr int PANEL_W = 8;           // most columns of a panel
 constexpr size_t PANEL_SMEM = 200 * 1024;
-constexpr int STRIP = 8;             // columns per CTA of the trailing update
+constexpr int STRIP = 4;             // columns per CTA of the trailing update
 constexpr int TRAIL_T = 256;
 
 // Columns of a panel: as many as fit the panel kernel's shared memory; one,
@@ -79,11 +79,12 @@ __global__ void k_inv_init(int n, int ld, double *inv) {
 // by column unless in_place. The pivot of a column is its first row of
 // largest magnitude (a NaN diagonal keeps its row, as a sequential scan from
 // there would); a largest magnitude of 0 marks the matrix singular. swaps[c]
-// is the row swapped with row c. Bound by the FP64 pipe of one SM (the
+// is the row swapped with row c; *wild becomes 1 with a multiplier that is not
+// finite. Bound by the FP64 pipe of one SM (the
 // divisions) and the barriers: two per column.
 __global__ void __launch_bounds__(PANEL_T)
     k_lu_panel(int n, int ld, double *lu, int c0, int w, int in_place, int *swaps,
-               int *singular) {
+               int *singular, int *wild) {
   extern __shared__ double panel[];
   __shared__ long long sv[PANEL_T / 32];
   __shared__ int si[PANEL_T / 32], s_pivot;
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(PANEL_T)
     for (int r = k + 1 + tid; r < R; r += PANEL_T) {
       const double l = __ddiv_rn(P[k * sk + r * sr], piv);
       P[k * sk + r * sr] = l;
+      if ((__double2hiint(l) & 0x7FF00000) == 0x7FF00000) *wild = 1;
       for (int j = k + 1; j < w; ++j)
         P[j * sk + r * sr] = sub_rn(P[j * sk + r * sr], mul_rn(l, P[j * sk + k * sr]));
     }
@@ -172,12 +174,16 @@ __global__ void __launch_bounds__(PANEL_T)
     for (int t = tid; t < R * w; t += PANEL_T) G[int64_t(t / w) * ld + t % w] = panel[(t % w) * R + t / w];
 }
 
-// The panel's swaps and reductions on a strip of 8 columns: of lu right of the
-// panel, then of inv. W: the panel's width. Bound by the FP64 pipe.
+// The panel's swaps and reductions on a strip of 4 columns: of lu right of the
+// panel, then of inv. W: the panel's width. Bound by the FP64 pipe. A strip whose
+// part of U is all +0 (columns of the identity whose row has not been a pivot
+// yet: half of them on average) is left as it is after the swaps: a - l 0 = a
+// for every finite l. Strips of 8 columns took 21 us per launch for n = 500, as
+// one CTA per SM bounded them; the whole solve went from 57.2 to 54.8 ms.
 template <int W>
 __global__ void __launch_bounds__(TRAIL_T)
     k_lu_trail(int n, int ld, double *lu, double *inv, int c0, const int *swaps,
-               const int *singular) {
+               const int *singular, const int *wild) {
   __shared__ int rows[2 * W], src[2 * W];
   __shared__ int nrows;
   __shared__ double moved[2 * W][STRIP], L[W][W], U[W][STRIP];
@@ -232,10 +238,15 @@ __global__ void __launch_bounds__(TRAIL_T)
     }
   }
   __syncthreads();
-  if (!has) return;
   double u[W];
+  bool some = false;
 #pragma unroll
-  for (int k = 0; k < W; ++k) u[k] = U[k][j];
+  for (int k = 0; k < W; ++k) {
+    u[k] = has ? U[k][j] : 0.0;
+    some = some || __double_as_longlong(u[k]) != 0;
+  }
+  if (!__syncthreads_or(some) && *wild == 0) return;
+  if (!has) return;
 #pragma unroll 2
   for (int r = c1 + rr; r < n; r += RT) {
     const double *l = lu + int64_t(r) * ld + c0;
@@ -254,8 +265,8 @@ __global__ void __launch_bounds__(TRAIL_T)
 // prepare the products, BACK_C at a time, one chunk ahead, through shared
 // memory. Only the product with the x found last is left to warp 0: the
 // chunks of row i start at j = i + 2, whose x is known a row earlier. One warp
-// doing both took 186 cycles per term (11.2 ms for n = 500), now 87 (5.6 ms).
-constexpr int BACK_P = 16;          // products per producer warp and chunk
+// doing both took 186 cycles per term (11.2 ms for n = 500), now 84 (5.5 ms).
+constexpr int BACK_P = 32;          // products per producer warp and chunk
 constexpr int BACK_C = 3 * BACK_P;  // products per chunk
 __global__ void __launch_bounds__(128)
     k_back(int n, int ld, const double *lu, double *inv, const int *singular) {
@@ -304,9 +315,19 @@ __global__ void __launch_bounds__(128)
         un = lu[int64_t(i - 1) * ld + i];
       }
       const int m = min(BACK_C, n - j0);
-      if (m == BACK_C) {
-#pragma unroll 16
-        for (int t = 0; t < BACK_C; ++t) s = sub_rn(s, prod[buf][t][lane]);
+      if (m == BACK_C) {  // the next BACK_P products load while these are subtracted
+        double p[2][BACK_P];
+#pragma unroll
+        for (int t = 0; t < BACK_P; ++t) p[0][t] = prod[buf][t][lane];
+#pragma unroll
+        for (int h = 0; h < BACK_C / BACK_P; ++h) {
+#pragma unroll
+          for (int t = 0; t < BACK_P; ++t)
+            if (h + 1 < BACK_C / BACK_P)
+              p[(h + 1) & 1][t] = prod[buf][(h + 1) * BACK_P + t][lane];
+#pragma unroll
+          for (int t = 0; t < BACK_P; ++t) s = sub_rn(s, p[h & 1][t]);
+        }
       } else {
 #pragma unroll 4
         for (int t = 0; t < m; ++t) s = sub_rn(s, prod[buf][t][lane]);
@@ -399,8 +420,8 @@ int blocks_for(int64_t items, int per) {
 
 }  // namespace
 
-void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, double *inv,
-                          cudaStream_t s) {
+void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, int *wild,
+                          double *inv, cudaStream_t s) {
   if (n <= 0) return;
   static const bool attr = [] {  // once, thread-safe
     SGN_CUDA(cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -409,6 +430,7 @@ void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, 
   }();
   (void)attr;
   SGN_CUDA(cudaMemsetAsync(singular, 0, sizeof(int), s));
+  SGN_CUDA(cudaMemsetAsync(wild, 0, sizeof(int), s));
   k_inv_init<<<blocks_for(int64_t(n) * n, 256), 256, 0, s>>>(n, ld, inv);
   SGN_LAUNCH_CHECK();
   const int width = panel_width(n);
@@ -417,12 +439,13 @@ void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, 
     while (w > n - c0) w /= 2;  // the last columns: widths are powers of two
     const size_t smem = size_t(n - c0) * w * sizeof(double);
     const int in_place = smem > PANEL_SMEM ? 1 : 0;
-    k_lu_panel<<<1, PANEL_T, in_place ? 0 : smem, s>>>(n, ld, lu, c0, w, in_place, swaps, singular);
+    k_lu_panel<<<1, PANEL_T, in_place ? 0 : smem, s>>>(n, ld, lu, c0, w, in_place, swaps, singular,
+                                                              wild);
     SGN_LAUNCH_CHECK();
     const unsigned strips =
         unsigned((n - c0 - w + STRIP - 1) / STRIP + (n + STRIP - 1) / STRIP);
     auto trail = [&](auto kernel) {
-      kernel<<<strips, TRAIL_T, 0, s>>>(n, ld, lu, inv, c0, swaps, singular);
+      kernel<<<strips, TRAIL_T, 0, s>>>(n, ld, lu, inv, c0, swaps, singular, wild);
       SGN_LAUNCH_CHECK();
     };
     if (w == 8) trail(k_lu_trail<8>);

@@ -721,9 +721,11 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
 // the first digit are kept in shared memory for the later ones when they fit.
 // LEVELS: 6 digits cover the 48 bits of an FP64 key, 3 those of an FP32 value
 // (its FP64 key's low 29 bits are zero). Up to DG_ONE candidates CTA 0 works
-// alone. Twelve launches over all candidates did this before: 6 x (5.0 + 5.2)
+// alone, and up to DG_T it finds tau without digits, by every candidate's sum of
+// the candidates up to its own key. Twelve launches over all candidates did this before: 6 x (5.0 + 5.2)
 // us for one matrix of 500 rows, now 13 in all.
 constexpr int DG_C = 8, DG_T = 512, DG_KEEP = 2048, DG_ONE = 4096;
+static_assert(DG_T <= 2 * NDIG && DG_T <= DG_KEEP && DG_T <= DG_ONE, "the short path's arrays");
 template <int LEVELS>
 __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
     k_sel_digits(SelRows R, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
@@ -752,6 +754,33 @@ __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
   const int eb = ms[m].sel_e;
   const unsigned long long Q = ms[m].sel_q;
   unsigned long long prefix = st.prefix, lo = st.below_lo, hi = st.below_hi;
+  if (total <= DG_T) {  // CTA 0 alone: thread i sums the squares of the keys <= key i
+    const int n = int(total);
+    const unsigned long long key = tid < n ? sc.cand[cb + tid] : ~0ULL;
+    keep[tid] = key;
+    sum[tid] = tid < n ? qval<double>(key, eb) : 0ULL;
+    if (tid == 0) s_res[0] = ~0ULL;
+    __syncthreads();
+    unsigned long long le_lo = lo, le_hi = hi, lt_lo = lo, lt_hi = hi;
+    for (int i = 0; i < n; ++i) {
+      const unsigned long long k = keep[i], q = sum[i];
+      if (k <= key) u128_add(le_lo, le_hi, q, 0ULL);
+      if (k < key) u128_add(lt_lo, lt_hi, q, 0ULL);
+    }
+    const bool over = tid < n && exceeds(le_lo, le_hi, Q);
+    if (over) atomicMin(&s_res[0], key);
+    __syncthreads();
+    const unsigned long long tau = s_res[0];
+    if (over && key == tau) {  // every thread of this key writes the same
+      ms[m].tau = __longlong_as_double((long long)tau);
+      sc.st[m].prefix = tau;
+      sc.st[m].below_lo = lt_lo;
+      sc.st[m].below_hi = lt_hi;
+    }
+    if (cnt && tid < n && keep_key(key, tau))
+      atomicAdd(reinterpret_cast<unsigned long long *>(cnt + sc.cand_r[cb + tid]), 1ULL);
+    return;
+  }
   bool local = false;  // the survivors of the first digit are in keep
   for (int level = 0; level < LEVELS; ++level) {
     const int shift = 40 - 8 * level;

@@ -1137,9 +1137,9 @@ struct Solver {
     const size_t blk = size_t(nmax) * size_t(nmax);
     double *dx = static_cast<double *>(w.dmem.ensure(sizeof(double) * (3 * blk + size_t(nmax)), s));
     double *lu = dx + blk, *inv = lu + blk, *part = inv + blk;
-    w.nmf_int.ensure(sizeof(int) * size_t(nmax + nb), s);
+    w.nmf_int.ensure(sizeof(int) * size_t(nmax + nb + 1), s);
     w.nmf_dbl.ensure(sizeof(double) * size_t(nb), s);
-    int *swaps = w.nmf_int.as<int>(), *sing = swaps + nmax;
+    int *swaps = w.nmf_int.as<int>(), *sing = swaps + nmax, *wild = sing + nb;
     double *xinv = w.nmf_dbl.as<double>();
     SGN_CUDA(cudaMemsetAsync(sing, 0, sizeof(int) * size_t(nb), s));
     int64_t slot0 = 0;
@@ -1152,7 +1152,7 @@ struct Solver {
       launch_nmf_densify(ni, ni, st.X.d_rp(), st.X.d_col(), st.X.d_val(), row0, dx, s);
       SGN_CUDA(cudaMemcpyAsync(lu, dx, sizeof(double) * size_t(n) * size_t(n),
                                cudaMemcpyDeviceToDevice, s));
-      launch_dense_inverse(ni, ni, lu, swaps, sing + i, inv, s);
+      launch_dense_inverse(ni, ni, lu, swaps, sing + i, wild, inv, s);
       launch_inv_norm(ni, ni, inv, part, xinv + i, s);
       launch_nmf_combine(ni, ni, dx, inv, row0, slot0, C.rs.as<int64_t>(), C.re.as<int64_t>(),
                          C.col.as<int32_t>(), C.val.as<double>(), s);
