@@ -35,6 +35,11 @@ struct CopyChunk {
 };
 void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s);
 
+// Copies bytes (a multiple of 8) of device memory into mapped host memory, then
+// stores seq to *flag there (the data is visible before the flag).
+void launch_publish(const void *src, void *dst, size_t bytes, unsigned *flag, unsigned seq,
+                    cudaStream_t s);
+
 // Matrix-wide statistics for the server's footprint model. Initialise
 // min_gap_bits to the bits of +inf and the rest to 0; then min_gap_bits holds
 // the bits of min over rows with a positive gap of |a_ii| - sum_{j!=i}|a_ij|,

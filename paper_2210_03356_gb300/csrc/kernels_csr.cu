@@ -136,6 +136,19 @@ __global__ void k_copy_chunks(int count, const CopyChunk *chunks) {
   }
 }
 
+// ------------------------------------------------------------ readback
+// bytes (a multiple of 8) of src into mapped host memory, then the flag: the
+// host polls it instead of a copy's completion.
+constexpr int PUB_T = 1024;
+__global__ void __launch_bounds__(PUB_T)
+    k_publish(const unsigned long long *src, unsigned long long *dst, int64_t words,
+              volatile unsigned *flag, unsigned seq) {
+  for (int64_t i = threadIdx.x; i < words; i += PUB_T) dst[i] = src[i];
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) *flag = seq;
+}
+
 // ------------------------------------------------------------ footprint statistics
 // Per row: diagonal magnitude, off-diagonal sum and farthest column, folded
 // into the matrix-wide Gershgorin gap, row-sum bound and half-bandwidth.
@@ -607,6 +620,14 @@ void launch_validate_batch(int count, const ValidateJob *jobs, const int64_t *ro
 void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s) {
   if (count < 1) return;
   k_copy_chunks<<<count < 152 * 8 ? count : 152 * 8, 256, 0, s>>>(count, chunks);
+  SGN_LAUNCH_CHECK();
+}
+
+void launch_publish(const void *src, void *dst, size_t bytes, unsigned *flag, unsigned seq,
+                    cudaStream_t s) {
+  k_publish<<<1, PUB_T, 0, s>>>(static_cast<const unsigned long long *>(src),
+                                static_cast<unsigned long long *>(dst), int64_t(bytes / 8), flag,
+                                seq);
   SGN_LAUNCH_CHECK();
 }
 

@@ -260,16 +260,19 @@ struct HostMirror {
   double *mults = nullptr;  // of the last product, per matrix
   int64_t *tot = nullptr;
   ExtractBlock *xb = nullptr;
+  unsigned *flag = nullptr;  // the last publication that reached the host
+  unsigned seq = 0;          // the last one queued
   int nb = 0;
   void alloc(int n) {
     nb = n;
-    size_t bytes = MatPack::bytes(nb) + ProductHead::bytes(nb) + sizeof(double) * size_t(nb) +
+    size_t bytes = 64 + MatPack::bytes(nb) + ProductHead::bytes(nb) + sizeof(double) * size_t(nb) +
                    sizeof(ExtractBlock) * nb + 64 + 1024;
     if (bytes > cap) {
       if (p) cudaFreeHost(p);
       p = nullptr;
       SGN_CUDA(cudaMallocHost(&p, bytes));
       cap = bytes;
+      *static_cast<unsigned *>(p) = seq;
     }
     char *c = static_cast<char *>(p);
     auto take = [&](size_t b) {
@@ -277,6 +280,7 @@ struct HostMirror {
       c += (b + 63) & ~size_t(63);
       return r;
     };
+    flag = reinterpret_cast<unsigned *>(take(sizeof(unsigned)));
     pack = MatPack::at(take(MatPack::bytes(nb)), nb);
     head = reinterpret_cast<ProductHead *>(take(ProductHead::bytes(nb)));
     mults = reinterpret_cast<double *>(take(sizeof(double) * nb));
@@ -362,6 +366,25 @@ struct Solver {
     sync(s);
     stg.used = 0;
   }
+  // Reads device memory back into the host mirror and waits for the stream up
+  // to here. A kernel writes the mirror (mapped memory) and a flag that is polled:
+  // about 4 us less GPU idle time per wait than a copy and
+  // cudaStreamSynchronize, four waits an iteration. The stream is queried from
+  // time to time, so that an error ends the wait.
+  void fetch(void *dst, const void *src, size_t bytes) {
+    const unsigned seq = ++hm.seq;
+    launch_publish(src, dst, bytes, hm.flag, seq, s);
+    prof_sync_point(s);
+    for (unsigned spin = 1; __atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) != seq; ++spin)
+      if (spin % 65536 == 0) {
+        const cudaError_t e = cudaStreamQuery(s);
+        if (e == cudaErrorNotReady) continue;
+        SGN_CUDA(e);
+        if (__atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) == seq) break;
+        throw Error(SIGN_ECUDA, "a readback did not reach the host");
+      }
+    stg.used = 0;
+  }
   // h2d from host memory of any kind, through the pinned arena.
   template <typename T>
   void put(void *dst, const T *src, size_t count) {
@@ -414,9 +437,7 @@ struct Solver {
   // the last product's values for the host, and the round's per-matrix values
   ProductHead *head_dev() { return w.counters.as<ProductHead>(); }
   MatPack pack_dev(int nb) { return MatPack::at(w.ms.ensure(MatPack::bytes(nb), s), nb); }
-  void read_pack(int nb) {
-    d2h(reinterpret_cast<char *>(hm.pack.ms), w.ms.p, MatPack::bytes(nb), s);
-  }
+  void fetch_pack(int nb) { fetch(hm.pack.ms, w.ms.p, MatPack::bytes(nb)); }
 
   // ---------------------------------------------------------------- product
   // C = A B for a stage. Enqueues everything; on return C is allocated and the
@@ -501,8 +522,7 @@ struct Solver {
       launch_scan(N, w.ub.as<int64_t>(), C.rs.template as<int64_t>(), w.scan_tmp.as<int64_t>(), s,
                   nullptr, nullptr, &head->tot[0]);
     }
-    d2h(reinterpret_cast<char *>(hm.head), head, ProductHead::bytes(nb), s);
-    wait();
+    fetch(hm.head, head, ProductHead::bytes(nb));
     const int *const ctr = hm.head->ctr;
     for (int i = 0; i < nb; ++i) hm.mults[i] = double(hm.head->mults[i]);
     int64_t slots = hm.head->tot[0];
@@ -936,10 +956,9 @@ struct Solver {
       launch_budget_x2(nb, st.d_moff.template as<int64_t>(), w.x2.as<double>(), o.switch_resid,
                        w.ms.as<MatScalars>(), s);
     }
-    read_pack(nb);
     std::vector<unsigned long long> dcount(dp.nd);
     if (dp.any()) d2h(dcount.data(), w.dcount.p, size_t(dp.nd), s);
-    wait();
+    fetch_pack(nb);
     for (int d = 0; d < dp.nd; ++d) {  // the dense path's T: its nonzeros and multiply-adds
       int i = dp.mat[d];
       hm.pack.nnz[i] += int64_t(dcount[d]);
@@ -1253,11 +1272,10 @@ struct Solver {
         launch_drop_sums(nb, st.d_moff.template as<int64_t>(), w.dropped.as<double>(), d_act,
                          exact ? w.sel.p : nullptr, pk.ms, pk.dsum, s);
       }
-      read_pack(nb);
       const bool capped = exact && w.sel_shift > 0;
       if (capped)
         d2h(reinterpret_cast<unsigned long long *>(hm.tot), select_overflow(w.sel.p, nb), 1, s);
-      wait();
+      fetch_pack(nb);
       if (!capped || hm.tot[0] == 0) break;
       select_threshold(st, in, d_act, true);  // the crossing bucket outgrew the room
     }
@@ -1306,8 +1324,7 @@ struct Solver {
     int nbm = int(st.mats.size());
     launch_scan(N, w.cnt.as<int64_t>(), st.Xh.d_rp(), w.scan_tmp.as<int64_t>(), s,
                 st.d_seg.template as<int32_t>(), pack_dev(nbm).ex);
-    read_pack(nbm);
-    wait();
+    fetch_pack(nbm);
     for (int i = 0; i < nbm; ++i) {
       hms[i].nnz_bar = hm.pack.ms[i].nnz_bar;
       hms[i].beta = hm.pack.ms[i].beta;  // NMF sets its own budget after the check
