@@ -26,12 +26,13 @@ void launch_validate_batch(int count, const ValidateJob *jobs, const int64_t *ro
                            int64_t total_rows, int *flags, cudaStream_t s);
 
 // Copies `count` chunks (src, dst: device-accessible pointers, e.g. device
-// memory or mapped pinned host memory; bytes a multiple of 4, the chunks not
-// overlapping) in one launch.
+// memory or mapped pinned host memory; addresses and bytes multiples of 4, the
+// chunks not overlapping) in one launch. host_src: src is host memory.
 struct CopyChunk {
   const void *src;
   void *dst;
   int64_t bytes;
+  int host_src;
 };
 void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s);
 

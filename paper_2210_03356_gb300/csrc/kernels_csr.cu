@@ -106,32 +106,74 @@ __global__ void k_validate_batch(int count, const ValidateJob *jobs, const int64
 }
 
 // ------------------------------------------------------------ gathered copies
-// One CTA per chunk (grid-stride): 16-byte words when both ends and the
-// length allow it, else 4-byte words (every chunk's length is a multiple of 4).
+// One CTA per chunk (grid-stride), 16-byte words with up to three 4-byte words
+// before and after them (every chunk's length and address is a multiple of 4).
+// Where the two sides are offset against each other, the far side (host memory,
+// whose accesses should be whole lines: src of a chunk read from the host, else
+// dst) is taken in aligned 16-byte words and the near one word by word. A
+// batch's results go into arrays packed one after another, which are seldom
+// aligned: 1.2 GB took 11.5 ms in 4-byte words, now 9.1 (8.9 where both start on
+// a line).
 __global__ void k_copy_chunks(int count, const CopyChunk *chunks) {
+  constexpr int U = 4;  // 16-byte words per thread in flight
+  const int T = blockDim.x, t = threadIdx.x;
   for (int c = blockIdx.x; c < count; c += gridDim.x) {
     const CopyChunk ch = chunks[c];
-    const uintptr_t a = reinterpret_cast<uintptr_t>(ch.src), b = reinterpret_cast<uintptr_t>(ch.dst);
-    if (((a | b | uintptr_t(ch.bytes)) & 15u) == 0) {
-      // four 16-byte words per thread in flight (the far side may be host memory)
-      const int4 *s4 = static_cast<const int4 *>(ch.src);
-      int4 *d4 = static_cast<int4 *>(ch.dst);
-      const int64_t n4 = ch.bytes >> 4;
-      const int64_t T = blockDim.x;
-      int64_t i = threadIdx.x;
-      for (; i + 3 * T < n4; i += 4 * T) {
-        const int4 v0 = s4[i], v1 = s4[i + T], v2 = s4[i + 2 * T], v3 = s4[i + 3 * T];
-        d4[i] = v0;
-        d4[i + T] = v1;
-        d4[i + 2 * T] = v2;
-        d4[i + 3 * T] = v3;
+    const uint32_t *s1 = static_cast<const uint32_t *>(ch.src);
+    uint32_t *d1 = static_cast<uint32_t *>(ch.dst);
+    const int64_t n1 = ch.bytes >> 2;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(s1), b = reinterpret_cast<uintptr_t>(d1);
+    const uintptr_t far = ch.host_src ? a : b;
+    const int64_t head = min(n1, int64_t((16u - (far & 15u)) & 15u) >> 2);
+    const int64_t n4 = (n1 - head) >> 2, tail = head + 4 * n4;
+    if (t < head) d1[t] = s1[t];
+    if (t < n1 - tail) d1[tail + t] = s1[tail + t];
+    s1 += head;
+    d1 += head;
+    const bool same = ((a ^ b) & 15u) == 0;
+    if (same) {
+      const int4 *s4 = reinterpret_cast<const int4 *>(s1);
+      int4 *d4 = reinterpret_cast<int4 *>(d1);
+      for (int64_t i = t; i < n4; i += U * T) {
+        int4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) v[u] = s4[i + u * T];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) d4[i + u * T] = v[u];
       }
-      for (; i < n4; i += T) d4[i] = s4[i];
+    } else if (ch.host_src) {
+      const int4 *s4 = reinterpret_cast<const int4 *>(s1);
+      for (int64_t i = t; i < n4; i += U * T) {
+        int4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) v[u] = s4[i + u * T];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) {
+            uint32_t *d = d1 + 4 * (i + u * T);
+            d[0] = uint32_t(v[u].x);
+            d[1] = uint32_t(v[u].y);
+            d[2] = uint32_t(v[u].z);
+            d[3] = uint32_t(v[u].w);
+          }
+      }
     } else {
-      const uint32_t *s1 = static_cast<const uint32_t *>(ch.src);
-      uint32_t *d1 = static_cast<uint32_t *>(ch.dst);
-      const int64_t n1 = ch.bytes >> 2;
-      for (int64_t i = threadIdx.x; i < n1; i += blockDim.x) d1[i] = s1[i];
+      int4 *d4 = reinterpret_cast<int4 *>(d1);
+      for (int64_t i = t; i < n4; i += U * T) {
+        int4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) {
+            const uint32_t *s = s1 + 4 * (i + u * T);
+            v[u] = make_int4(int(s[0]), int(s[1]), int(s[2]), int(s[3]));
+          }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + u * T < n4) d4[i + u * T] = v[u];
+      }
     }
   }
 }

@@ -88,11 +88,12 @@ thread_local Staging g_xfer_stage;
 
 struct Gather {
   std::vector<CopyChunk> chunks;
+  int host_src = 0;  // the sources are host memory
   void add(const void *src, void *dst, int64_t bytes) {
     const int64_t step = int64_t(1) << 20;
     for (int64_t o = 0; o < bytes; o += step)
       chunks.push_back(CopyChunk{static_cast<const char *>(src) + o, static_cast<char *>(dst) + o,
-                                 std::min(step, bytes - o)});
+                                 std::min(step, bytes - o), host_src});
   }
   size_t staged_bytes() const { return sizeof(CopyChunk) * chunks.size() + 64; }
   // queues the copies on s; the arena must have room for staged_bytes(); list
@@ -207,6 +208,7 @@ sign_status sign_create_batch(int count, const int64_t *n, const int64_t *nnz,
     // device arrays, or host arrays that are all pinned and mapped: one
     // gather kernel reads them
     Gather g;
+    g.host_src = on_device ? 0 : 1;
     std::vector<const void *> src(3 * size_t(count), nullptr);
     bool gather = true;
     for (int i = 0; i < count && gather; ++i) {
