@@ -61,6 +61,13 @@ void launch_gersh(int64_t n, const int64_t *rp, const int32_t *col, const double
 int64_t scan_tmp_elems(int64_t n);
 void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s,
                  const int32_t *seg = nullptr, int64_t *eoff = nullptr, int64_t *total = nullptr);
+// Up to SCAN_JOBS scans of n values at once; tmp holds scan_tmp_elems(n) for each.
+constexpr int SCAN_JOBS = 3;
+struct ScanJobs {
+  const int64_t *cnt[SCAN_JOBS];
+  int64_t *out[SCAN_JOBS], *total[SCAN_JOBS];  // total: nullable
+};
+void launch_scans(int64_t n, int jobs, const ScanJobs &J, int64_t *tmp, cudaStream_t s);
 
 // One block of a block-diagonal assembly: rows [row0, row0+nrows) of a source
 // CSR whose column indices are shifted by col_shift on the way.
@@ -174,12 +181,18 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // dslot (nullable, per matrix): matrices with dslot[m] >= 0 take the dense
 // path; their rows get no sparse work, and in MODE_UPDATE a whole row of
 // slots (moff gives the matrix sizes).
-void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, const int *active,
-                   int mode, int groups, float group_margin, int band, float band_min_eff,
+// nnzA: A's entries (or more). bspans, cspans (fc nullable): the band layouts of
+// B's rows and of the product's.
+struct BandSpans {  // of each row: fc and nf (see Band) and span = nf, scanned into pos
+  int32_t *fc = nullptr, *nf = nullptr;
+  int64_t *span = nullptr;
+};
+void launch_bounds(int64_t n, const Rows &A, int64_t nnzA, const Rows &B, const int32_t *seg,
+                   const int *active, int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
-                   cudaStream_t s);
+                   const BandSpans &bspans, const BandSpans &cspans, cudaStream_t s);
 
 // Band layout of the rows of an FP32 operand: row k's values dense over the
 // columns [fc[k], fc[k] + nf[k]) (fc and nf multiples of 4, holes +0) at
@@ -201,13 +214,6 @@ struct BandOut {
 };
 constexpr int BAND_JW = 64;   // widest output hull of a band tile, in 32-column words
 constexpr int BAND_KT = 312;  // widest k hull (A rows' columns) of a band tile
-// fc, nf and span[k] = nf[k] of each row (span is scanned into pos).
-void launch_band_spans(int64_t n, const Rows &R, int32_t *fc, int32_t *nf, int64_t *span,
-                       cudaStream_t s);
-// The same layout from a product's row column ranges [lo, lo + len) (the
-// first and last column of a product row are stored entries).
-void launch_band_spans_range(int64_t n, const int32_t *lo, const int32_t *len, int32_t *fc,
-                             int32_t *nf, int64_t *span, cudaStream_t s);
 // Writes the rows' bands (cleared first) from their CSR; rows with skip[r]
 // set (skip nullable) are left as they are.
 void launch_band_fill(int64_t n, const Rows &R, const float *val, const int64_t *pos,
@@ -217,7 +223,7 @@ void launch_band_fill(int64_t n, const Rows &R, const float *val, const int64_t 
 // (SQUARE, with the partial sums of launch_numeric) or 1.5 A - 0.5 A B
 // (UPDATE), A's rows as CSR (its stored k) and both operands as bands. In
 // SQUARE, bandC (val nullable) receives the band of the tiles' rows of C, laid
-// out by launch_band_spans_range.
+// out by launch_bounds (cspans).
 void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, const Band &bandA,
                          const Band &bandB, const BandOut &bandC, const int32_t *lo,
                          const int32_t *len, const int32_t *lists, int *counters,

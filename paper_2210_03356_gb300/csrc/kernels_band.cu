@@ -74,43 +74,6 @@ __device__ __forceinline__ int warp_max(int v) {
 }
 
 // ---------------------------------------------------------------- band layout
-__global__ void k_band_spans(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
-                             int32_t *fc, int32_t *nf, int64_t *span) {
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
-       r += int64_t(gridDim.x) * blockDim.x) {
-    int64_t a = rs[r], b = re[r];
-    int32_t f = 0, w = 0;
-    if (b > a) {
-      int32_t first = col[a], last = col[b - 1];
-      f = first & ~3;
-      w = ((last + 4) & ~3) - f;
-    }
-    fc[r] = f;
-    nf[r] = w;
-    span[r] = w;
-  }
-}
-
-// The band layout of the rows of a product from their column ranges
-// [lo, lo + len): the first and last column of a product row are stored
-// entries (each is the first or last column of some B_k), so this is the
-// layout k_band_spans gives for the finished rows.
-__global__ void k_band_spans_range(int64_t n, const int32_t *lo, const int32_t *len, int32_t *fc,
-                                   int32_t *nf, int64_t *span) {
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
-       r += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t L = len[r];
-    int32_t f = 0, w = 0;
-    if (L > 0) {
-      f = lo[r] & ~3;
-      w = ((lo[r] + L - 1 + 4) & ~3) - f;
-    }
-    fc[r] = f;
-    nf[r] = w;
-    span[r] = w;
-  }
-}
-
 constexpr int FILL_LPR = 8;  // lanes per row of the band layout
 
 // FILL_LPR lanes per row (rows with skip[r] set are left alone): the row's
@@ -506,24 +469,6 @@ int sm_count_band() {
 }
 
 }  // namespace
-
-void launch_band_spans(int64_t n, const Rows &R, int32_t *fc, int32_t *nf, int64_t *span,
-                       cudaStream_t s) {
-  if (n == 0) return;
-  int64_t g = (n + 255) / 256;
-  if (g > int64_t(sm_count_band()) * 8) g = int64_t(sm_count_band()) * 8;
-  k_band_spans<<<unsigned(g), 256, 0, s>>>(n, R.rs, R.re, R.col, fc, nf, span);
-  SGN_LAUNCH_CHECK();
-}
-
-void launch_band_spans_range(int64_t n, const int32_t *lo, const int32_t *len, int32_t *fc,
-                             int32_t *nf, int64_t *span, cudaStream_t s) {
-  if (n == 0) return;
-  int64_t g = (n + 255) / 256;
-  if (g > int64_t(sm_count_band()) * 8) g = int64_t(sm_count_band()) * 8;
-  k_band_spans_range<<<unsigned(g), 256, 0, s>>>(n, lo, len, fc, nf, span);
-  SGN_LAUNCH_CHECK();
-}
 
 void launch_band_fill(int64_t n, const Rows &R, const float *val, const int64_t *pos,
                       const int32_t *fc, const int32_t *nf, const unsigned char *skip, float *bval,

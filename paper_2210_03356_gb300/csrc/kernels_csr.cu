@@ -260,9 +260,11 @@ __device__ int64_t block_excl_scan(int64_t v, int64_t *sm, int64_t *total) {
   return r;
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(int64_t n, const int64_t *cnt,
-                                                        int64_t *tmp) {
+// blockIdx.y: the scan, its tile totals at tmp + blockIdx.y * tmp_stride.
+__global__ void __launch_bounds__(SCAN_T)
+    k_scan_reduce(int64_t n, ScanJobs J, int64_t *tmp, int64_t tmp_stride) {
   __shared__ int64_t sm[33];
+  const int64_t *cnt = blockIdx.y == 0 ? J.cnt[0] : blockIdx.y == 1 ? J.cnt[1] : J.cnt[2];
   int64_t base = int64_t(blockIdx.x) * SCAN_TILE + int64_t(threadIdx.x) * SCAN_ITEMS;
   int64_t v = 0;
 #pragma unroll
@@ -270,16 +272,22 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(int64_t n, const int64_t
     if (base + i < n) v += cnt[base + i];
   int64_t total;
   block_excl_scan(v, sm, &total);
-  if (threadIdx.x == 0) tmp[blockIdx.x] = total;
+  if (threadIdx.x == 0) tmp[blockIdx.y * tmp_stride + blockIdx.x] = total;
 }
 
 // A tile's scan: the tiles before it are added from their totals in tmp (a
 // single tile has none). seg, eoff (nullable): the scan's value at the end of
 // each matrix; total (nullable): the sum of all.
 __global__ void __launch_bounds__(SCAN_T)
-    k_scan_final(int64_t n, const int64_t *cnt, const int64_t *tmp, int64_t *out,
-                 const int32_t *seg, int64_t *eoff, int64_t *total) {
+    k_scan_final(int64_t n, ScanJobs J, const int64_t *tmp, int64_t tmp_stride,
+                 const int32_t *seg, int64_t *eoff) {
   __shared__ int64_t sm[33];
+  const int y = blockIdx.y;  // picked by comparison: an indexed parameter is copied to local memory
+  static_assert(SCAN_JOBS == 3, "three to pick from");
+  const int64_t *cnt = y == 0 ? J.cnt[0] : y == 1 ? J.cnt[1] : J.cnt[2];
+  int64_t *const out = y == 0 ? J.out[0] : y == 1 ? J.out[1] : J.out[2];
+  int64_t *const total = y == 0 ? J.total[0] : y == 1 ? J.total[1] : J.total[2];
+  tmp += blockIdx.y * tmp_stride;
   int64_t before = 0;
   if (blockIdx.x > 0) {
     int64_t v = 0;
@@ -675,21 +683,38 @@ void launch_publish(const void *src, void *dst, size_t bytes, unsigned *flag, un
 
 int64_t scan_tmp_elems(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
 
-void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s,
-                 const int32_t *seg, int64_t *eoff, int64_t *total) {
-  int64_t nblocks = (n + SCAN_TILE - 1) / SCAN_TILE;
+static void run_scans(int64_t n, int jobs, const ScanJobs &J, int64_t *tmp, const int32_t *seg,
+                      int64_t *eoff, cudaStream_t s) {
+  const int64_t nblocks = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (nblocks == 0) {
-    SGN_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), s));
+    for (int j = 0; j < jobs; ++j) {
+      SGN_CUDA(cudaMemsetAsync(J.out[j], 0, sizeof(int64_t), s));
+      if (J.total[j]) SGN_CUDA(cudaMemsetAsync(J.total[j], 0, sizeof(int64_t), s));
+    }
     if (eoff) SGN_CUDA(cudaMemsetAsync(eoff, 0, sizeof(int64_t), s));
-    if (total) SGN_CUDA(cudaMemsetAsync(total, 0, sizeof(int64_t), s));
     return;
   }
+  const dim3 grid{unsigned(nblocks), unsigned(jobs)};
+  const int64_t stride = scan_tmp_elems(n);
   if (nblocks > 1) {
-    k_scan_reduce<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp);
+    k_scan_reduce<<<grid, SCAN_T, 0, s>>>(n, J, tmp, stride);
     SGN_LAUNCH_CHECK();
   }
-  k_scan_final<<<unsigned(nblocks), SCAN_T, 0, s>>>(n, cnt, tmp, out, seg, eoff, total);
+  k_scan_final<<<grid, SCAN_T, 0, s>>>(n, J, tmp, stride, seg, eoff);
   SGN_LAUNCH_CHECK();
+}
+
+void launch_scans(int64_t n, int jobs, const ScanJobs &J, int64_t *tmp, cudaStream_t s) {
+  run_scans(n, jobs, J, tmp, nullptr, nullptr, s);
+}
+
+void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cudaStream_t s,
+                 const int32_t *seg, int64_t *eoff, int64_t *total) {
+  ScanJobs J = {};
+  J.cnt[0] = cnt;
+  J.out[0] = out;
+  J.total[0] = total;
+  run_scans(n, 1, J, tmp, seg, eoff, s);
 }
 
 void launch_assemble_rows(int nblocks, const AsmBlock *blocks, const int64_t *boff, int64_t n_dst,

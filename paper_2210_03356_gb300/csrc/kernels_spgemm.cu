@@ -89,8 +89,7 @@ __device__ __forceinline__ int64_t lower_bound(const int32_t *a, int64_t lo, int
   return lo;
 }
 
-constexpr int BOUNDS_TILE = 256;  // rows per CTA of k_bounds; lists keep this order
-static_assert(BOUNDS_TILE % 16 == 0, "band tiles are aligned groups of 16 rows");
+constexpr int BOUNDS_T = 256;  // threads of k_bounds
 // A 16-row group goes to a band tile when its multiply-adds are at least a
 // fraction band_min_eff (a schedule option, 0.08 by default) of the tile's
 // estimated FMA slots: the band kernel spends about 2.5 instructions per slot,
@@ -115,17 +114,29 @@ __device__ __forceinline__ float lane_use(float avg, int g) {
 // be streamed.
 constexpr float STREAM_AVG = 64.0f;
 
+// The band layout of a row from its first and last column (last < first: empty).
+__device__ __forceinline__ void put_span(const BandSpans &bs, int64_t r, int first, int last) {
+  const int f = last < first ? 0 : first & ~3;
+  const int w = last < first ? 0 : ((last + 4) & ~3) - f;
+  bs.fc[r] = f;
+  bs.nf[r] = w;
+  bs.span[r] = w;
+}
+
 // Per row k of B: (first column, last column, entries, 0), so that k_bounds
 // reads one 16-byte record per k instead of a chain of dependent loads. ends
 // (nullable; FP64 products): of a row with at least 32 entries, the 31st
-// column and the 31st from its end (see stream_rows).
+// column and the 31st from its end (see stream_rows). bs (fc nullable): the
+// band layout of B's rows.
 __global__ void k_row_info(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
-                           int4 *info, int2 *ends) {
+                           int4 *info, int2 *ends, BandSpans bs) {
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     const int64_t a = rs[r], b = re[r];
-    info[r] = b > a ? make_int4(col[a], col[b - 1], int(b - a), 0) : make_int4(0, -1, 0, 0);
+    const int4 x = b > a ? make_int4(col[a], col[b - 1], int(b - a), 0) : make_int4(0, -1, 0, 0);
+    info[r] = x;
     if (ends && b - a >= 32) ends[r] = make_int2(col[a + 30], col[b - 31]);
+    if (bs.fc) put_span(bs, r, x.x, x.y);
   }
 }
 
@@ -179,187 +190,211 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
   return cls;
 }
 
+// Over the 16 lanes of a half warp.
+__device__ __forceinline__ int half_min(unsigned hm, int v) { return __reduce_min_sync(hm, v); }
+__device__ __forceinline__ int half_max(unsigned hm, int v) { return __reduce_max_sync(hm, v); }
+__device__ __forceinline__ int half_sum(unsigned hm, int v) { return __reduce_add_sync(hm, v); }
+
+// Bounds, class and lists of the rows of a product, TILE rows at a time per
+// CTA, L lanes per row (its A entries L apart, four B records per lane in
+// flight). Bound by the latency of row -> k -> record and, where rows are many
+// and short, by atomics on single addresses (list lengths, multiply-adds),
+// which are therefore made once per tile. With a lane per row throughout, an
+// atomic per warp and the band decision by one lane per 16 rows, 16 products
+// took 0.52 ms at 6001 rows and 0.79 at 262144, now 0.23 and 0.41 (with the
+// rows' records and the band layouts' widths). cs (fc nullable): the band layout of
+// the product's rows, whose first and last columns [lo, lo + len) are stored
+// entries (each is the first or last column of some B_k).
 // counters: [RC_*] list lengths, [RC_QUEUE + RC_*] work-queue heads of the numeric kernels.
-__global__ void __launch_bounds__(BOUNDS_TILE)
+template <int L, int TILE>
+__global__ void __launch_bounds__(BOUNDS_T)
     k_bounds(int64_t n, const int64_t *ars, const int64_t *are, const int32_t *acol,
              const int4 *binfo, const int32_t *seg,
              const int *active, int mode, int groups, float group_margin, int band,
              float band_min_eff, const int *dslot,
              const int64_t *moff, int32_t *lo, int32_t *len, int64_t *ub, int32_t *lists,
              int *counters, unsigned long long *mults, double *band_work,
-             unsigned char *bandrow) {
-  __shared__ unsigned char s_cls[BOUNDS_TILE];
-  __shared__ int s_cnt[BOUNDS_TILE / 32][RC_N];
+             unsigned char *bandrow, BandSpans cs) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int ROWS = BOUNDS_T / L;  // rows of one pass
+  constexpr int NW = (TILE + 31) / 32;  // warps with rows in the second part
+  static_assert(TILE % ROWS == 0 && TILE <= BOUNDS_T, "whole passes, a thread per row");
+  static_assert(TILE % 16 == 0, "band tiles are aligned groups of 16 rows");
+  __shared__ unsigned char s_cls[TILE];
+  __shared__ int s_cnt[NW][RC_N];
   __shared__ int s_base[RC_N];
+  __shared__ unsigned long long s_mult, s_band_work;
   // per-row statistics of the band decision (rows of sparse work only)
-  __shared__ int s_seg[BOUNDS_TILE], s_lo[BOUNDS_TILE], s_L[BOUNDS_TILE];
-  __shared__ int s_kf[BOUNDS_TILE], s_kl[BOUNDS_TILE], s_na[BOUNDS_TILE];
-  __shared__ float s_wk[BOUNDS_TILE];
-  __shared__ unsigned char s_band[BOUNDS_TILE / 16];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = BOUNDS_TILE / 32;
+  __shared__ int s_seg[TILE], s_lo[TILE], s_L[TILE];
+  __shared__ int s_kf[TILE], s_kl[TILE], s_na[TILE];
+  __shared__ float s_wk[TILE];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  const int64_t ntiles = (n + BOUNDS_TILE - 1) / BOUNDS_TILE;
+  const int64_t ntiles = (n + TILE - 1) / TILE;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t t0 = tile * BOUNDS_TILE;
-    // One thread per row: its own pass over A_i (four B records in flight),
-    // with no reductions across lanes. Rows of more than BOUNDS_LONG entries
-    // are left to the whole warp afterwards.
-    const int i = threadIdx.x;
-    const int64_t r = t0 + i;
-    int cls = RC_NONE;
-    bool longrow = false;
-    s_seg[i] = -1;  // not eligible for a band tile
-    int m = 0;
-    int64_t a0 = 0, a1 = 0;
-    unsigned long long mywork = 0;  // the row's multiply-adds
-    if (r < n) {
-      m = seg[r];
-      if (!active[m] || (dslot && dslot[m] >= 0)) {
-        // inactive, or on the dense path: no sparse work; a dense row of an
-        // update gets a whole row of slots for 1.5 X - 0.5 X T
-        const bool dense = active[m] && dslot && dslot[m] >= 0;
-        ub[r] = dense && mode == MODE_UPDATE ? moff[m + 1] - moff[m] : 0;
-        len[r] = 0;
-        lo[r] = 0;
-      } else {
+    const int64_t t0 = tile * TILE;
+    const int m0 = seg[t0];
+    if (threadIdx.x == 0) s_mult = s_band_work = 0ULL;
+    unsigned long long mywork = 0;  // multiply-adds of matrix m0 (leaders)
+    auto add_work = [&](int m, unsigned long long w) {
+      if (m == m0)
+        mywork += w;
+      else
+        atomicAdd(&mults[m], w);
+    };
+#pragma unroll 1
+    for (int i0 = 0; i0 < TILE; i0 += ROWS) {
+      const int i = i0 + threadIdx.x / L, gl = threadIdx.x % L;
+      const int64_t r = t0 + i;
+      int cls = RC_NONE, m = 0;
+      bool work = false, longrow = false;  // the row has sparse work; walked by the warp
+      int64_t a0 = 0, a1 = 0;
+      int32_t mn = INT_MAX, mx = -1, kf = INT_MAX, kl = -1;
+      int64_t wk = 0;
+      if (gl == 0) s_seg[i] = -1;  // not eligible for a band tile
+      if (r < n) {
+        m = seg[r];
         a0 = ars[r];
         a1 = are[r];
-        if (a1 - a0 > BOUNDS_LONG) {
-          longrow = true;
+        if (!active[m] || (dslot && dslot[m] >= 0)) {
+          // inactive, or on the dense path: no sparse work; a dense row of an
+          // update gets a whole row of slots for 1.5 X - 0.5 X T
+          if (gl == 0) {
+            const bool dense = active[m] && dslot && dslot[m] >= 0;
+            ub[r] = dense && mode == MODE_UPDATE ? moff[m + 1] - moff[m] : 0;
+            len[r] = 0;
+            lo[r] = 0;
+            if (cs.fc) put_span(cs, r, 0, -1);
+          }
         } else {
-          int32_t mn = INT_MAX, mx = -1;
-          int64_t wk = 0;
-          int64_t p = a0;
-          for (; p + 4 <= a1; p += 4) {
-            const int32_t k0 = acol[p], k1 = acol[p + 1], k2 = acol[p + 2], k3 = acol[p + 3];
-            const int4 b0 = binfo[k0], b1 = binfo[k1], b2 = binfo[k2], b3 = binfo[k3];
-            wk += int64_t(b0.z) + b1.z + b2.z + b3.z;
-            // an empty B row has first column 0 and last -1: no effect on either
-            mn = min(mn, min(min(b0.z ? b0.x : INT_MAX, b1.z ? b1.x : INT_MAX),
-                             min(b2.z ? b2.x : INT_MAX, b3.z ? b3.x : INT_MAX)));
-            mx = max(mx, max(max(b0.y, b1.y), max(b2.y, b3.y)));
+          work = true;
+          // one lane per row: rows of more than BOUNDS_LONG entries are left to the warp
+          longrow = L == 1 && a1 - a0 > BOUNDS_LONG;
+          if (a1 > a0) {
+            kf = acol[a0];
+            kl = acol[a1 - 1];
           }
-          for (; p < a1; ++p) {
-            const int4 bi = binfo[acol[p]];
-            wk += bi.z;
-            if (bi.z > 0) mn = min(mn, bi.x);
-            mx = max(mx, bi.y);
+          if (!longrow) {
+            for (int64_t p = a0 + gl; p < a1; p += 4 * L) {
+              int32_t k[4];
+              int4 b[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) k[u] = p + u * L < a1 ? acol[p + u * L] : -1;
+#pragma unroll
+              for (int u = 0; u < 4; ++u) b[u] = k[u] >= 0 ? binfo[k[u]] : make_int4(0, -1, 0, 0);
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                wk += b[u].z;
+                // an empty B row has first column 0 and last -1: no effect on either
+                mn = min(mn, b[u].z ? b[u].x : INT_MAX);
+                mx = max(mx, b[u].y);
+              }
+            }
           }
-          const int32_t kf = a1 > a0 ? acol[a0] : INT_MAX, kl = a1 > a0 ? acol[a1 - 1] : -1;
-          if (mode == MODE_UPDATE && a1 > a0) {  // the columns of X_i itself (ascending)
-            mn = min(mn, kf);
-            mx = max(mx, kl);
-          }
-          mywork = (unsigned long long)wk;
-          cls = bounds_row(r, m, a1 - a0, mn, mx, kf, kl, wk, mode, groups, group_margin, band,
-                           lo, len, ub, s_seg + i, s_lo + i, s_L + i, s_kf + i, s_kl + i,
-                           s_na + i, s_wk + i);
         }
       }
-    }
-    s_cls[i] = (unsigned char)cls;
-    // long rows: the warp walks each with its lanes striding over A_i
-    unsigned lm = __ballot_sync(0xffffffffu, longrow);
-    while (lm) {
-      const int src = __ffs(lm) - 1;
-      lm &= lm - 1;
-      const int li = warp * 32 + src;
-      const int64_t lr = t0 + li;
-      const int lmat = __shfl_sync(0xffffffffu, m, src);
-      const int64_t la0 = __shfl_sync(0xffffffffu, a0, src), la1 = __shfl_sync(0xffffffffu, a1, src);
-      int32_t mn = INT_MAX, mx = -1;
-      int64_t wk = 0;
-      for (int64_t p = la0 + lane; p < la1; p += 32) {
-        const int4 bi = binfo[acol[p]];
-        wk += bi.z;
-        if (bi.z > 0) mn = min(mn, bi.x);
-        mx = max(mx, bi.y);
-      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        wk += __shfl_xor_sync(0xffffffffu, wk, o);
+      for (int o = L / 2; o > 0; o >>= 1) {
+        mn = min(mn, __shfl_xor_sync(FULL, mn, o));
+        mx = max(mx, __shfl_xor_sync(FULL, mx, o));
+        wk += __shfl_xor_sync(FULL, wk, o);
       }
-      if (lane == src) {
-        const int32_t kf = acol[la0], kl = acol[la1 - 1];
-        if (mode == MODE_UPDATE) {
+      if constexpr (L == 1) {  // long rows: the warp walks each with its lanes striding over A_i
+        unsigned lm = __ballot_sync(FULL, longrow);
+        while (lm) {
+          const int src = __ffs(lm) - 1;
+          lm &= lm - 1;
+          const int64_t la0 = __shfl_sync(FULL, a0, src), la1 = __shfl_sync(FULL, a1, src);
+          int32_t lmn = INT_MAX, lmx = -1;
+          int64_t lwk = 0;
+          for (int64_t p = la0 + lane; p < la1; p += 32) {
+            const int4 bi = binfo[acol[p]];
+            lwk += bi.z;
+            if (bi.z > 0) lmn = min(lmn, bi.x);
+            lmx = max(lmx, bi.y);
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            lmn = min(lmn, __shfl_xor_sync(FULL, lmn, o));
+            lmx = max(lmx, __shfl_xor_sync(FULL, lmx, o));
+            lwk += __shfl_xor_sync(FULL, lwk, o);
+          }
+          if (lane == src) {
+            mn = lmn;
+            mx = lmx;
+            wk = lwk;
+          }
+        }
+      }
+      if (work && gl == 0) {
+        if (mode == MODE_UPDATE && a1 > a0) {  // the columns of X_i itself (ascending)
           mn = min(mn, kf);
           mx = max(mx, kl);
         }
-        mywork = (unsigned long long)wk;
-        s_cls[li] = (unsigned char)bounds_row(lr, lmat, la1 - la0, mn, mx, kf, kl, wk, mode,
-                                              groups, group_margin, band, lo, len, ub,
-                                              s_seg + li, s_lo + li, s_L + li, s_kf + li,
-                                              s_kl + li, s_na + li, s_wk + li);
+        add_work(m, (unsigned long long)wk);
+        cls = bounds_row(r, m, a1 - a0, mn, mx, kf, kl, wk, mode, groups, group_margin, band, lo,
+                         len, ub, s_seg + i, s_lo + i, s_L + i, s_kf + i, s_kl + i, s_na + i,
+                         s_wk + i);
+        if (cs.fc) put_span(cs, r, mx < 0 ? 0 : mn, mx);
       }
-    }
-    // multiply-adds per matrix: one atomic per warp where its rows are of one matrix
-    if (__all_sync(0xffffffffu, m == __shfl_sync(0xffffffffu, m, 0) || mywork == 0)) {
-      unsigned long long sum = mywork;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0 && sum) atomicAdd(&mults[m], sum);
-    } else if (mywork) {
-      atomicAdd(&mults[m], mywork);
+      if (gl == 0) s_cls[i] = (unsigned char)cls;
     }
     __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mywork += __shfl_xor_sync(FULL, mywork, o);
+    if (lane == 0 && mywork) atomicAdd(&s_mult, mywork);
+    // from here on a thread per row
+    const int i = threadIdx.x;
     // band tiles: aligned groups of 16 rows of one matrix, all with sparse
     // work, whose estimated FMA slots the multiply-adds fill well enough
-    if (band && threadIdx.x < BOUNDS_TILE / 16) {
-      const int b0 = threadIdx.x * 16;
-      bool ok = s_seg[b0] >= 0;
-      int jlo = INT_MAX, jhi = -1, klo = INT_MAX, khi = -1;
-      float wsum = 0.0f, nsum = 0.0f;
-      double wexact = 0.0;
-      for (int i = b0; i < b0 + 16 && ok; ++i) {
-        ok = s_seg[i] == s_seg[b0];
-        if (s_L[i] > 0) {
-          jlo = min(jlo, s_lo[i]);
-          jhi = max(jhi, s_lo[i] + s_L[i] - 1);
+    bool inband = false;
+    if (band && i < TILE) {
+      const unsigned hm = 0xffffu << (lane & 16);
+      const int sg = s_seg[i];
+      if (__all_sync(hm, sg >= 0 && sg == s_seg[i & ~15])) {
+        const bool some = s_L[i] > 0;
+        const int jlo = half_min(hm, some ? s_lo[i] : INT_MAX);
+        const int jhi = half_max(hm, some ? s_lo[i] + s_L[i] - 1 : -1);
+        const int klo = half_min(hm, s_kf[i]), khi = half_max(hm, s_kl[i]);
+        if (jhi >= 0 && khi >= 0 && khi - klo < BAND_KT - 3) {
+          const int nwords = (jhi >> 5) - (jlo >> 5) + 1;
+          if (nwords <= BAND_JW) {  // below 2^20 multiply-adds per row: sums exact in integers
+            const int wsum = half_sum(hm, int(s_wk[i])), nsum = half_sum(hm, s_na[i]);
+            const float bavg = float(wsum) / fmaxf(float(nsum), 1.0f);  // mean entries of a B row
+            const float kc = fminf(float(khi - klo + 1), bavg + 35.0f);
+            const float slots = 16.0f * 32.0f * float(nwords) * kc;
+            inband = float(wsum) >= band_min_eff * slots;
+            if (inband && (lane & 15) == 0 && band_work)
+              atomicAdd(&s_band_work, (unsigned long long)wsum);
+          }
         }
-        klo = min(klo, s_kf[i]);
-        khi = max(khi, s_kl[i]);
-        wsum += s_wk[i];
-        wexact += double(s_wk[i]);
-        nsum += float(s_na[i]);
       }
-      if (ok && jhi >= 0 && khi >= 0) {
-        const int nwords = (jhi >> 5) - (jlo >> 5) + 1;
-        const float bavg = wsum / fmaxf(nsum, 1.0f);  // mean entries of a B row
-        const float kc = fminf(float(khi - klo + 1), bavg + 35.0f);
-        const float slots = 16.0f * 32.0f * float(nwords) * kc;
-        ok = nwords <= BAND_JW && khi - klo < BAND_KT - 3 && wsum >= band_min_eff * slots;
-      } else {
-        ok = false;
-      }
-      s_band[threadIdx.x] = ok ? 1 : 0;
-      if (ok && band_work) atomicAdd(band_work, wexact);  // multiply-adds of the band tiles
     }
-    __syncthreads();
     // ordered compaction of the tile's rows into one list per class
-    int my = s_cls[threadIdx.x];
-    const bool inband = band && s_band[threadIdx.x >> 4];
-    if (inband) my = (threadIdx.x & 15) == 0 ? RC_BAND : RC_NONE;
-    if (bandrow && t0 + threadIdx.x < n) bandrow[t0 + threadIdx.x] = inband ? 1 : 0;
+    int my = i < TILE ? s_cls[i] : int(RC_NONE);
+    if (inband) my = (i & 15) == 0 ? RC_BAND : RC_NONE;
+    if (bandrow && i < TILE && t0 + i < n) bandrow[t0 + i] = inband ? 1 : 0;
     unsigned bal[RC_N];
 #pragma unroll
     for (int c = 0; c < RC_N; ++c) {
-      bal[c] = __ballot_sync(0xffffffffu, my == c);
-      if (lane == 0) s_cnt[warp][c] = __popc(bal[c]);
+      bal[c] = __ballot_sync(FULL, my == c);
+      if (lane == 0 && warp < NW) s_cnt[warp][c] = __popc(bal[c]);
     }
     __syncthreads();
-    if (threadIdx.x < RC_N) {
-      int c = threadIdx.x, tot = 0;
-      for (int w = 0; w < nw; ++w) tot += s_cnt[w][c];
-      s_base[c] = tot ? atomicAdd(&counters[c], tot) : 0;
+    if (i < RC_N) {
+      int tot = 0;
+      for (int w = 0; w < NW; ++w) tot += s_cnt[w][i];
+      s_base[i] = tot ? atomicAdd(&counters[i], tot) : 0;
+    } else if (i == 32) {
+      if (s_mult) atomicAdd(&mults[m0], s_mult);
+      if (s_band_work) atomicAdd(band_work, double(s_band_work));  // of the band tiles
     }
     __syncthreads();
     if (my < RC_N) {
       int off = s_base[my];
       for (int w = 0; w < warp; ++w) off += s_cnt[w][my];
       off += __popc(bal[my] & lt);
-      lists[int64_t(my) * n + off] = int32_t(t0 + threadIdx.x);
+      lists[int64_t(my) * n + off] = int32_t(t0 + i);
     }
     __syncthreads();
   }
@@ -1196,21 +1231,33 @@ int grid_cap(int64_t items, int per_block, int per_sm) {
 
 }  // namespace
 
-void launch_bounds(int64_t n, const Rows &A, const Rows &B, const int32_t *seg, const int *active,
+void launch_bounds(int64_t n, const Rows &A, int64_t nnzA, const Rows &B, const int32_t *seg,
+                   const int *active,
                    int mode, int groups, float group_margin, int band, float band_min_eff,
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
-                   cudaStream_t s) {
+                   const BandSpans &bspans, const BandSpans &cspans, cudaStream_t s) {
   if (n == 0) return;
-  k_row_info<<<grid_cap(n, 256, 8), 256, 0, s>>>(n, B.rs, B.re, B.col, binfo, ends);
+  k_row_info<<<grid_cap(n, 256, 8), 256, 0, s>>>(n, B.rs, B.re, B.col, binfo, ends, bspans);
   SGN_LAUNCH_CHECK();
-  int tiles = int((n + BOUNDS_TILE - 1) / BOUNDS_TILE);
-  int g = tiles < sm_count() * 8 ? tiles : sm_count() * 8;
-  k_bounds<<<g, BOUNDS_TILE, 0, s>>>(n, A.rs, A.re, A.col, binfo, seg, active, mode, groups,
-                                     group_margin, band, band_min_eff, dslot, moff, lo, len, ub,
-                                     lists, counters, mults, band_work, bandrow);
-  SGN_LAUNCH_CHECK();
+  auto run = [&](auto kern, int tile) {
+    kern<<<grid_cap(n, tile, 8), BOUNDS_T, 0, s>>>(n, A.rs, A.re, A.col, binfo, seg, active, mode,
+                                                   groups, group_margin, band, band_min_eff, dslot,
+                                                   moff, lo, len, ub, lists, counters, mults,
+                                                   band_work, bandrow, cspans);
+    SGN_LAUNCH_CHECK();
+  };
+  // Few rows: 16 lanes each, for the latency of a row. Rows of many entries,
+  // where a lane per row would not fill the chip: 8. Otherwise a lane per row,
+  // whose chain of loads before the first entry serves the most rows at once
+  // (the bounds of 24 products of a batch of 512 banded matrices: 3.5 ms, with 8 lanes 4.6)
+  if (n < 152 * 64)
+    run(k_bounds<16, 16>, 16);
+  else if (n < 152 * 8 * 256 && nnzA / n >= 16)
+    run(k_bounds<8, 64>, 64);
+  else
+    run(k_bounds<1, 256>, 256);
 }
 
 template <typename T, int MODE, int G, int LOOP = LOOP_ROW>

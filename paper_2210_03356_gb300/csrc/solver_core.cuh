@@ -454,7 +454,7 @@ struct Solver {
     w.wlist.ensure(sizeof(int32_t) * size_t(RC_N) * size_t(N), s);
     w.counters.ensure(ProductHead::bytes(nb), s);
     ProductHead *const head = head_dev();
-    w.scan_tmp.ensure(sizeof(int64_t) * size_t(scan_tmp_elems(N)), s);
+    w.scan_tmp.ensure(sizeof(int64_t) * SCAN_JOBS * size_t(scan_tmp_elems(N)), s);
     SGN_CUDA(cudaMemsetAsync(head, 0, ProductHead::bytes(nb), s));
     // band tiles (FP32): in SQUARE the bands of X (both operands) and of T
     // (the output, for the update) are laid out here, their sizes read with
@@ -465,14 +465,39 @@ struct Solver {
     int2 *ends = sizeof(T) == 8
                      ? static_cast<int2 *>(w.ends.ensure(sizeof(int2) * size_t(N > 0 ? N : 1), s))
                      : nullptr;
+    ScanJobs scans = {};
+    int jobs = 0;
+    auto layout = [&](BandBuf &b, int64_t *total) {  // its spans, to be filled in, and their scan
+      b.filled = false;
+      BandSpans bs;
+      bs.fc = static_cast<int32_t *>(b.fc.ensure(sizeof(int32_t) * size_t(N), s));
+      bs.nf = static_cast<int32_t *>(b.nf.ensure(sizeof(int32_t) * size_t(N), s));
+      bs.span = static_cast<int64_t *>(b.span.ensure(sizeof(int64_t) * size_t(N), s));
+      scans.cnt[jobs] = bs.span;
+      scans.out[jobs] = static_cast<int64_t *>(b.pos.ensure(sizeof(int64_t) * size_t(N + 1), s));
+      scans.total[jobs++] = total;
+      return bs;
+    };
+    C.n = N;
+    C.rs.ensure(sizeof(int64_t) * size_t(N + 1), s);
+    C.re.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
     {
       ProfScope ps(KC_BOUNDS, s);
-      if (band && mode == MODE_SQUARE) w.bandrow.ensure(size_t(N > 0 ? N : 1), s);
+      BandSpans bspans, cspans;
+      if (band && mode == MODE_SQUARE) {
+        w.bandrow.ensure(size_t(N > 0 ? N : 1), s);
+        w.bt_rows_done = false;
+        bspans = layout(w.bx, &head->tot[1]);
+        cspans = layout(w.bt, &head->tot[2]);
+      } else if (band && !b_is_square_t) {  // B is not the square's T: its own layout
+        w.bt_rows_done = false;
+        bspans = layout(w.bt, &head->tot[2]);
+      }
       // schedule: FP64 rows by lane use (or all on 32 lanes), FP32 rows in pairs (or one per warp)
       const int groups = few                ? 0
                          : sizeof(T) == 8 ? (o.group_margin < 0.0 ? 0 : 1)
                                           : (o.pair_rows ? 2 : 0);
-      launch_bounds(N, A, B, st.d_seg.template as<int32_t>(), active, mode, groups,
+      launch_bounds(N, A, nnzA, B, st.d_seg.template as<int32_t>(), active, mode, groups,
                     float(o.group_margin), band ? 1 : 0, float(o.band_min_eff),
                     dp && dp->any() ? w.dslot.as<int>() : nullptr,
                     st.d_moff.template as<int64_t>(), w.lo.as<int32_t>(),
@@ -480,47 +505,14 @@ struct Solver {
                     head->ctr, head->mults, &head->band_work,
                     band && mode == MODE_SQUARE ? w.bandrow.as<unsigned char>() : nullptr,
                     static_cast<int4 *>(w.binfo.ensure(sizeof(int4) * size_t(N > 0 ? N : 1), s)),
-                    ends, s);
-      if (band) {
-        if (mode == MODE_SQUARE) {
-          for (BandBuf *b : {&w.bx, &w.bt}) {
-            b->filled = false;
-            b->fc.ensure(sizeof(int32_t) * size_t(N), s);
-            b->nf.ensure(sizeof(int32_t) * size_t(N), s);
-            b->span.ensure(sizeof(int64_t) * size_t(N), s);
-            b->pos.ensure(sizeof(int64_t) * size_t(N + 1), s);
-          }
-          w.bt_rows_done = false;
-          launch_band_spans(N, B, w.bx.fc.as<int32_t>(), w.bx.nf.as<int32_t>(),
-                            w.bx.span.as<int64_t>(), s);
-          launch_scan(N, w.bx.span.as<int64_t>(), w.bx.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[1]);
-          launch_band_spans_range(N, w.lo.as<int32_t>(), w.len.as<int32_t>(),
-                                  w.bt.fc.as<int32_t>(), w.bt.nf.as<int32_t>(),
-                                  w.bt.span.as<int64_t>(), s);
-          launch_scan(N, w.bt.span.as<int64_t>(), w.bt.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[2]);
-        } else if (!b_is_square_t) {  // B is not the square's T: its own layout
-          w.bt.filled = false;
-          w.bt_rows_done = false;
-          w.bt.fc.ensure(sizeof(int32_t) * size_t(N), s);
-          w.bt.nf.ensure(sizeof(int32_t) * size_t(N), s);
-          w.bt.span.ensure(sizeof(int64_t) * size_t(N), s);
-          w.bt.pos.ensure(sizeof(int64_t) * size_t(N + 1), s);
-          launch_band_spans(N, B, w.bt.fc.as<int32_t>(), w.bt.nf.as<int32_t>(),
-                            w.bt.span.as<int64_t>(), s);
-          launch_scan(N, w.bt.span.as<int64_t>(), w.bt.pos.as<int64_t>(),
-                      w.scan_tmp.as<int64_t>(), s, nullptr, nullptr, &head->tot[2]);
-        }
-      }
+                    ends, bspans, cspans, s);
     }
-    C.n = N;
-    C.rs.ensure(sizeof(int64_t) * size_t(N + 1), s);
-    C.re.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
     {
       ProfScope ps(KC_SCAN, s);
-      launch_scan(N, w.ub.as<int64_t>(), C.rs.template as<int64_t>(), w.scan_tmp.as<int64_t>(), s,
-                  nullptr, nullptr, &head->tot[0]);
+      scans.cnt[jobs] = w.ub.as<int64_t>();
+      scans.out[jobs] = C.rs.template as<int64_t>();
+      scans.total[jobs++] = &head->tot[0];
+      launch_scans(N, jobs, scans, w.scan_tmp.as<int64_t>(), s);
     }
     fetch(hm.head, head, ProductHead::bytes(nb));
     const int *const ctr = hm.head->ctr;
