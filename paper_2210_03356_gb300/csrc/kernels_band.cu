@@ -84,6 +84,7 @@ __global__ void k_band_fill(int64_t n, const int64_t *rs, const int64_t *re, con
                             const float *val, const int64_t *pos, const int32_t *fc,
                             const int32_t *nf, const unsigned char *skip, float *bval,
                             unsigned *bmask) {
+  after_previous();
   // FILL_LPR lanes per row, 32 / FILL_LPR rows per warp at a time
   constexpr int L = FILL_LPR;
   const int lane = threadIdx.x & 31, g = lane / L, gl = lane % L;
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(BT_WARPS * 32, BT_CTAS)
            Band A, Band B, BandOut Cb, const int32_t *lo, const int32_t *len,
            const int32_t *list, int *counters, int cls, const int64_t *cs, int64_t *ce,
            int32_t *ccol, float *cval, double *part) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char band_smem[];
   BandSmem &sm = reinterpret_cast<BandSmem *>(band_smem)[threadIdx.x >> 5];
   constexpr unsigned FULL = 0xffffffffu;
@@ -476,9 +478,8 @@ void launch_band_fill(int64_t n, const Rows &R, const float *val, const int64_t 
   if (n == 0) return;
   int64_t g = (n + 8 * (32 / FILL_LPR) - 1) / (8 * (32 / FILL_LPR));  // 8 warps per CTA
   if (g > int64_t(sm_count_band()) * 16) g = int64_t(sm_count_band()) * 16;
-  k_band_fill<<<unsigned(g), 256, 0, s>>>(n, R.rs, R.re, R.col, val, pos, fc, nf, skip, bval,
-                                          bmask);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_band_fill, unsigned(g), 256, 0, s, n, R.rs, R.re, R.col, val, pos, fc, nf, skip,
+              bval, bmask);
 }
 
 void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, const Band &bandA,
@@ -499,14 +500,11 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
   (void)attr;
   const int g = sm_count_band() * BT_CTAS;
   if (mode == MODE_SQUARE)
-    k_band<MODE_SQUARE><<<g, BT_WARPS * 32, smem, s>>>(A.rs, A.re, A.col, aval, bandA, bandB,
-                                                       bandC, lo, len, list, counters, RC_BAND, cs,
-                                                       ce, ccol, cval, part);
+    launch_next(k_band<MODE_SQUARE>, g, BT_WARPS * 32, smem, s, A.rs, A.re, A.col, aval, bandA,
+                bandB, bandC, lo, len, list, counters, RC_BAND, cs, ce, ccol, cval, part);
   else
-    k_band<MODE_UPDATE><<<g, BT_WARPS * 32, smem, s>>>(A.rs, A.re, A.col, aval, bandA, bandB,
-                                                       BandOut{}, lo, len, list, counters, RC_BAND,
-                                                       cs, ce, ccol, cval, part);
-  SGN_LAUNCH_CHECK();
+    launch_next(k_band<MODE_UPDATE>, g, BT_WARPS * 32, smem, s, A.rs, A.re, A.col, aval, bandA,
+                bandB, BandOut{}, lo, len, list, counters, RC_BAND, cs, ce, ccol, cval, part);
 }
 
 }  // namespace sgn

@@ -48,6 +48,7 @@ int grid_for(int64_t items, int per_block, int cap = 152 * 16) {
 // ------------------------------------------------------------ validation
 __global__ void k_validate(int64_t n, int64_t nnz, const int64_t *rp, const int32_t *col,
                            const double *val, int *flag) {
+  after_previous();
   int lane = lane_id();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (rp[0] != 0 || rp[n] != nnz) atomicOr(flag, 1);
@@ -75,6 +76,7 @@ __global__ void k_validate(int64_t n, int64_t nnz, const int64_t *rp, const int3
 // row pointer.
 __global__ void k_validate_batch(int count, const ValidateJob *jobs, const int64_t *row_off,
                                  int *flags) {
+  after_previous();
   const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (tid < count) {
     const ValidateJob &j = jobs[tid];
@@ -185,6 +187,7 @@ constexpr int PUB_T = 1024;
 __global__ void __launch_bounds__(PUB_T)
     k_publish(const unsigned long long *src, unsigned long long *dst, int64_t words,
               volatile unsigned *flag, unsigned seq) {
+  after_previous();
   for (int64_t i = threadIdx.x; i < words; i += PUB_T) dst[i] = src[i];
   __threadfence_system();
   __syncthreads();
@@ -196,6 +199,7 @@ __global__ void __launch_bounds__(PUB_T)
 // into the matrix-wide Gershgorin gap, row-sum bound and half-bandwidth.
 __global__ void k_gersh(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
                         GershStats *g) {
+  after_previous();
   int lane = lane_id();
   for_each_row_warp(n, [&](int64_t r) {
     double diag = 0.0, off = 0.0;
@@ -263,6 +267,7 @@ __device__ int64_t block_excl_scan(int64_t v, int64_t *sm, int64_t *total) {
 // blockIdx.y: the scan, its tile totals at tmp + blockIdx.y * tmp_stride.
 __global__ void __launch_bounds__(SCAN_T)
     k_scan_reduce(int64_t n, ScanJobs J, int64_t *tmp, int64_t tmp_stride) {
+  after_previous();
   __shared__ int64_t sm[33];
   const int64_t *cnt = blockIdx.y == 0 ? J.cnt[0] : blockIdx.y == 1 ? J.cnt[1] : J.cnt[2];
   int64_t base = int64_t(blockIdx.x) * SCAN_TILE + int64_t(threadIdx.x) * SCAN_ITEMS;
@@ -281,6 +286,7 @@ __global__ void __launch_bounds__(SCAN_T)
 __global__ void __launch_bounds__(SCAN_T)
     k_scan_final(int64_t n, ScanJobs J, const int64_t *tmp, int64_t tmp_stride,
                  const int32_t *seg, int64_t *eoff) {
+  after_previous();
   __shared__ int64_t sm[33];
   const int y = blockIdx.y;  // picked by comparison: an indexed parameter is copied to local memory
   static_assert(SCAN_JOBS == 3, "three to pick from");
@@ -333,6 +339,7 @@ __device__ __forceinline__ int find_block(const int64_t *off, int nb, int64_t r)
 
 __global__ void k_asm_lens(int nblocks, const AsmBlock *blocks, const int64_t *boff, int64_t n,
                            int64_t *lens) {
+  after_previous();
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     int b = find_block(boff, nblocks, r);
@@ -344,6 +351,7 @@ __global__ void k_asm_lens(int nblocks, const AsmBlock *blocks, const int64_t *b
 
 __global__ void k_asm_vals(int nblocks, const AsmBlock *blocks, const int64_t *boff, int64_t n,
                            const int64_t *drp, int32_t *dcol, void *dval, int dst_f32) {
+  after_previous();
   // 8 lanes per row, four rows per warp at a time (rows are short)
   constexpr int L = 8;
   const int lane = lane_id(), gl = lane % L;
@@ -376,6 +384,7 @@ __global__ void k_asm_vals(int nblocks, const AsmBlock *blocks, const int64_t *b
 }
 
 __global__ void k_fill_seg(int nb, const int64_t *moff, int64_t n, int32_t *seg) {
+  after_previous();
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x)
     seg[r] = find_block(moff, nb, r);
@@ -415,6 +424,7 @@ __device__ __forceinline__ void add128(unsigned long long *lohi, unsigned long l
 
 __global__ void k_absmax(int64_t n, const int32_t *seg, const int64_t *rp, const double *val,
                          unsigned long long *mmax) {
+  after_previous();
   for_each_row_group8(n, [&](int64_t r, bool has, int gl) {
     double m = 0.0;
     if (has)
@@ -429,6 +439,7 @@ __global__ void k_absmax(int64_t n, const int32_t *seg, const int64_t *rp, const
 __global__ void k_colsum(int64_t n, const int32_t *seg, const int64_t *rp, const int32_t *col,
                          const double *val, const unsigned long long *mmax,
                          unsigned long long *colsum) {
+  after_previous();
   for_each_row_group8(n, [&](int64_t r, bool has, int gl) {
     if (!has) return;
     double M = __longlong_as_double((long long)mmax[seg[r]]);
@@ -445,6 +456,7 @@ __global__ void k_colsum(int64_t n, const int32_t *seg, const int64_t *rp, const
 // A whole warp stays in the loop (max_into); its lanes past the end add nothing.
 __global__ void k_colmax_hi(int64_t n, const int32_t *seg, const unsigned long long *colsum,
                             unsigned long long *maxhi) {
+  after_previous();
   for (int64_t j0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane_id(); j0 < n;
        j0 += int64_t(gridDim.x) * blockDim.x) {
     const int64_t j = j0 + lane_id() < n ? j0 + lane_id() : n - 1;
@@ -454,6 +466,7 @@ __global__ void k_colmax_hi(int64_t n, const int32_t *seg, const unsigned long l
 
 __global__ void k_colmax_lo(int64_t n, const int32_t *seg, const unsigned long long *colsum,
                             const unsigned long long *maxhi, unsigned long long *maxlo) {
+  after_previous();
   for (int64_t j0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane_id(); j0 < n;
        j0 += int64_t(gridDim.x) * blockDim.x) {
     const int64_t j = j0 + lane_id() < n ? j0 + lane_id() : n - 1;
@@ -465,6 +478,7 @@ __global__ void k_colmax_lo(int64_t n, const int32_t *seg, const unsigned long l
 __global__ void k_norm_final(int nb, const unsigned long long *mmax,
                              const unsigned long long *maxhi, const unsigned long long *maxlo,
                              double *norm) {
+  after_previous();
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= nb) return;
   double M = __longlong_as_double((long long)mmax[m]);
@@ -481,6 +495,7 @@ __global__ void k_norm_final(int nb, const unsigned long long *mmax,
 
 __global__ void k_scale(int64_t n, const int32_t *seg, const int64_t *rp, double *val,
                         const double *norm) {
+  after_previous();
   for_each_row_group8(n, [&](int64_t r, bool has, int gl) {
     if (!has) return;
     double s = norm[seg[r]];
@@ -489,6 +504,7 @@ __global__ void k_scale(int64_t n, const int32_t *seg, const int64_t *rp, double
 }
 
 __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64_t *out) {
+  after_previous();
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m <= nb) out[m] = rp[moff[m]];
 }
@@ -504,6 +520,7 @@ __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp,
 // out[m] = the sum of part over matrix m's rows.
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
     k_seg_reduce(const int64_t *moff, const double *part, double *out) {
+  after_previous();
   __shared__ double sm[RED_T];
   cg::cluster_group cl = cg::this_cluster();
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
@@ -523,6 +540,7 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(3 * RED_LANES)
     k_check_scalars(const int64_t *moff, const double *part, const int64_t *rs, const int64_t *re,
                     double c4, double tol_stage, double switch_resid, MatScalars *ms,
                     int64_t *nnz) {
+  after_previous();
   __shared__ double sm[2][RED_T];
   __shared__ unsigned long long s_cnt;
   cg::cluster_group cl = cg::this_cluster();
@@ -560,6 +578,7 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(3 * RED_LANES)
 
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
     k_seg_count(const int64_t *moff, const int64_t *rs, const int64_t *re, int64_t *out) {
+  after_previous();
   __shared__ unsigned long long sm;  // CTA 0: the matrix's count
   cg::cluster_group cl = cg::this_cluster();
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
@@ -577,6 +596,7 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
 // blockIdx.y walks the blocks; the gridDim.x CTAs of a block share its rows
 // and entries, so that a large matrix is copied by many SMs.
 __global__ void k_extract(int nblocks, const ExtractBlock *blocks) {
+  after_previous();
   for (int b = blockIdx.y; b < nblocks; b += gridDim.y) {
     const ExtractBlock B = blocks[b];
     const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -593,6 +613,7 @@ __global__ void k_extract(int nblocks, const ExtractBlock *blocks) {
 }
 
 __global__ void k_row_lengths(int64_t n, const int64_t *rs, const int64_t *re, int64_t *out) {
+  after_previous();
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x)
     out[r] = re[r] - rs[r];
@@ -601,6 +622,7 @@ __global__ void k_row_lengths(int64_t n, const int64_t *rs, const int64_t *re, i
 __global__ void k_compact_rows(int64_t n, const int64_t *rs, const int64_t *re,
                                const int32_t *col, const void *val, int vsize, const int64_t *orp,
                                int32_t *ocol, void *oval) {
+  after_previous();
   int lane = lane_id();
   for_each_row_warp(n, [&](int64_t r) {
     int64_t b = rs[r], e = re[r], d = orp[r];
@@ -619,23 +641,21 @@ __global__ void k_compact_rows(int64_t n, const int64_t *rs, const int64_t *re,
 void launch_row_lengths(int64_t n, const int64_t *rs, const int64_t *re, int64_t *out,
                         cudaStream_t s) {
   if (n == 0) return;
-  k_row_lengths<<<grid_for(n, 256), 256, 0, s>>>(n, rs, re, out);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_row_lengths, grid_for(n, 256), 256, 0, s, n, rs, re, out);
 }
 
 void launch_compact_rows(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
                          const void *val, int vsize, const int64_t *orp, int32_t *ocol,
                          void *oval, cudaStream_t s) {
   if (n == 0) return;
-  k_compact_rows<<<grid_for(n, 8), 256, 0, s>>>(n, rs, re, col, val, vsize, orp, ocol, oval);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_compact_rows, grid_for(n, 8), 256, 0, s, n, rs, re, col, val, vsize, orp, ocol,
+              oval);
 }
 
 void launch_seg_count(int nb, const int64_t *moff, const int64_t *rs, const int64_t *re,
                       int64_t *out, cudaStream_t s) {
   if (nb == 0) return;
-  k_seg_count<<<unsigned(nb) * RED_C, RED_T, 0, s>>>(moff, rs, re, out);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_seg_count, unsigned(nb) * RED_C, RED_T, 0, s, moff, rs, re, out);
 }
 
 void launch_extract(int nblocks, const ExtractBlock *blocks, int64_t max_entries, cudaStream_t s) {
@@ -643,28 +663,24 @@ void launch_extract(int nblocks, const ExtractBlock *blocks, int64_t max_entries
   // about 8 entries per thread of a 512-thread CTA, at most 152 CTAs per block
   const int64_t per = (max_entries + 4095) / 4096;
   dim3 grid(unsigned(per < 1 ? 1 : (per > 152 ? 152 : per)), unsigned(nblocks < 65535 ? nblocks : 65535));
-  k_extract<<<grid, 512, 0, s>>>(nblocks, blocks);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_extract, grid, 512, 0, s, nblocks, blocks);
 }
 
 void launch_gersh(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
                   GershStats *g, cudaStream_t s) {
-  k_gersh<<<grid_for(n, 8), 256, 0, s>>>(n, rp, col, val, g);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_gersh, grid_for(n, 8), 256, 0, s, n, rp, col, val, g);
 }
 
 void launch_validate(int64_t n, int64_t nnz, const int64_t *rp, const int32_t *col,
                      const double *val, int *flag, cudaStream_t s) {
-  k_validate<<<grid_for(n, 8), 256, 0, s>>>(n, nnz, rp, col, val, flag);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_validate, grid_for(n, 8), 256, 0, s, n, nnz, rp, col, val, flag);
 }
 
 void launch_validate_batch(int count, const ValidateJob *jobs, const int64_t *row_off,
                            int64_t total_rows, int *flags, cudaStream_t s) {
   if (count < 1) return;
   const int64_t items = total_rows > count ? total_rows : count;
-  k_validate_batch<<<grid_for(items, 32), 256, 0, s>>>(count, jobs, row_off, flags);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_validate_batch, grid_for(items, 32), 256, 0, s, count, jobs, row_off, flags);
 }
 
 void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s) {
@@ -675,10 +691,8 @@ void launch_copy_chunks(int count, const CopyChunk *chunks, cudaStream_t s) {
 
 void launch_publish(const void *src, void *dst, size_t bytes, unsigned *flag, unsigned seq,
                     cudaStream_t s) {
-  k_publish<<<1, PUB_T, 0, s>>>(static_cast<const unsigned long long *>(src),
-                                static_cast<unsigned long long *>(dst), int64_t(bytes / 8), flag,
-                                seq);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_publish, 1, PUB_T, 0, s, static_cast<const unsigned long long *>(src),
+              static_cast<unsigned long long *>(dst), int64_t(bytes / 8), flag, seq);
 }
 
 int64_t scan_tmp_elems(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
@@ -697,11 +711,9 @@ static void run_scans(int64_t n, int jobs, const ScanJobs &J, int64_t *tmp, cons
   const dim3 grid{unsigned(nblocks), unsigned(jobs)};
   const int64_t stride = scan_tmp_elems(n);
   if (nblocks > 1) {
-    k_scan_reduce<<<grid, SCAN_T, 0, s>>>(n, J, tmp, stride);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_scan_reduce, grid, SCAN_T, 0, s, n, J, tmp, stride);
   }
-  k_scan_final<<<grid, SCAN_T, 0, s>>>(n, J, tmp, stride, seg, eoff);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_scan_final, grid, SCAN_T, 0, s, n, J, tmp, stride, seg, eoff);
 }
 
 void launch_scans(int64_t n, int jobs, const ScanJobs &J, int64_t *tmp, cudaStream_t s) {
@@ -720,8 +732,7 @@ void launch_scan(int64_t n, const int64_t *cnt, int64_t *out, int64_t *tmp, cuda
 void launch_assemble_rows(int nblocks, const AsmBlock *blocks, const int64_t *boff, int64_t n_dst,
                           int64_t *lens, int64_t *dst_rp, int64_t *scan_tmp, cudaStream_t s) {
   if (n_dst > 0) {
-    k_asm_lens<<<grid_for(n_dst, 256), 256, 0, s>>>(nblocks, blocks, boff, n_dst, lens);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_asm_lens, grid_for(n_dst, 256), 256, 0, s, nblocks, blocks, boff, n_dst, lens);
   }
   launch_scan(n_dst, lens, dst_rp, scan_tmp, s);
 }
@@ -730,15 +741,13 @@ void launch_assemble_vals(int nblocks, const AsmBlock *blocks, const int64_t *bo
                           const int64_t *dst_rp, int32_t *dst_col, void *dst_val, int dst_f32,
                           cudaStream_t s) {
   if (n_dst == 0) return;
-  k_asm_vals<<<grid_for(n_dst, 32), 256, 0, s>>>(nblocks, blocks, boff, n_dst, dst_rp, dst_col,
-                                                  dst_val, dst_f32);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_asm_vals, grid_for(n_dst, 32), 256, 0, s, nblocks, blocks, boff, n_dst, dst_rp,
+              dst_col, dst_val, dst_f32);
 }
 
 void launch_fill_seg(int nb, const int64_t *moff, int64_t n, int32_t *seg, cudaStream_t s) {
   if (n == 0) return;
-  k_fill_seg<<<grid_for(n, 256), 256, 0, s>>>(nb, moff, n, seg);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_fill_seg, grid_for(n, 256), 256, 0, s, nb, moff, n, seg);
 }
 
 void launch_onenorm(int nb, const int64_t *moff, const int32_t *seg, int64_t n, const int64_t *rp,
@@ -750,44 +759,35 @@ void launch_onenorm(int nb, const int64_t *moff, const int32_t *seg, int64_t n, 
   unsigned long long *maxhi = mmax + nb;        // nb
   unsigned long long *maxlo = maxhi + nb;       // nb
   SGN_CUDA(cudaMemsetAsync(work, 0, sizeof(unsigned long long) * size_t(2 * n + 3 * nb), s));
-  k_absmax<<<grid_for(n, 32), 256, 0, s>>>(n, seg, rp, val, mmax);
-  SGN_LAUNCH_CHECK();
-  k_colsum<<<grid_for(n, 32), 256, 0, s>>>(n, seg, rp, col, val, mmax, colsum);
-  SGN_LAUNCH_CHECK();
-  k_colmax_hi<<<grid_for(n, 256), 256, 0, s>>>(n, seg, colsum, maxhi);
-  SGN_LAUNCH_CHECK();
-  k_colmax_lo<<<grid_for(n, 256), 256, 0, s>>>(n, seg, colsum, maxhi, maxlo);
-  SGN_LAUNCH_CHECK();
-  k_norm_final<<<(nb + 127) / 128, 128, 0, s>>>(nb, mmax, maxhi, maxlo, norm);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_absmax, grid_for(n, 32), 256, 0, s, n, seg, rp, val, mmax);
+  launch_next(k_colsum, grid_for(n, 32), 256, 0, s, n, seg, rp, col, val, mmax, colsum);
+  launch_next(k_colmax_hi, grid_for(n, 256), 256, 0, s, n, seg, colsum, maxhi);
+  launch_next(k_colmax_lo, grid_for(n, 256), 256, 0, s, n, seg, colsum, maxhi, maxlo);
+  launch_next(k_norm_final, (nb + 127) / 128, 128, 0, s, nb, mmax, maxhi, maxlo, norm);
 }
 
 void launch_scale(int64_t n, const int32_t *seg, const int64_t *rp, double *val,
                   const double *norm, cudaStream_t s) {
-  k_scale<<<grid_for(n, 32), 256, 0, s>>>(n, seg, rp, val, norm);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_scale, grid_for(n, 32), 256, 0, s, n, seg, rp, val, norm);
 }
 
 void launch_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64_t *out,
                            cudaStream_t s) {
-  k_gather_offsets<<<(nb + 1 + 127) / 128, 128, 0, s>>>(nb, moff, rp, out);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_gather_offsets, (nb + 1 + 127) / 128, 128, 0, s, nb, moff, rp, out);
 }
 
 void launch_seg_reduce(int nb, const int64_t *moff, const double *part, double *out,
                        cudaStream_t s) {
   if (nb == 0) return;
-  k_seg_reduce<<<unsigned(nb) * RED_C, RED_LANES, 0, s>>>(moff, part, out);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_seg_reduce, unsigned(nb) * RED_C, RED_LANES, 0, s, moff, part, out);
 }
 
 void launch_check_scalars(int nb, const int64_t *moff, const double *part, const int64_t *rs,
                           const int64_t *re, double c4, double tol_stage, double switch_resid,
                           MatScalars *ms, int64_t *nnz, cudaStream_t s) {
   if (nb == 0) return;
-  k_check_scalars<<<unsigned(nb) * RED_C, 3 * RED_LANES, 0, s>>>(moff, part, rs, re, c4, tol_stage,
-                                                                switch_resid, ms, nnz);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_check_scalars, unsigned(nb) * RED_C, 3 * RED_LANES, 0, s, moff, part, rs, re, c4,
+              tol_stage, switch_resid, ms, nnz);
 }
 
 }  // namespace sgn

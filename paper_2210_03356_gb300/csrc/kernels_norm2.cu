@@ -39,6 +39,7 @@ __device__ __forceinline__ int exp_of(unsigned long long bits) {
 
 __global__ void k_n2_init(int64_t n, const int32_t *seg, const int64_t *moff, const MatScalars *ms,
                           double sw, double *v) {
+  after_previous();
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     const int m = seg[r];
@@ -50,6 +51,7 @@ __global__ void k_n2_init(int64_t n, const int32_t *seg, const int64_t *moff, co
 __global__ void k_n2_absmax(int64_t n, const int32_t *seg, const int64_t *rs, const int64_t *re,
                             const void *val, int f32, const MatScalars *ms, double sw,
                             unsigned long long *xmax) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -68,6 +70,7 @@ __global__ void k_n2_spmv(int64_t n, const int32_t *seg, const int64_t *rs, cons
                           const int32_t *col, const void *val, int f32, const MatScalars *ms,
                           double sw, const double *v, double *y, unsigned long long *ymax,
                           double *part) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -90,6 +93,7 @@ __global__ void k_n2_spmv_t(int64_t n, const int32_t *seg, const int64_t *rs, co
                             const int32_t *col, const void *val, int f32, const MatScalars *ms,
                             double sw, const double *y, const unsigned long long *xmax,
                             const unsigned long long *ymax, unsigned long long *zacc) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -119,6 +123,7 @@ __global__ void k_n2_spmv_t(int64_t n, const int32_t *seg, const int64_t *rs, co
 __global__ void k_n2_zfinal(int64_t n, const int32_t *seg, const MatScalars *ms, double sw,
                             const unsigned long long *xmax, const unsigned long long *ymax,
                             unsigned long long *zacc, double *z, double *part) {
+  after_previous();
   for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
        j += int64_t(gridDim.x) * blockDim.x) {
     const int m = seg[j];
@@ -143,6 +148,7 @@ __global__ void k_n2_zfinal(int64_t n, const int32_t *seg, const MatScalars *ms,
 // every later step gives the same ||X v||)
 __global__ void k_n2_scale(int64_t n, const int32_t *seg, const MatScalars *ms, double sw,
                            const double *z, const double *nz2, double *v) {
+  after_previous();
   for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < n;
        j += int64_t(gridDim.x) * blockDim.x) {
     if (!wanted(ms, seg[j], sw)) continue;
@@ -152,6 +158,7 @@ __global__ void k_n2_scale(int64_t n, const int32_t *seg, const MatScalars *ms, 
 }
 
 __global__ void k_n2_final(int nb, const double *ny2, double *x2) {
+  after_previous();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m < nb) x2[m] = __dsqrt_rn(ny2[m]);
 }
@@ -159,6 +166,7 @@ __global__ void k_n2_final(int nb, const double *ny2, double *x2) {
 // Eq. (1.18) with x = x2 for the matrices in the adaptive phase
 __global__ void k_budget_x2(int nb, const int64_t *moff, const double *x2, double switch_resid,
                             MatScalars *ms) {
+  after_previous();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= nb) return;
   const double r = ms[m].r;
@@ -190,35 +198,28 @@ void launch_norm2_est(int nb, const int64_t *moff, const int32_t *seg, int64_t n
   const double sw = switch_resid;
   SGN_CUDA(cudaMemsetAsync(wk.xmax, 0, sizeof(unsigned long long) * size_t(nb), s));
   SGN_CUDA(cudaMemsetAsync(wk.zacc, 0, sizeof(unsigned long long) * 2 * size_t(n), s));
-  k_n2_init<<<gr, 256, 0, s>>>(n, seg, moff, ms, sw, wk.v);
-  SGN_LAUNCH_CHECK();
-  k_n2_absmax<<<gw, 256, 0, s>>>(n, seg, X.rs, X.re, val, val_f32, ms, sw, wk.xmax);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_n2_init, gr, 256, 0, s, n, seg, moff, ms, sw, wk.v);
+  launch_next(k_n2_absmax, gw, 256, 0, s, n, seg, X.rs, X.re, val, val_f32, ms, sw, wk.xmax);
   for (int step = 0; step <= NORM2_STEPS; ++step) {
     SGN_CUDA(cudaMemsetAsync(wk.ymax, 0, sizeof(unsigned long long) * size_t(nb), s));
-    k_n2_spmv<<<gw, 256, 0, s>>>(n, seg, X.rs, X.re, X.col, val, val_f32, ms, sw, wk.v, wk.y,
-                                 wk.ymax, wk.part);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_n2_spmv, gw, 256, 0, s, n, seg, X.rs, X.re, X.col, val, val_f32, ms, sw, wk.v,
+                wk.y, wk.ymax, wk.part);
     if (step == NORM2_STEPS) break;
-    k_n2_spmv_t<<<gw, 256, 0, s>>>(n, seg, X.rs, X.re, X.col, val, val_f32, ms, sw, wk.y,
-                                   wk.xmax, wk.ymax, wk.zacc);
-    SGN_LAUNCH_CHECK();
-    k_n2_zfinal<<<gr, 256, 0, s>>>(n, seg, ms, sw, wk.xmax, wk.ymax, wk.zacc, wk.z, wk.part);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_n2_spmv_t, gw, 256, 0, s, n, seg, X.rs, X.re, X.col, val, val_f32, ms, sw, wk.y,
+                wk.xmax, wk.ymax, wk.zacc);
+    launch_next(k_n2_zfinal, gr, 256, 0, s, n, seg, ms, sw, wk.xmax, wk.ymax, wk.zacc, wk.z,
+                wk.part);
     launch_seg_reduce(nb, moff, wk.part, wk.nrm, s);
-    k_n2_scale<<<gr, 256, 0, s>>>(n, seg, ms, sw, wk.z, wk.nrm, wk.v);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_n2_scale, gr, 256, 0, s, n, seg, ms, sw, wk.z, wk.nrm, wk.v);
   }
   launch_seg_reduce(nb, moff, wk.part, wk.nrm, s);
-  k_n2_final<<<(nb + 127) / 128, 128, 0, s>>>(nb, wk.nrm, x2);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_n2_final, (nb + 127) / 128, 128, 0, s, nb, wk.nrm, x2);
 }
 
 void launch_budget_x2(int nb, const int64_t *moff, const double *x2, double switch_resid,
                       MatScalars *ms, cudaStream_t s) {
   if (nb == 0) return;
-  k_budget_x2<<<(nb + 127) / 128, 128, 0, s>>>(nb, moff, x2, switch_resid, ms);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_budget_x2, (nb + 127) / 128, 128, 0, s, nb, moff, x2, switch_resid, ms);
 }
 
 }  // namespace sgn

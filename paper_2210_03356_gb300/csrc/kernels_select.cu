@@ -40,6 +40,7 @@ constexpr int NDIG = 256;         // digit buckets
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 __global__ void k_select_bound(int nb, const int *active, MatScalars *ms) {
+  after_previous();
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= nb || !active[m]) return;
   int64_t c = ms[m].nnz_bar;
@@ -257,6 +258,7 @@ __device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, 
 // Clears the matrix's histogram, minimum and candidate count.
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
     k_sel_prepare(SelRows R, MatScalars *ms, SelScratch sc) {
+  after_previous();
   __shared__ unsigned long long s_cnt;  // CTA 0: the matrix's entries
   cg::cluster_group cl = cg::this_cluster();
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
@@ -371,6 +373,7 @@ template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS)
     k_sel_hist0(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
                 SelScratch sc) {
+  after_previous();
   using K = typename KeyT<T>::K;
   __shared__ uint32_t s_h[3][NB0];
   __shared__ unsigned long long s_min, s_below[2];
@@ -518,6 +521,7 @@ __device__ __forceinline__ int warp_crossing(const unsigned long long *h, int nb
 // One warp per matrix: the level-0 bucket where the exact sums cross Q (never
 // the sum below the pivot, bucket 0).
 __global__ void k_sel_find0(int nb, const int *active, const MatScalars *ms, SelScratch sc) {
+  after_previous();
   const int m = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (m >= nb) return;
@@ -585,6 +589,7 @@ template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS)
     k_sel_extract(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
                   SelScratch sc, int64_t *cnt, double *dropped) {
+  after_previous();
   using K = typename KeyT<T>::K;
   __shared__ ChunkRows cr;
   __shared__ K s_lo[RPC], s_up[RPC];
@@ -692,6 +697,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
     k_drop_sums(const int64_t *moff, const double *dropped, const int *active, int exact,
                 SelScratch sc, const MatScalars *ms, double *sums) {
+  after_previous();
   __shared__ double sm[RED_T];
   cg::cluster_group cl = cg::this_cluster();
   const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
@@ -729,6 +735,7 @@ static_assert(DG_T <= 2 * NDIG && DG_T <= DG_KEEP && DG_T <= DG_ONE, "the short 
 template <int LEVELS>
 __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
     k_sel_digits(SelRows R, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
+  after_previous();
   __shared__ uint32_t h[3][NDIG];
   __shared__ unsigned long long sum[NDIG * 2];
   __shared__ unsigned long long keep[DG_KEEP];
@@ -867,6 +874,7 @@ __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
 __global__ void k_filter_count(int64_t n, const int32_t *seg, const int *active,
                                const int64_t *rs, const int64_t *re, const void *val, int f32,
                                const MatScalars *ms, int64_t *cnt, double *dropped) {
+  after_previous();
   int lane = lane_id();
   int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -927,6 +935,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
     k_filter_write(int64_t n, int rpc, const int32_t *seg, const int *active, const int64_t *rs,
                    const int64_t *re, const int32_t *col, const T *val, const MatScalars *ms,
                    const int64_t *orp, int32_t *ocol, T *oval) {
+  after_previous();
   using K = typename KeyT<T>::K;
   __shared__ ChunkRows cr;
   __shared__ int64_t s_out[RPC], s_oend[RPC];
@@ -997,6 +1006,7 @@ int grid_for(int64_t items, int per_block, int cap = 152 * 16) {
 }
 
 __global__ void k_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms) {
+  after_previous();
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m < nb) ms[m].nnz_bar = nnz[m];
 }
@@ -1004,13 +1014,11 @@ __global__ void k_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms) {
 }  // namespace
 
 void launch_store_nnz_bar(int nb, const int64_t *nnz, MatScalars *ms, cudaStream_t s) {
-  k_store_nnz_bar<<<(nb + 127) / 128, 128, 0, s>>>(nb, nnz, ms);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_store_nnz_bar, (nb + 127) / 128, 128, 0, s, nb, nnz, ms);
 }
 
 void launch_select_bound(int nb, const int *active, MatScalars *ms, cudaStream_t s) {
-  k_select_bound<<<(nb + 127) / 128, 128, 0, s>>>(nb, active, ms);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_select_bound, (nb + 127) / 128, 128, 0, s, nb, active, ms);
 }
 
 const unsigned long long *select_overflow(void *scratch, int nb) {
@@ -1035,26 +1043,22 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *act
                          cudaStream_t s) {
   {
     ProfScope ps(KC_SEL_HIST, s, 0.0, 0.0);
-    k_sel_prepare<<<unsigned(nb) * RED_C, RED_T, 0, s>>>(R, ms, sc);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_sel_prepare, unsigned(nb) * RED_C, RED_T, 0, s, R, ms, sc);
     sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
-      k_sel_hist0<T, lpr.value><<<g, SEL_THREADS, 0, s>>>(R, rpc, active, val, ms, sc);
-      SGN_LAUNCH_CHECK();
+      launch_next(k_sel_hist0<T, lpr.value>, g, SEL_THREADS, 0, s, R, rpc, active, val, ms, sc);
     });
-    k_sel_find0<<<(nb + 3) / 4, 128, 0, s>>>(nb, active, ms, sc);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_sel_find0, (nb + 3) / 4, 128, 0, s, nb, active, ms, sc);
   }
   {
     ProfScope ps(KC_SEL_EXTRACT, s, 0.0, 0.0);
     sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
-      k_sel_extract<T, lpr.value><<<g, SEL_THREADS, 0, s>>>(R, rpc, active, val, ms, sc, cnt,
-                                                           dropped);
-      SGN_LAUNCH_CHECK();
+      launch_next(k_sel_extract<T, lpr.value>, g, SEL_THREADS, 0, s, R, rpc, active, val, ms, sc,
+                  cnt, dropped);
     });
   }
   ProfScope ps(KC_SEL_DIGITS, s, 0.0, 0.0);
-  k_sel_digits<sizeof(T) == 4 ? 3 : 6><<<unsigned(nb) * DG_C, DG_T, 0, s>>>(R, active, sc, ms, cnt);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_sel_digits<sizeof(T) == 4 ? 3 : 6>, unsigned(nb) * DG_C, DG_T, 0, s, R, active, sc,
+              ms, cnt);
 }
 
 void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
@@ -1073,18 +1077,16 @@ void launch_drop_sums(int nb, const int64_t *moff, const double *dropped, const 
                       void *scratch, const MatScalars *ms, double *sums, cudaStream_t s) {
   if (nb == 0) return;
   const SelScratch sc = scratch ? carve(scratch, nb, 1) : SelScratch{};
-  k_drop_sums<<<unsigned(nb) * RED_C, RED_LANES, 0, s>>>(moff, dropped, active, scratch ? 1 : 0, sc,
-                                                        ms, sums);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_drop_sums, unsigned(nb) * RED_C, RED_LANES, 0, s, moff, dropped, active,
+              scratch ? 1 : 0, sc, ms, sums);
 }
 
 void launch_filter_count(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,
                          const int64_t *re, const void *val, int val_f32, const MatScalars *ms,
                          int64_t *cnt, double *dropped, cudaStream_t s) {
   if (n == 0) return;
-  k_filter_count<<<grid_for(n, 8), 256, 0, s>>>(n, seg, active, rs, re, val, val_f32, ms, cnt,
-                                                 dropped);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_filter_count, grid_for(n, 8), 256, 0, s, n, seg, active, rs, re, val, val_f32, ms,
+              cnt, dropped);
 }
 
 void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int *active,
@@ -1093,14 +1095,13 @@ void launch_filter_write(int64_t n, int64_t nvals, const int32_t *seg, const int
                          void *oval, cudaStream_t s) {
   sel_pass(n, nvals, [&](auto lpr, int rpc, int g) {
     if (val_f32)
-      k_filter_write<float, lpr.value><<<g, SEL_THREADS, 0, s>>>(
-          n, rpc, seg, active, rs, re, col, static_cast<const float *>(val), ms, orp, ocol,
-          static_cast<float *>(oval));
+      launch_next(k_filter_write<float, lpr.value>, g, SEL_THREADS, 0, s, n, rpc, seg, active, rs,
+                  re, col, static_cast<const float *>(val), ms, orp, ocol,
+                  static_cast<float *>(oval));
     else
-      k_filter_write<double, lpr.value><<<g, SEL_THREADS, 0, s>>>(
-          n, rpc, seg, active, rs, re, col, static_cast<const double *>(val), ms, orp, ocol,
-          static_cast<double *>(oval));
-    SGN_LAUNCH_CHECK();
+      launch_next(k_filter_write<double, lpr.value>, g, SEL_THREADS, 0, s, n, rpc, seg, active, rs,
+                  re, col, static_cast<const double *>(val), ms, orp, ocol,
+                  static_cast<double *>(oval));
   });
 }
 

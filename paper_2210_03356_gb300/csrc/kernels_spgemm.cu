@@ -130,6 +130,7 @@ __device__ __forceinline__ void put_span(const BandSpans &bs, int64_t r, int fir
 // band layout of B's rows.
 __global__ void k_row_info(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
                            int4 *info, int2 *ends, BandSpans bs) {
+  after_previous();
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     const int64_t a = rs[r], b = re[r];
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(BOUNDS_T)
              const int64_t *moff, int32_t *lo, int32_t *len, int64_t *ub, int32_t *lists,
              int *counters, unsigned long long *mults, double *band_work,
              unsigned char *bandrow, BandSpans cs) {
+  after_previous();
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int ROWS = BOUNDS_T / L;  // rows of one pass
   constexpr int NW = (TILE + 31) / 32;  // warps with rows in the second part
@@ -794,6 +796,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
                 const int2 *ends, const int32_t *lo, const int32_t *len, const int32_t *list,
                 int *counters, int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval,
                 double *part) {
+  after_previous();
   constexpr bool PAIR = LOOP == LOOP_PAIR;
   static_assert(!PAIR || G == 16, "pairs are two 16-lane groups");
   static_assert(LOOP != LOOP_AHEAD || G == 32, "a warp per row");
@@ -940,6 +943,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
 __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
                              const int32_t *seg, const int64_t *moff, int sh, int stride,
                              int *off) {
+  after_previous();
   const int lane = lane_id();
   const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -986,6 +990,7 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
                const int32_t *seg, const int64_t *moff, const int *off, int sh, int stride,
                const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
                int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
+  after_previous();
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
@@ -1174,6 +1179,7 @@ template <typename T>
 __global__ void k_rows_empty(int64_t n, const int64_t *ars, const int64_t *are, const T *aval,
                              const int32_t *len, const int32_t *seg, const int *dslot,
                              const int64_t *cs, int64_t *ce, double *part) {
+  after_previous();
   int lane = lane_id();
   const int g = lane >> 3, gl = lane & 7;  // four groups of 8 lanes
   int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -1239,14 +1245,12 @@ void launch_bounds(int64_t n, const Rows &A, int64_t nnzA, const Rows &B, const 
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
                    const BandSpans &bspans, const BandSpans &cspans, cudaStream_t s) {
   if (n == 0) return;
-  k_row_info<<<grid_cap(n, 256, 8), 256, 0, s>>>(n, B.rs, B.re, B.col, binfo, ends, bspans);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_row_info, grid_cap(n, 256, 8), 256, 0, s, n, B.rs, B.re, B.col, binfo, ends,
+              bspans);
   auto run = [&](auto kern, int tile) {
-    kern<<<grid_cap(n, tile, 8), BOUNDS_T, 0, s>>>(n, A.rs, A.re, A.col, binfo, seg, active, mode,
-                                                   groups, group_margin, band, band_min_eff, dslot,
-                                                   moff, lo, len, ub, lists, counters, mults,
-                                                   band_work, bandrow, cspans);
-    SGN_LAUNCH_CHECK();
+    launch_next(kern, grid_cap(n, tile, 8), BOUNDS_T, 0, s, n, A.rs, A.re, A.col, binfo, seg,
+                active, mode, groups, group_margin, band, band_min_eff, dslot, moff, lo, len, ub,
+                lists, counters, mults, band_work, bandrow, cspans);
   };
   // Few rows: 16 lanes each, for the latency of a row. Rows of many entries,
   // where a lane per row would not fill the chip: 8. Otherwise a lane per row,
@@ -1266,11 +1270,10 @@ static void group_launch(int rows, int64_t n, const Rows &A, const T *aval, cons
                          const int32_t *lists, int *ctr, int cls, const int64_t *cs, int64_t *ce,
                          int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   if (rows <= 0) return;
-  k_num_group<T, MODE, G, LOOP><<<grid_cap(rows, WARPS_PER_CTA * (32 / G), group_occ<T, LOOP>()),
-                                  WARPS_PER_CTA * 32, 0, s>>>(
-      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, ends, lo, len, lists + int64_t(cls) * n,
-      ctr, cls, cs, ce, ccol, cval, part);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_num_group<T, MODE, G, LOOP>,
+              grid_cap(rows, WARPS_PER_CTA * (32 / G), group_occ<T, LOOP>()), WARPS_PER_CTA * 32, 0,
+              s, A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, ends, lo, len,
+              lists + int64_t(cls) * n, ctr, cls, cs, ce, ccol, cval, part);
 }
 
 template <typename T, int MODE>
@@ -1306,10 +1309,9 @@ static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, c
     return true;
   }();
   (void)attr;
-  k_num_wide<T, MODE, P><<<grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()), WIDE_WARPS * 32, sm, s>>>(
-      A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg, wt.moff, wt.off, wt.sh, wt.stride,
-      lo, len, list, ctr, cls, cs, ce, ccol, cval, part);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_num_wide<T, MODE, P>, grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()),
+              WIDE_WARPS * 32, sm, s, A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg,
+              wt.moff, wt.off, wt.sh, wt.stride, lo, len, list, ctr, cls, cs, ce, ccol, cval, part);
 }
 
 template <typename T, int MODE>
@@ -1331,8 +1333,8 @@ static void wide_launch_p(int rows, int p, const Rows &A, const T *aval, const R
 void launch_col_blocks(int64_t n, const Rows &B, const int32_t *seg, const int64_t *moff, int sh,
                        int stride, int *off, cudaStream_t s) {
   if (n == 0) return;
-  k_col_blocks<<<grid_cap(n, 8, 16), 256, 0, s>>>(n, B.rs, B.re, B.col, seg, moff, sh, stride, off);
-  SGN_LAUNCH_CHECK();
+  launch_next(k_col_blocks, grid_cap(n, 8, 16), 256, 0, s, n, B.rs, B.re, B.col, seg, moff, sh,
+              stride, off);
 }
 
 int wide_block_shift(int64_t max_n) {
@@ -1381,9 +1383,8 @@ void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Row
   int64_t listed = 0;
   for (int c = 0; c < RC_N; ++c) listed += int64_t(rows[c]) * (c == RC_BAND ? 16 : 1);
   if (listed < n) {
-    k_rows_empty<T><<<grid_cap(n, 8 * 32, 16), 256, 0, s>>>(
-        n, A.rs, A.re, aval, len, seg, dslot, cs, ce, mode == MODE_SQUARE ? part : nullptr);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_rows_empty<T>, grid_cap(n, 8 * 32, 16), 256, 0, s, n, A.rs, A.re, aval, len, seg,
+                dslot, cs, ce, mode == MODE_SQUARE ? part : nullptr);
   }
   if (shared) return;
   if (mode == MODE_SQUARE)
