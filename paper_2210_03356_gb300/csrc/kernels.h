@@ -158,12 +158,10 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // range [lo, lo+len) of the row (including A's own row in MODE_UPDATE), the
 // slot size ub[i] = min(len, work + (UPDATE ? nnz(A_i) : 0)) >= nnz(C_i), and
 // work of the row = sum_{k in A_i} nnz(B_k), its multiply-adds, added into
-// mults[m] (zeroed by the caller). Non-empty
-// rows are listed, in row order within tiles, by the numeric kernel that takes
-// them: lists holds RC_N lists of n entries (32-, 16- or 8-lane groups, one
-// CTA per row, band tiles); counters[c] is the length of list c and
-// counters[RC_QUEUE + c] the work-queue head of its kernel (all zeroed by the
-// caller). groups: 0 keeps every warp-sized row on 32 lanes; 1 (FP64
+// mults[m]. Non-empty rows are listed, in row order within tiles, by the
+// numeric kernel that takes them: lists holds RC_N lists of n entries (32-, 16-
+// or 8-lane groups, wide rows, band tiles); counters[c] is the length of list c
+// and counters[RC_QUEUE + c] the work-queue head of its kernel. groups: 0 keeps every warp-sized row on 32 lanes; 1 (FP64
 // products, bound by the FP64 pipe) picks 32, 16 or 8 lanes by lane
 // utilisation, a narrower group only when it raises the use by more than
 // group_margin; 2 (FP32 products) lists every row of extent <= 512 in the
@@ -173,7 +171,7 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // FMA slots (by the work estimate in k_bounds; at the default 0.08 the tile
 // costs fewer instructions than the row-wise product) go to the band list
 // instead, and their
-// multiply-adds are added to *band_work (nullable; zeroed by the caller);
+// multiply-adds are added to *band_work (nullable);
 // bandrow (nullable) gets 1 for the rows of band tiles, 0 for the others.
 // binfo: scratch of n records (B's rows' first/last column and length; B has
 // n rows, as every operand of a stage). ends (nullable; FP64 products): n
@@ -181,8 +179,9 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // dslot (nullable, per matrix): matrices with dslot[m] >= 0 take the dense
 // path; their rows get no sparse work, and in MODE_UPDATE a whole row of
 // slots (moff gives the matrix sizes).
-// nnzA: A's entries (or more). bspans, cspans (fc nullable): the band layouts of
-// B's rows and of the product's.
+// head: the block that holds counters, mults and band_work, cleared first
+// (head_bytes, a multiple of 8). nnzA: A's entries (or more). bspans, cspans (fc
+// nullable): the band layouts of B's rows and of the product's.
 struct BandSpans {  // of each row: fc and nf (see Band) and span = nf, scanned into pos
   int32_t *fc = nullptr, *nf = nullptr;
   int64_t *span = nullptr;
@@ -192,7 +191,8 @@ void launch_bounds(int64_t n, const Rows &A, int64_t nnzA, const Rows &B, const 
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
-                   const BandSpans &bspans, const BandSpans &cspans, cudaStream_t s);
+                   const BandSpans &bspans, const BandSpans &cspans, void *head,
+                   size_t head_bytes, cudaStream_t s);
 
 // Band layout of the rows of an FP32 operand: row k's values dense over the
 // columns [fc[k], fc[k] + nf[k]) (fc and nf multiples of 4, holes +0) at

@@ -127,10 +127,14 @@ __device__ __forceinline__ void put_span(const BandSpans &bs, int64_t r, int fir
 // reads one 16-byte record per k instead of a chain of dependent loads. ends
 // (nullable; FP64 products): of a row with at least 32 entries, the 31st
 // column and the 31st from its end (see stream_rows). bs (fc nullable): the
-// band layout of B's rows.
+// band layout of B's rows. Also clears the `words` of the product's head, which
+// k_bounds adds to (a memset of its own would stand between the kernels).
 __global__ void k_row_info(int64_t n, const int64_t *rs, const int64_t *re, const int32_t *col,
-                           int4 *info, int2 *ends, BandSpans bs) {
+                           int4 *info, int2 *ends, BandSpans bs, unsigned long long *head,
+                           int words) {
   after_previous();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x)
+    head[i] = 0ULL;
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
     const int64_t a = rs[r], b = re[r];
@@ -1243,10 +1247,14 @@ void launch_bounds(int64_t n, const Rows &A, int64_t nnzA, const Rows &B, const 
                    const int *dslot, const int64_t *moff, int32_t *lo, int32_t *len,
                    int64_t *ub, int32_t *lists, int *counters, unsigned long long *mults,
                    double *band_work, unsigned char *bandrow, int4 *binfo, int2 *ends,
-                   const BandSpans &bspans, const BandSpans &cspans, cudaStream_t s) {
-  if (n == 0) return;
+                   const BandSpans &bspans, const BandSpans &cspans, void *head,
+                   size_t head_bytes, cudaStream_t s) {
+  if (n == 0) {
+    SGN_CUDA(cudaMemsetAsync(head, 0, head_bytes, s));
+    return;
+  }
   launch_next(k_row_info, grid_cap(n, 256, 8), 256, 0, s, n, B.rs, B.re, B.col, binfo, ends,
-              bspans);
+              bspans, static_cast<unsigned long long *>(head), int(head_bytes / 8));
   auto run = [&](auto kern, int tile) {
     launch_next(kern, grid_cap(n, tile, 8), BOUNDS_T, 0, s, n, A.rs, A.re, A.col, binfo, seg,
                 active, mode, groups, group_margin, band, band_min_eff, dslot, moff, lo, len, ub,

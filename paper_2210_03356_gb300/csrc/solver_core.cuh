@@ -455,7 +455,6 @@ struct Solver {
     w.counters.ensure(ProductHead::bytes(nb), s);
     ProductHead *const head = head_dev();
     w.scan_tmp.ensure(sizeof(int64_t) * SCAN_JOBS * size_t(scan_tmp_elems(N)), s);
-    SGN_CUDA(cudaMemsetAsync(head, 0, ProductHead::bytes(nb), s));
     // band tiles (FP32): in SQUARE the bands of X (both operands) and of T
     // (the output, for the update) are laid out here, their sizes read with
     // the slot total below; the band tiles write the rows of T's band they
@@ -505,7 +504,7 @@ struct Solver {
                     head->ctr, head->mults, &head->band_work,
                     band && mode == MODE_SQUARE ? w.bandrow.as<unsigned char>() : nullptr,
                     static_cast<int4 *>(w.binfo.ensure(sizeof(int4) * size_t(N > 0 ? N : 1), s)),
-                    ends, bspans, cspans, s);
+                    ends, bspans, cspans, head, ProductHead::bytes(nb), s);
     }
     {
       ProfScope ps(KC_SCAN, s);
