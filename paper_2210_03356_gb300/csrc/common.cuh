@@ -41,10 +41,9 @@ void count_launch();
 // chain of some 20 kernels, each of 3 to 5 us for a small matrix: the solve of
 // a tridiagonal matrix of order 500 went from 1.43 to 1.12 ms, that of a banded
 // one of order 6001 from 3.44 to 3.00.
-// Kernels whose few CTAs each want an SM to themselves are launched in the
-// ordinary way (the dense products, the copies, the inverse of an NMF step):
-// CTAs placed early pile up where the kernel before left room, and that
-// inverse took 56.4 ms for 54.9.
+// Long kernels whose few CTAs each want an SM to themselves (the dense products,
+// the copies, an inverse's back substitution) are launched in the ordinary way:
+// CTAs placed early settle where the kernel before left room.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -85,6 +85,7 @@ __global__ void k_inv_init(int n, int ld, double *inv) {
 __global__ void __launch_bounds__(PANEL_T)
     k_lu_panel(int n, int ld, double *lu, int c0, int w, int in_place, int *swaps,
                int *singular, int *wild) {
+  after_previous();
   extern __shared__ double panel[];
   __shared__ long long sv[PANEL_T / 32];
   __shared__ int si[PANEL_T / 32], s_pivot;
@@ -184,6 +185,7 @@ template <int W>
 __global__ void __launch_bounds__(TRAIL_T)
     k_lu_trail(int n, int ld, double *lu, double *inv, int c0, const int *swaps,
                const int *singular, const int *wild) {
+  after_previous();
   __shared__ int rows[2 * W], src[2 * W];
   __shared__ int nrows;
   __shared__ double moved[2 * W][STRIP], L[W][W], U[W][STRIP];
@@ -439,14 +441,12 @@ void launch_dense_inverse(int n, int ld, double *lu, int *swaps, int *singular, 
     while (w > n - c0) w /= 2;  // the last columns: widths are powers of two
     const size_t smem = size_t(n - c0) * w * sizeof(double);
     const int in_place = smem > PANEL_SMEM ? 1 : 0;
-    k_lu_panel<<<1, PANEL_T, in_place ? 0 : smem, s>>>(n, ld, lu, c0, w, in_place, swaps, singular,
-                                                              wild);
-    SGN_LAUNCH_CHECK();
+    launch_next(k_lu_panel, 1, PANEL_T, in_place ? 0 : smem, s, n, ld, lu, c0, w, in_place, swaps,
+                singular, wild);
     const unsigned strips =
         unsigned((n - c0 - w + STRIP - 1) / STRIP + (n + STRIP - 1) / STRIP);
     auto trail = [&](auto kernel) {
-      kernel<<<strips, TRAIL_T, 0, s>>>(n, ld, lu, inv, c0, swaps, singular, wild);
-      SGN_LAUNCH_CHECK();
+      launch_next(kernel, strips, TRAIL_T, 0, s, n, ld, lu, inv, c0, swaps, singular, wild);
     };
     if (w == 8) trail(k_lu_trail<8>);
     else if (w == 4) trail(k_lu_trail<4>);
