@@ -582,7 +582,7 @@ constexpr int EX_U = 4;  // entries per lane of a row loaded at once
 // matrix without a crossing already has its tau (the smallest key above b),
 // so every entry is decided here. k_sel_digits adds the kept candidates
 // once tau is final; the dropped candidates' squares come from the select's
-// exact sums (k_sel_drop_fix). Rows of inactive matrices get 0 and 0.
+// exact sums (k_drop_sums). Rows of inactive matrices get 0 and 0.
 // Per row two bounds on the keys decide: below s_lo an entry is dropped, from
 // s_up on it is kept, between it is a candidate (a NaN is dropped).
 template <typename T, int LPR>
