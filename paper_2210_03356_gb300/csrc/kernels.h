@@ -151,8 +151,9 @@ struct Rows {
 // windows of wide rows (RC_CTA), or band tiles of 16 rows (FP32 only; the list holds each
 // tile's first row).
 enum RowClass { RC_G32 = 0, RC_CTA = 1, RC_G16 = 2, RC_G8 = 3, RC_BAND = 4, RC_NONE = 5, RC_N = 5 };
-constexpr int RC_QUEUE = RC_N;        // counters[RC_QUEUE + c]: work-queue head of class c
-constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
+constexpr int RC_QUEUE = RC_N;         // counters[RC_QUEUE + c]: work-queue head of class c
+constexpr int RC_EMPTY = 2 * RC_N;     // counters[RC_EMPTY]: rows without output (in band tiles too)
+constexpr int RC_COUNTERS = 2 * RC_N + 2;  // ints in the counters array (8-byte padded)
 
 // Per row i of C = A B (rows of inactive matrices are empty): the column
 // range [lo, lo+len) of the row (including A's own row in MODE_UPDATE), the
@@ -160,8 +161,10 @@ constexpr int RC_COUNTERS = 2 * RC_N;  // ints in the counters array
 // work of the row = sum_{k in A_i} nnz(B_k), its multiply-adds, added into
 // mults[m]. Non-empty rows are listed, in row order within tiles, by the
 // numeric kernel that takes them: lists holds RC_N lists of n entries (32-, 16-
-// or 8-lane groups, wide rows, band tiles); counters[c] is the length of list c
-// and counters[RC_QUEUE + c] the work-queue head of its kernel. groups: 0 keeps every warp-sized row on 32 lanes; 1 (FP64
+// or 8-lane groups, wide rows, band tiles); counters[c] is the length of list c,
+// counters[RC_QUEUE + c] the work-queue head of its kernel and
+// counters[RC_EMPTY] the number of rows without output (len 0), which no list
+// or a band tile beside other rows holds. groups: 0 keeps every warp-sized row on 32 lanes; 1 (FP64
 // products, bound by the FP64 pipe) picks 32, 16 or 8 lanes by lane
 // utilisation, a narrower group only when it raises the use by more than
 // group_margin; 2 (FP32 products) lists every row of extent <= 512 in the
@@ -235,11 +238,11 @@ void launch_band_product(int64_t n, int mode, const Rows &A, const float *aval, 
 // The part entries of dense-path matrices (dslot nullable; dslot[seg[i]] >= 0)
 // are left to the dense path. ends: from launch_bounds (FP64; null for FP32).
 // rows: the list lengths (counters[RC_*]) on the host; empty classes are not
-// launched. few: every listed row is in the 32-lane class (groups = 0) and runs
+// launched. empty: counters[RC_EMPTY], whose rows' ends and sums are written here. few: every listed row is in the 32-lane class (groups = 0) and runs
 // with its loads ahead of its sums (rows too few to hide them otherwise); shared:
 // they are left to launch_numeric_wide.
 template <typename T>
-void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Rows &A, const T *aval,
+void launch_numeric(int64_t n, const int *rows, int empty, bool shared, bool few, const Rows &A, const T *aval,
                     const Rows &B, const T *bval, int mode, const int2 *ends, const int32_t *lo,
                     const int32_t *len, const int32_t *seg, const int *dslot,
                     const int32_t *lists, int *counters, const int64_t *cs, int64_t *ce,

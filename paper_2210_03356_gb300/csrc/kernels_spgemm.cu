@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(BOUNDS_T)
     }
     // ordered compaction of the tile's rows into one list per class
     int my = i < TILE ? s_cls[i] : int(RC_NONE);
+    const bool empty = i < TILE && t0 + i < n && my == RC_NONE;
     if (inband) my = (i & 15) == 0 ? RC_BAND : RC_NONE;
     if (bandrow && i < TILE && t0 + i < n) bandrow[t0 + i] = inband ? 1 : 0;
     unsigned bal[RC_N];
@@ -386,7 +387,7 @@ __global__ void __launch_bounds__(BOUNDS_T)
       bal[c] = __ballot_sync(FULL, my == c);
       if (lane == 0 && warp < NW) s_cnt[warp][c] = __popc(bal[c]);
     }
-    __syncthreads();
+    const int nempty = __syncthreads_count(empty);
     if (i < RC_N) {
       int tot = 0;
       for (int w = 0; w < NW; ++w) tot += s_cnt[w][i];
@@ -394,6 +395,7 @@ __global__ void __launch_bounds__(BOUNDS_T)
     } else if (i == 32) {
       if (s_mult) atomicAdd(&mults[m0], s_mult);
       if (s_band_work) atomicAdd(band_work, double(s_band_work));  // of the band tiles
+      if (nempty) atomicAdd(&counters[RC_EMPTY], nempty);
     }
     __syncthreads();
     if (my < RC_N) {
@@ -1174,7 +1176,8 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
   }
 }
 
-// Rows with an empty column range: their slot stays empty (ce = cs) and, in
+// Rows with an empty column range, also those of a band tile whose other rows
+// have output (k_band passes over them): their slot stays empty (ce = cs) and, in
 // MODE_SQUARE, they still contribute (0 - 1)^2 = 1 for the missing diagonal
 // and sum_k a_ik^2 to the norms. The rows of dense-path matrices (dslot[seg]
 // >= 0) are empty here too, but their norms come from the dense blocks: their
@@ -1382,15 +1385,13 @@ template void launch_numeric_wide<float>(int64_t, int, int, double, const Rows &
                                          cudaStream_t);
 
 template <typename T>
-void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Rows &A, const T *aval,
+void launch_numeric(int64_t n, const int *rows, int empty, bool shared, bool few, const Rows &A, const T *aval,
                     const Rows &B, const T *bval, int mode, const int2 *ends, const int32_t *lo,
                     const int32_t *len, const int32_t *seg, const int *dslot,
                     const int32_t *lists, int *counters, const int64_t *cs, int64_t *ce,
                     int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   if (n == 0) return;
-  int64_t listed = 0;
-  for (int c = 0; c < RC_N; ++c) listed += int64_t(rows[c]) * (c == RC_BAND ? 16 : 1);
-  if (listed < n) {
+  if (empty > 0) {
     launch_next(k_rows_empty<T>, grid_cap(n, 8 * 32, 16), 256, 0, s, n, A.rs, A.re, aval, len, seg,
                 dslot, cs, ce, mode == MODE_SQUARE ? part : nullptr);
   }
@@ -1403,12 +1404,12 @@ void launch_numeric(int64_t n, const int *rows, bool shared, bool few, const Row
                                ce, ccol, cval, part, s);
 }
 
-template void launch_numeric<double>(int64_t, const int *, bool, bool, const Rows &, const double *,
+template void launch_numeric<double>(int64_t, const int *, int, bool, bool, const Rows &, const double *,
                                      const Rows &, const double *, int, const int2 *,
                                      const int32_t *, const int32_t *, const int32_t *,
                                      const int *, const int32_t *, int *, const int64_t *,
                                      int64_t *, int32_t *, double *, double *, cudaStream_t);
-template void launch_numeric<float>(int64_t, const int *, bool, bool, const Rows &, const float *,
+template void launch_numeric<float>(int64_t, const int *, int, bool, bool, const Rows &, const float *,
                                     const Rows &, const float *, int, const int2 *,
                                     const int32_t *, const int32_t *, const int32_t *, const int *,
                                     const int32_t *, int *, const int64_t *, int64_t *, int32_t *,

@@ -575,7 +575,7 @@ struct Solver {
       int rows[RC_N];
       std::copy(ctr, ctr + RC_N, rows);
       const int wide_rows[2] = {rows[RC_CTA], shared ? rows[RC_G32] : 0};
-      launch_numeric<T>(N, rows, shared, few, A, aval, B, bval, mode, ends, w.lo.as<int32_t>(),
+      launch_numeric<T>(N, rows, ctr[RC_EMPTY], shared, few, A, aval, B, bval, mode, ends, w.lo.as<int32_t>(),
                         w.len.as<int32_t>(), st.d_seg.template as<int32_t>(),
                         dp && dp->any() ? w.dslot.as<int>() : nullptr, w.wlist.as<int32_t>(),
                         head->ctr, C.rs.template as<int64_t>(),
