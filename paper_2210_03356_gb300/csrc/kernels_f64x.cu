@@ -37,7 +37,8 @@
 // (BF16) MMAs per accumulator and stage. Steps share an accumulator while its
 // products stay within 4096 per entry (all of a level for K <= 512, one step
 // for K > 2048); then the epilogue warps drain both accumulators into the
-// CTA's tile of integers (global scratch, 256 KB, stays in L2).
+// CTA's tiles of integers (global scratch, 2 x 256 KB, stay in L2), the last
+// run of a whole tile into C.
 // What bounds it: the tensor pipe and, behind it, the L2 reads of the operand
 // planes, 16 KB per pair and slice here against 24 KB when every pair loads
 // its own two planes, and the FP64 pipe (16 cycles per warp instruction) when
@@ -172,8 +173,8 @@ __device__ __forceinline__ void xtile_of(int t, const SliceJob *jobs, const int 
 }
 
 // maps[2 j]: the digits of A of job j as one (8 M) x K array, maps[2 j + 1]
-// those of Bt as (8 N) x K; digit s of row r is row (s - 1) rows + r. tiles: one
-// integer tile per CTA; parts: two per part (levels 9 .. 4, levels 3 and 2).
+// those of Bt as (8 N) x K; digit s of row r is row (s - 1) rows + r. tiles and
+// parts: two integer tiles (levels 9 .. 4, levels 3 and 2) per CTA and per part.
 __global__ void __launch_bounds__(XTHREADS, 1)
     k_gemm_slices(const SliceJob *jobs, const CUtensorMap *maps, const int *tile_start,
                   int njobs, XPlan pl, long long *tiles, long long *parts, int *err) {
@@ -304,11 +305,11 @@ __global__ void __launch_bounds__(XTHREADS, 1)
       int j, m0, n0;
       xtile_of(un.tile, jobs, tile_start, njobs, j, m0, n0);
       const SliceJob J = jobs[j];
-      // this warp's part of the integer tiles: [chunk][column][lane]; a part has a
-      // second one for the levels 3 and 2
-      long long *const low =
-          (part ? parts + size_t(u - pl.nfull) * (2 * XM * XN) : tiles + size_t(blockIdx.x) * (XM * XN)) +
-          size_t(warp - 2) * (XM * XN / 8) + lane;
+      // this warp's part of the integer tiles, [chunk][column][lane]: one for the
+      // levels 9 .. 4 and one for 3 and 2
+      long long *const low = (part ? parts + size_t(u - pl.nfull) * (2 * XM * XN)
+                                   : tiles + size_t(blockIdx.x) * (2 * XM * XN)) +
+                             size_t(warp - 2) * (XM * XN / 8) + lane;
       const int gr = m0 + q * 32 + lane;
       const int ea = gr < J.M ? J.ea[gr] : 0;
       const int nk = (J.K + XK - 1) / XK;
@@ -328,6 +329,8 @@ __global__ void __launch_bounds__(XTHREADS, 1)
             const bool both = ta < l;  // the lower level's accumulator was written
             const bool high = lp == XLP - 1;
             const bool first = high ? first_high : first_low;
+            // a whole tile's last run: its sums are complete and go into C
+            const bool into_c = high && !part && e == un.s1;
 #pragma unroll 1
             for (int c = 0; c < XN / 64; ++c) {
               uint32_t v0[32], v1[32];
@@ -340,8 +343,8 @@ __global__ void __launch_bounds__(XTHREADS, 1)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v0[i] = 0u;
               }
-              long long *const lc = low + c * 32 * 32 + (high && part ? XM * XN : 0);
-              if (!high || part) {  // into an integer tile
+              long long *const lc = low + c * 32 * 32 + (high ? XM * XN : 0);
+              if (!into_c) {  // into an integer tile
                 const int sh = high ? 0 : 2 * DIGIT_BITS * lp;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -357,46 +360,46 @@ __global__ void __launch_bounds__(XTHREADS, 1)
                 }
                 continue;
               }
-              // levels 3 and 2: C = [C +] 2^(e_i + f_j - 63) L + 2^(e_i + f_j - 21) H
+              // C = [C +] 2^(e_i + f_j - 63) L + 2^(e_i + f_j - 21) H, H and L exact as
+              // where the tile is cut into parts: the same bits either way
               const int gc = n0 + col;
               if (gr >= J.M) continue;
               double *const crow = J.C + int64_t(gr) * J.ldc + gc;
-              const bool with_low = first;
-              const bool add = !first || k0 > 0 || J.accum;  // C holds earlier terms
-              auto pair_of = [&](int k, const double2 &old) {  // columns gc + k, gc + k + 1
-                const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + k);
-                double r[2];
+              const long long *const ll = lc - XM * XN;
+              const bool add = k0 > 0 || J.accum;  // C holds earlier K blocks
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                  const int sc = ea + (i ? eb.y : eb.x);
-                  r[i] = scaled_int(acc_int(v0[k + i]) * (1 << DIGIT_BITS) + acc_int(v1[k + i]),
-                                    sc - 3 * DIGIT_BITS);
-                  if (with_low) r[i] += scaled_int(lc[(k + i) * 32], sc - 9 * DIGIT_BITS);
-                  if (add) r[i] += i ? old.y : old.x;
+              for (int h = 0; h < 4; ++h) {
+                // eight columns: all loads in flight before any store (N and ldc even,
+                // C 16-byte aligned: column pairs)
+                long long hs[8], ls[8];
+                double2 o[4];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  hs[i] = first ? 0ll : lc[(8 * h + i) * 32];
+                  ls[i] = ll[(8 * h + i) * 32];
                 }
-                return make_double2(r[0], r[1]);
-              };
-              if (gc + 32 <= J.N) {
+                if (add) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  double2 o[8];  // eight loads of the row in flight before any store
-                  if (add) {
+                  for (int i = 0; i < 4; ++i)
+                    if (gc + 8 * h + 2 * i < J.N)
+                      o[i] = reinterpret_cast<const double2 *>(crow)[4 * h + i];
+                }
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                      o[i] = reinterpret_cast<const double2 *>(crow)[8 * h + i];
+                for (int i = 0; i < 8; i += 2) {
+                  const int x = 8 * h + i;
+                  if (gc + x >= J.N) break;
+                  const int2 eb = *reinterpret_cast<const int2 *>(J.eb + gc + x);
+                  double r[2];
+#pragma unroll
+                  for (int p = 0; p < 2; ++p) {
+                    const int sc = ea + (p ? eb.y : eb.x);
+                    r[p] = scaled_int(hs[i + p] + acc_int(v0[x + p]) * (1 << DIGIT_BITS) +
+                                          acc_int(v1[x + p]),
+                                      sc - 3 * DIGIT_BITS);
+                    r[p] += scaled_int(ls[i + p], sc - 9 * DIGIT_BITS);
+                    if (add) r[p] += p ? o[i / 2].y : o[i / 2].x;
                   }
-#pragma unroll
-                  for (int i = 0; i < 8; ++i)
-                    reinterpret_cast<double2 *>(crow)[8 * h + i] =
-                        pair_of(16 * h + 2 * i, add ? o[i] : make_double2(0.0, 0.0));
-                }
-              } else {
-                // ragged last chunk (N and ldc even, C 16-byte aligned: column pairs)
-#pragma unroll
-                for (int k = 0; k < 32; k += 2) {
-                  if (gc + k >= J.N) break;
-                  double2 *const cp = reinterpret_cast<double2 *>(crow + k);
-                  *cp = pair_of(k, add ? *cp : make_double2(0.0, 0.0));
+                  reinterpret_cast<double2 *>(crow)[x / 2] = make_double2(r[0], r[1]);
                 }
               }
             }
@@ -812,7 +815,7 @@ static XPlan slice_plan(int ntiles, bool one_block) {
 size_t slice_jobs_scratch_bytes(int njobs, int ntiles) {
   const XPlan pl = slice_plan(ntiles, true);
   return scratch_maps_bytes_x(njobs) +
-         XTILE_BYTES * (size_t(std::min(ntiles, slice_ctas())) + 2 * size_t(pl.ntail) * pl.parts);
+         2 * XTILE_BYTES * (size_t(std::min(ntiles, slice_ctas())) + size_t(pl.ntail) * pl.parts);
 }
 
 void launch_slices(int rows, int K, const double *x, int ldx, int transpose, uint16_t *digits,
@@ -859,7 +862,7 @@ void launch_slice_jobs(int njobs, const SliceJob *jobs_host, SliceJob *jobs_dev,
   unsigned char *sc = static_cast<unsigned char *>(scratch);
   const int *starts = reinterpret_cast<const int *>(sc + size_t(njobs) * 2 * sizeof(CUtensorMap));
   long long *tiles = reinterpret_cast<long long *>(sc + scratch_maps_bytes_x(njobs));
-  long long *parts = tiles + size_t(std::min(ntiles, slice_ctas())) * (XM * XN);
+  long long *parts = tiles + size_t(std::min(ntiles, slice_ctas())) * (2 * XM * XN);
   k_gemm_slices<<<std::min(pl.units(), slice_ctas()), XTHREADS, XSMEM, s>>>(
       jobs_dev, reinterpret_cast<const CUtensorMap *>(sc), starts, njobs, pl, tiles, parts, err);
   SGN_LAUNCH_CHECK();
