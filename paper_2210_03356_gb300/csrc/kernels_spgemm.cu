@@ -56,6 +56,10 @@ template <>
 struct SqAcc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add_sq(double v) { s = __fma_rn(v, v, s); }
+  __device__ __forceinline__ void merge(const SqAcc &o) { s += o.s; }
+  __device__ __forceinline__ SqAcc from_lane_xor(unsigned mask, int o) const {
+    return SqAcc{__shfl_xor_sync(mask, s, o)};
+  }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
@@ -74,8 +78,36 @@ struct SqAcc<float> {
     add(p);
     lo = __fadd_rn(lo, e);
   }
+  __device__ __forceinline__ void merge(const SqAcc &o) {  // the same with *this and o exchanged
+    const float l = __fadd_rn(lo, o.lo);
+    lo = 0.0f;
+    add(o.hi);
+    lo = __fadd_rn(l, lo);
+  }
+  __device__ __forceinline__ SqAcc from_lane_xor(unsigned mask, int o) const {
+    return SqAcc{__shfl_xor_sync(mask, hi, o), __shfl_xor_sync(mask, lo, o)};
+  }
   __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
 };
+
+// The total of a row's 32 partial sums, 32 / G on each of the G lanes of mask
+// (lane gl holds gl, gl + G, ..): added 16 apart, 8 apart and so on, the same
+// additions for every G.
+template <typename T, int G>
+__device__ __forceinline__ double sum_of_32(SqAcc<T> (&p)[32 / G], unsigned mask) {
+  constexpr int N = 32 / G;
+  if constexpr (N == 1) {
+    p[0].merge(p[0].from_lane_xor(mask, 16));
+  } else {
+#pragma unroll
+    for (int u = 0; u < N / 2; ++u) p[u].merge(p[u + N / 2]);
+  }
+  double v = p[0].value();
+  if constexpr (N == 4) v += p[1].value();
+#pragma unroll
+  for (int o = G < 16 ? G / 2 : 8; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o, G);
+  return v;
+}
 
 __device__ __forceinline__ int64_t lower_bound(const int32_t *a, int64_t lo, int64_t hi,
                                                int64_t v) {
@@ -787,6 +819,10 @@ template <> struct WarpOcc<float> { static constexpr int value = 10; };
 // G lanes per row, 32/G rows per warp; each group owns WARP_W*G/32 slots of
 // its warp's accumulator and runs the ascending-k accumulation of its own row
 // with group-wide barriers, so the result is the same as with a whole warp.
+// A row's sums of squares are 32 partial sums, of the columns lo + p, lo + p + 32,
+// ... (the diagonal's square is added last) and of every 32nd entry of X_i, in
+// ascending order, then added by sum_of_32: whatever lanes a row runs on, which
+// depends on the other rows of the launch too, its part of the residual is the same.
 // LOOP: LOOP_PAIR (with G = 16): the two rows of a warp share its k-loop
 // (pair_rows); the rest of the kernel is that of 16-lane groups. LOOP_AHEAD
 // (with G = 32): the k-loop of ahead_rows.
@@ -889,50 +925,58 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
           __syncwarp(gmask);
         }
         int64_t out = cs[r];
-        SqAcc<T> racc;
+        SqAcc<T> racc[NG];  // 32 partial sums per row, NG to a lane
         double rdiag = 0.0;
         bool diag = false;
-        for (int s0 = 0; s0 < L; s0 += G) {
-          int s = s0 + gl;
-          int fl = 0;
-          if (s < L) {
-            // touched: a product or, in an update, x_ij
-            fl = MODE == MODE_UPDATE ? f[s] : 0;
-            if (!fl && !untouched(acc[s])) fl = 1;
-          }
-          unsigned m = (__ballot_sync(gmask, fl != 0) >> (g * G)) & gbits;
-          if (fl) {
-            int64_t pos = out + __popc(m & lt);
-            int32_t cj = c0 + s;
-            T v = acc[s];
-            if (MODE == MODE_UPDATE && !(fl & 2)) v = ns_combine(T(0), v);
-            ccol[pos] = cj;
-            cval[pos] = v;
-            if (MODE == MODE_SQUARE) {
-              if (cj == r) {  // (t_ii - 1)^2 in FP64, once per row
-                double d = double(v) - 1.0;
-                rdiag = d * d;
-                diag = true;
-              } else {
-                racc.add_sq(v);
+        for (int s32 = 0; s32 < L; s32 += 32) {
+#pragma unroll
+          for (int u = 0; u < NG; ++u) {
+            const int s0 = s32 + u * G;
+            if (u > 0 && s0 >= L) break;
+            int s = s0 + gl;
+            int fl = 0;
+            if (s < L) {
+              // touched: a product or, in an update, x_ij
+              fl = MODE == MODE_UPDATE ? f[s] : 0;
+              if (!fl && !untouched(acc[s])) fl = 1;
+            }
+            unsigned m = (__ballot_sync(gmask, fl != 0) >> (g * G)) & gbits;
+            if (fl) {
+              int64_t pos = out + __popc(m & lt);
+              int32_t cj = c0 + s;
+              T v = acc[s];
+              if (MODE == MODE_UPDATE && !(fl & 2)) v = ns_combine(T(0), v);
+              ccol[pos] = cj;
+              cval[pos] = v;
+              if (MODE == MODE_SQUARE) {
+                if (cj == r) {  // (t_ii - 1)^2 in FP64, once per row
+                  double d = double(v) - 1.0;
+                  rdiag = d * d;
+                  diag = true;
+                } else {
+                  racc[u].add_sq(v);
+                }
               }
             }
+            out += __popc(m);
           }
-          out += __popc(m);
         }
         if (gl == 0) ce[r] = out;
         if (MODE == MODE_SQUARE) {
-          SqAcc<T> xacc;
-          for (int64_t p = a0 + gl; p < a1; p += G) xacc.add_sq(aval[p]);
-          double rs = racc.value() + rdiag, xs = xacc.value();
-  #pragma unroll
-          for (int o = G / 2; o > 0; o >>= 1) {
-            rs += __shfl_xor_sync(gmask, rs, o, G);
-            xs += __shfl_xor_sync(gmask, xs, o, G);
+          SqAcc<T> xacc[NG];
+          for (int64_t p = a0 + gl; p < a1; p += 4 * G) {  // four loads in flight
+            T x[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) x[t] = p + t * G < a1 ? aval[p + t * G] : T(0);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              if (p + t * G < a1) xacc[t % NG].add_sq(x[t]);
           }
-          bool any_diag = __any_sync(gmask, diag);
+          const double rs = sum_of_32<T, G>(racc, gmask), xs = sum_of_32<T, G>(xacc, gmask);
+          const unsigned dm = __ballot_sync(gmask, diag);
+          const double rd = __shfl_sync(gmask, rdiag, dm ? __ffs(dm) - 1 : 0, G);
           if (gl == 0) {
-            part[2 * int64_t(r)] = any_diag ? rs : rs + 1.0;
+            part[2 * int64_t(r)] = rs + (dm ? rd : 1.0);
             part[2 * int64_t(r) + 1] = xs;
           }
         }
@@ -977,6 +1021,10 @@ __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, co
 // to add up their entry counts before each writes its part. P follows the
 // mean length of B's rows: enough entries of B_k per warp to fill its lanes
 // (an FP64 instruction costs the pipe the same whatever its active lanes).
+// A row's sums of squares are 256 partial sums, of every 256th column counted
+// from the row's first one and of every 256th entry of X_i, added pairwise in
+// eighths of 32 (8 / P of them to a warp) and those in order: the same for every P
+// and window. Rows of the 32-lane class take that class's sums instead.
 // One CTA per row with a barrier per k took 12.0 and 6.0 ms for the update and
 // the square of the 16^3 Laplacian's FP32 iterate just below the dense path's
 // density, now 7.8 and 4.0.
@@ -989,7 +1037,7 @@ constexpr size_t wide_smem() {
   return size_t(WIDE_WARPS) * WARP_W * (sizeof(T) + (MODE == MODE_UPDATE ? 1 : 0));
 }
 
-template <typename T, int MODE, int P>
+template <typename T, int MODE, int P, bool NARROW>
 __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
     k_num_wide(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
                const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
@@ -1000,8 +1048,9 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
+  constexpr int NQ = WIDE_WARPS / P;     // eighths of a row's sums per warp
   __shared__ int s_idx[NG], s_cnt[WIDE_WARPS];
-  __shared__ double s_red[2][WIDE_WARPS];
+  __shared__ double s_red[2][NG * WIDE_WARPS];
   __shared__ int s_diag[WIDE_WARPS];
   const int lane = lane_id(), w = threadIdx.x >> 5, g = w / P, wr = w % P;
   const unsigned lt = (1u << lane) - 1u;
@@ -1025,7 +1074,9 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
     const int b0 = int((lo[r] - base) >> sh), b1 = int((int64_t(lo[r]) + len[r] - 1 - base) >> sh);
     const int bpw = min(WARP_W >> sh, (b1 - b0 + P) / P);  // blocks per warp and window
     int64_t out = cs[r];
-    double rs = 0.0;
+    SqAcc<T> racc[1];  // NARROW: the sums of k_num_group, by warp 0
+    double rdiag = 0.0;
+    double rq[NQ] = {};
     bool diag = false;
     for (int win = b0; win <= b1; win += P * bpw) {
       const int w0 = win + wr * bpw, w1 = min(w0 + bpw, b1 + 1);  // this warp's blocks
@@ -1128,48 +1179,101 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
           if (MODE == MODE_UPDATE && !(fl & 2)) v = ns_combine(T(0), v);
           ccol[pos] = int32_t(cj);
           cval[pos] = v;
-          if (MODE == MODE_SQUARE) {
-            double d = double(v);
-            if (cj == r) {
-              d = d - 1.0;
-              diag = true;
-            }
-            rs += d * d;
-          }
         }
         at += __popc(mk);
+      }
+      if constexpr (MODE == MODE_SQUARE) {
+        // the squares of the window's columns, from the accumulators of all the
+        // row's warps; column i is counted from the row's first one
+        const int d = int(lo[r] - base) - (win << sh);  // column i is i + d of the window
+        const int i0 = max(0, -d), i1 = min(len[r], (P * bpw << sh) - d);
+        const int idiag = r - lo[r];
+        auto value_at = [&](int i, T &v) {
+          if (i < i0 || i >= i1) return false;
+          const int o = P == 1 ? 0 : ((i + d) >> sh) / bpw;  // the warp that holds it
+          v = acc[(o - wr) * WARP_W + (i + d) - (o * bpw << sh)];
+          return !untouched(v);
+        };
+        T v;
+        if constexpr (NARROW) {
+          if (wr == 0)
+            for (int i = (i0 & ~31) + lane; i - lane < i1; i += 32)
+              if (value_at(i, v)) {
+                if (i == idiag) {
+                  const double t = double(v) - 1.0;
+                  rdiag = t * t;
+                  diag = true;
+                } else {
+                  racc[0].add_sq(v);
+                }
+              }
+        } else {
+          for (int i8 = i0 & ~255; i8 < i1; i8 += 256)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+              const int i = i8 + 32 * (wr + q * P) + lane;
+              if (value_at(i, v)) {
+                double t = double(v);
+                if (i == idiag) {
+                  t = t - 1.0;
+                  diag = true;
+                }
+                rq[q] += t * t;
+              }
+            }
+        }
       }
       row_sync();  // s_cnt and the accumulators are free again
     }
     if (wr == 0 && lane == 0) ce[r] = out;
-    if (MODE == MODE_SQUARE) {
-      double xs = 0.0;
-      for (int64_t p = a0 + wr * 32 + lane; p < a1; p += P * 32) {
-        const double x = double(aval[p]);
-        xs += x * x;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        rs += __shfl_xor_sync(FULL, rs, o);
-        xs += __shfl_xor_sync(FULL, xs, o);
-      }
-      const bool dg = __any_sync(FULL, diag);
-      if (lane == 0) {
-        s_red[0][w] = rs;
-        s_red[1][w] = xs;
-        s_diag[w] = dg ? 1 : 0;
-      }
-      row_sync();
-      if (wr == 0 && lane == 0) {
-        double a = 0.0, b = 0.0;
-        int any = 0;
-        for (int i = 0; i < P; ++i) {
-          a += s_red[0][w + i];
-          b += s_red[1][w + i];
-          any |= s_diag[w + i];
+    if constexpr (MODE == MODE_SQUARE) {
+      const unsigned dm = __ballot_sync(FULL, diag);
+      if constexpr (NARROW) {
+        if (wr == 0) {
+          SqAcc<T> xacc[1];
+          for (int64_t p = a0 + lane; p < a1; p += 32) xacc[0].add_sq(aval[p]);
+          const double rs = sum_of_32<T, 32>(racc, FULL), xs = sum_of_32<T, 32>(xacc, FULL);
+          const double rd = __shfl_sync(FULL, rdiag, dm ? __ffs(dm) - 1 : 0);
+          if (lane == 0) {
+            part[2 * int64_t(r)] = rs + (dm ? rd : 1.0);
+            part[2 * int64_t(r) + 1] = xs;
+          }
         }
-        part[2 * int64_t(r)] = any ? a : a + 1.0;
-        part[2 * int64_t(r) + 1] = b;
+      } else {
+        double xq[NQ] = {};
+        for (int64_t p = a0; p < a1; p += 256)
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            const int64_t i = p + 32 * (wr + q * P) + lane;
+            const double x = i < a1 ? double(aval[i]) : 0.0;
+            xq[q] += x * x;
+          }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          double a = rq[q], b = xq[q];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(FULL, a, o);
+            b += __shfl_xor_sync(FULL, b, o);
+          }
+          if (lane == 0) {
+            s_red[0][g * WIDE_WARPS + wr + q * P] = a;
+            s_red[1][g * WIDE_WARPS + wr + q * P] = b;
+          }
+        }
+        if (lane == 0) s_diag[w] = dm ? 1 : 0;
+        row_sync();
+        if (wr == 0 && lane == 0) {
+          double a = 0.0, b = 0.0;
+          int any = 0;
+          for (int i = 0; i < WIDE_WARPS; ++i) {
+            a += s_red[0][g * WIDE_WARPS + i];
+            b += s_red[1][g * WIDE_WARPS + i];
+          }
+          for (int i = 0; i < P; ++i) any |= s_diag[w + i];
+          part[2 * int64_t(r)] = any ? a : a + 1.0;
+          part[2 * int64_t(r) + 1] = b;
+        }
       }
     }
     row_sync();  // s_idx and s_red are read
@@ -1308,19 +1412,19 @@ static void num_launch(int64_t n, const int *rows, bool few, const Rows &A, cons
                              cs, ce, ccol, cval, part, s);
 }
 
-template <typename T, int MODE, int P>
+template <typename T, int MODE, int P, bool NARROW>
 static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, const T *bval,
                         const WideTable &wt, const int32_t *lo, const int32_t *len,
                         const int32_t *list, int *ctr, int cls, const int64_t *cs, int64_t *ce,
                         int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   constexpr size_t sm = wide_smem<T, MODE>();
   static const bool attr = [] {  // once, thread-safe
-    SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P>,
+    SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P, NARROW>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
     return true;
   }();
   (void)attr;
-  launch_next(k_num_wide<T, MODE, P>, grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()),
+  launch_next(k_num_wide<T, MODE, P, NARROW>, grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()),
               WIDE_WARPS * 32, sm, s, A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg,
               wt.moff, wt.off, wt.sh, wt.stride, lo, len, list, ctr, cls, cs, ce, ccol, cval, part);
 }
@@ -1331,13 +1435,21 @@ static void wide_launch_p(int rows, int p, const Rows &A, const T *aval, const R
                           const int32_t *len, const int32_t *list, int *ctr, int cls,
                           const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                           cudaStream_t s) {
-#define SGN_WIDE(P) \
-  wide_launch<T, MODE, P>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cls, cs, ce, ccol, cval, \
+#define SGN_WIDE(P, NARROW) \
+  wide_launch<T, MODE, P, NARROW>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cls, cs, ce, ccol, cval, \
                           part, s)
-  if (p >= 8) SGN_WIDE(8);
-  else if (p >= 4) SGN_WIDE(4);
-  else if (p >= 2) SGN_WIDE(2);
-  else SGN_WIDE(1);
+  if (cls != RC_CTA) {  // rows of the 32-lane class
+    if (p >= 8) SGN_WIDE(8, true);
+    else SGN_WIDE(4, true);
+  } else if (p >= 8) {
+    SGN_WIDE(8, false);
+  } else if (p >= 4) {
+    SGN_WIDE(4, false);
+  } else if (p >= 2) {
+    SGN_WIDE(2, false);
+  } else {
+    SGN_WIDE(1, false);
+  }
 #undef SGN_WIDE
 }
 

@@ -58,3 +58,43 @@ def test_fp64_dense_path_alone_and_in_a_batch(sg):
         assert res.status == alone.status and res.iters == alone.iters
         assert np.array_equal(res.col, alone.col)
         assert np.array_equal(res.val.view(np.uint64), alone.val.view(np.uint64))
+
+
+# ---------------------------------------------------------------- checks of the iterates
+def _long_rows(n, per, seed):
+    """n <= 1024 rows of about `per` entries each, within one warp's accumulator."""
+    rng = np.random.default_rng(seed)
+    d = np.where(rng.random((n, n)) < per / n, rng.uniform(-0.2, 0.2, (n, n)) / per, 0.0)
+    d[np.arange(n), np.arange(n)] = rng.choice([-1.0, 1.0], n) * (1.0 + rng.random(n))
+    return w.csr_from_dense(d)
+
+
+SUMS = ("resid_k", "xnorm_k", "beta_k")
+MATS = {
+    "tridiagonal": lambda: w.tridiagonal(500),      # 8 lanes a row, or 32 when rows are few
+    "banded": lambda: w.banded(700, 9, 41),         # 16 and 32 lanes
+    "long": lambda: _long_rows(600, 220, 5),        # several warps a row when rows are few
+    "wide": lambda: w.laplacian(40, 2),             # rows of several warps, windows
+    "scattered": lambda: w.sprand_like(1500, 0.006, seed=3),
+}
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("name", sorted(MATS))
+def test_checks_alone_and_in_batches(sg, name, prec):
+    """Alone, beside a few rows (2432 in all or less) and beside many, among
+    matrices of shorter and of longer rows: the sums behind the residual are the
+    same bits. (Without band tiles, whose sums go by 4 columns from a multiple
+    of 4 of the launch.)"""
+    a = MATS[name]()
+    kw = dict(tol=1e-8, filter="exact", prec=prec, dense_frac=2.0, max_iter=8, fp32_band=0)
+    alone = sg.solve(a, **kw)
+    small, long, wide = w.tridiagonal(301), _long_rows(500, 400, 8), w.laplacian(36, 2)
+    for rest in ([small], [long], [w.tridiagonal(5000)], [wide, long, wide]):
+        for mats, at in (([a] + rest, 0), (rest + [a], len(rest))):
+            res = sg.solve_batch(mats, **kw)[at]
+            assert res.status == alone.status and res.iters == alone.iters
+            assert np.array_equal(res.val.view(np.uint64), alone.val.view(np.uint64))
+            for k in SUMS:
+                assert np.array_equal(res.trace[k].view(np.uint64),
+                                      alone.trace[k].view(np.uint64)), (k, len(rest))
