@@ -113,10 +113,11 @@ typedef struct {
   int method;          /* sign_method; SIGN_METHOD_NSF                       */
   /* Schedule: which kernel runs which rows. It changes the speed; every
    * schedule gives the same products bit for bit (each still adds its terms
-   * in ascending k), and so the same iterates and results, except where a
-   * residual within a rounding of a threshold (tol, fp32_until,
-   * switch_resid) is summed in another order. sign_tune_batch picks one by
-   * timing. */
+   * in ascending k), and so the same iterates and results. The sums behind a
+   * residual are the same for every schedule too, except between band tiles
+   * and row-wise rows: there a residual within a rounding of a threshold
+   * (fp32_until, switch_resid) may fall on its other side. sign_tune_batch
+   * picks one by timing. */
   double band_min_eff; /* an FP32 group of 16 rows runs as a band tile when its
                           multiply-adds fill at least this fraction of the
                           tile's FMA slots (>= 0); 0.08                     */
@@ -319,8 +320,12 @@ sign_status sign_dense_product_f64(int M, int N, int K, const double *A, int lda
  * lanes). An admitted request joins the next round of its lane's entry
  * stage beside the requests already in flight; each
  * request's arithmetic is that of a lone sign_solve with the server's
- * options, so its result is the same alone or in any mix. A request whose
- * predicted footprint alone exceeds mem_budget is refused at submission.
+ * options, so its result is the same alone or in any mix, whatever the other
+ * requests are. (In the FP32 stage of the mixed mode a band tile sums a
+ * row's squares by its columns' place in the launch: a residual within a
+ * rounding of fp32_until or switch_resid may fall on its other side there.)
+ * A request whose predicted footprint alone exceeds mem_budget is refused
+ * at submission.
  *
  * Predicted footprint (bytes) of a request, from its n, nnz, Gershgorin
  * gap delta = min_i (|a_ii| - sum_{j!=i} |a_ij|), row-sum bound
