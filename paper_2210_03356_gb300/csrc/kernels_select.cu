@@ -542,31 +542,52 @@ __global__ void k_sel_find0(int nb, const int *active, const MatScalars *ms, Sel
   if (lane == 0) sc.st[m] = st;
 }
 
-// Per-lane square sums of dropped entries: FP32 values exactly in FP32 pairs
-// (scaled by 2^96), FP64 values by FMA.
-struct DropSum {
-  float hi = 0.0f, lo = 0.0f;
-  double d = 0.0;
-  __device__ __forceinline__ void add(float x) { ff_add_sq48(x, hi, lo); }
-  __device__ __forceinline__ void add(double x) { d = __fma_rn(x, x, d); }
-  // the total over each group of W lanes (W divides 32), valid in every lane
-  template <typename T, int W>
-  __device__ __forceinline__ double group_total() {
-    if constexpr (sizeof(T) == 4) {
-      if (!__any_sync(0xffffffffu, hi != 0.0f)) return 0.0;
+// Square sums of a row's dropped entries: 32 partial sums, of every 32nd entry
+// of the row, 32 / W on each of its W lanes (lane gl holds gl, gl + W, ..), added
+// 16 apart, 8 apart and so on, the same additions for every W. FP32 values exactly in
+// FP32 pairs (scaled by 2^96), FP64 values by FMA.
+template <typename T, int W>
+struct DropSum;
+template <int W>
+struct DropSum<float, W> {
+  static constexpr int N = 32 / W;
+  float hi[N] = {}, lo[N] = {};
+  __device__ __forceinline__ void add(float x, int u) { ff_add_sq48(x, hi[u], lo[u]); }
+  __device__ __forceinline__ double total() {  // valid in every lane of the W
+    bool any = false;
 #pragma unroll
-      for (int o = W / 2; o > 0; o >>= 1) {
-        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o, W);
-        const float l2 = __shfl_xor_sync(0xffffffffu, lo, o, W);
-        ff_add(hi, lo, h2, l2);
-      }
-      return (double(hi) + double(lo)) * 0x1p-96;  // exact scaling, one rounding as ldexp
-    } else {
-      if (!__any_sync(0xffffffffu, d != 0.0)) return 0.0;  // FP64 adds only for rows that drop
+    for (int u = 0; u < N; ++u) any = any || hi[u] != 0.0f;
+    if (!__any_sync(0xffffffffu, any)) return 0.0;
 #pragma unroll
-      for (int o = W / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o, W);
-      return d;
+    for (int h = N / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int u = 0; u < h; ++u) ff_add(hi[u], lo[u], hi[u + h], lo[u + h]);
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, hi[0], o, W);
+      const float l2 = __shfl_xor_sync(0xffffffffu, lo[0], o, W);
+      ff_add(hi[0], lo[0], h2, l2);
     }
+    return (double(hi[0]) + double(lo[0])) * 0x1p-96;  // exact scaling, one rounding as ldexp
+  }
+};
+template <int W>
+struct DropSum<double, W> {
+  static constexpr int N = 32 / W;
+  double d[N] = {};
+  __device__ __forceinline__ void add(double x, int u) { d[u] = __fma_rn(x, x, d[u]); }
+  __device__ __forceinline__ double total() {
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < N; ++u) any = any || d[u] != 0.0;
+    if (!__any_sync(0xffffffffu, any)) return 0.0;  // FP64 adds only for rows that drop
+#pragma unroll
+    for (int h = N / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int u = 0; u < h; ++u) d[u] += d[u + h];
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) d[0] += __shfl_xor_sync(0xffffffffu, d[0], o, W);
+    return d[0];
   }
 };
 
@@ -586,7 +607,7 @@ constexpr int EX_U = 4;  // entries per lane of a row loaded at once
 // Per row two bounds on the keys decide: below s_lo an entry is dropped, from
 // s_up on it is kept, between it is a candidate (a NaN is dropped).
 template <typename T, int LPR>
-__global__ void __launch_bounds__(SEL_THREADS)
+__global__ void __launch_bounds__(SEL_THREADS, 4)
     k_sel_extract(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
                   SelScratch sc, int64_t *cnt, double *dropped) {
   after_previous();
@@ -631,7 +652,8 @@ __global__ void __launch_bounds__(SEL_THREADS)
       const int64_t e0 = has ? cr.b[i] : 0, e1 = has ? cr.e[i] : 0;
       const K lo = has ? s_lo[i] : K(0), up = has ? s_up[i] : K(0);
       int c = 0;
-      DropSum ds;
+      DropSum<T, LPR> ds;
+      static_assert(EX_U % (32 / LPR) == 0, "entry u of a lane belongs to partial sum u % N");
       for (int64_t p0 = e0;; p0 += LPR * EX_U) {
         // the warp's rows together (loops of their own would run one by one)
         if (!__any_sync(0xffffffffu, p0 < e1)) break;
@@ -653,7 +675,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
           if (key >= up && key <= KeyT<T>::kInf)
             ++c;
           else
-            ds.add(x[u]);
+            ds.add(x[u], u % ds.N);
         }
         if (n) {  // the row's candidates of this round, in one reservation
           const int m = cr.m[i];
@@ -679,7 +701,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
       if (!cnt) continue;
 #pragma unroll
       for (int o = LPR / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o, LPR);
-      const double d = ds.group_total<T, LPR>();
+      const double d = ds.total();
       if (gl == 0 && has) {
         cnt[r] = c;
         dropped[r] = d;

@@ -98,3 +98,18 @@ def test_checks_alone_and_in_batches(sg, name, prec):
             for k in SUMS:
                 assert np.array_equal(res.trace[k].view(np.uint64),
                                       alone.trace[k].view(np.uint64)), (k, len(rest))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("filt", ["exact", "bound"])
+@pytest.mark.parametrize("name", ["tridiagonal", "banded", "long"])
+def test_dropped_norms_alone_and_in_a_batch(sg, name, filt, prec):
+    """The filter's passes take 32 lanes a row up to 9727 rows, 8 beyond."""
+    a = MATS[name]()
+    kw = dict(tol=1e-8, filter=filt, prec=prec, dense_frac=2.0, fp32_band=0)
+    alone = sg.solve(a, **kw)
+    res = sg.solve_batch([w.tridiagonal(12001), a], **kw)[1]
+    if filt == "exact":
+        assert (alone.trace["fnorm_k"] > 0).any()
+    for k in SUMS + ("tau_k", "fnorm_k"):
+        assert np.array_equal(res.trace[k].view(np.uint64), alone.trace[k].view(np.uint64)), k
