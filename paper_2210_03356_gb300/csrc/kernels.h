@@ -503,11 +503,13 @@ struct DenseBuf {
   float *X_hi, *X_lo, *XT_hi, *XT_lo, *TT_hi, *TT_lo, *P;
   int n, ld;
   int64_t row0;  // the matrix's first row in the stage
+  int64_t grp0;  // row groups of the blocks before it (densify_groups each)
 };
-// The nd dense blocks (leading dimensions up to max_ld) from the stage's CSR:
-// every element of X and X^T is written.
-void launch_densify(int nd, int max_ld, const int64_t *rp, const int32_t *col, const float *val,
-                    const DenseBuf *bufs, cudaStream_t s);
+// The nd dense blocks (leading dimensions up to max_ld, `groups` row groups in
+// all) from the stage's CSR: every element of X and X^T is written.
+int64_t densify_groups(int ld);
+void launch_densify(int nd, int64_t groups, int max_ld, const int64_t *rp, const int32_t *col,
+                    const float *val, const DenseBuf *bufs, cudaStream_t s);
 // dslot[m] = index into bufs for matrices on the dense path, -1 otherwise.
 void launch_dense_resid(int64_t n, const int32_t *seg, const int *dslot, const int64_t *moff,
                         const DenseBuf *bufs, double *part, unsigned long long *tcount,

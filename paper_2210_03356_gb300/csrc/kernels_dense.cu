@@ -311,18 +311,25 @@ __global__ void __launch_bounds__(256)
 // per element. A CTA takes 32 rows, 128 columns at a time, through a
 // shared-memory tile, so that X^T is written in 128-byte rows as well; writing
 // it entry by entry into zeroed blocks took 340 us for a full 4096 x 4096
-// iterate after 80 us of zeroing, now 107 us in all.
+// iterate after 80 us of zeroing, now 107 us in all. blockIdx.x counts the row
+// groups of all blocks (grp0: a block's first), blockIdx.y parts of the columns.
 constexpr int DT_R = 32, DT_C = 128;  // tile rows and columns
 constexpr int DT_LPR = 8;             // lanes reading a row's entries
 __global__ void __launch_bounds__(DT_R *DT_LPR)
-    k_densify(const int64_t *rp, const int32_t *col, const float *val, const DenseBuf *bufs) {
+    k_densify(int nd, const int64_t *rp, const int32_t *col, const float *val,
+              const DenseBuf *bufs) {
   __shared__ float tile[DT_R][DT_C + 1];  // rows and columns both read without conflicts
-  const DenseBuf B = bufs[blockIdx.z];
-  const int i0 = blockIdx.x * DT_R;
+  int dlo = 0, dhi = nd - 1;
+  while (dlo < dhi) {  // the last block with grp0 <= blockIdx.x
+    const int mid = (dlo + dhi + 1) >> 1;
+    if (bufs[mid].grp0 <= int64_t(blockIdx.x)) dlo = mid; else dhi = mid - 1;
+  }
+  const DenseBuf B = bufs[dlo];
+  const int i0 = int(blockIdx.x - B.grp0) * DT_R;
   const int nchunks = (B.ld + DT_C - 1) / DT_C;
   const int per = (nchunks + int(gridDim.y) - 1) / int(gridDim.y);
   const int c0 = blockIdx.y * per, c1 = min(nchunks, c0 + per);
-  if (i0 >= B.ld || c0 >= c1) return;
+  if (c0 >= c1) return;
   const int row = threadIdx.x / DT_LPR, gl = threadIdx.x % DT_LPR;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned gmask = ((1u << DT_LPR) - 1u) << (lane / DT_LPR * DT_LPR);
@@ -567,14 +574,15 @@ void launch_split(int rows, int cols, const float *in, int ldi, int transpose, f
   SGN_LAUNCH_CHECK();
 }
 
-void launch_densify(int nd, int max_ld, const int64_t *rp, const int32_t *col, const float *val,
-                    const DenseBuf *bufs, cudaStream_t s) {
+int64_t densify_groups(int ld) { return (ld + DT_R - 1) / DT_R; }
+
+void launch_densify(int nd, int64_t groups, int max_ld, const int64_t *rp, const int32_t *col,
+                    const float *val, const DenseBuf *bufs, cudaStream_t s) {
   if (nd == 0) return;
   // column parts so that a few row groups still fill the chip
-  const int gx = (max_ld + DT_R - 1) / DT_R, chunks = (max_ld + DT_C - 1) / DT_C;
-  const int want = (152 * 6 + gx * nd - 1) / (gx * nd);
-  const dim3 grid(unsigned(gx), unsigned(std::max(1, std::min(want, chunks))), unsigned(nd));
-  k_densify<<<grid, DT_R * DT_LPR, 0, s>>>(rp, col, val, bufs);
+  const int64_t chunks = (max_ld + DT_C - 1) / DT_C, want = (152 * 6 + groups - 1) / groups;
+  const dim3 grid(unsigned(groups), unsigned(std::max<int64_t>(1, std::min(want, chunks))));
+  k_densify<<<grid, DT_R * DT_LPR, 0, s>>>(nd, rp, col, val, bufs);
   SGN_LAUNCH_CHECK();
 }
 

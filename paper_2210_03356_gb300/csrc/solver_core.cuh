@@ -217,6 +217,7 @@ struct DensePlan {
   std::vector<DenseBuf64> bufs64; // ... or of the DenseBuf64 array (FP64 stage)
   std::vector<int> mat;           // stage slot of each dense matrix
   int nd = 0, max_ld = 0;
+  int64_t groups = 0;             // row groups of the FP32 blocks (densify_groups)
   bool any() const { return nd > 0; }
 };
 
@@ -693,6 +694,8 @@ struct Solver {
         b.n = int(n);
         b.ld = ld;
         b.row0 = st.moff[i];
+        b.grp0 = dp.groups;
+        dp.groups += densify_groups(ld);
         dp.bufs.push_back(b);
       } else {
         DenseBuf64 b = {};
@@ -774,7 +777,7 @@ struct Solver {
       const DenseBuf *bufs = w.dbufs.as<DenseBuf>();
       if (mode == MODE_SQUARE) {
         // every element of X and X^T is written here and of T^T and P by the products
-        launch_densify(dp.nd, dp.max_ld, st.X.d_rp(), st.X.d_col(),
+        launch_densify(dp.nd, dp.groups, dp.max_ld, st.X.d_rp(), st.X.d_col(),
                        reinterpret_cast<const float *>(st.X.val.p), bufs, s);
       }
       {
