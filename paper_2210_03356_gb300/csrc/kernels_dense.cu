@@ -276,12 +276,14 @@ __global__ void __launch_bounds__(256)
 }
 
 // The same of the transpose: out[i][j] = in[j][i], through a 64 x 64 tile, so that
-// both sides move whole 128-byte lines.
+// both sides move whole 128-byte lines. The tiles are numbered along blockIdx.x,
+// those of a column of out's rows first: neither side is bound by a grid's limits.
 constexpr int ST = 64;
 __global__ void __launch_bounds__(256)
     k_split_cols(int rows, int cols, const float *in, int ldi, float *hi, float *lo, int ldo) {
   __shared__ float tile[ST][ST + 1];
-  const int i0 = blockIdx.x * ST, j0 = blockIdx.y * ST;  // of out
+  const unsigned ti = unsigned(rows - 1) / ST + 1;
+  const int i0 = int(blockIdx.x % ti) * ST, j0 = int(blockIdx.x / ti) * ST;  // of out
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
 #pragma unroll
   for (int a = 0; a < ST; a += 8)
@@ -564,8 +566,8 @@ void launch_split(int rows, int cols, const float *in, int ldi, int transpose, f
                   float *lo, int ldo, cudaStream_t s) {
   if (rows <= 0 || ldo <= 0) return;
   if (transpose) {
-    const dim3 grid(unsigned((rows + ST - 1) / ST), unsigned((ldo + ST - 1) / ST));
-    k_split_cols<<<grid, 256, 0, s>>>(rows, cols, in, ldi, hi, lo, ldo);
+    const int64_t tiles = int64_t((rows - 1) / ST + 1) * ((ldo - 1) / ST + 1);
+    k_split_cols<<<unsigned(tiles), 256, 0, s>>>(rows, cols, in, ldi, hi, lo, ldo);
   } else {
     const int64_t total = int64_t(rows) * (ldo / 4);
     k_split_rows<<<int(std::min<int64_t>((total + 255) / 256, 152 * 32)), 256, 0, s>>>(

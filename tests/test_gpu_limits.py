@@ -34,3 +34,13 @@ def test_many_dense_blocks(sg, count):
         assert np.array_equal(col, ref.col)
         assert np.array_equal(val.view(np.uint64), ref.val.view(np.uint64))
     b.close()
+
+
+@pytest.mark.parametrize("m,n,k", [(4, 4, 64), (5, 4, 4194300), (3, 68, 4194312)])
+def test_long_fp32_product(sg, m, n, k):
+    """Entries of -1, 0 and 1: every partial sum is an integer below 2^24, exact."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(k)
+    a = torch.randint(-1, 2, (m, k), device="cuda", generator=g).float()
+    b = torch.randint(-1, 2, (k, n), device="cuda", generator=g).float()
+    assert torch.equal(sg.dense_product(a, b).double(), a.double() @ b.double())
