@@ -315,7 +315,7 @@ void launch_budget_x2(int nb, const int64_t *moff, const double *x2, double swit
 // The values a threshold is selected over: row r holds entries [rs[r], re[r])
 // of matrix seg[r], whose rows start at moff[m]; rs == nullptr means one flat
 // array of flat_nnz values of matrix 0, cut into rows of kFlatRow values.
-// cshift: the candidate room of a matrix is its entry count >> cshift.
+// cshift: the candidate room of a matrix is its entry count >> cshift, at first.
 constexpr int64_t kFlatRow = 1024;
 struct SelRows {
   int64_t nrows;
@@ -330,8 +330,8 @@ struct SelRows {
 // Threshold selection (EXACT) for every active matrix; writes ms[m].tau.
 // The scratch holds, 256-byte aligned each: the level-0 histograms
 // (kSelBuckets 128-bit sums per matrix), one minimum per matrix, one select
-// state of at most kSelStateBytes per matrix, the overflow flag and the
-// candidate counts, and room for cap candidates (8-byte key + row).
+// state of at most kSelStateBytes per matrix, two flags, the candidate counts
+// and regions, and room for cap candidates (8-byte key + row).
 // kSelBuckets: the buckets from b / sqrt(2^62) to b, 16 per octave, and one
 // sum below.
 constexpr int kSelBuckets = 512;
@@ -339,16 +339,18 @@ constexpr size_t kSelStateBytes = 64;
 constexpr size_t sel_align(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t select_scratch_bytes(int nb, int64_t cap) {
   return sel_align(size_t(nb) * kSelBuckets * 2 * 8) + sel_align(size_t(nb) * 8) +
-         sel_align(size_t(nb) * kSelStateBytes) + sel_align(size_t(nb + 1) * 8) +
+         sel_align(size_t(nb) * kSelStateBytes) + sel_align((3 * size_t(nb) + 2) * 8) +
          sel_align(size_t(cap > 0 ? cap : 1) * 8) + sel_align(size_t(cap > 0 ? cap : 1) * 4);
 }
 // nvals: the values (or slots) of all rows, which sizes the launches. With row
 // lists the entries per matrix are counted into ms[m].nnz_bar; for a flat array
 // nnz_bar holds them already.
-// cand_cap is the scratch's candidate room, at least nvals >> R.cshift. When a
-// matrix has more candidates than its room, *select_overflow is set and the
-// thresholds (and counts) are not valid: the caller selects again with room
-// for every value (cshift 0). With cshift 0 it cannot happen.
+// cand_cap is the scratch's candidate room, at least nvals >> R.cshift, shared by
+// all matrices: one with more candidates than its entries >> cshift has them
+// taken again in a second pass. When there are more than cand_cap in all,
+// *select_overflow is set and the thresholds (and counts) are not valid: the
+// caller selects again with room for every value (cshift 0), where it cannot
+// happen.
 // cnt, dropped (nullable, R.nrows each; R must have rows rs/re): the
 // filter's per-row kept counts and dropped sums of squares under the
 // selected tau, as launch_filter_count gives them, except that the squares of

@@ -64,7 +64,10 @@ struct SelScratch {
   unsigned long long *minabove;  // nb
   SelState *st;                  // nb
   unsigned long long *overflow;  // 1: set when a matrix has more candidates than room
+  unsigned long long *redo;      // 1: the candidates are taken again, into exact regions
   unsigned long long *ncand;     // nb; may count past the room
+  unsigned long long *cbase;     // nb: matrix m's candidates lie at [cbase, cbase + croom)
+  unsigned long long *croom;     // nb
   unsigned long long *cand;      // cap
   int *cand_r;                   // cap
 };
@@ -83,22 +86,15 @@ SelScratch carve(void *base, int nb, int64_t cap) {
   s.st = reinterpret_cast<SelState *>(p);
   p += align_up(size_t(nb) * kSelStateBytes);
   s.overflow = reinterpret_cast<unsigned long long *>(p);
-  s.ncand = s.overflow + 1;
-  p += align_up(size_t(nb + 1) * 8);
+  s.redo = s.overflow + 1;
+  s.ncand = s.overflow + 2;
+  s.cbase = s.ncand + nb;
+  s.croom = s.cbase + nb;
+  p += align_up((3 * size_t(nb) + 2) * 8);
   s.cand = reinterpret_cast<unsigned long long *>(p);
   p += align_up(size_t(cap > 0 ? cap : 1) * 8);
   s.cand_r = reinterpret_cast<int *>(p);
   return s;
-}
-
-// Matrix m's candidate region: its entries start at slot rs[moff[m]], and the
-// region is that range of slots (shifted right by cshift when the room is a
-// sixteenth of the slots), so the regions of different matrices are disjoint.
-__device__ __forceinline__ unsigned long long cand_base(const SelRows &R, int m) {
-  return R.rs ? (unsigned long long)(R.rs[R.moff[m]] >> R.cshift) : 0ULL;
-}
-__device__ __forceinline__ unsigned long long cand_room(const SelRows &R, const MatScalars &ms) {
-  return (unsigned long long)(ms.nnz_bar >> R.cshift);
 }
 
 // Rows of the values to select over: row r holds entries [rs[r], re[r]) and
@@ -255,7 +251,8 @@ __device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, 
 // q >= 1 (the key of 2^(e - 31 - 1023)) and the pivot's bucket: a power of two
 // fraction below b / sqrt(nnz_bar), so that no rounding lifts it above. b = 0,
 // +inf or NaN: no key is summed (tiny = all ones), every q counts as 0.
-// Clears the matrix's histogram, minimum and candidate count.
+// Clears the matrix's histogram, minimum and candidate count, and sets its
+// candidate region.
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
     k_sel_prepare(SelRows R, MatScalars *ms, SelScratch sc) {
   after_previous();
@@ -275,8 +272,12 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
   if (q != 0 || threadIdx.x) return;
   sc.minabove[m] = ~0ULL;
   sc.ncand[m] = 0ULL;
-  if (m == 0) *sc.overflow = 0ULL;
+  if (m == 0) *sc.overflow = *sc.redo = 0ULL;
   if (R.rs) ms[m].nnz_bar = int64_t(s_cnt);
+  // the candidate region: the matrix's range of slots, shifted right by cshift
+  // when the room is a fraction of the slots, so the regions are disjoint
+  sc.cbase[m] = R.rs ? (unsigned long long)(R.rs[R.moff[m]] >> R.cshift) : 0ULL;
+  sc.croom[m] = (unsigned long long)(ms[m].nnz_bar >> R.cshift);
   const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
   const int e = int(bkey >> 52);
   if (bkey == 0ULL || e >= 0x7FF) {  // b <= 0 (sign bit) is caught here as well
@@ -609,8 +610,9 @@ constexpr int EX_U = 4;  // entries per lane of a row loaded at once
 template <typename T, int LPR>
 __global__ void __launch_bounds__(SEL_THREADS, 4)
     k_sel_extract(SelRows R, int rpc, const int *active, const T *val, const MatScalars *ms,
-                  SelScratch sc, int64_t *cnt, double *dropped) {
+                  SelScratch sc, int64_t *cnt, double *dropped, const unsigned long long *run) {
   after_previous();
+  if (run && *run == 0ULL) return;
   using K = typename KeyT<T>::K;
   __shared__ ChunkRows cr;
   __shared__ K s_lo[RPC], s_up[RPC];
@@ -632,8 +634,8 @@ __global__ void __launch_bounds__(SEL_THREADS, 4)
         const K top = KeyT<T>::ceil_key(next);
         const K above = KeyT<T>::floor_key((unsigned long long)__double_as_longlong(ms[mt].b)) + 1;
         s_up[t] = above < top ? above : top;
-        s_cbase[t] = cand_base(R, mt);
-        s_room[t] = cand_room(R, ms[mt]);
+        s_cbase[t] = sc.cbase[mt];
+        s_room[t] = sc.croom[mt];
       } else {
         const unsigned long long above = sc.minabove[mt];  // tau without a crossing
         s_lo[t] = s_up[t] = KeyT<T>::ceil_key(above == ~0ULL ? INF_KEY : above);
@@ -710,6 +712,43 @@ __global__ void __launch_bounds__(SEL_THREADS, 4)
   }
 }
 
+// After a first pass with regions of a fraction of the entries (cshift > 0): if
+// a matrix had more candidates than its region, the counts, which are complete,
+// become the regions of a second pass, as long as they fit the room in all.
+// One CTA; only stages above 2^28 slots come here.
+constexpr int REG_T = 1024;
+__global__ void __launch_bounds__(REG_T) k_sel_regions(int nb, unsigned long long cap,
+                                                       SelScratch sc) {
+  after_previous();
+  __shared__ unsigned long long s[REG_T];
+  if (*sc.overflow == 0ULL) return;
+  const int t = threadIdx.x, per = (nb - 1) / REG_T + 1;
+  const int m0 = min(nb, t * per), m1 = min(nb, m0 + per);
+  unsigned long long sum = 0;
+  for (int m = m0; m < m1; ++m) sum += sc.ncand[m];
+  s[t] = sum;
+  __syncthreads();
+  for (int o = 1; o < REG_T; o <<= 1) {  // inclusive prefix sums
+    const unsigned long long y = t >= o ? s[t - o] : 0ULL;
+    __syncthreads();
+    s[t] += y;
+    __syncthreads();
+  }
+  if (s[REG_T - 1] > cap) return;  // the caller selects again with room for every value
+  unsigned long long at = s[t] - sum;
+  for (int m = m0; m < m1; ++m) {
+    const unsigned long long k = sc.ncand[m];
+    sc.cbase[m] = at;
+    sc.croom[m] = k;
+    sc.ncand[m] = 0ULL;
+    at += k;
+  }
+  if (t == 0) {
+    *sc.overflow = 0ULL;
+    *sc.redo = 1ULL;
+  }
+}
+
 // sums[m] = the dropped squares of matrix m's rows plus, with the select's
 // scratch, those of the dropped candidates: the exact sum of their q
 // (the select's sum below tau minus its sum below the crossing bucket) in
@@ -775,7 +814,7 @@ __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
     }
     return;
   }
-  const unsigned long long room = cand_room(R, ms[m]), cb = cand_base(R, m);
+  const unsigned long long room = sc.croom[m], cb = sc.cbase[m];
   const unsigned long long total = sc.ncand[m] < room ? sc.ncand[m] : room;
   const bool one = total <= DG_ONE;
   if (one && rank != 0) return;
@@ -1060,9 +1099,9 @@ static void sel_pass(int64_t nrows, int64_t nvals, F f) {
 }
 
 template <typename T>
-static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *active, const T *val,
-                         MatScalars *ms, const SelScratch &sc, int64_t *cnt, double *dropped,
-                         cudaStream_t s) {
+static void select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
+                         const int *active, const T *val, MatScalars *ms, const SelScratch &sc,
+                         int64_t *cnt, double *dropped, cudaStream_t s) {
   {
     ProfScope ps(KC_SEL_HIST, s, 0.0, 0.0);
     launch_next(k_sel_prepare, unsigned(nb) * RED_C, RED_T, 0, s, R, ms, sc);
@@ -1073,10 +1112,17 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, const int *act
   }
   {
     ProfScope ps(KC_SEL_EXTRACT, s, 0.0, 0.0);
-    sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
-      launch_next(k_sel_extract<T, lpr.value>, g, SEL_THREADS, 0, s, R, rpc, active, val, ms, sc,
-                  cnt, dropped);
-    });
+    auto extract = [&](const unsigned long long *run) {
+      sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
+        launch_next(k_sel_extract<T, lpr.value>, g, SEL_THREADS, 0, s, R, rpc, active, val, ms, sc,
+                    cnt, dropped, run);
+      });
+    };
+    extract(nullptr);
+    if (R.cshift > 0) {
+      launch_next(k_sel_regions, 1, REG_T, 0, s, nb, (unsigned long long)cand_cap, sc);
+      extract(sc.redo);
+    }
   }
   ProfScope ps(KC_SEL_DIGITS, s, 0.0, 0.0);
   launch_next(k_sel_digits<sizeof(T) == 4 ? 3 : 6>, unsigned(nb) * DG_C, DG_T, 0, s, R, active, sc,
@@ -1088,11 +1134,11 @@ void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_c
                          void *scratch, int64_t *cnt, double *dropped, cudaStream_t s) {
   const SelScratch sc = carve(scratch, nb, cand_cap);
   if (val_f32)
-    select_exact<float>(nb, R, nvals, active, static_cast<const float *>(val), ms, sc, cnt, dropped,
-                        s);
+    select_exact<float>(nb, R, nvals, cand_cap, active, static_cast<const float *>(val), ms, sc,
+                        cnt, dropped, s);
   else
-    select_exact<double>(nb, R, nvals, active, static_cast<const double *>(val), ms, sc, cnt,
-                         dropped, s);
+    select_exact<double>(nb, R, nvals, cand_cap, active, static_cast<const double *>(val), ms, sc,
+                         cnt, dropped, s);
 }
 
 void launch_drop_sums(int nb, const int64_t *moff, const double *dropped, const int *active,

@@ -1214,8 +1214,9 @@ struct Solver {
     int nb = int(st.mats.size());
     if (o.filter == SIGN_FILTER_EXACT) {
       const int64_t big = int64_t(1) << 28;
-      w.sel_shift = full_room || in.slots <= big ? 0 : 4;
-      const int64_t cap = w.sel_shift ? std::max(big, in.slots >> w.sel_shift) : in.slots;
+      const int64_t cap = full_room ? in.slots : std::min(in.slots, std::max(big, in.slots / 16));
+      w.sel_shift = 0;  // the largest regions that the room holds for every matrix at once
+      while ((in.slots >> w.sel_shift) > cap) ++w.sel_shift;
       w.sel.ensure(select_scratch_bytes(nb, cap), s);
       w.dropped.ensure(sizeof(double) * size_t(N > 0 ? N : 1), s);
       w.cnt.ensure(sizeof(int64_t) * size_t(N > 0 ? N : 1), s);
