@@ -23,6 +23,7 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/sign.h"
@@ -48,6 +49,12 @@ constexpr size_t BIG_BUFFER = size_t(4) << 30;
 constexpr int64_t FEW_ROWS = 152 * 16;
 // From this mean length of B's rows several warps share each of the few rows.
 constexpr double SHARED_B = 192.0;
+// Readbacks of more bytes are copies, one CTA writes the others. A solve of 1024
+// matrices of order 16 (a readback of 131 KB): 2.30 ms written, 2.34 copied; of
+// 2048: 3.70 and 3.67; of 8192: 12.7 and 12.4.
+constexpr size_t PUBLISH_MAX = size_t(192) << 10;
+// Polls of a readback before the waiting thread lets others run.
+constexpr unsigned SPINS_BEFORE_YIELD = 4096;
 
 // ------------------------------------------------------------------ CSR
 template <typename T>
@@ -370,20 +377,38 @@ struct Solver {
   // Reads device memory back into the host mirror and waits for the stream up
   // to here. A kernel writes the mirror (mapped memory) and a flag that is polled:
   // about 4 us less GPU idle time per wait than a copy and
-  // cudaStreamSynchronize, four waits an iteration. The stream is queried from
-  // time to time, so that an error ends the wait.
+  // cudaStreamSynchronize, four waits an iteration. The poll follows the device's
+  // scheduling flag as cudaStreamSynchronize does: it gives the core away at
+  // every turn (yield), never (spin), or, by default, once the wait is longer
+  // than most; a process that asked for blocking waits, and more than one CTA
+  // should write, get a copy and a synchronize. The stream is queried from time to
+  // time, so that an error ends the wait.
   void fetch(void *dst, const void *src, size_t bytes) {
+    unsigned sched = 0;
+    SGN_CUDA(cudaGetDeviceFlags(&sched));
+    sched &= cudaDeviceScheduleMask;
+    if (bytes > PUBLISH_MAX || sched == cudaDeviceScheduleBlockingSync) {
+      SGN_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+      wait();
+      return;
+    }
     const unsigned seq = ++hm.seq;
     launch_publish(src, dst, bytes, hm.flag, seq, s);
     prof_sync_point(s);
-    for (unsigned spin = 1; __atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) != seq; ++spin)
+    const unsigned busy = sched == cudaDeviceScheduleYield  ? 0u
+                          : sched == cudaDeviceScheduleSpin ? ~0u
+                                                            : SPINS_BEFORE_YIELD;
+    for (unsigned spin = 1; __atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) != seq; ++spin) {
       if (spin % 65536 == 0) {
         const cudaError_t e = cudaStreamQuery(s);
-        if (e == cudaErrorNotReady) continue;
-        SGN_CUDA(e);
-        if (__atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) == seq) break;
-        throw Error(SIGN_ECUDA, "a readback did not reach the host");
+        if (e != cudaErrorNotReady) {
+          SGN_CUDA(e);
+          if (__atomic_load_n(hm.flag, __ATOMIC_ACQUIRE) == seq) break;
+          throw Error(SIGN_ECUDA, "a readback did not reach the host");
+        }
       }
+      if (spin > busy) std::this_thread::yield();
+    }
     stg.used = 0;
   }
   // h2d from host memory of any kind, through the pinned arena.
