@@ -519,76 +519,118 @@ __global__ void k_gather_offsets(int nb, const int64_t *moff, const int64_t *rp,
 
 // out[m] = the sum of part over matrix m's rows.
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
-    k_seg_reduce(const int64_t *moff, const double *part, double *out) {
+    k_seg_reduce(int nb, int per, const int64_t *moff, const double *part, double *out) {
   after_previous();
   __shared__ double sm[RED_T];
   cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
-  const int t = q * RED_LANES + threadIdx.x;
-  cl.sync();  // CTA 0 has started: its shared memory may be written
-  *cl.map_shared_rank(&sm[t], 0) = seg_partial(part, 1, 0, moff[m], moff[m + 1], t);
-  cl.sync();
-  if (q != 0) return;
-  seg_tree(sm);
-  if (threadIdx.x == 0) out[m] = sm[0];
+  const int q = int(cl.block_rank()), t = q * RED_LANES + threadIdx.x;
+  auto solo = [&](int m) {
+    seg_sum_solo(sm, part, 1, 0, moff[m], moff[m + 1]);
+    if (threadIdx.x == 0) out[m] = sm[0];
+  };
+  auto joint = [&](int m) {
+    cl.sync();  // CTA 0 has started, and read its sums: its shared memory may be written
+    *cl.map_shared_rank(&sm[t], 0) = seg_partial(part, 1, 0, moff[m], moff[m + 1], t);
+    cl.sync();
+    if (q != 0) return;
+    seg_tree(sm);
+    if (threadIdx.x == 0) out[m] = sm[0];
+  };
+  cluster_each(nb, per, moff, blockIdx.x / RED_C, q, solo, joint);
 }
 
-// The check of a round in one launch: per matrix the sums of the two columns of
-// part (warps 0 and 1 of each CTA), the entries of T (warp 2) and from them r,
-// x, beta and b.
-__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(3 * RED_LANES)
-    k_check_scalars(const int64_t *moff, const double *part, const int64_t *rs, const int64_t *re,
-                    double c4, double tol_stage, double switch_resid, MatScalars *ms,
-                    int64_t *nnz) {
-  after_previous();
-  __shared__ double sm[2][RED_T];
-  __shared__ unsigned long long s_cnt;
-  cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / RED_C, q = int(cl.block_rank()), c = threadIdx.x / RED_LANES;
-  const int t = q * RED_LANES + lane_id();
-  if (threadIdx.x == 0) s_cnt = 0ULL;
-  cl.sync();  // CTA 0 has started: its shared memory may be written
-  const int64_t b = moff[m], e = moff[m + 1];
-  if (c < 2) {
-    *cl.map_shared_rank(&sm[c][t], 0) = seg_partial(part, 2, c, b, e, t);
-  } else {
-    const unsigned long long k = seg_entries(rs, re, b, e, t, RED_T);
-    if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
-  }
-  cl.sync();
-  if (q != 0) return;
-  if (c < 2) seg_tree(sm[c]);
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double sn = __dsqrt_rn(double(e - b));
-  const double r = __ddiv_rn(__dsqrt_rn(sm[0][0]), sn);
-  const double x = __ddiv_rn(__dsqrt_rn(sm[1][0]), sn);
+// r, x, beta and b of a matrix of n rows from its sums of squares, and its entries.
+__device__ __forceinline__ void put_scalars(int64_t n, double rsum, double xsum, int64_t entries,
+                                            double c4, double tol_stage, double switch_resid,
+                                            MatScalars &ms, int64_t &nnz) {
+  const double sn = __dsqrt_rn(double(n));
+  const double r = __ddiv_rn(__dsqrt_rn(rsum), sn);
+  const double x = __ddiv_rn(__dsqrt_rn(xsum), sn);
   double beta;
   if (r >= switch_resid)
     beta = __dmul_rn(c4, tol_stage);
   else
     beta = __ddiv_rn(__dmul_rn(__dmul_rn(0.75, r), r),
                      __dadd_rn(__dmul_rn(3.0, x), __dmul_rn(__dmul_rn(x, x), x)));
-  ms[m].r = r;
-  ms[m].x = x;
-  ms[m].beta = beta;
-  ms[m].b = __dmul_rn(sn, beta);
-  nnz[m] = int64_t(s_cnt);
+  ms.r = r;
+  ms.x = x;
+  ms.beta = beta;
+  ms.b = __dmul_rn(sn, beta);
+  nnz = entries;
+}
+
+// The check of a round in one launch: per matrix the sums of the two columns of
+// part (warps 0 and 1 of each CTA), the entries of T (warp 2) and from them r,
+// x, beta and b.
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(3 * RED_LANES)
+    k_check_scalars(int nb, int per, const int64_t *moff, const double *part, const int64_t *rs,
+                    const int64_t *re, double c4, double tol_stage, double switch_resid,
+                    MatScalars *ms, int64_t *nnz) {
+  after_previous();
+  __shared__ double sm[2][RED_T];
+  __shared__ unsigned long long s_cnt;
+  cg::cluster_group cl = cg::this_cluster();
+  const int q = int(cl.block_rank()), c = threadIdx.x / RED_LANES;
+  const int t = q * RED_LANES + lane_id();
+  auto put = [&](int m) {
+    put_scalars(moff[m + 1] - moff[m], sm[0][0], sm[1][0], int64_t(s_cnt), c4, tol_stage,
+                switch_resid, ms[m], nnz[m]);
+  };
+  auto solo = [&](int m) {
+    const int64_t b = moff[m], e = moff[m + 1];
+    if (c < 2) {
+      seg_sum_solo(sm[c], part, 2, c, b, e);
+    } else {
+      const unsigned long long k = seg_entries(rs, re, b, e, lane_id(), 32);
+      if (lane_id() == 0) s_cnt = k;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) put(m);
+  };
+  auto joint = [&](int m) {
+    if (threadIdx.x == 0) s_cnt = 0ULL;
+    cl.sync();  // CTA 0 has started, and read its sums: its shared memory may be written
+    const int64_t b = moff[m], e = moff[m + 1];
+    if (c < 2) {
+      *cl.map_shared_rank(&sm[c][t], 0) = seg_partial(part, 2, c, b, e, t);
+    } else {
+      const unsigned long long k = seg_entries(rs, re, b, e, t, RED_T);
+      if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
+    }
+    cl.sync();
+    if (q != 0) return;
+    if (c < 2) seg_tree(sm[c]);
+    __syncthreads();
+    if (threadIdx.x == 0) put(m);
+  };
+  cluster_each(nb, per, moff, blockIdx.x / RED_C, q, solo, joint);
 }
 
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
-    k_seg_count(const int64_t *moff, const int64_t *rs, const int64_t *re, int64_t *out) {
+    k_seg_count(int nb, int per, const int64_t *moff, const int64_t *rs, const int64_t *re,
+                int64_t *out) {
   after_previous();
-  __shared__ unsigned long long sm;  // CTA 0: the matrix's count
+  __shared__ unsigned long long sm;  // the matrix's count (joint: CTA 0's)
   cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
-  if (threadIdx.x == 0) sm = 0ULL;
-  cl.sync();
-  const unsigned long long k = seg_entries(rs, re, moff[m], moff[m + 1], q * RED_T + threadIdx.x,
-                                           RED_C * RED_T);
-  if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&sm, 0), k);
-  cl.sync();
-  if (q == 0 && threadIdx.x == 0) out[m] = int64_t(sm);
+  const int q = int(cl.block_rank());
+  auto solo = [&](int m) {
+    if (threadIdx.x == 0) sm = 0ULL;
+    __syncthreads();
+    const unsigned long long k = seg_entries(rs, re, moff[m], moff[m + 1], threadIdx.x, RED_T);
+    if (lane_id() == 0 && k) atomicAdd(&sm, k);
+    __syncthreads();
+    if (threadIdx.x == 0) out[m] = int64_t(sm);
+  };
+  auto joint = [&](int m) {
+    if (threadIdx.x == 0) sm = 0ULL;
+    cl.sync();
+    const unsigned long long k = seg_entries(rs, re, moff[m], moff[m + 1], q * RED_T + threadIdx.x,
+                                             RED_C * RED_T);
+    if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&sm, 0), k);
+    cl.sync();
+    if (q == 0 && threadIdx.x == 0) out[m] = int64_t(sm);
+  };
+  cluster_each(nb, per, moff, blockIdx.x / RED_C, q, solo, joint);
 }
 
 // One CTA per extracted matrix: rebased row pointers, shifted columns,
@@ -655,7 +697,8 @@ void launch_compact_rows(int64_t n, const int64_t *rs, const int64_t *re, const 
 void launch_seg_count(int nb, const int64_t *moff, const int64_t *rs, const int64_t *re,
                       int64_t *out, cudaStream_t s) {
   if (nb == 0) return;
-  launch_next(k_seg_count, unsigned(nb) * RED_C, RED_T, 0, s, moff, rs, re, out);
+  launch_next(k_seg_count, cluster_ctas(nb), RED_T, 0, s, nb, cluster_matrices(nb), moff, rs, re,
+              out);
 }
 
 void launch_extract(int nblocks, const ExtractBlock *blocks, int64_t max_entries, cudaStream_t s) {
@@ -779,15 +822,16 @@ void launch_gather_offsets(int nb, const int64_t *moff, const int64_t *rp, int64
 void launch_seg_reduce(int nb, const int64_t *moff, const double *part, double *out,
                        cudaStream_t s) {
   if (nb == 0) return;
-  launch_next(k_seg_reduce, unsigned(nb) * RED_C, RED_LANES, 0, s, moff, part, out);
+  launch_next(k_seg_reduce, cluster_ctas(nb), RED_LANES, 0, s, nb, cluster_matrices(nb), moff, part,
+              out);
 }
 
 void launch_check_scalars(int nb, const int64_t *moff, const double *part, const int64_t *rs,
                           const int64_t *re, double c4, double tol_stage, double switch_resid,
                           MatScalars *ms, int64_t *nnz, cudaStream_t s) {
   if (nb == 0) return;
-  launch_next(k_check_scalars, unsigned(nb) * RED_C, 3 * RED_LANES, 0, s, moff, part, rs, re, c4,
-              tol_stage, switch_resid, ms, nnz);
+  launch_next(k_check_scalars, cluster_ctas(nb), 3 * RED_LANES, 0, s, nb, cluster_matrices(nb), moff,
+              part, rs, re, c4, tol_stage, switch_resid, ms, nnz);
 }
 
 }  // namespace sgn

@@ -246,34 +246,18 @@ __device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, 
   return qval<T>(wide, eb);
 }
 
-// Per matrix, by a cluster: nnz_bar = its entries (row lists), e (the biased
-// exponent of b, 1 for a subnormal b), Q = q(b), the smallest key with
-// q >= 1 (the key of 2^(e - 31 - 1023)) and the pivot's bucket: a power of two
-// fraction below b / sqrt(nnz_bar), so that no rounding lifts it above. b = 0,
-// +inf or NaN: no key is summed (tiny = all ones), every q counts as 0.
-// Clears the matrix's histogram, minimum and candidate count, and sets its
-// candidate region.
-__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
-    k_sel_prepare(SelRows R, MatScalars *ms, SelScratch sc) {
-  after_previous();
-  __shared__ unsigned long long s_cnt;  // CTA 0: the matrix's entries
-  cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
-  if (threadIdx.x == 0) s_cnt = 0ULL;
-  cl.sync();
-  for (int t = q * RED_T + threadIdx.x; t < 2 * NB0; t += RED_C * RED_T)
-    sc.hist0[size_t(m) * NB0 * 2 + t] = 0ULL;
-  if (R.rs) {
-    const unsigned long long k = seg_entries(R.rs, R.re, R.moff[m], R.moff[m + 1],
-                                             q * RED_T + threadIdx.x, RED_C * RED_T);
-    if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
-  }
-  cl.sync();
-  if (q != 0 || threadIdx.x) return;
+// A matrix of `entries` stored values (row lists; a flat array's nnz_bar is set):
+// nnz_bar, e (the biased exponent of b, 1 for a subnormal b), Q = q(b), the
+// smallest key with q >= 1 (the key of 2^(e - 31 - 1023)) and the pivot's bucket: a
+// power of two fraction below b / sqrt(nnz_bar), so that no rounding lifts it above.
+// b = 0, +inf or NaN: no key is summed (tiny = all ones), every q counts as 0.
+// Clears the matrix's minimum and candidate count, and sets its candidate region.
+__device__ __forceinline__ void prepare_matrix(int m, const SelRows &R, unsigned long long entries,
+                                               MatScalars *ms, const SelScratch &sc) {
   sc.minabove[m] = ~0ULL;
   sc.ncand[m] = 0ULL;
   if (m == 0) *sc.overflow = *sc.redo = 0ULL;
-  if (R.rs) ms[m].nnz_bar = int64_t(s_cnt);
+  if (R.rs) ms[m].nnz_bar = int64_t(entries);
   // the candidate region: the matrix's range of slots, shifted right by cshift
   // when the room is a fraction of the slots, so the regions are disjoint
   sc.cbase[m] = R.rs ? (unsigned long long)(R.rs[R.moff[m]] >> R.cshift) : 0ULL;
@@ -295,6 +279,42 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
   const double pivot = ms[m].b / sqrt(double(N)) * 0.999;
   const int base = int((unsigned long long)__double_as_longlong(pivot) >> 48);
   ms[m].sel_base = pivot < 0x1p-1000 && base > 0 ? base - 1 : base;  // rounding near underflow
+}
+
+// prepare_matrix of every matrix, its entries counted and its histogram cleared by a
+// cluster or (many small matrices) by a CTA. A flat array is one matrix (R.moff null).
+__global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_T)
+    k_sel_prepare(int nb, int per, SelRows R, MatScalars *ms, SelScratch sc) {
+  after_previous();
+  __shared__ unsigned long long s_cnt;  // the matrix's entries (joint: CTA 0's)
+  cg::cluster_group cl = cg::this_cluster();
+  const int q = int(cl.block_rank());
+  auto clear = [&](int m, int first, int step) {
+    for (int t = first; t < 2 * NB0; t += step) sc.hist0[size_t(m) * NB0 * 2 + t] = 0ULL;
+  };
+  auto solo = [&](int m) {
+    if (threadIdx.x == 0) s_cnt = 0ULL;
+    __syncthreads();
+    clear(m, threadIdx.x, RED_T);
+    const unsigned long long k =
+        seg_entries(R.rs, R.re, R.moff[m], R.moff[m + 1], threadIdx.x, RED_T);
+    if (lane_id() == 0 && k) atomicAdd(&s_cnt, k);
+    __syncthreads();
+    if (threadIdx.x == 0) prepare_matrix(m, R, s_cnt, ms, sc);
+  };
+  auto joint = [&](int m) {
+    if (threadIdx.x == 0) s_cnt = 0ULL;
+    cl.sync();
+    clear(m, q * RED_T + threadIdx.x, RED_C * RED_T);
+    if (R.rs) {
+      const unsigned long long k = seg_entries(R.rs, R.re, R.moff[m], R.moff[m + 1],
+                                               q * RED_T + threadIdx.x, RED_C * RED_T);
+      if (lane_id() == 0 && k) atomicAdd(cl.map_shared_rank(&s_cnt, 0), k);
+    }
+    cl.sync();
+    if (q == 0 && threadIdx.x == 0) prepare_matrix(m, R, s_cnt, ms, sc);
+  };
+  cluster_each(nb, per, R.moff, blockIdx.x / RED_C, q, solo, joint);
 }
 
 // (lo, hi) += (alo, ahi) atomically in memory; exact, order-independent.
@@ -755,30 +775,37 @@ __global__ void __launch_bounds__(REG_T) k_sel_regions(int nb, unsigned long lon
 // grid steps 2^(2e - 62). A candidate's magnitude is at least b / sqrt(1.1
 // nnz) (a bucket spans a factor 2^(1/16)), so its q is above 2^62 / (1.1 nnz)
 // and its flooring to an integer is far below the FP64 rounding of the sum.
+__device__ __forceinline__ double drop_sum(int m, double sum, const int *active, int exact,
+                                           const SelScratch &sc, const MatScalars *ms) {
+  if (!(exact && active[m] && sc.st[m].found)) return sum;
+  const SelState st = sc.st[m];
+  const unsigned long long lo = st.below_lo - st.below0_lo;
+  const unsigned long long hi =
+      st.below_hi - st.below0_hi - (st.below_lo < st.below0_lo ? 1ULL : 0ULL);
+  const double qs = __fma_rn(double(hi), 18446744073709551616.0, double(lo));
+  return __dadd_rn(sum, ldexp(qs, 2 * (ms[m].sel_e - 1023) - 62));
+}
+
 __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
-    k_drop_sums(const int64_t *moff, const double *dropped, const int *active, int exact,
-                SelScratch sc, const MatScalars *ms, double *sums) {
+    k_drop_sums(int nb, int per, const int64_t *moff, const double *dropped, const int *active,
+                int exact, SelScratch sc, const MatScalars *ms, double *sums) {
   after_previous();
   __shared__ double sm[RED_T];
   cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / RED_C, q = int(cl.block_rank());
-  const int t = q * RED_LANES + threadIdx.x;
-  cl.sync();  // CTA 0 has started: its shared memory may be written
-  *cl.map_shared_rank(&sm[t], 0) = seg_partial(dropped, 1, 0, moff[m], moff[m + 1], t);
-  cl.sync();
-  if (q != 0) return;
-  seg_tree(sm);
-  if (threadIdx.x != 0) return;
-  double sum = sm[0];
-  if (exact && active[m] && sc.st[m].found) {
-    const SelState st = sc.st[m];
-    const unsigned long long lo = st.below_lo - st.below0_lo;
-    const unsigned long long hi =
-        st.below_hi - st.below0_hi - (st.below_lo < st.below0_lo ? 1ULL : 0ULL);
-    const double qs = __fma_rn(double(hi), 18446744073709551616.0, double(lo));
-    sum = __dadd_rn(sum, ldexp(qs, 2 * (ms[m].sel_e - 1023) - 62));
-  }
-  sums[m] = sum;
+  const int q = int(cl.block_rank()), t = q * RED_LANES + threadIdx.x;
+  auto solo = [&](int m) {
+    seg_sum_solo(sm, dropped, 1, 0, moff[m], moff[m + 1]);
+    if (threadIdx.x == 0) sums[m] = drop_sum(m, sm[0], active, exact, sc, ms);
+  };
+  auto joint = [&](int m) {
+    cl.sync();  // CTA 0 has started, and read its sums: its shared memory may be written
+    *cl.map_shared_rank(&sm[t], 0) = seg_partial(dropped, 1, 0, moff[m], moff[m + 1], t);
+    cl.sync();
+    if (q != 0) return;
+    seg_tree(sm);
+    if (threadIdx.x == 0) sums[m] = drop_sum(m, sm[0], active, exact, sc, ms);
+  };
+  cluster_each(nb, per, moff, blockIdx.x / RED_C, q, solo, joint);
 }
 
 // The digits below the crossing bucket, tau and the kept candidates' counts of
@@ -787,42 +814,41 @@ __global__ void __cluster_dims__(RED_C, 1, 1) __launch_bounds__(RED_LANES)
 // distributed shared memory and finds the crossing. The candidates that match
 // the first digit are kept in shared memory for the later ones when they fit.
 // LEVELS: 6 digits cover the 48 bits of an FP64 key, 3 those of an FP32 value
-// (its FP64 key's low 29 bits are zero). Up to DG_ONE candidates CTA 0 works
+// (its FP64 key's low 29 bits are zero). Up to DG_ONE candidates one CTA works
 // alone, and up to DG_T it finds tau without digits, by every candidate's sum of
-// the candidates up to its own key. Twelve launches over all candidates did this before: 6 x (5.0 + 5.2)
+// the candidates up to its own key. Of many matrices a cluster has several (see
+// seg.cuh): those that one CTA takes alone side by side, then the others one after
+// another. Twelve launches over all candidates did this before: 6 x (5.0 + 5.2)
 // us for one matrix of 500 rows, now 13 in all.
 constexpr int DG_C = 8, DG_T = 512, DG_KEEP = 2048, DG_ONE = 4096;
+static_assert(DG_C == RED_C, "clusters and groups of seg.cuh");
 static_assert(DG_T <= 2 * NDIG && DG_T <= DG_KEEP && DG_T <= DG_ONE, "the short path's arrays");
+struct DgShared {
+  uint32_t h[3][NDIG];
+  unsigned long long sum[NDIG * 2];
+  unsigned long long keep[DG_KEEP];
+  unsigned long long s_res[3];  // CTA 0: prefix and sum below it
+  int s_nkeep;
+};
+
+// Matrix m, which has a crossing, by nc CTAs (1 or the cluster's DG_C).
 template <int LEVELS>
-__global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
-    k_sel_digits(SelRows R, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
-  after_previous();
-  __shared__ uint32_t h[3][NDIG];
-  __shared__ unsigned long long sum[NDIG * 2];
-  __shared__ unsigned long long keep[DG_KEEP];
-  __shared__ unsigned long long s_res[3];  // CTA 0: prefix and sum below it
-  __shared__ int s_nkeep;
+__device__ __forceinline__ void digits_matrix(int m, int nc, int rank, unsigned long long total,
+                                              DgShared &sh, const SelScratch &sc, MatScalars *ms,
+                                              int64_t *cnt) {
+  auto &h = sh.h;
+  auto &sum = sh.sum;
+  auto &keep = sh.keep;
+  auto &s_res = sh.s_res;
+  int &s_nkeep = sh.s_nkeep;
   cg::cluster_group cl = cg::this_cluster();
-  const int m = blockIdx.x / DG_C, rank = int(cl.block_rank()), tid = threadIdx.x;
-  if (!active[m]) return;  // the whole cluster, as every return before the loop
+  const int tid = threadIdx.x;
   const SelState st = sc.st[m];
-  if (!st.found) {
-    if (rank == 0 && tid == 0) {
-      const unsigned long long k = sc.minabove[m];
-      ms[m].tau = k == ~0ULL ? __longlong_as_double(0x7ff0000000000000LL)
-                             : __longlong_as_double((long long)k);
-    }
-    return;
-  }
-  const unsigned long long room = sc.croom[m], cb = sc.cbase[m];
-  const unsigned long long total = sc.ncand[m] < room ? sc.ncand[m] : room;
-  const bool one = total <= DG_ONE;
-  if (one && rank != 0) return;
-  const int nc = one ? 1 : DG_C;
+  const unsigned long long cb = sc.cbase[m];
   const int eb = ms[m].sel_e;
   const unsigned long long Q = ms[m].sel_q;
   unsigned long long prefix = st.prefix, lo = st.below_lo, hi = st.below_hi;
-  if (total <= DG_T) {  // CTA 0 alone: thread i sums the squares of the keys <= key i
+  if (total <= DG_T) {  // one CTA alone: thread i sums the squares of the keys <= key i
     const int n = int(total);
     const unsigned long long key = tid < n ? sc.cand[cb + tid] : ~0ULL;
     keep[tid] = key;
@@ -929,6 +955,34 @@ __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T)
         atomicAdd(reinterpret_cast<unsigned long long *>(cnt + sc.cand_r[cb + i]), 1ULL);
   }
   if (nc > 1) cl.sync();  // CTA 0's shared memory is read until here
+}
+
+template <int LEVELS>
+__global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T, 3)
+    k_sel_digits(int nb, int per, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
+  after_previous();
+  __shared__ DgShared sh;
+  const int rank = int(cg::this_cluster().block_rank()), g0 = blockIdx.x / DG_C * per;
+  // i = -1: this CTA's own matrix, alone; then those of the whole cluster, the same m
+  // for all its CTAs
+  for (int i = rank < per ? -1 : 0; i < per; ++i) {
+    const int m = i < 0 ? g0 + rank : g0 + i;
+    if (m >= nb || !active[m]) continue;
+    if (!sc.st[m].found) {
+      if (i < 0 && threadIdx.x == 0) {
+        const unsigned long long k = sc.minabove[m];
+        ms[m].tau = k == ~0ULL ? __longlong_as_double(0x7ff0000000000000LL)
+                               : __longlong_as_double((long long)k);
+      }
+      if (per == 1) break;
+      continue;
+    }
+    const unsigned long long total = min(sc.ncand[m], sc.croom[m]);
+    if ((total <= DG_ONE) != (i < 0)) continue;
+    __syncthreads();  // sh is free
+    digits_matrix<LEVELS>(m, i < 0 ? 1 : DG_C, i < 0 ? 0 : rank, total, sh, sc, ms, cnt);
+    if (per == 1) break;
+  }
 }
 
 // ------------------------------------------------------------ filter
@@ -1104,7 +1158,7 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_c
                          int64_t *cnt, double *dropped, cudaStream_t s) {
   {
     ProfScope ps(KC_SEL_HIST, s, 0.0, 0.0);
-    launch_next(k_sel_prepare, unsigned(nb) * RED_C, RED_T, 0, s, R, ms, sc);
+    launch_next(k_sel_prepare, cluster_ctas(nb), RED_T, 0, s, nb, cluster_matrices(nb), R, ms, sc);
     sel_pass(R.nrows, nvals, [&](auto lpr, int rpc, int g) {
       launch_next(k_sel_hist0<T, lpr.value>, g, SEL_THREADS, 0, s, R, rpc, active, val, ms, sc);
     });
@@ -1125,8 +1179,8 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_c
     }
   }
   ProfScope ps(KC_SEL_DIGITS, s, 0.0, 0.0);
-  launch_next(k_sel_digits<sizeof(T) == 4 ? 3 : 6>, unsigned(nb) * DG_C, DG_T, 0, s, R, active, sc,
-              ms, cnt);
+  launch_next(k_sel_digits<sizeof(T) == 4 ? 3 : 6>, cluster_ctas(nb), DG_T, 0, s, nb,
+              cluster_matrices(nb), active, sc, ms, cnt);
 }
 
 void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,
@@ -1145,8 +1199,8 @@ void launch_drop_sums(int nb, const int64_t *moff, const double *dropped, const 
                       void *scratch, const MatScalars *ms, double *sums, cudaStream_t s) {
   if (nb == 0) return;
   const SelScratch sc = scratch ? carve(scratch, nb, 1) : SelScratch{};
-  launch_next(k_drop_sums, unsigned(nb) * RED_C, RED_LANES, 0, s, moff, dropped, active,
-              scratch ? 1 : 0, sc, ms, sums);
+  launch_next(k_drop_sums, cluster_ctas(nb), RED_LANES, 0, s, nb, cluster_matrices(nb), moff, dropped,
+              active, scratch ? 1 : 0, sc, ms, sums);
 }
 
 void launch_filter_count(int64_t n, const int32_t *seg, const int *active, const int64_t *rs,

@@ -1,5 +1,5 @@
 // Sums over the rows of a matrix by a cluster of RED_C CTAs, one warp of each
-// per summed component.
+// per summed component; or, of many small matrices, by one CTA each.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -12,6 +12,35 @@ constexpr int RED_C = 8;    // CTAs per matrix (the portable cluster size)
 constexpr int RED_LANES = RED_T / RED_C;
 constexpr int RED_U = 32;   // rows loaded at once, the next ones while these are added
 static_assert(RED_LANES == 32, "one warp of each CTA per component");
+
+// Matrices per cluster in a launch over nb matrices: one, or from GROUP_NB on
+// (every SM then has CTAs enough) RED_C. Of these, each CTA takes one of its own if
+// that is small (solo); the larger ones are then taken by the whole cluster, one
+// after another (joint), as a lone one is. The sums are the same either way. A
+// cluster for each of 32768 matrices of order 16 took 1.20 ms per check, 0.82 for the
+// select's preparation and histogram, 0.71 per digit search and 49 ms per solve,
+// now 0.28, 0.27, 0.41 and 35; 1024 such matrices 2.30 ms, now 1.90.
+constexpr int GROUP_NB = 1024;
+constexpr int64_t SOLO_ROWS = 2048;
+inline int cluster_matrices(int nb) { return nb >= GROUP_NB ? RED_C : 1; }
+inline unsigned cluster_ctas(int nb) {
+  const int per = cluster_matrices(nb);
+  return unsigned((nb + per - 1) / per) * RED_C;
+}
+// solo(m) and joint(m) for the matrices of cluster `cluster`, by CTA q of it.
+template <typename S, typename J>
+__device__ __forceinline__ void cluster_each(int nb, int per, const int64_t *moff, int cluster,
+                                             int q, S solo, J joint) {
+  if (per == 1) {
+    joint(cluster);
+    return;
+  }
+  const int g0 = cluster * per, g1 = min(nb, g0 + per);
+  auto small = [&](int m) { return moff[m + 1] - moff[m] <= SOLO_ROWS; };
+  if (g0 + q < g1 && small(g0 + q)) solo(g0 + q);
+  for (int m = g0; m < g1; ++m)
+    if (!small(m)) joint(m);
+}
 
 // acc + v as a fused multiply-add (v * 1 is exact): in a chain of dependent FP64
 // additions a DFMA takes 64 cycles, a DADD 76. In PTX, so that it stays one.
@@ -66,6 +95,16 @@ __device__ __forceinline__ void seg_tree(double *sm) {
     for (int i = lane; i < s; i += 32) sm[i] += sm[i + s];
     __syncwarp();
   }
+}
+
+// The partial sums of component c of the rows [b, e), all by one warp, then their sum
+// in sm[0].
+__device__ __forceinline__ void seg_sum_solo(double *sm, const double *part, int ncomp, int c,
+                                             int64_t b, int64_t e) {
+  const int lane = threadIdx.x & 31;
+  for (int t = lane; t < RED_T; t += 32) sm[t] = seg_partial(part, ncomp, c, b, e, t);
+  __syncwarp();
+  seg_tree(sm);
 }
 
 // Warp q of a matrix's cluster: its share of the entries of the rows [b, e).

@@ -113,3 +113,34 @@ def test_dropped_norms_alone_and_in_a_batch(sg, name, filt, prec):
         assert (alone.trace["fnorm_k"] > 0).any()
     for k in SUMS + ("tau_k", "fnorm_k"):
         assert np.array_equal(res.trace[k].view(np.uint64), alone.trace[k].view(np.uint64)), k
+
+
+@pytest.mark.parametrize("kw", [dict(filter="exact"), dict(filter="exact", prec=1, fp32_band=0),
+                                dict(filter="bound"), dict(filter="none", max_iter=2),
+                                dict(filter="exact", budget_norm=1)], ids=str)
+def test_many_matrices(sg, kw):
+    """From 1024 matrices on a cluster has eight of them, a CTA for each when all are
+    small; those with larger ones (2049 and 3000 rows, thousands of candidates) are taken by
+    the whole cluster, and the last one has fewer. Every matrix as alone."""
+    kw = dict(tol=1e-8, dense_frac=2.0, **kw)
+    base = [w.tridiagonal(16), w.banded(40, 3, 5), w.tridiagonal(1), _long_rows(60, 30, 2)]
+    mats = [base[i % 4] for i in range(1030)]
+    special = {0: w.tridiagonal(2048), 9: w.banded(3000, 9, 7), 10: w.tridiagonal(2049),
+               17: w.laplacian(20, 2), 1029: w.banded(2500, 10, 8)}
+    for i, a in special.items():
+        mats[i] = a
+    out = sg.solve_batch(mats, **kw)
+    alone = {i: sg.solve(a, **kw) for i, a in special.items()}
+    alone.update({100 + i: sg.solve(base[i], **kw) for i in range(4)})
+    for i, ref in alone.items():
+        same = [i] if i in special else [j for j in range(i % 4, 1030, 4) if j not in special]
+        for j in same:
+            res = out[j]
+            assert res.status == ref.status and res.iters == ref.iters
+            assert np.array_equal(res.col, ref.col)
+            assert np.array_equal(res.val.view(np.uint64), ref.val.view(np.uint64))
+            for k in SUMS + ("tau_k", "fnorm_k"):
+                assert np.array_equal(res.trace[k].view(np.uint64),
+                                      ref.trace[k].view(np.uint64)), (i, j, k)
+            for k in ("nnz_t", "nnz_bar"):
+                assert np.array_equal(res.trace[k], ref.trace[k])
