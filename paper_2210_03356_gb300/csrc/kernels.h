@@ -148,9 +148,10 @@ struct Rows {
 };
 
 // Row classes of the numeric kernels: groups of 32, 16 or 8 lanes per row,
-// windows of wide rows (RC_CTA), or band tiles of 16 rows (FP32 only; the list holds each
-// tile's first row).
-enum RowClass { RC_G32 = 0, RC_CTA = 1, RC_G16 = 2, RC_G8 = 3, RC_BAND = 4, RC_NONE = 5, RC_N = 5 };
+// windows of wide rows (RC_CTA) and of those above LONG_W columns (RC_LONG), or
+// band tiles of 16 rows (FP32 only; the list holds each tile's first row).
+enum RowClass { RC_G32 = 0, RC_CTA = 1, RC_G16 = 2, RC_G8 = 3, RC_BAND = 4, RC_LONG = 5, RC_NONE = 6, RC_N = 6 };
+constexpr int LONG_W = 8192;
 constexpr int RC_QUEUE = RC_N;         // counters[RC_QUEUE + c]: work-queue head of class c
 constexpr int RC_EMPTY = 2 * RC_N;     // counters[RC_EMPTY]: rows without output (in band tiles too)
 constexpr int RC_COUNTERS = 2 * RC_N + 2;  // ints in the counters array (8-byte padded)
@@ -247,13 +248,14 @@ void launch_numeric(int64_t n, const int *rows, int empty, bool shared, bool few
                     const int32_t *len, const int32_t *seg, const int *dslot,
                     const int32_t *lists, int *counters, const int64_t *cs, int64_t *ce,
                     int32_t *ccol, T *cval, double *part, cudaStream_t s);
-// The rows of more than WARP_W columns (cls = RC_CTA, `rows` of them), or the few
+// The rows of more than WARP_W columns (cls = RC_CTA or RC_LONG, `rows` of them), or the few
 // rows of the 32-lane class (cls = RC_G32), by windows of several warps.
 // mean_b: the mean length of the B rows that products read. wt: the rows'
-// matrices, the column-block table of B (launch_col_blocks: n * stride ints;
-// null: binary search in its place), its block width 1 << sh and row stride,
-// (max matrix order >> sh) + 2.
+// matrices, the records of B's rows (launch_bounds), the column-block table of B
+// (launch_col_blocks: n * stride ints; null: binary search in its place), its block
+// width 1 << sh and row stride, (max matrix order >> sh) + 2.
 struct WideTable {
+  const int4 *binfo;
   const int32_t *seg;
   const int64_t *moff;
   const int *off;

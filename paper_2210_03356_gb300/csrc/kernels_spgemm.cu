@@ -198,7 +198,7 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
     const int32_t L = mx - mn + 1;
     const int64_t bound = wk + (mode == MODE_UPDATE ? na : 0);
     if (L > WARP_W) {
-      cls = RC_CTA;
+      cls = L > LONG_W ? RC_LONG : RC_CTA;
     } else if (!groups) {
       cls = RC_G32;
     } else if (groups == GROUPS_PAIRS) {
@@ -1028,24 +1028,35 @@ __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, co
 // One CTA per row with a barrier per k took 12.0 and 6.0 ms for the update and
 // the square of the 16^3 Laplacian's FP32 iterate just below the dense path's
 // density, now 7.8 and 4.0.
+// Rows of more than LONG_W columns (WIDE_LONG) always take eight warps, and a warp
+// looks through the k by the first and last columns of their B rows, 128 at a time,
+// before it locates any: such a row has many windows and most k fall into few of
+// them. With one warp that located every k in every window the FP64 products of a
+// solve of a tridiagonal matrix of order 65536 with one full row took 3.5 s (1.1 s
+// with one CTA per row before that), now 0.086.
 constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_K = 4;  // k whose first 32 entries are loaded ahead
-template <typename T>
-constexpr int wide_occ() { return sizeof(T) == 8 ? 3 : 5; }  // CTAs per SM
+enum { WIDE_ROWS = 0, WIDE_NARROW = 1, WIDE_LONG = 2 };
+template <typename T, int KIND>
+constexpr int wide_occ() {  // CTAs per SM
+  return KIND == WIDE_LONG ? 2 : sizeof(T) == 8 ? 3 : 5;
+}
 template <typename T, int MODE>
 constexpr size_t wide_smem() {
   return size_t(WIDE_WARPS) * WARP_W * (sizeof(T) + (MODE == MODE_UPDATE ? 1 : 0));
 }
 
-template <typename T, int MODE, int P, bool NARROW>
-__global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
+template <typename T, int MODE, int P, int KIND>
+__global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
     k_num_wide(const int64_t *ars, const int64_t *are, const int32_t *acol, const T *aval,
                const int64_t *brs, const int64_t *bre, const int32_t *bcol, const T *bval,
-               const int32_t *seg, const int64_t *moff, const int *off, int sh, int stride,
-               const int32_t *lo, const int32_t *len, const int32_t *list, int *counters,
-               int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
+               const int4 *binfo, const int32_t *seg, const int64_t *moff, const int *off, int sh,
+               int stride, const int32_t *lo, const int32_t *len, const int32_t *list,
+               int *counters, int cls, const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part) {
   after_previous();
   constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool NARROW = KIND == WIDE_NARROW;
+  constexpr int KB = KIND == WIDE_LONG ? 4 : 1;  // groups of 32 k looked at together
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
   constexpr int NQ = WIDE_WARPS / P;     // eighths of a row's sums per warp
@@ -1089,50 +1100,70 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T>())
       }
       __syncwarp();
       if (has) {
-        for (int64_t pb = a0; pb < a1; pb += 32) {
-          T av = T(0);
-          int64_t qs = 0;
-          int qn = 0;
-          if (pb + lane < a1) {
-            const int32_t k = acol[pb + lane];
-            av = aval[pb + lane];
-            qs = brs[k];
-            if (off) {
-              const int *o = off + int64_t(k) * stride;
-              const int o0 = o[w0];
-              qn = o[w1] - o0;
-              qs += o0;
-            } else {
-              const int64_t e = bre[k];
-              qs = lower_bound(bcol, qs, e, c0);
-              qn = int(lower_bound(bcol, qs, e, c0 + W) - qs);
-            }
-          }
-          unsigned todo = __ballot_sync(FULL, qn > 0);
-          while (todo) {  // ascending k, WIDE_K at a time
-            T a[WIDE_K], v[WIDE_K];
-            int64_t q0[WIDE_K];
-            int nn[WIDE_K], j[WIDE_K];
+        for (int64_t pb = a0; pb < a1; pb += 32 * KB) {
+          int32_t kk[KB];
+          bool hit[KB];
 #pragma unroll
-            for (int t = 0; t < WIDE_K; ++t) {
-              const int src = todo ? __ffs(todo) - 1 : 0;
-              const bool any = todo != 0;
-              todo &= todo - 1;
-              a[t] = __shfl_sync(FULL, av, src);
-              q0[t] = __shfl_sync(FULL, qs, src);
-              nn[t] = __shfl_sync(FULL, qn, src);
-              if (!any) nn[t] = 0;
-              if (lane < nn[t]) {
-                j[t] = int(bcol[q0[t] + lane] - c0);
-                v[t] = bval[q0[t] + lane];
+          for (int u = 0; u < KB; ++u) {
+            const int64_t p = pb + 32 * u + lane;
+            hit[u] = p < a1;
+            kk[u] = hit[u] ? acol[p] : 0;
+          }
+          if constexpr (KIND == WIDE_LONG) {
+            int4 bi[KB];
+#pragma unroll
+            for (int u = 0; u < KB; ++u) bi[u] = binfo[kk[u]];
+#pragma unroll
+            for (int u = 0; u < KB; ++u)
+              hit[u] = hit[u] && bi[u].z > 0 && bi[u].x < c0 + W && bi[u].y >= c0;
+          }
+#pragma unroll
+          for (int u = 0; u < KB; ++u) {
+            if (KIND == WIDE_LONG && !__any_sync(FULL, hit[u])) continue;
+            T av = T(0);
+            int64_t qs = 0;
+            int qn = 0;
+            if (hit[u]) {
+              const int32_t k = kk[u];
+              av = aval[pb + 32 * u + lane];
+              qs = brs[k];
+              if (off) {
+                const int *o = off + int64_t(k) * stride;
+                const int o0 = o[w0];
+                qn = o[w1] - o0;
+                qs += o0;
+              } else {
+                const int64_t e = bre[k];
+                qs = lower_bound(bcol, qs, e, c0);
+                qn = int(lower_bound(bcol, qs, e, c0 + W) - qs);
               }
             }
-#pragma unroll
-            for (int t = 0; t < WIDE_K; ++t) {
-              if (lane < nn[t]) mac(acc, j[t], a[t], v[t]);
-              if (nn[t] > 32)
-                accumulate_k<T, 32>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, lane);
-              __syncwarp();
+            unsigned todo = __ballot_sync(FULL, qn > 0);
+            while (todo) {  // ascending k, WIDE_K at a time
+              T a[WIDE_K], v[WIDE_K];
+              int64_t q0[WIDE_K];
+              int nn[WIDE_K], j[WIDE_K];
+  #pragma unroll
+              for (int t = 0; t < WIDE_K; ++t) {
+                const int src = todo ? __ffs(todo) - 1 : 0;
+                const bool any = todo != 0;
+                todo &= todo - 1;
+                a[t] = __shfl_sync(FULL, av, src);
+                q0[t] = __shfl_sync(FULL, qs, src);
+                nn[t] = __shfl_sync(FULL, qn, src);
+                if (!any) nn[t] = 0;
+                if (lane < nn[t]) {
+                  j[t] = int(bcol[q0[t] + lane] - c0);
+                  v[t] = bval[q0[t] + lane];
+                }
+              }
+  #pragma unroll
+              for (int t = 0; t < WIDE_K; ++t) {
+                if (lane < nn[t]) mac(acc, j[t], a[t], v[t]);
+                if (nn[t] > 32)
+                  accumulate_k<T, 32>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, lane);
+                __syncwarp();
+              }
             }
           }
         }
@@ -1412,21 +1443,22 @@ static void num_launch(int64_t n, const int *rows, bool few, const Rows &A, cons
                              cs, ce, ccol, cval, part, s);
 }
 
-template <typename T, int MODE, int P, bool NARROW>
+template <typename T, int MODE, int P, int KIND>
 static void wide_launch(int rows, const Rows &A, const T *aval, const Rows &B, const T *bval,
                         const WideTable &wt, const int32_t *lo, const int32_t *len,
                         const int32_t *list, int *ctr, int cls, const int64_t *cs, int64_t *ce,
                         int32_t *ccol, T *cval, double *part, cudaStream_t s) {
   constexpr size_t sm = wide_smem<T, MODE>();
   static const bool attr = [] {  // once, thread-safe
-    SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P, NARROW>,
+    SGN_CUDA(cudaFuncSetAttribute(k_num_wide<T, MODE, P, KIND>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
     return true;
   }();
   (void)attr;
-  launch_next(k_num_wide<T, MODE, P, NARROW>, grid_cap(rows, WIDE_WARPS / P, wide_occ<T>()),
-              WIDE_WARPS * 32, sm, s, A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.seg,
-              wt.moff, wt.off, wt.sh, wt.stride, lo, len, list, ctr, cls, cs, ce, ccol, cval, part);
+  launch_next(k_num_wide<T, MODE, P, KIND>, grid_cap(rows, WIDE_WARPS / P, wide_occ<T, KIND>()),
+              WIDE_WARPS * 32, sm, s, A.rs, A.re, A.col, aval, B.rs, B.re, B.col, bval, wt.binfo,
+              wt.seg, wt.moff, wt.off, wt.sh, wt.stride, lo, len, list, ctr, cls, cs, ce, ccol,
+              cval, part);
 }
 
 template <typename T, int MODE>
@@ -1435,20 +1467,22 @@ static void wide_launch_p(int rows, int p, const Rows &A, const T *aval, const R
                           const int32_t *len, const int32_t *list, int *ctr, int cls,
                           const int64_t *cs, int64_t *ce, int32_t *ccol, T *cval, double *part,
                           cudaStream_t s) {
-#define SGN_WIDE(P, NARROW) \
-  wide_launch<T, MODE, P, NARROW>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cls, cs, ce, ccol, cval, \
-                          part, s)
-  if (cls != RC_CTA) {  // rows of the 32-lane class
-    if (p >= 8) SGN_WIDE(8, true);
-    else SGN_WIDE(4, true);
+#define SGN_WIDE(P, KIND) \
+  wide_launch<T, MODE, P, KIND>(rows, A, aval, B, bval, wt, lo, len, list, ctr, cls, cs, ce, ccol, \
+                                cval, part, s)
+  if (cls == RC_LONG) {
+    SGN_WIDE(8, WIDE_LONG);
+  } else if (cls != RC_CTA) {  // rows of the 32-lane class
+    if (p >= 8) SGN_WIDE(8, WIDE_NARROW);
+    else SGN_WIDE(4, WIDE_NARROW);
   } else if (p >= 8) {
-    SGN_WIDE(8, false);
+    SGN_WIDE(8, WIDE_ROWS);
   } else if (p >= 4) {
-    SGN_WIDE(4, false);
+    SGN_WIDE(4, WIDE_ROWS);
   } else if (p >= 2) {
-    SGN_WIDE(2, false);
+    SGN_WIDE(2, WIDE_ROWS);
   } else {
-    SGN_WIDE(1, false);
+    SGN_WIDE(1, WIDE_ROWS);
   }
 #undef SGN_WIDE
 }

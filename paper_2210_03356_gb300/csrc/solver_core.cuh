@@ -600,14 +600,15 @@ struct Solver {
       const bool shared = few && mean_b >= SHARED_B;
       int rows[RC_N];
       std::copy(ctr, ctr + RC_N, rows);
-      const int wide_rows[2] = {rows[RC_CTA], shared ? rows[RC_G32] : 0};
+      const int wide_cls[3] = {RC_CTA, RC_LONG, RC_G32};
+      const int wide_rows[3] = {rows[RC_CTA], rows[RC_LONG], shared ? rows[RC_G32] : 0};
       launch_numeric<T>(N, rows, ctr[RC_EMPTY], shared, few, A, aval, B, bval, mode, ends, w.lo.as<int32_t>(),
                         w.len.as<int32_t>(), st.d_seg.template as<int32_t>(),
                         dp && dp->any() ? w.dslot.as<int>() : nullptr, w.wlist.as<int32_t>(),
                         head->ctr, C.rs.template as<int64_t>(),
                         C.re.template as<int64_t>(), C.col.template as<int32_t>(), C.d_val(),
                         mode == MODE_SQUARE ? w.part.as<double>() : nullptr, s);
-      if (wide_rows[0] + wide_rows[1] > 0) {
+      if (wide_rows[0] + wide_rows[1] + wide_rows[2] > 0) {
         int64_t max_n = 0;
         for (size_t i = 0; i + 1 < st.moff.size(); ++i)
           max_n = std::max(max_n, st.moff[i + 1] - st.moff[i]);
@@ -620,10 +621,10 @@ struct Solver {
           launch_col_blocks(N, B, st.d_seg.template as<int32_t>(),
                             st.d_moff.template as<int64_t>(), sh, stride, off, s);
         }
-        const WideTable wt{st.d_seg.template as<int32_t>(), st.d_moff.template as<int64_t>(), off,
-                           sh, stride};
-        for (int i = 0; i < 2; ++i)
-          launch_numeric_wide<T>(N, i ? RC_G32 : RC_CTA, wide_rows[i], mean_b, A, aval, B, bval,
+        const WideTable wt{w.binfo.as<int4>(), st.d_seg.template as<int32_t>(),
+                           st.d_moff.template as<int64_t>(), off, sh, stride};
+        for (int i = 0; i < 3; ++i)
+          launch_numeric_wide<T>(N, wide_cls[i], wide_rows[i], mean_b, A, aval, B, bval,
                                  mode, wt, w.lo.as<int32_t>(), w.len.as<int32_t>(),
                                  w.wlist.as<int32_t>(), head->ctr,
                                  C.rs.template as<int64_t>(), C.re.template as<int64_t>(),
