@@ -148,8 +148,9 @@ struct Rows {
 };
 
 // Row classes of the numeric kernels: groups of 32, 16 or 8 lanes per row,
-// windows of wide rows (RC_CTA) and of those above LONG_W columns (RC_LONG), or
-// band tiles of 16 rows (FP32 only; the list holds each tile's first row).
+// windows of wide rows (RC_CTA) and of those above LONG_W columns whose B rows fall
+// into few windows (RC_LONG), or band tiles of 16 rows (FP32 only; the list holds each
+// tile's first row).
 enum RowClass { RC_G32 = 0, RC_CTA = 1, RC_G16 = 2, RC_G8 = 3, RC_BAND = 4, RC_LONG = 5, RC_NONE = 6, RC_N = 6 };
 constexpr int LONG_W = 8192;
 constexpr int RC_QUEUE = RC_N;         // counters[RC_QUEUE + c]: work-queue head of class c

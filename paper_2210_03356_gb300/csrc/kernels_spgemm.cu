@@ -90,6 +90,12 @@ struct SqAcc<float> {
   __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
 };
 
+// (t_ii - 1)^2 of the diagonal entry v, 1 where none is stored.
+__device__ __forceinline__ double diag_square(bool stored, double v) {
+  const double d = stored ? v - 1.0 : -1.0;
+  return d * d;
+}
+
 // The total of a row's 32 partial sums, 32 / G on each of the G lanes of mask
 // (lane gl holds gl, gl + G, ..): added 16 apart, 8 apart and so on, the same
 // additions for every G.
@@ -198,7 +204,7 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
     const int32_t L = mx - mn + 1;
     const int64_t bound = wk + (mode == MODE_UPDATE ? na : 0);
     if (L > WARP_W) {
-      cls = L > LONG_W ? RC_LONG : RC_CTA;
+      cls = RC_CTA;
     } else if (!groups) {
       cls = RC_G32;
     } else if (groups == GROUPS_PAIRS) {
@@ -225,6 +231,24 @@ __device__ __forceinline__ int bounds_row(int64_t r, int m, int64_t na, int32_t 
     *swk = float(wk);
   }
   return cls;
+}
+
+// Whether a row of L > LONG_W columns goes to RC_LONG: it has many pairs of a window and
+// 32 k, each a step of its warps, and the B rows (16 of them are looked at) fall into
+// less than about a quarter of the windows. Scattered B rows do not: the FP32 squares of
+// a matrix of order 20000 with 7 and 258 scattered entries a row take 15.4 ms that
+// way, 12.9 with RC_CTA's rows.
+__device__ __forceinline__ bool long_row(const int32_t *acol, const int4 *binfo, int64_t a0,
+                                         int64_t a1, int L) {
+  constexpr int SAMPLES = 16;
+  if (int64_t(L / WARP_W) * ((a1 - a0) / 32) < 64) return false;  // a1 - a0 >= 32 from here on
+  int64_t extent = 0;
+#pragma unroll 4
+  for (int i = 0; i < SAMPLES; ++i) {
+    const int4 b = binfo[acol[a0 + i * ((a1 - a0) / SAMPLES)]];
+    extent += b.z ? b.y - b.x + 1 : 0;
+  }
+  return (extent / SAMPLES + WARP_W) * 4 < L;
 }
 
 // Over the 16 lanes of a half warp.
@@ -374,6 +398,8 @@ __global__ void __launch_bounds__(BOUNDS_T)
                          len, ub, s_seg + i, s_lo + i, s_L + i, s_kf + i, s_kl + i, s_na + i,
                          s_wk + i);
         if (cs.fc) put_span(cs, r, mx < 0 ? 0 : mn, mx);
+        if (cls == RC_CTA && mx - mn >= LONG_W && long_row(acol, binfo, a0, a1, mx - mn + 1))
+          cls = RC_LONG;
       }
       if (gl == 0) s_cls[i] = (unsigned char)cls;
     }
@@ -926,7 +952,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
         }
         int64_t out = cs[r];
         SqAcc<T> racc[NG];  // 32 partial sums per row, NG to a lane
-        double rdiag = 0.0;
+        T vdiag = T(0);     // t_ii, whose square is added last
         bool diag = false;
         for (int s32 = 0; s32 < L; s32 += 32) {
 #pragma unroll
@@ -949,9 +975,8 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
               ccol[pos] = cj;
               cval[pos] = v;
               if (MODE == MODE_SQUARE) {
-                if (cj == r) {  // (t_ii - 1)^2 in FP64, once per row
-                  double d = double(v) - 1.0;
-                  rdiag = d * d;
+                if (cj == r) {
+                  vdiag = v;
                   diag = true;
                 } else {
                   racc[u].add_sq(v);
@@ -974,9 +999,9 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, group_occ<T, LOOP>())
           }
           const double rs = sum_of_32<T, G>(racc, gmask), xs = sum_of_32<T, G>(xacc, gmask);
           const unsigned dm = __ballot_sync(gmask, diag);
-          const double rd = __shfl_sync(gmask, rdiag, dm ? __ffs(dm) - 1 : 0, G);
+          const T vd = __shfl_sync(gmask, vdiag, dm ? __ffs(dm) - 1 : 0, G);
           if (gl == 0) {
-            part[2 * int64_t(r)] = rs + (dm ? rd : 1.0);
+            part[2 * int64_t(r)] = rs + diag_square(dm != 0, vd);
             part[2 * int64_t(r) + 1] = xs;
           }
         }
@@ -1021,17 +1046,18 @@ __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, co
 // to add up their entry counts before each writes its part. P follows the
 // mean length of B's rows: enough entries of B_k per warp to fill its lanes
 // (an FP64 instruction costs the pipe the same whatever its active lanes).
-// A row's sums of squares are 256 partial sums, of every 256th column counted
-// from the row's first one and of every 256th entry of X_i, added pairwise in
-// eighths of 32 (8 / P of them to a warp) and those in order: the same for every P
-// and window. Rows of the 32-lane class take that class's sums instead.
+// A row's sums of squares are 256 partial sums, of every 256th column and of every
+// 256th entry of X_i in ascending order, 256 / P to a warp, added 128 apart, 64
+// apart and so on, the diagonal's last: the same for every P and window (and for every first column that
+// the 256 are counted from, which is the window's). One warp adds its squares as it
+// writes the row; several read each other's accumulators. Rows of the 32-lane class
+// take that class's 32 sums.
 // One CTA per row with a barrier per k took 12.0 and 6.0 ms for the update and
 // the square of the 16^3 Laplacian's FP32 iterate just below the dense path's
 // density, now 7.8 and 4.0.
-// Rows of more than LONG_W columns (WIDE_LONG) always take eight warps, and a warp
-// looks through the k by the first and last columns of their B rows, 128 at a time,
-// before it locates any: such a row has many windows and most k fall into few of
-// them. With one warp that located every k in every window the FP64 products of a
+// The rows of RC_LONG (WIDE_LONG) always take eight warps, and a warp looks through
+// the k by the first and last columns of their B rows, 128 at a time, before it locates
+// any: such a row has many windows and most k fall into few of them. With one warp that located every k in every window the FP64 products of a
 // solve of a tridiagonal matrix of order 65536 with one full row took 3.5 s (1.1 s
 // with one CTA per row before that), now 0.086.
 constexpr int WIDE_WARPS = 8;
@@ -1056,13 +1082,13 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
   after_previous();
   constexpr unsigned FULL = 0xffffffffu;
   constexpr bool NARROW = KIND == WIDE_NARROW;
-  constexpr int KB = KIND == WIDE_LONG ? 4 : 1;  // groups of 32 k looked at together
   constexpr int NG = WIDE_WARPS / P;     // rows in flight per CTA
   extern __shared__ __align__(16) unsigned char wide_smem_raw[];
   constexpr int NQ = WIDE_WARPS / P;     // eighths of a row's sums per warp
   __shared__ int s_idx[NG], s_cnt[WIDE_WARPS];
-  __shared__ double s_red[2][NG * WIDE_WARPS];
+  __shared__ double s_red[2][MODE == MODE_SQUARE && P > 1 ? WIDE_WARPS : 1][32];
   __shared__ int s_diag[WIDE_WARPS];
+  __shared__ T s_vdiag[WIDE_WARPS];
   const int lane = lane_id(), w = threadIdx.x >> 5, g = w / P, wr = w % P;
   const unsigned lt = (1u << lane) - 1u;
   T *acc = reinterpret_cast<T *>(wide_smem_raw) + w * WARP_W;
@@ -1086,8 +1112,12 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
     const int bpw = min(WARP_W >> sh, (b1 - b0 + P) / P);  // blocks per warp and window
     int64_t out = cs[r];
     SqAcc<T> racc[1];  // NARROW: the sums of k_num_group, by warp 0
-    double rdiag = 0.0;
+    // FP64: indexed at run time and so kept in local memory. In registers through the
+    // k loop they cost it its loads in flight (two squares of a matrix of order 20000
+    // with 7 and 258 scattered entries a row: 13.0 ms, now 11.6); the FP32 words are better unrolled
+    // (12.8 ms against 11.0).
     double rq[NQ] = {};
+    T vdiag = T(0);  // t_ii, whose square is added last
     bool diag = false;
     for (int win = b0; win <= b1; win += P * bpw) {
       const int w0 = win + wr * bpw, w1 = min(w0 + bpw, b1 + 1);  // this warp's blocks
@@ -1100,71 +1130,90 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
       }
       __syncwarp();
       if (has) {
-        for (int64_t pb = a0; pb < a1; pb += 32 * KB) {
-          int32_t kk[KB];
-          bool hit[KB];
+        // lane t's k: the factor and the part of its B row in the window
+        auto add_rows = [&](T av, int64_t qs, int qn) {
+          unsigned todo = __ballot_sync(FULL, qn > 0);
+          while (todo) {  // ascending k, WIDE_K at a time
+            T a[WIDE_K], v[WIDE_K];
+            int64_t q0[WIDE_K];
+            int nn[WIDE_K], j[WIDE_K];
 #pragma unroll
-          for (int u = 0; u < KB; ++u) {
-            const int64_t p = pb + 32 * u + lane;
-            hit[u] = p < a1;
-            kk[u] = hit[u] ? acol[p] : 0;
+            for (int t = 0; t < WIDE_K; ++t) {
+              const int src = todo ? __ffs(todo) - 1 : 0;
+              const bool any = todo != 0;
+              todo &= todo - 1;
+              a[t] = __shfl_sync(FULL, av, src);
+              q0[t] = __shfl_sync(FULL, qs, src);
+              nn[t] = __shfl_sync(FULL, qn, src);
+              if (!any) nn[t] = 0;
+              if (lane < nn[t]) {
+                j[t] = int(bcol[q0[t] + lane] - c0);
+                v[t] = bval[q0[t] + lane];
+              }
+            }
+#pragma unroll
+            for (int t = 0; t < WIDE_K; ++t) {
+              if (lane < nn[t]) mac(acc, j[t], a[t], v[t]);
+              if (nn[t] > 32)
+                accumulate_k<T, 32>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, lane);
+              __syncwarp();
+            }
           }
-          if constexpr (KIND == WIDE_LONG) {
+        };
+        // the part of row k of B in the window
+        auto locate = [&](int32_t k, int64_t &qs, int &qn) {
+          qs = brs[k];
+          if (off) {
+            const int *o = off + int64_t(k) * stride;
+            const int o0 = o[w0];
+            qn = o[w1] - o0;
+            qs += o0;
+          } else {
+            const int64_t e = bre[k];
+            qs = lower_bound(bcol, qs, e, c0);
+            qn = int(lower_bound(bcol, qs, e, c0 + W) - qs);
+          }
+        };
+        if constexpr (KIND == WIDE_LONG) {
+          constexpr int KB = 4;  // groups of 32 k looked at together
+          for (int64_t pb = a0; pb < a1; pb += 32 * KB) {
+            int32_t kk[KB];
+            bool hit[KB];
             int4 bi[KB];
+#pragma unroll
+            for (int u = 0; u < KB; ++u) {
+              hit[u] = pb + 32 * u + lane < a1;
+              kk[u] = hit[u] ? acol[pb + 32 * u + lane] : 0;
+            }
 #pragma unroll
             for (int u = 0; u < KB; ++u) bi[u] = binfo[kk[u]];
 #pragma unroll
             for (int u = 0; u < KB; ++u)
               hit[u] = hit[u] && bi[u].z > 0 && bi[u].x < c0 + W && bi[u].y >= c0;
-          }
 #pragma unroll
-          for (int u = 0; u < KB; ++u) {
-            if (KIND == WIDE_LONG && !__any_sync(FULL, hit[u])) continue;
+            for (int u = 0; u < KB; ++u) {
+              if (!__any_sync(FULL, hit[u])) continue;
+              T av = T(0);
+              int64_t qs = 0;
+              int qn = 0;
+              if (hit[u]) {
+                av = aval[pb + 32 * u + lane];
+                locate(kk[u], qs, qn);
+              }
+              add_rows(av, qs, qn);
+            }
+          }
+        } else {
+          for (int64_t pb = a0; pb < a1; pb += 32) {
             T av = T(0);
             int64_t qs = 0;
             int qn = 0;
-            if (hit[u]) {
-              const int32_t k = kk[u];
-              av = aval[pb + 32 * u + lane];
-              qs = brs[k];
-              if (off) {
-                const int *o = off + int64_t(k) * stride;
-                const int o0 = o[w0];
-                qn = o[w1] - o0;
-                qs += o0;
-              } else {
-                const int64_t e = bre[k];
-                qs = lower_bound(bcol, qs, e, c0);
-                qn = int(lower_bound(bcol, qs, e, c0 + W) - qs);
-              }
+            if (pb + lane < a1) {
+              const int32_t k = acol[pb + lane];
+              av = aval[pb + lane];
+              locate(k, qs, qn);
             }
-            unsigned todo = __ballot_sync(FULL, qn > 0);
-            while (todo) {  // ascending k, WIDE_K at a time
-              T a[WIDE_K], v[WIDE_K];
-              int64_t q0[WIDE_K];
-              int nn[WIDE_K], j[WIDE_K];
-  #pragma unroll
-              for (int t = 0; t < WIDE_K; ++t) {
-                const int src = todo ? __ffs(todo) - 1 : 0;
-                const bool any = todo != 0;
-                todo &= todo - 1;
-                a[t] = __shfl_sync(FULL, av, src);
-                q0[t] = __shfl_sync(FULL, qs, src);
-                nn[t] = __shfl_sync(FULL, qn, src);
-                if (!any) nn[t] = 0;
-                if (lane < nn[t]) {
-                  j[t] = int(bcol[q0[t] + lane] - c0);
-                  v[t] = bval[q0[t] + lane];
-                }
-              }
-  #pragma unroll
-              for (int t = 0; t < WIDE_K; ++t) {
-                if (lane < nn[t]) mac(acc, j[t], a[t], v[t]);
-                if (nn[t] > 32)
-                  accumulate_k<T, 32>(a[t], q0[t] + 32, q0[t] + nn[t], bcol, bval, c0, acc, lane);
-                __syncwarp();
-              }
-            }
+            add_rows(av, qs, qn);
           }
         }
         if (MODE == MODE_UPDATE) {  // x_ij of the window
@@ -1185,11 +1234,11 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
         if (!fl && !untouched(acc[s])) fl = 1;
         return fl;
       };
-      int cnt = 0;
-      for (int s0 = 0; s0 < W; s0 += 32)
-        cnt += __popc(__ballot_sync(FULL, touched(s0 + lane) != 0));
       int64_t at = out;
       if constexpr (P > 1) {
+        int cnt = 0;
+        for (int s0 = 0; s0 < W; s0 += 32)
+          cnt += __popc(__ballot_sync(FULL, touched(s0 + lane) != 0));
         if (lane == 0) s_cnt[w] = cnt;
         row_sync();
         for (int i = 0; i < P; ++i) {
@@ -1197,10 +1246,8 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
           if (i < wr) at += ci;
           out += ci;
         }
-      } else {
-        out += cnt;
       }
-      for (int s0 = 0; s0 < W; s0 += 32) {
+      auto emit = [&](int s0, auto also) {
         const int s = s0 + lane, fl = touched(s);
         const unsigned mk = __ballot_sync(FULL, fl != 0);
         if (fl) {
@@ -1210,48 +1257,67 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
           if (MODE == MODE_UPDATE && !(fl & 2)) v = ns_combine(T(0), v);
           ccol[pos] = int32_t(cj);
           cval[pos] = v;
+          also(cj, v);
         }
         at += __popc(mk);
+      };
+      if constexpr (P == 1 && MODE == MODE_SQUARE) {
+#pragma unroll 1
+        for (int s0 = 0; s0 < W; s0 += 32)
+          emit(s0, [&](int64_t cj, T v) {
+            if (cj == r) {
+              vdiag = v;
+              diag = true;
+            } else {
+              double &sum = rq[s0 / 32 % NQ];
+              sum = __fma_rn(double(v), double(v), sum);
+            }
+          });
+      } else {
+        for (int s0 = 0; s0 < W; s0 += 32) emit(s0, [](int64_t, T) {});
       }
-      if constexpr (MODE == MODE_SQUARE) {
-        // the squares of the window's columns, from the accumulators of all the
-        // row's warps; column i is counted from the row's first one
-        const int d = int(lo[r] - base) - (win << sh);  // column i is i + d of the window
-        const int i0 = max(0, -d), i1 = min(len[r], (P * bpw << sh) - d);
-        const int idiag = r - lo[r];
-        auto value_at = [&](int i, T &v) {
-          if (i < i0 || i >= i1) return false;
-          const int o = P == 1 ? 0 : ((i + d) >> sh) / bpw;  // the warp that holds it
-          v = acc[(o - wr) * WARP_W + (i + d) - (o * bpw << sh)];
-          return !untouched(v);
+      if constexpr (P == 1) out = at;
+      if constexpr (MODE == MODE_SQUARE && P > 1) {
+        // the squares of the window's columns, from the accumulators of all the row's
+        // warps: words of 32 columns, each within one warp's (o, up to column oend)
+        const int words = ((min(win + P * bpw, b1 + 1) - win) << sh) / 32;
+        const int bcol = bpw << sh, idiag = int(r - base) - (win << sh);
+        const T *const row = acc - wr * WARP_W + lane;
+        int o = 0, oend = bcol;
+        auto square = [&](int j, auto add) {
+          while (32 * j >= oend) {
+            ++o;
+            oend += bcol;
+          }
+          const T v = row[o * (WARP_W - bcol) + 32 * j];
+          if (untouched(v)) return;
+          if (32 * j + lane == idiag) {
+            vdiag = v;
+            diag = true;
+          } else {
+            add(v);
+          }
         };
-        T v;
         if constexpr (NARROW) {
           if (wr == 0)
-            for (int i = (i0 & ~31) + lane; i - lane < i1; i += 32)
-              if (value_at(i, v)) {
-                if (i == idiag) {
-                  const double t = double(v) - 1.0;
-                  rdiag = t * t;
-                  diag = true;
-                } else {
-                  racc[0].add_sq(v);
-                }
-              }
+            for (int j = 0; j < words; ++j) square(j, [&](T v) { racc[0].add_sq(v); });
         } else {
-          for (int i8 = i0 & ~255; i8 < i1; i8 += 256)
+          auto add_to = [&](int j, double &sum) {
+            square(j, [&](T v) { sum = __fma_rn(double(v), double(v), sum); });
+          };
+          if constexpr (sizeof(T) == 4 || NQ == 1) {
+            for (int j8 = wr; j8 < words; j8 += 8)
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-              const int i = i8 + 32 * (wr + q * P) + lane;
-              if (value_at(i, v)) {
-                double t = double(v);
-                if (i == idiag) {
-                  t = t - 1.0;
-                  diag = true;
-                }
-                rq[q] += t * t;
-              }
+              for (int q = 0; q < NQ; ++q)
+                if (j8 + q * P < words) add_to(j8 + q * P, rq[q]);
+          } else {
+            int q = 0;
+#pragma unroll 1
+            for (int j = wr; j < words; j += P) {
+              add_to(j, rq[q]);
+              q = (q + 1) % NQ;
             }
+          }
         }
       }
       row_sync();  // s_cnt and the accumulators are free again
@@ -1264,9 +1330,9 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
           SqAcc<T> xacc[1];
           for (int64_t p = a0 + lane; p < a1; p += 32) xacc[0].add_sq(aval[p]);
           const double rs = sum_of_32<T, 32>(racc, FULL), xs = sum_of_32<T, 32>(xacc, FULL);
-          const double rd = __shfl_sync(FULL, rdiag, dm ? __ffs(dm) - 1 : 0);
+          const T vd = __shfl_sync(FULL, vdiag, dm ? __ffs(dm) - 1 : 0);
           if (lane == 0) {
-            part[2 * int64_t(r)] = rs + (dm ? rd : 1.0);
+            part[2 * int64_t(r)] = rs + diag_square(dm != 0, vd);
             part[2 * int64_t(r) + 1] = xs;
           }
         }
@@ -1276,34 +1342,61 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, wide_occ<T, KIND>())
 #pragma unroll
           for (int q = 0; q < NQ; ++q) {
             const int64_t i = p + 32 * (wr + q * P) + lane;
-            const double x = i < a1 ? double(aval[i]) : 0.0;
-            xq[q] += x * x;
+            if (i < a1) {
+              const double x = double(aval[i]);
+              xq[q] = __fma_rn(x, x, xq[q]);
+            }
           }
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-          double a = rq[q], b = xq[q];
+        for (int h = NQ / 2; h > 0; h >>= 1)  // 128, 64, 32 apart: in this lane
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(FULL, a, o);
-            b += __shfl_xor_sync(FULL, b, o);
+          for (int q = 0; q < h; ++q) {
+            rq[q] += rq[q + h];
+            xq[q] += xq[q + h];
           }
+        double rs = rq[0], xs = xq[0];
+        bool any = dm != 0;
+        T vd = __shfl_sync(FULL, vdiag, dm ? __ffs(dm) - 1 : 0);
+        if constexpr (P > 1) {  // in those of the other warps
+          s_red[0][w][lane] = rs;
+          s_red[1][w][lane] = xs;
           if (lane == 0) {
-            s_red[0][g * WIDE_WARPS + wr + q * P] = a;
-            s_red[1][g * WIDE_WARPS + wr + q * P] = b;
+            s_diag[w] = any;
+            s_vdiag[w] = vd;
+          }
+          row_sync();
+          if (wr == 0) {
+            double a[P], b[P];
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+              a[i] = s_red[0][w + i][lane];
+              b[i] = s_red[1][w + i][lane];
+              if (s_diag[w + i]) {
+                any = true;
+                vd = s_vdiag[w + i];
+              }
+            }
+#pragma unroll
+            for (int h = P / 2; h > 0; h >>= 1)
+#pragma unroll
+              for (int i = 0; i < h; ++i) {
+                a[i] += a[i + h];
+                b[i] += b[i + h];
+              }
+            rs = a[0];
+            xs = b[0];
           }
         }
-        if (lane == 0) s_diag[w] = dm ? 1 : 0;
-        row_sync();
-        if (wr == 0 && lane == 0) {
-          double a = 0.0, b = 0.0;
-          int any = 0;
-          for (int i = 0; i < WIDE_WARPS; ++i) {
-            a += s_red[0][g * WIDE_WARPS + i];
-            b += s_red[1][g * WIDE_WARPS + i];
+        if (wr == 0) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            rs += __shfl_xor_sync(FULL, rs, o);
+            xs += __shfl_xor_sync(FULL, xs, o);
           }
-          for (int i = 0; i < P; ++i) any |= s_diag[w + i];
-          part[2 * int64_t(r)] = any ? a : a + 1.0;
-          part[2 * int64_t(r) + 1] = b;
+          if (lane == 0) {
+            part[2 * int64_t(r)] = rs + diag_square(any, vd);
+            part[2 * int64_t(r) + 1] = xs;
+          }
         }
       }
     }
