@@ -1063,9 +1063,13 @@ __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, co
 constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_K = 4;  // k whose first 32 entries are loaded ahead
 enum { WIDE_ROWS = 0, WIDE_NARROW = 1, WIDE_LONG = 2 };
+// CTAs per SM: FP64 as many as the accumulators leave room for; FP32 four, with 64
+// registers a thread (P = 2 and 4 spill up to 84 B). Five (48) spilled up to 300 B:
+// squares and updates of the 16^3 Laplacian's solve 2.19 and 3.51 ms, with four 1.87
+// and 3.21; of the 45^2 Laplacian's 1.77 and 2.52, with four 1.58 and 2.32.
 template <typename T, int KIND>
-constexpr int wide_occ() {  // CTAs per SM
-  return KIND == WIDE_LONG ? 2 : sizeof(T) == 8 ? 3 : 5;
+constexpr int wide_occ() {
+  return KIND == WIDE_LONG ? 2 : sizeof(T) == 8 ? 3 : 4;
 }
 template <typename T, int MODE>
 constexpr size_t wide_smem() {
