@@ -303,7 +303,9 @@ sign_status sign_dense_product(int M, int N, int K, const float *A, int lda, con
  * error of an entry stays below about 2^-41 (K/4096) 2^(e_i + f_j), with
  * 2^e_i, 2^f_j bounding row i of A and column j of B (an FP64 dot product's
  * bound); K is taken in blocks of 4096, each summed exactly, the blocks
- * added in FP64. Needs N and ldc even and C 16-byte aligned, else
+ * added in FP64. A call takes device workspace for the digits, 16 (M + N)
+ * bytes per column of A (K rounded up to 8), and up to 240 MB for integer
+ * sums (0.5 MB per tile of 128 x 256 in flight). Needs N and ldc even and C 16-byte aligned, else
  * SIGN_EINVAL; SIGN_ETIMEOUT if a bounded wait on the tensor cores gave up.
  * Returns after cuda_stream has finished. */
 sign_status sign_dense_product_f64(int M, int N, int K, const double *A, int lda, const double *B,
@@ -341,7 +343,9 @@ sign_status sign_dense_product_f64(int M, int N, int K, const double *A, int lda
  * products' upper-bound slots counted twice); 80 bytes per n^2 entry the
  * dense path's FP64 blocks and digit planes, taken when the fill is
  * predicted to reach a quarter of the row; 24 bytes per input entry the
- * input and its scaled copy. */
+ * input and its scaled copy. The model does not count what a lane keeps
+ * whatever its requests are: workspaces of bytes per row and, once a request
+ * took the FP64 dense path, up to 240 MB of integer sums. */
 typedef struct sign_server_s *sign_server_t;
 
 typedef struct {

@@ -43,12 +43,13 @@
 // planes, 16 KB per pair and slice here against 24 KB when every pair loads
 // its own two planes, and the FP64 pipe (16 cycles per warp instruction) when
 // every pair is added into C in FP64, as an earlier form did: 6.07 ms at
-// 4096^3 and 3.69 ms at 2744^3 (GB300), now 3.70 and 1.98 ms (1.34 PFLOP/s on
+// 4096^3 and 3.69 ms at 2744^3 (GB300), now 3.47 and 1.91 ms (1.43 PFLOP/s on
 // the tensor pipe at 4096^3).
 // Tiles of a last, partial wave are cut into S parts of about equal pairs, each
 // a work unit of its own that leaves its integers in scratch; k_slices_finish
 // adds them up (exactly, in any order) and writes C. 2744^3 has 242 tiles: two
-// waves of 152 become 1 2/3 (2.31 -> 1.98 ms), 1024^3 has 32: 0.29 -> 0.088 ms.
+// waves of 152 become 1 2/3 (2.31 -> 1.98 ms when it came), 1024^3 has 32: 0.29 ->
+// 0.087 ms.
 // Every wait has a clock budget, as in the split-TF32 kernel.
 #include <stdint.h>
 

@@ -7,8 +7,9 @@
 // subtraction per entry), the forward substitution L y = P e for each column
 // e of the identity and the back substitution U x = y, both with their sums
 // in ascending index order. Every operation is an explicitly rounded FP64
-// operation and every entry takes its operations in that order, so the inverse
-// is the same on every run and for every blocking.
+// operation and every entry takes its operations in that order (but for those
+// with a zero that k_lu_trail leaves out), so the inverse is the same on every run
+// and for every blocking.
 //
 // The forward substitution rides along with the elimination: the identity's
 // rows are swapped and reduced like those of the matrix, [A | I] -> [U | y].
@@ -179,7 +180,9 @@ __global__ void __launch_bounds__(PANEL_T)
 // panel, then of inv. W: the panel's width. Bound by the FP64 pipe. A strip whose
 // part of U is all +0 (columns of the identity whose row has not been a pivot
 // yet: half of them on average) is left as it is after the swaps: a - l 0 = a
-// for every finite l. Strips of 8 columns took 21 us per launch for n = 500, as
+// for every finite l, but that -0 - l 0 is +0 for l < 0. So U may keep a zero of the
+// other sign, which the inverse does not show: y never holds -0 (it starts from the
+// identity), and s - (+-0) x = s for every other s. Strips of 8 columns took 21 us per launch for n = 500, as
 // one CTA per SM bounded them; the whole solve went from 57.2 to 54.8 ms.
 template <int W>
 __global__ void __launch_bounds__(TRAIL_T)

@@ -254,15 +254,16 @@ __device__ __forceinline__ unsigned long long q_bucket(typename KeyT<T>::K key, 
 // Clears the matrix's minimum and candidate count, and sets its candidate region.
 __device__ __forceinline__ void prepare_matrix(int m, const SelRows &R, unsigned long long entries,
                                                MatScalars *ms, const SelScratch &sc) {
+  const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
+  const int64_t nnz = R.rs ? int64_t(entries) : ms[m].nnz_bar;
   sc.minabove[m] = ~0ULL;
   sc.ncand[m] = 0ULL;
   if (m == 0) *sc.overflow = *sc.redo = 0ULL;
-  if (R.rs) ms[m].nnz_bar = int64_t(entries);
+  if (R.rs) ms[m].nnz_bar = nnz;
   // the candidate region: the matrix's range of slots, shifted right by cshift
   // when the room is a fraction of the slots, so the regions are disjoint
   sc.cbase[m] = R.rs ? (unsigned long long)(R.rs[R.moff[m]] >> R.cshift) : 0ULL;
-  sc.croom[m] = (unsigned long long)(ms[m].nnz_bar >> R.cshift);
-  const unsigned long long bkey = (unsigned long long)__double_as_longlong(ms[m].b);
+  sc.croom[m] = (unsigned long long)(nnz >> R.cshift);
   const int e = int(bkey >> 52);
   if (bkey == 0ULL || e >= 0x7FF) {  // b <= 0 (sign bit) is caught here as well
     ms[m].sel_e = 0;
@@ -275,8 +276,8 @@ __device__ __forceinline__ void prepare_matrix(int m, const SelRows &R, unsigned
   ms[m].sel_e = eb;
   ms[m].sel_q = qval<double>(bkey, eb);
   ms[m].tiny = eb > 32 ? (unsigned long long)(eb - 31) << 52 : 0ULL;
-  const int64_t N = ms[m].nnz_bar > 1 ? ms[m].nnz_bar : 1;
-  const double pivot = ms[m].b / sqrt(double(N)) * 0.999;
+  const int64_t N = nnz > 1 ? nnz : 1;
+  const double pivot = __longlong_as_double((long long)bkey) / sqrt(double(N)) * 0.999;
   const int base = int((unsigned long long)__double_as_longlong(pivot) >> 48);
   ms[m].sel_base = pivot < 0x1p-1000 && base > 0 ? base - 1 : base;  // rounding near underflow
 }
@@ -831,9 +832,13 @@ struct DgShared {
   int s_nkeep;
 };
 
-// Matrix m, which has a crossing, by nc CTAs (1 or the cluster's DG_C).
+// Matrix m, which has a crossing, by nc CTAs (1 or the cluster's DG_C). prefix, lo,
+// hi: the key bits known so far and the sum below them; cb: the first of its `total`
+// candidates.
 template <int LEVELS>
-__device__ __forceinline__ void digits_matrix(int m, int nc, int rank, unsigned long long total,
+__device__ __forceinline__ void digits_matrix(int m, int nc, int rank, unsigned long long prefix,
+                                              unsigned long long lo, unsigned long long hi,
+                                              unsigned long long cb, unsigned long long total,
                                               DgShared &sh, const SelScratch &sc, MatScalars *ms,
                                               int64_t *cnt) {
   auto &h = sh.h;
@@ -843,11 +848,8 @@ __device__ __forceinline__ void digits_matrix(int m, int nc, int rank, unsigned 
   int &s_nkeep = sh.s_nkeep;
   cg::cluster_group cl = cg::this_cluster();
   const int tid = threadIdx.x;
-  const SelState st = sc.st[m];
-  const unsigned long long cb = sc.cbase[m];
   const int eb = ms[m].sel_e;
   const unsigned long long Q = ms[m].sel_q;
-  unsigned long long prefix = st.prefix, lo = st.below_lo, hi = st.below_hi;
   if (total <= DG_T) {  // one CTA alone: thread i sums the squares of the keys <= key i
     const int n = int(total);
     const unsigned long long key = tid < n ? sc.cand[cb + tid] : ~0ULL;
@@ -957,31 +959,37 @@ __device__ __forceinline__ void digits_matrix(int m, int nc, int rank, unsigned 
   if (nc > 1) cl.sync();  // CTA 0's shared memory is read until here
 }
 
-template <int LEVELS>
+// MANY: RED_C matrices per cluster (see seg.cuh), else one.
+template <int LEVELS, bool MANY>
 __global__ void __cluster_dims__(DG_C, 1, 1) __launch_bounds__(DG_T, 3)
-    k_sel_digits(int nb, int per, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
+    k_sel_digits(int nb, const int *active, SelScratch sc, MatScalars *ms, int64_t *cnt) {
   after_previous();
   __shared__ DgShared sh;
-  const int rank = int(cg::this_cluster().block_rank()), g0 = blockIdx.x / DG_C * per;
-  // i = -1: this CTA's own matrix, alone; then those of the whole cluster, the same m
-  // for all its CTAs
-  for (int i = rank < per ? -1 : 0; i < per; ++i) {
-    const int m = i < 0 ? g0 + rank : g0 + i;
-    if (m >= nb || !active[m]) continue;
-    if (!sc.st[m].found) {
-      if (i < 0 && threadIdx.x == 0) {
+  const int rank = int(cg::this_cluster().block_rank()), cluster = blockIdx.x / DG_C;
+  constexpr int PER = MANY ? RED_C : 1;
+  // i = -1: this CTA's own matrix, if one CTA does; then those of the whole cluster, the
+  // same m for all its CTAs. A lone matrix (i = 0) is either.
+  for (int i = MANY ? -1 : 0; i < PER; ++i) {
+    const int m = cluster * PER + (i < 0 ? rank : i);
+    if (m >= nb) continue;
+    // loaded together, before any of them is looked at
+    const int act = active[m];
+    const SelState st = sc.st[m];
+    const unsigned long long total = min(sc.ncand[m], sc.croom[m]), cb = sc.cbase[m];
+    if (!act) continue;
+    const bool solo = total <= DG_ONE, mine = MANY ? i < 0 : rank == 0;
+    if (!st.found) {
+      if (mine && threadIdx.x == 0) {
         const unsigned long long k = sc.minabove[m];
         ms[m].tau = k == ~0ULL ? __longlong_as_double(0x7ff0000000000000LL)
                                : __longlong_as_double((long long)k);
       }
-      if (per == 1) break;
       continue;
     }
-    const unsigned long long total = min(sc.ncand[m], sc.croom[m]);
-    if ((total <= DG_ONE) != (i < 0)) continue;
-    __syncthreads();  // sh is free
-    digits_matrix<LEVELS>(m, i < 0 ? 1 : DG_C, i < 0 ? 0 : rank, total, sh, sc, ms, cnt);
-    if (per == 1) break;
+    if (solo ? !mine : i < 0) continue;
+    if (MANY && i >= 0) __syncthreads();  // sh is free
+    digits_matrix<LEVELS>(m, solo ? 1 : DG_C, solo ? 0 : rank, st.prefix, st.below_lo, st.below_hi,
+                          cb, total, sh, sc, ms, cnt);
   }
 }
 
@@ -1179,8 +1187,11 @@ static void select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_c
     }
   }
   ProfScope ps(KC_SEL_DIGITS, s, 0.0, 0.0);
-  launch_next(k_sel_digits<sizeof(T) == 4 ? 3 : 6>, cluster_ctas(nb), DG_T, 0, s, nb,
-              cluster_matrices(nb), active, sc, ms, cnt);
+  constexpr int LEVELS = sizeof(T) == 4 ? 3 : 6;
+  if (cluster_matrices(nb) > 1)
+    launch_next(k_sel_digits<LEVELS, true>, cluster_ctas(nb), DG_T, 0, s, nb, active, sc, ms, cnt);
+  else
+    launch_next(k_sel_digits<LEVELS, false>, cluster_ctas(nb), DG_T, 0, s, nb, active, sc, ms, cnt);
 }
 
 void launch_select_exact(int nb, const SelRows &R, int64_t nvals, int64_t cand_cap,

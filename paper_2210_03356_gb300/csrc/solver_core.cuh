@@ -364,7 +364,13 @@ struct Solver {
   Stage<float> s32;          // FP32 stage of the mixed mode
   Stage<double> s64;
   Staging stg;
+  unsigned sched = schedule_flag();  // how this solver's waits poll (see fetch)
 
+  static unsigned schedule_flag() {
+    unsigned f = 0;
+    SGN_CUDA(cudaGetDeviceFlags(&f));
+    return f & cudaDeviceScheduleMask;
+  }
   ~Solver() {
     if (stg.used) cudaStreamSynchronize(s);  // copies from the arena may be in flight
   }
@@ -384,9 +390,6 @@ struct Solver {
   // should write, get a copy and a synchronize. The stream is queried from time to
   // time, so that an error ends the wait.
   void fetch(void *dst, const void *src, size_t bytes) {
-    unsigned sched = 0;
-    SGN_CUDA(cudaGetDeviceFlags(&sched));
-    sched &= cudaDeviceScheduleMask;
     if (bytes > PUBLISH_MAX || sched == cudaDeviceScheduleBlockingSync) {
       SGN_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
       wait();
