@@ -1234,9 +1234,9 @@ struct Solver {
     return live > 0;
   }
 
-  // Above 2^28 values the candidate room is a sixteenth of them (at least
-  // 2^28); filter_rows selects again with full room if the crossing bucket
-  // held more.
+  // Above 2^28 values the candidate room, shared by all matrices, is a sixteenth of
+  // them (at least 2^28); filter_rows selects again with full room if the crossing
+  // buckets held more.
   template <typename T>
   void select_threshold(Stage<T> &st, Slotted<T> &in, const int *d_act, bool full_room = false) {
     int64_t N = st.moff.back();
