@@ -366,10 +366,13 @@ struct Solver {
   Staging stg;
   unsigned sched = schedule_flag();  // how this solver's waits poll (see fetch)
 
-  static unsigned schedule_flag() {
+  // Never throws (a server's worker makes its solvers outside any handler): where the
+  // flag cannot be read, the waits poll as by default.
+  static unsigned schedule_flag() noexcept {
     unsigned f = 0;
-    SGN_CUDA(cudaGetDeviceFlags(&f));
-    return f & cudaDeviceScheduleMask;
+    if (cudaGetDeviceFlags(&f) == cudaSuccess) return f & cudaDeviceScheduleMask;
+    cudaGetLastError();
+    return cudaDeviceScheduleAuto;
   }
   ~Solver() {
     if (stg.used) cudaStreamSynchronize(s);  // copies from the arena may be in flight
