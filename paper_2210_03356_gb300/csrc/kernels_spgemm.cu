@@ -1059,7 +1059,7 @@ __global__ void k_col_blocks(int64_t n, const int64_t *rs, const int64_t *re, co
 // the k by the first and last columns of their B rows, 128 at a time, before it locates
 // any: such a row has many windows and most k fall into few of them. With one warp that located every k in every window the FP64 products of a
 // solve of a tridiagonal matrix of order 65536 with one full row took 3.5 s (1.1 s
-// with one CTA per row before that), now 0.086.
+// with one CTA per row before that), now 0.088.
 constexpr int WIDE_WARPS = 8;
 constexpr int WIDE_K = 4;  // k whose first 32 entries are loaded ahead
 enum { WIDE_ROWS = 0, WIDE_NARROW = 1, WIDE_LONG = 2 };
@@ -1607,7 +1607,11 @@ void launch_numeric_wide(int64_t n, int cls, int rows, double mean_b, const Rows
   // warps per row: about 64 (FP32) or 128 (FP64) entries of a B row per warp, a
   // pass for each where rows are few
   const double per = cls != RC_CTA ? 32.0 : sizeof(T) == 8 ? 128.0 : 64.0;
-  const int p = mean_b >= 8 * per ? 8 : mean_b >= 4 * per ? 4 : mean_b >= 2 * per ? 2 : 1;
+  int p = mean_b >= 8 * per ? 8 : mean_b >= 4 * per ? 4 : mean_b >= 2 * per ? 2 : 1;
+  // and all eight where the rows leave warps idle: beside one full row, the rows that
+  // have it among their k are as wide, and the mean says nothing of them (the solve of
+  // a tridiagonal matrix of order 65536 with one full row: 216 ms without, 171 with)
+  while (p < 8 && int64_t(rows) * p < int64_t(sm_count()) * 16) p *= 2;
   const int32_t *list = lists + int64_t(cls) * n;
   if (mode == MODE_SQUARE)
     wide_launch_p<T, MODE_SQUARE>(rows, p, A, aval, B, bval, wt, lo, len, list, counters, cls, cs,
